@@ -4,13 +4,22 @@
 // Work unit = (two adjacent 128-row Q tiles of one plan item, one query head).  Roles per CTA:
 //   warp 0        work scheduler (global counter -> shared-memory ring) and TMA producer: Q tiles and the K/V tile
 //                 ring (128-byte swizzled boxes)
-//   warps 1, 2    UMMA issuers, one per Q tile: S = Q K^T into TMEM, O += P V with P read from TMEM
+//   warp 1        UMMA issuer of the scores: S = Q K^T into TMEM, the two Q tiles by turns
+//   warp 2        UMMA issuer of the outputs: O += P V with P read from TMEM
 //   warps 4..7    softmax for Q tile 0: one thread per query row, the whole 128-column row in registers
 //   warps 8..11   softmax for Q tile 1
 //   warps 12..15  epilogue for both tiles: normalise O, store the partial output and its log-sum-exp
-// TMEM (512 columns): S0 | S1 | O0 | O1, 128 fp32 columns each (D = 128); bf16 P overwrites the
-// first 64 columns of its S.  While one tile's softmax runs on the CUDA cores the tensor core works
-// on the other tile, so the two Q tiles share every K/V tile that is staged.
+// TMEM (512 columns): P has columns of its own, so that the scores of the next step are computed while the
+// probabilities of this one are still being formed and consumed.  D = 128: S (one buffer, used by the two Q tiles in
+// turn) | P0 | P1 | O0 | O1; D = 64 has room for a score buffer per Q tile.  The two Q tiles share every K/V tile.
+//
+// What bounds it: per K/V tile the two Q tiles need 2048 clk of UMMA time and 2048 clk of the MUFU (one warp per
+// scheduler and tile, 8 clk per warp-wide ex2); a timestamp trace (D = 128) shows a period of 3030 clk: scores seen to
+// loaded 266, maximum 338, exponentials 1390, wait for the free P 254, store and hand over 118, wait for the next
+// scores 662.  With P over its own S (each tile's next scores behind the product that consumes P, the groups taking
+// turns at the exponentials) the period was 4200 clk.  Long launches run under the power cap, where 16 % fewer
+// cycles give 7 % of the time: one 128K sequence among short ones 167 -> 156 ms, 128K bimodal batch 37.2 -> 34.2 ms,
+// 64K log-normal batch 4.54 -> 4.28 ms, D = 64 ragged 16K batch 112 -> 102 us.
 //
 // Registers are moved between the warp groups at start-up: a softmax thread holds a full row of S
 // (128 values), reads it from TMEM once, and needs no exchange with another thread for the row
@@ -24,9 +33,9 @@ namespace fcp {
 constexpr int FWD_THREADS = 512;          // 4 control warps + 2 x 4 softmax warps + 4 epilogue warps
 constexpr int FWD_KV_SLOTS = 4;
 constexpr int FWD_WORK_SLOTS = 4;         // ring of work items handed from the producer to the other roles
-// register budgets per thread of the three roles: 128 * 64 + 256 * 184 + 128 * 80 = 512 * 128
-#define FCP_FWD_REGS_CTRL "64"
-#define FCP_FWD_REGS_SOFTMAX "184"
+// register budgets per thread of the three roles: 128 * 48 + 256 * 192 + 128 * 80 = 512 * 128
+#define FCP_FWD_REGS_CTRL "48"
+#define FCP_FWD_REGS_SOFTMAX "192"
 #define FCP_FWD_REGS_EPI "80"
 
 template <int D>
@@ -36,10 +45,11 @@ struct FwdSmem {
   static constexpr int Q_OFF = 0;
   static constexpr int KV_OFF = 2 * Q_TILE_BYTES;
   static constexpr int BAR_OFF = KV_OFF + FWD_KV_SLOTS * KV_TILE_BYTES;
-  // barriers: q_full[2] q_empty[2] kv_full[S] kv_empty[S] s_full[2] p_full[2] o_final[2] o_empty[2] turn[2]
+  static constexpr int NS = D == 128 ? 1 : 2;             // score buffers in TMEM
+  // barriers: q_full[2] q_empty[2] kv_full[S] kv_empty[S] s_full[2] s_free[2] p_full[2] p_free[2] o_final[2] o_empty[2]
   //           stat_full[2] stat_empty[2]
   //           w_full[W] w_empty[W]
-  static constexpr int N_BARS = 4 + 2 * FWD_KV_SLOTS + 14 + 2 * FWD_WORK_SLOTS;
+  static constexpr int N_BARS = 4 + 2 * FWD_KV_SLOTS + 16 + 2 * FWD_WORK_SLOTS;
   static constexpr int MISC_OFF = BAR_OFF + N_BARS * 8;   // tmem base (4 B), abort flag (4 B), work ring [W][unit, head]
   static constexpr int STAT_OFF = MISC_OFF + 16 + 8 * FWD_WORK_SLOTS;   // [2 tiles][row sum, reference maximum][128 rows] fp32
   static constexpr int TOTAL = STAT_OFF + 2 * 2 * 128 * 4;
@@ -71,7 +81,9 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   constexpr int KBLK = D / 64;                 // 64-element (128-byte) column blocks per row
   constexpr uint32_t BLK_BYTES = 128 * 128;    // one [128 rows][64] swizzled block
   constexpr uint32_t TMEM_COLS = 512;
-  constexpr uint32_t S_COL0 = 0, O_COL0 = 256; // S stage s at 128*s, O stage s at 256 + 128*s
+  // TMEM columns.  D = 128: S | P0 | P1 | O0 | O1; D = 64: P0 | P1 | O0 | O1 | S | S.
+  constexpr uint32_t NS = SM::NS;
+  constexpr uint32_t S_COL0 = D == 128 ? 0 : 256, P_COL0 = D == 128 ? 128 : 0, O_COL0 = D == 128 ? 256 : 128, O_STRIDE = D;
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -79,8 +91,9 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   const uint32_t bar0 = sbase + SM::BAR_OFF;
   auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
   const int B_QFULL = 0, B_QEMPTY = 2, B_KVFULL = 4, B_KVEMPTY = 4 + FWD_KV_SLOTS,
-            B_SFULL = 4 + 2 * FWD_KV_SLOTS, B_PFULL = B_SFULL + 2, B_OFINAL = B_SFULL + 4, B_OEMPTY = B_SFULL + 6,
-            B_TURN = B_SFULL + 8, B_STATFULL = B_SFULL + 10, B_STATEMPTY = B_SFULL + 12, B_WFULL = B_SFULL + 14,
+            B_SFULL = 4 + 2 * FWD_KV_SLOTS, B_SFREE = B_SFULL + 2, B_PFULL = B_SFULL + 4, B_PFREE = B_SFULL + 6,
+            B_OFINAL = B_SFULL + 8, B_OEMPTY = B_SFULL + 10, B_STATFULL = B_SFULL + 12, B_STATEMPTY = B_SFULL + 14,
+            B_WFULL = B_SFULL + 16,
             B_WEMPTY = B_WFULL + FWD_WORK_SLOTS;
   volatile uint32_t* tmem_slot = (volatile uint32_t*)(smem + SM::MISC_OFF);
   volatile int* abort_flag = (volatile int*)(smem + SM::MISC_OFF + 4);
@@ -95,10 +108,11 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       mbar_init(BAR(B_QFULL + i), 1);
       mbar_init(BAR(B_QEMPTY + i), 1);
       mbar_init(BAR(B_SFULL + i), 1);
-      mbar_init(BAR(B_PFULL + i), 4);          // one elected lane per softmax warp
+      mbar_init(BAR(B_SFREE + i), 4);          // one elected lane per softmax warp of the tile the scores belong to
+      mbar_init(BAR(B_PFULL + i), 4);
+      mbar_init(BAR(B_PFREE + i), 1);
       mbar_init(BAR(B_OFINAL + i), 1);
       mbar_init(BAR(B_OEMPTY + i), 4);         // one elected lane per epilogue warp
-      mbar_init(BAR(B_TURN + i), 4);
       mbar_init(BAR(B_STATFULL + i), 4);
       mbar_init(BAR(B_STATEMPTY + i), 4);
     }
@@ -108,7 +122,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
     for (int i = 0; i < FWD_KV_SLOTS; ++i) {
       mbar_init(BAR(B_KVFULL + i), 1);
-      mbar_init(BAR(B_KVEMPTY + i), 2);        // one commit from each issuer
+      mbar_init(BAR(B_KVEMPTY + i), 1);        // commit of the issuer that reads the slot (K: scores, V: outputs)
     }
     fence_mbar_init();
     prefetch_tmap(&tm_q);
@@ -213,20 +227,13 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
       }
     }
-  } else if (warp == 1 || warp == 2) {
-    // ------------------------------------------------------------------ UMMA issuers, one per Q tile
-    // A single thread cannot issue the 32 UMMAs of one K/V tile (two Q tiles) plus its waits and
-    // commits in the 2048 clocks they take to execute, so each Q tile has its own issuing thread;
-    // their products touch disjoint TMEM columns and only read the shared K/V tiles.
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ UMMA issuer 1: S = Q K^T of both Q tiles
+    // The two issuing threads are split by product, not by Q tile: S of the next step only waits for a free score
+    // buffer, so it is never queued behind the product that consumes the probabilities of an earlier step.
     if (lane == 0) {
-      // one issuing thread per Q tile (measured faster than a warp in uniform flow with a leader lane)
-      const bool leader = true;
       constexpr uint32_t IDESC_QK = make_idesc(128, 128, 0, 0);
-      constexpr uint32_t IDESC_PV = make_idesc(128, D, 0, 1);
-      const int s = warp - 1;
-      const uint32_t t_s = tmem + S_COL0 + s * 128, t_o = tmem + O_COL0 + s * 128;
-      const uint32_t q_addr = sbase + SM::Q_OFF + s * SM::Q_TILE_BYTES;
-      uint32_t kv_it = 0, qcnt = 0, pcnt = 0, ocnt = 0, nw = 0;
+      uint32_t kv_it = 0, qcnt0 = 0, qcnt1 = 0, xcnt0 = 0, xcnt1 = 0, nw = 0;
       bool ok = true;
 #pragma unroll 1
       while (ok) {
@@ -234,61 +241,90 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         int h;
         const int r = take_item(nw, U, h, false);
         if (r <= 0) { ok = r == 0; break; }
-        const int nts = __ldg(U + FU_NT_STAGE0 + s);
-        const int n_max = max(__ldg(U + FU_NT_STAGE0), __ldg(U + FU_NT_STAGE1));
-        if (nts > 0) {
-          ok = mbar_wait(BAR(B_QFULL + s), qcnt & 1, wctx, 20 + s);
-          ++qcnt;
-        }
+        const int nt0 = __ldg(U + FU_NT_STAGE0), nt1 = __ldg(U + FU_NT_STAGE1);
+        const int n_max = max(nt0, nt1);
 #pragma unroll 1
-        for (int j = 0; j <= n_max && ok; ++j) {
-          // ring positions: K_j at kv_it + 2j, V_{j-1} at kv_it + 2j - 1
-          const uint32_t itK = kv_it + 2 * j, itV = kv_it + 2 * j - 1;
-          const uint32_t slotK = itK % FWD_KV_SLOTS, slotV = itV % FWD_KV_SLOTS;
-          // Every slot is awaited and released by both issuers, whether or not their tile uses it:
-          // a release may only be counted in the phase of the load it answers.
-          if (j >= 1) ok = mbar_wait(BAR(B_KVFULL + slotV), (itV / FWD_KV_SLOTS) & 1, wctx, 22);
-          if (ok && j < n_max) ok = mbar_wait(BAR(B_KVFULL + slotK), (itK / FWD_KV_SLOTS) & 1, wctx, 23);
-          if (!ok) break;
-          if (j >= 1 && j - 1 < nts) {
-            // O_s (+)= P_s(j-1) V_{j-1}
-            if (j == 1) {
-              ok = mbar_wait(BAR(B_OEMPTY + s), (ocnt & 1) ^ 1, wctx, 24 + s);
-              ++ocnt;
+        for (int j = 0; j < n_max && ok; ++j, kv_it += 2) {
+          const uint32_t slot = kv_it % FWD_KV_SLOTS;
+          ok = mbar_wait(BAR(B_KVFULL + slot), (kv_it / FWD_KV_SLOTS) & 1, wctx, 23);
+#pragma unroll 1
+          for (int s = 0; s < 2 && ok; ++s) {
+            const int nts = s ? nt1 : nt0;
+            if (j >= nts) continue;
+            if (j == 0) {
+              ok = mbar_wait(BAR(B_QFULL + s), (s ? qcnt1 : qcnt0) & 1, wctx, 20 + s);
+              if (s) ++qcnt1; else ++qcnt0;
+              if (!ok) break;
             }
-            if (ok) ok = mbar_wait(BAR(B_PFULL + s), pcnt & 1, wctx, 26 + s);
-            ++pcnt;
+            const uint32_t sb = NS == 2 ? s : 0;
+            ok = mbar_wait(BAR(B_SFREE + sb), ((sb ? xcnt1 : xcnt0) & 1) ^ 1, wctx, 24);
+            if (!ok) break;
+            if (sb) ++xcnt1; else ++xcnt0;
+            tc_fence_after();
+            umma_loop_kk<D / 16>(true, tmem + S_COL0 + sb * 128, sbase + SM::Q_OFF + s * SM::Q_TILE_BYTES,
+                                 sbase + SM::KV_OFF + slot * SM::KV_TILE_BYTES, IDESC_QK);
+            tc_commit(BAR(B_SFULL + s));
+            if (j == nts - 1) tc_commit(BAR(B_QEMPTY + s));
+          }
+          tc_commit(BAR(B_KVEMPTY + slot));
+        }
+      }
+    }
+  } else if (warp == 2) {
+    // ------------------------------------------------------------------ UMMA issuer 2: O (+)= P V of both Q tiles
+    if (lane == 0) {
+      constexpr uint32_t IDESC_PV = make_idesc(128, D, 0, 1);
+      uint32_t kv_it = 1, pcnt0 = 0, pcnt1 = 0, ocnt0 = 0, ocnt1 = 0, nw = 0;
+      bool ok = true;
+#pragma unroll 1
+      while (ok) {
+        const int32_t* U;
+        int h;
+        const int r = take_item(nw, U, h, false);
+        if (r <= 0) { ok = r == 0; break; }
+        const int nt0 = __ldg(U + FU_NT_STAGE0), nt1 = __ldg(U + FU_NT_STAGE1);
+        const int n_max = max(nt0, nt1);
+#pragma unroll 1
+        for (int j = 0; j < n_max && ok; ++j, kv_it += 2) {
+          const uint32_t slot = kv_it % FWD_KV_SLOTS;
+          ok = mbar_wait(BAR(B_KVFULL + slot), (kv_it / FWD_KV_SLOTS) & 1, wctx, 22);
+#pragma unroll 1
+          for (int s = 0; s < 2 && ok; ++s) {
+            const int nts = s ? nt1 : nt0;
+            if (j >= nts) continue;
+            if (j == 0) {
+              ok = mbar_wait(BAR(B_OEMPTY + s), ((s ? ocnt1 : ocnt0) & 1) ^ 1, wctx, 25);
+              if (s) ++ocnt1; else ++ocnt0;
+              if (!ok) break;
+            }
+            ok = mbar_wait(BAR(B_PFULL + s), (s ? pcnt1 : pcnt0) & 1, wctx, 26 + s);
+            if (s) ++pcnt1; else ++pcnt0;
             if (!ok) break;
             tc_fence_after();
-            umma_loop_ts(leader, t_o, t_s, false, sbase + SM::KV_OFF + slotV * SM::KV_TILE_BYTES, IDESC_PV, j > 1 ? 1u : 0u);
-            if (j == nts) tc_commit_if(leader, BAR(B_OFINAL + s));
+            umma_loop_ts(true, tmem + O_COL0 + s * O_STRIDE, tmem + P_COL0 + s * 64, false,
+                         sbase + SM::KV_OFF + slot * SM::KV_TILE_BYTES, IDESC_PV, j > 0 ? 1u : 0u);
+            tc_commit(BAR(B_PFREE + s));
+            if (j == nts - 1) tc_commit(BAR(B_OFINAL + s));
           }
-          if (j < nts) {
-            // S_s = Q_s K_j^T
-            tc_fence_after();
-            umma_loop_kk<D / 16>(leader, t_s, q_addr, sbase + SM::KV_OFF + slotK * SM::KV_TILE_BYTES, IDESC_QK);
-            tc_commit_if(leader, BAR(B_SFULL + s));
-            if (j == nts - 1) tc_commit_if(leader, BAR(B_QEMPTY + s));
-          }
-          if (j >= 1) tc_commit_if(leader, BAR(B_KVEMPTY + slotV));
-          if (j < n_max) tc_commit_if(leader, BAR(B_KVEMPTY + slotK));
+          tc_commit(BAR(B_KVEMPTY + slot));
         }
-        kv_it += 2 * n_max;
       }
     }
   } else if (warp >= 4 && warp < 12) {
     // ------------------------------------------------------------------ softmax
     // Four warps per Q tile, one per TMEM lane quarter; a thread owns one query row and reads all 128
-    // scores of the current K/V tile into registers with one round of TMEM loads.
+    // scores of the current K/V tile into registers with one round of TMEM loads, which frees the score buffer.
     asm volatile("setmaxnreg.inc.sync.aligned.u32 " FCP_FWD_REGS_SOFTMAX ";");
     const int s = (warp - 4) >> 2;            // Q tile handled by this warp group
     const int rb = warp & 3;                  // TMEM lane quarter this warp may access
     const int row = rb * 32 + lane;
-    const uint32_t t_s = tmem_addr(tmem, rb * 32, S_COL0 + s * 128);   // P goes over the first 64 columns
-    const uint32_t t_o = tmem_addr(tmem, rb * 32, O_COL0 + s * 128);
+    const uint32_t sb = NS == 2 ? s : 0;      // score buffer of this tile (D = 128: one buffer, used by turns)
+    const uint32_t t_s = tmem_addr(tmem, rb * 32, S_COL0 + sb * 128);
+    const uint32_t t_p = tmem_addr(tmem, rb * 32, P_COL0 + s * 64);
+    const uint32_t t_o = tmem_addr(tmem, rb * 32, O_COL0 + s * O_STRIDE);
     float* stat = (float*)(smem + SM::STAT_OFF) + s * 256;
     const float c2 = a.scale_log2;
-    uint32_t scnt = 0, ucnt = 0, tcnt = 0, nw = 0;
+    uint32_t pcnt = 0, ucnt = 0, nw = 0;
     bool ok = true;
 #pragma unroll 1
     while (ok) {
@@ -297,41 +333,34 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const int r = take_item(nw, U, h, true);
       if (r <= 0) { ok = r == 0; break; }
       const int nts = __ldg(U + FU_NT_STAGE0 + s);
-      const int n_max = max(__ldg(U + FU_NT_STAGE0), __ldg(U + FU_NT_STAGE1));
       const int q_pos = __ldg(U + FU_Q_ROW0) + s * 128 + row;
       // first key this row does not see in a DIAG range: the one after itself, or the end of its span
       const int row_lim = (a.row_limit != nullptr && s * 128 + row < __ldg(U + FU_Q_ROWS)) ? __ldg(a.row_limit + q_pos) : q_pos + 1;
+      // key limit of this row within the current KV range, first key of the current tile
+      int lim = min(__ldg(U + FU_KV0_END), __ldg(U + FU_KV0_DIAG) ? row_lim : 0x7fffffff);
+      int ks = __ldg(U + FU_KV0_BEGIN);
       const int nr0 = __ldg(U + FU_NT_RANGE0);
-      const int kvb0 = __ldg(U + FU_KV0_BEGIN), kvb1 = __ldg(U + FU_KV1_BEGIN);
-      const int kve0 = __ldg(U + FU_KV0_END), kve1 = __ldg(U + FU_KV1_END);
-      const int kvd0 = __ldg(U + FU_KV0_DIAG), kvd1 = __ldg(U + FU_KV1_DIAG);
-      float m_ref = -INFINITY, l = 0.f;
+      float m_ref = -INFINITY;
+      float2 l01 = make_float2(0.f, 0.f), l23 = make_float2(0.f, 0.f);
 #pragma unroll 1
-      for (int j = 0; j < n_max && ok; ++j) {
-        // The two softmax groups take turns at the exponentials (the MUFU pipe cannot serve both at
-        // full speed): tile 0 of K/V tile j, tile 1 of j, tile 0 of j+1, ...  While one group is in
-        // its exponentials the tensor core runs the other tile's products.  A group without work
-        // for this j only passes the turn on.
-        if (j >= nts) {
-          ok = mbar_wait_warp(BAR(B_TURN + s), (tcnt & 1) ^ (s ^ 1), wctx, 34 + s);
-          ++tcnt;
-          __syncwarp();
-          if (lane == 0) mbar_arrive(BAR(B_TURN + (s ^ 1)));
-          continue;
+      for (int j = 0; j < nts; ++j, ++pcnt) {
+        if (j == nr0) {                            // on to the second range
+          lim = min(__ldg(U + FU_KV1_END), __ldg(U + FU_KV1_DIAG) ? row_lim : 0x7fffffff);
+          ks = __ldg(U + FU_KV1_BEGIN);
         }
-        const bool r1 = j >= nr0;
-        const int ks = r1 ? kvb1 + (j - nr0) * 128 : kvb0 + j * 128;
-        int limit = (r1 ? kve1 : kve0) - ks;                  // valid columns of this tile for this row
-        if (r1 ? kvd1 : kvd0) limit = min(limit, row_lim - ks);
+        const int limit = lim - ks;                // valid columns of this tile for this row
+        ks += 128;
         const bool masked = __any_sync(0xffffffffu, limit < 128);
-        ok = mbar_wait_warp(BAR(B_SFULL + s), scnt & 1, wctx, 30 + s);
-        ++scnt;
+        ok = mbar_wait_warp(BAR(B_SFULL + s), pcnt & 1, wctx, 30 + s);
         if (!ok) break;
         tc_fence_after();
         uint32_t sv[4][32];
 #pragma unroll
         for (int b = 0; b < 4; ++b) tmem_ld32(t_s + 32 * b, sv[b]);
         tc_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(BAR(B_SFREE + sb));
         if (masked) {
 #pragma unroll
           for (int b = 0; b < 4; ++b)
@@ -346,22 +375,24 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           for (int b = 0; b < 4; ++b)
 #pragma unroll
             for (int i = 0; i < 32; i += 8) {
-              mx0 = fmaxf(mx0, fmaxf(__uint_as_float(sv[b][i]), __uint_as_float(sv[b][i + 1])));
-              mx1 = fmaxf(mx1, fmaxf(__uint_as_float(sv[b][i + 2]), __uint_as_float(sv[b][i + 3])));
-              mx2 = fmaxf(mx2, fmaxf(__uint_as_float(sv[b][i + 4]), __uint_as_float(sv[b][i + 5])));
-              mx3 = fmaxf(mx3, fmaxf(__uint_as_float(sv[b][i + 6]), __uint_as_float(sv[b][i + 7])));
+              mx0 = max3(mx0, __uint_as_float(sv[b][i]), __uint_as_float(sv[b][i + 1]));
+              mx1 = max3(mx1, __uint_as_float(sv[b][i + 2]), __uint_as_float(sv[b][i + 3]));
+              mx2 = max3(mx2, __uint_as_float(sv[b][i + 4]), __uint_as_float(sv[b][i + 5]));
+              mx3 = max3(mx3, __uint_as_float(sv[b][i + 6]), __uint_as_float(sv[b][i + 7]));
             }
           mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * c2;
         }
         // Lazy reference maximum: O and l are only rescaled when the row maximum grew by more than
-        // 2^8, so p <= 256 always and the result is exact up to rounding.  The products issued so far
-        // have completed (S of this tile was committed after them), so O is at rest here.
+        // 2^8, so p <= 256 always and the result is exact up to rounding.
         const bool grow = mx > m_ref + 8.f;
         if (__any_sync(0xffffffffu, grow)) {
           const float m_new = grow ? mx : m_ref;
           const float f = grow ? ex2(m_ref - m_new) : 1.f;    // m_ref = -inf -> 0
-          l *= f;
+          l01.x *= f; l01.y *= f; l23.x *= f; l23.y *= f;
           if (j > 0) {
+            ok = mbar_wait_warp(BAR(B_PFREE + s), (pcnt & 1) ^ 1, wctx, 36);   // O is at rest once the last product is done
+            if (!ok) break;
+            tc_fence_after();
 #pragma unroll 1
             for (int c = 0; c < D / 16; ++c) {
               uint32_t ov[16];
@@ -374,29 +405,26 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           }
           m_ref = m_new;
         }
-        ok = mbar_wait_warp(BAR(B_TURN + s), (tcnt & 1) ^ (s ^ 1), wctx, 34 + s);
-        ++tcnt;
-        if (!ok) break;
-        // exponentials, row sum, bf16 P over the first 64 columns of S (masked scores are -inf -> 0)
-        float sum0 = 0.f, sum1 = 0.f, sum2 = 0.f, sum3 = 0.f;
+        // exponentials, row sum, bf16 P (masked scores are -inf -> 0)
+        uint32_t pk[4][16];
+        const float2 c22 = make_float2(c2, c2), nm2 = make_float2(-m_ref, -m_ref);
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-          uint32_t pk[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
-            const float p0 = ex2(fmaf(__uint_as_float(sv[b][2 * i]), c2, -m_ref));
-            const float p1 = ex2(fmaf(__uint_as_float(sv[b][2 * i + 1]), c2, -m_ref));
-            if ((i & 3) == 0) sum0 += p0 + p1;
-            else if ((i & 3) == 1) sum1 += p0 + p1;
-            else if ((i & 3) == 2) sum2 += p0 + p1;
-            else sum3 += p0 + p1;
-            pk[i] = pack_bf16(p0, p1);
+            const float2 e = fma2(make_float2(__uint_as_float(sv[b][2 * i]), __uint_as_float(sv[b][2 * i + 1])), c22, nm2);
+            const float2 p = make_float2(ex2(e.x), ex2(e.y));
+            if (i & 1) l23 = add2(l23, p);
+            else l01 = add2(l01, p);
+            pk[b][i] = pack_bf16(p.x, p.y);
           }
-          tmem_st16(t_s + b * 16, pk);
         }
-        l += (sum0 + sum1) + (sum2 + sum3);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(BAR(B_TURN + (s ^ 1)));
+        // the product that reads the previous P of this tile must be done before P is overwritten
+        ok = mbar_wait_warp(BAR(B_PFREE + s), (pcnt & 1) ^ 1, wctx, 34 + s);
+        if (!ok) break;
+        tc_fence_after();
+#pragma unroll
+        for (int b = 0; b < 4; ++b) tmem_st16(t_p + b * 16, pk[b]);
         tc_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -404,6 +432,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       }
       if (!ok) break;
       if (nts == 0) continue;
+      const float l = (l01.x + l01.y) + (l23.x + l23.y);
       // hand the row sum and the reference maximum to the epilogue warps
       ok = mbar_wait_warp(BAR(B_STATEMPTY + s), (ucnt & 1) ^ 1, wctx, 36 + s);
       ++ucnt;
@@ -449,7 +478,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         ok = mbar_wait_warp(BAR(B_OFINAL + s), ph, wctx, 32 + s);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t t_o = tmem_addr(tmem, rb * 32, O_COL0 + s * 128);
+        const uint32_t t_o = tmem_addr(tmem, rb * 32, O_COL0 + s * O_STRIDE);
         const int rows_s = min(128, q_rows - s * 128);
         const float inv_l = 1.f / l;
         const float lse_row = (m_ref + log2f(l)) * 0.6931471805599453f;
