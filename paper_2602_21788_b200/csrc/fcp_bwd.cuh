@@ -12,7 +12,7 @@
 //                                      (UMMA, smem x smem)      over dP^T
 //   T4  dK  += dS^T Q                  (UMMA, smem x smem)      TMEM cols [384,512); issued after T5 so
 //                                      that it runs while the drain warps read the dQ tile
-//   C3  dQ accumulator += tile         fp32 reductions to global memory (coalesced for D = 128)
+//   C3  dQ accumulator += tile         fp32 reductions to global memory, whole sectors per warp
 //
 // 16 warps: warp 0 TMA producer and work scheduler, warp 1 UMMA issuer (warps 2-3 idle), warps 4..11
 // the element-wise math C1/C2 (two warps per TMEM lane quarter, each half of the query columns),
@@ -63,10 +63,10 @@ struct BwdArgs {
   int32_t* counter;         // work counter, zero before the launch
   int64_t T, t_stride;
   float scale, scale_log2;
-  const float* delta_t;     // [hq_acc][t_stride], already multiplied by the softmax scale
-  const float* lse2_t;      // [hq_acc][t_stride], log2 units
+  const float* delta_t;     // [hq_acc][t_stride], minus delta, already multiplied by the softmax scale
+  const float* lse2_t;      // [hq_acc][t_stride], minus the log-sum-exp, log2 units
   const int32_t* first_query;   // [T] or nullptr (causal): first query (packed index) that sees key t
-  float* dq_acc;            // [T][hq_acc][D] fp32, zero-initialised
+  float* dq_acc;            // fp32, zero-initialised: [T][hq_acc][D] (D = 128), blocked for D = 64 (see dq_block)
   __nv_bfloat16* dk;        // [T][hkv][D]
   __nv_bfloat16* dv;
   int32_t* status;
@@ -128,6 +128,35 @@ __device__ __forceinline__ void red_add_f32(float* p, float v) {
 }
 __device__ __forceinline__ void red_add_v4_f32(float* p, float a, float b, float c, float d) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+// dQ accumulator of D = 64: per query head, blocks of 128 packed token rows (the last one of T % 128 rows), within a block
+// [D / 4][rows][4].  The dQ tile has the query rows along the TMEM lanes (a transposed one would be an M = 64 product at
+// half the rate), so a drain warp holds 32 consecutive rows, one per lane, and each of its 16-byte reductions covers 512
+// contiguous bytes whatever row the tile starts at; with plain rows every lane would touch a line of its own.  Returns
+// the address of (head, row t, columns 0..3); `step` is the distance in bytes to the next four columns.
+// Ragged 16K batch, D = 64: kernel 308 -> 221 us (249 without the pauses between the reductions).
+// At D = 128 the same layout is slower (128K bimodal batch 102 -> 117 ms): there the rate of the reductions in the L2
+// bounds, and the transposed tile's 128-byte scalar ones run faster than four-wide ones.
+template <int D>
+__device__ __forceinline__ char* dq_block(float* acc, int64_t T, int h, int64_t t, uint32_t& step) {
+  const int64_t blk = t >> 7;
+  step = 16u * (uint32_t)(blk == (T >> 7) ? (T & 127) : 128);
+  return reinterpret_cast<char*>(acc) + ((int64_t)h * T + (blk << 7)) * (D * 4) + (t & 127) * 16;
+}
+
+// Two element-wise operations of a math warp, as one two-wide instruction (WIDE) or two scalar ones.  Both give the same
+// bits.  Two-wide is faster at D = 64 (kernel -4 %), where the tile's products are short and the math warps are what
+// the tile waits for; at D = 128 it is slower (64K log-normal batch 12.9 -> 13.6 ms).
+template <bool WIDE>
+__device__ __forceinline__ float2 fma_pair(uint32_t x, uint32_t y, float2 m, float2 add) {
+  const float2 v = make_float2(__uint_as_float(x), __uint_as_float(y));
+  return WIDE ? fma2(v, m, add) : make_float2(fmaf(v.x, m.x, add.x), fmaf(v.y, m.y, add.y));
+}
+template <bool WIDE>
+__device__ __forceinline__ float2 mul_pair(float2 a, uint32_t bf16x2) {
+  const float2 b = make_float2(__uint_as_float(bf16x2 << 16), __uint_as_float(bf16x2 & 0xffff0000u));
+  return WIDE ? mul2(a, b) : make_float2(a.x * b.x, a.y * b.y);
 }
 
 template <int D>
@@ -344,6 +373,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const int row = rb * 32 + lane;             // key row of S^T / dP^T
     const int mtid = threadIdx.x - 128;         // 0..255 among the math threads
     const uint32_t t_s = tmem_addr(tmem, rb * 32, C_S + half * 64), t_dp = tmem_addr(tmem, rb * 32, C_DP + half * 64);
+    const float2 c22 = make_float2(a.scale_log2, a.scale_log2), s22 = make_float2(a.scale, a.scale);
     uint8_t* ds_row = smem + SM::DS_OFF + half * BLK_BYTES + row * 128;
     // this thread's share of the per-query-row statistics: lse2 (threads 0..127) or delta (128..255)
     const float* my_rows = (mtid < 128 ? a.lse2_t : a.delta_t) + (mtid & 127);
@@ -409,12 +439,10 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const float4 l4 = *reinterpret_cast<const float4*>(lse_c + 4 * i);
-            const float p0 = ex2(fmaf(__uint_as_float(sv[4 * i]), a.scale_log2, -l4.x));
-            const float p1 = ex2(fmaf(__uint_as_float(sv[4 * i + 1]), a.scale_log2, -l4.y));
-            const float p2 = ex2(fmaf(__uint_as_float(sv[4 * i + 2]), a.scale_log2, -l4.z));
-            const float p3 = ex2(fmaf(__uint_as_float(sv[4 * i + 3]), a.scale_log2, -l4.w));
-            pb[2 * i] = pack_bf16(p0, p1);
-            pb[2 * i + 1] = pack_bf16(p2, p3);
+            const float2 e0 = fma_pair<D == 64>(sv[4 * i], sv[4 * i + 1], c22, make_float2(l4.x, l4.y));
+            const float2 e1 = fma_pair<D == 64>(sv[4 * i + 2], sv[4 * i + 3], c22, make_float2(l4.z, l4.w));
+            pb[2 * i] = pack_bf16(ex2(e0.x), ex2(e0.y));
+            pb[2 * i + 1] = pack_bf16(ex2(e1.x), ex2(e1.y));
           }
           if (need_mask) {
             const uint32_t k32 = (uint32_t)(keep >> (32 * c));
@@ -445,12 +473,11 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           for (int i = 0; i < 8; ++i) {
             const float4 d4 = *reinterpret_cast<const float4*>(delta_c + 4 * i);
             const uint32_t pp = pa[2 * i], pq = pa[2 * i + 1];
-            const float d0 = __uint_as_float(pp << 16) * fmaf(__uint_as_float(dv_[4 * i]), a.scale, -d4.x);
-            const float d1 = __uint_as_float(pp & 0xffff0000u) * fmaf(__uint_as_float(dv_[4 * i + 1]), a.scale, -d4.y);
-            const float d2 = __uint_as_float(pq << 16) * fmaf(__uint_as_float(dv_[4 * i + 2]), a.scale, -d4.z);
-            const float d3 = __uint_as_float(pq & 0xffff0000u) * fmaf(__uint_as_float(dv_[4 * i + 3]), a.scale, -d4.w);
-            out[2 * i] = pack_bf16(d0, d1);
-            out[2 * i + 1] = pack_bf16(d2, d3);
+            const float2 f0 = fma_pair<D == 64>(dv_[4 * i], dv_[4 * i + 1], s22, make_float2(d4.x, d4.y));
+            const float2 f1 = fma_pair<D == 64>(dv_[4 * i + 2], dv_[4 * i + 3], s22, make_float2(d4.z, d4.w));
+            const float2 d0 = mul_pair<D == 64>(f0, pp), d1 = mul_pair<D == 64>(f1, pq);
+            out[2 * i] = pack_bf16(d0.x, d0.y);
+            out[2 * i + 1] = pack_bf16(d1.x, d1.y);
           }
 #pragma unroll
           for (int j = 0; j < 16; ++j) pa[j] = pb[j];
@@ -547,22 +574,22 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             }
           }
         } else {
-          float* dst = a.dq_acc + (((int64_t)q_row + row) * a.hq_acc + h) * D;
-#pragma unroll 1
-          for (int c16 = 0; c16 < D / 16; ++c16) {
-            uint32_t qv[16];
-            tmem_ld16(t_dq + c16 * 16, qv);
-            tc_wait_ld();
-            if (c16 == D / 16 - 1) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(BAR(B_DQEMPTY));
-            }
-            if (row < q_valid) {
+          uint32_t qv[D];
 #pragma unroll
-              for (int c = 0; c < 16; c += 4)
-                red_add_v4_f32(dst + c16 * 16 + c, __uint_as_float(qv[c]), __uint_as_float(qv[c + 1]),
-                               __uint_as_float(qv[c + 2]), __uint_as_float(qv[c + 3]));
+          for (int c = 0; c < D / 32; ++c) tmem_ld32(t_dq + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&qv[c * 32]));
+          tc_wait_ld();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(BAR(B_DQEMPTY));
+          uint32_t step;
+          char* dst = dq_block<D>(a.dq_acc, a.T, h, (int64_t)q_row + row, step);
+          if (row < q_valid) {
+#pragma unroll
+            for (int c = 0; c < D / 4; ++c) {
+              red_add_v4_f32(reinterpret_cast<float*>(dst), __uint_as_float(qv[4 * c]), __uint_as_float(qv[4 * c + 1]),
+                             __uint_as_float(qv[4 * c + 2]), __uint_as_float(qv[4 * c + 3]));
+              dst += step;
+              if ((c & 3) == 3) __nanosleep(200);
             }
           }
         }

@@ -148,8 +148,8 @@ __global__ void __launch_bounds__(256) fcp_merge_kernel(const int32_t* __restric
 }
 
 // ---------------------------------------------------------------------------------------------
-// Backward preprocess (HBM bound): delta[h][t] = scale * sum_c dO[t,h,c] * O[t,h,c], and the forward LSE
-// transposed to [h][t] in log2 units, the layout the backward kernel's per-tile loads want.
+// Backward preprocess (HBM bound): delta[h][t] = -scale * sum_c dO[t,h,c] * O[t,h,c], and minus the forward
+// LSE transposed to [h][t] in log2 units, the layout the backward kernel's per-tile loads want.
 // ---------------------------------------------------------------------------------------------
 template <int D>
 __global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
@@ -178,8 +178,8 @@ __global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* __r
 #pragma unroll
   for (int off = TPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
   if (row < T * hc && sub == 0) {
-    delta_t[hl * t_stride + t] = acc * scale;
-    lse2_t[hl * t_stride + t] = lse[src] * 1.4426950408889634f;
+    delta_t[hl * t_stride + t] = -acc * scale;
+    lse2_t[hl * t_stride + t] = lse[src] * -1.4426950408889634f;
   }
 }
 
@@ -199,6 +199,34 @@ __global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* __rest
       j = t * dst_row8 + dst_off8 + (i - t * row8);
     }
     reinterpret_cast<uint4*>(dq)[j] = pk;
+  }
+}
+
+// The same from the blocked accumulator of D = 64 (dq_block): one CTA per (block of 128 rows, head) reads the block's
+// contiguous 128 * D floats with lanes along the rows and turns it round in shared memory, so that both sides move
+// whole sectors.
+__global__ void __launch_bounds__(256) fcp_dq_convert_blocked_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq,
+                                                                     int64_t T, int hq, int h0) {
+  constexpr int D = 64;
+  constexpr int PITCH = D + 8;                // bf16 elements per row in shared memory: 16 bytes of padding
+  __shared__ __align__(16) __nv_bfloat16 tile[128 * PITCH];
+  const int64_t t0 = (int64_t)blockIdx.x * 128;
+  const int rows = (int)min((int64_t)128, T - t0);
+  const float4* src = reinterpret_cast<const float4*>(acc + ((int64_t)blockIdx.y * T + t0) * D);
+  const int row = threadIdx.x & 127;
+  if (row < rows) {
+#pragma unroll
+    for (int c = threadIdx.x >> 7; c < D / 4; c += 2) {
+      const float4 v = __ldcs(src + c * rows + row);
+      *reinterpret_cast<uint2*>(tile + row * PITCH + c * 4) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+    }
+  }
+  __syncthreads();
+  constexpr int TPR = D / 8;                  // threads per row, 16 bytes each
+  __nv_bfloat16* dst = dq + ((t0 * hq) + h0 + blockIdx.y) * (int64_t)D;
+  for (int r = threadIdx.x / TPR; r < rows; r += 256 / TPR) {
+    const int c = (threadIdx.x % TPR) * 8;
+    *reinterpret_cast<uint4*>(dst + (int64_t)r * hq * D + c) = *reinterpret_cast<const uint4*>(tile + r * PITCH + c);
   }
 }
 
@@ -552,7 +580,10 @@ int run_bwd(const fcp_plan* plan, const BwdTables& tb, const void* q, const void
     const int64_t n8 = T * hc * D / 8;
     const int blocks = (int)std::min<int64_t>((n8 + 255) / 256, (int64_t)tb.sm_count * 16);
     ProfScope ps(prof, 4, st);
-    fcp_dq_convert_kernel<<<blocks, 256, 0, st>>>(dq_acc, (__nv_bfloat16*)dq, n8, hc * D / 8, P.hq * D / 8, h0 * D / 8);
+    if (D == 128)
+      fcp_dq_convert_kernel<<<blocks, 256, 0, st>>>(dq_acc, (__nv_bfloat16*)dq, n8, hc * D / 8, P.hq * D / 8, h0 * D / 8);
+    else
+      fcp_dq_convert_blocked_kernel<<<dim3((unsigned)((T + 127) / 128), (unsigned)hc), 256, 0, st>>>(dq_acc, (__nv_bfloat16*)dq, T, P.hq, h0);
     FCP_CUDA_CHECK(cudaGetLastError());
   }
   return FCP_OK;
