@@ -1,8 +1,10 @@
 // Device side of libfcp: launchers behind the C ABI, the HBM-bound kernels (LSE merge, backward
 // preprocess, dQ conversion) and the glue around the tensor-core kernels of fcp_fwd.cuh and
 // fcp_bwd.cuh.  No call here allocates device memory except fcp_plan_upload.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "fcp_bwd.cuh"
@@ -233,19 +235,158 @@ __global__ void __launch_bounds__(256) fcp_dq_convert_blocked_kernel(const float
 // ---------------------------------------------------------------------------------------------
 // Plan upload / destroy / status
 // ---------------------------------------------------------------------------------------------
+// Device blocks for the plans' tables.  Every new batch uploads a plan and drops the one before it, and cudaMalloc,
+// cudaFree (which waits for the whole device), the device query and the kernel attributes cost milliseconds each time:
+// a 16K-token batch took 6.8 ms for 2.8 ms of kernels.  So a destroyed plan's block goes to a short list per device and
+// is handed to the next plan once the event recorded after the last compute call that read it has completed; nothing
+// waits for it.  The list holds at most 8 blocks and 32 MB (the oldest leave first), larger blocks are never kept, and
+// fcp_release_cached gives all idle ones back.
+struct PlanBlock {
+  void* dev = nullptr;           // tables
+  void* host = nullptr;          // pinned staging of the same size: one copy per upload
+  size_t bytes = 0;
+  cudaEvent_t used = nullptr;    // after the last compute call that read the block
+};
+
+namespace {
+constexpr int kMaxDevices = 64;
+constexpr size_t kBlockMin = size_t(64) << 10, kBlockKeepMax = size_t(8) << 20, kKeepBytes = size_t(32) << 20;
+constexpr size_t kKeepBlocks = 8;
+
+struct DeviceState {
+  std::mutex mu;
+  bool ready = false;            // device checked, attributes set, stream created
+  int sm_count = 0;
+  cudaStream_t copy = nullptr;   // uploads: complete without waiting for the work queued on the caller's stream
+  std::vector<PlanBlock*> idle;  // oldest first
+  size_t idle_bytes = 0;
+};
+DeviceState g_device[kMaxDevices];
+
+void free_block(PlanBlock* b) {
+  if (b->dev) cudaFree(b->dev);
+  if (b->host) cudaFreeHost(b->host);
+  if (b->used) cudaEventDestroy(b->used);
+  delete b;
+}
+
+// Once per device: architecture check, shared-memory opt-in of the tensor-core kernels, the upload stream.
+int device_setup(int dev, DeviceState& ds) {
+  if (ds.ready) return FCP_OK;
+  int major = 0, sms = 0;
+  FCP_CUDA_CHECK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+  FCP_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  if (major != 10) {
+    fcp_set_error("device %d is not sm_100: this library is built for sm_100a only", dev);
+    return FCP_ERR_CUDA;
+  }
+  FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<64>::DYN_BYTES));
+  FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<128>::DYN_BYTES));
+  FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_bwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<64>::DYN_BYTES));
+  FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_bwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<128>::DYN_BYTES));
+  FCP_CUDA_CHECK(cudaStreamCreateWithFlags(&ds.copy, cudaStreamNonBlocking));
+  ds.sm_count = sms;
+  ds.ready = true;
+  return FCP_OK;
+}
+
+// A block of at least `bytes`: the smallest idle one that fits and that no queued work reads any more; with a full list
+// the oldest one that fits, whose event the caller then waits for (a new block would push out one in use, and freeing
+// that waits for the whole device); else a new one.
+int acquire_block(DeviceState& ds, size_t bytes, PlanBlock** out) {
+  size_t best = ds.idle.size();
+  for (size_t i = 0; i < ds.idle.size(); ++i) {
+    PlanBlock* b = ds.idle[i];
+    if (b->bytes >= bytes && (best == ds.idle.size() || b->bytes < ds.idle[best]->bytes) &&
+        cudaEventQuery(b->used) == cudaSuccess)
+      best = i;
+  }
+  cudaGetLastError();            // cudaErrorNotReady of a query is no error
+  if (best == ds.idle.size() && ds.idle.size() >= kKeepBlocks)
+    for (best = 0; best < ds.idle.size() && ds.idle[best]->bytes < bytes;) ++best;
+  if (best < ds.idle.size()) {
+    *out = ds.idle[best];
+    ds.idle_bytes -= (*out)->bytes;
+    ds.idle.erase(ds.idle.begin() + best);
+    return FCP_OK;
+  }
+  PlanBlock* b = new PlanBlock();
+  b->bytes = kBlockMin;
+  while (b->bytes < bytes && b->bytes < kBlockKeepMax) b->bytes *= 2;
+  b->bytes = std::max(b->bytes, bytes);
+  cudaError_t e = cudaMalloc(&b->dev, b->bytes);
+  if (e == cudaSuccess) e = cudaMallocHost(&b->host, b->bytes);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->used, cudaEventDisableTiming);
+  if (e != cudaSuccess) {
+    free_block(b);
+    fcp_set_error("plan upload failed: %s", cudaGetErrorString(e));
+    return FCP_ERR_CUDA;
+  }
+  *out = b;
+  return FCP_OK;
+}
+
+// `keep`: the event of the block covers all work that may still read it.  Otherwise (and for large blocks) the memory
+// is freed, which waits for the device.
+void return_block(int dev, PlanBlock* b, bool keep) {
+  if (!keep || b->bytes > kBlockKeepMax || dev < 0 || dev >= kMaxDevices) {
+    free_block(b);
+    return;
+  }
+  DeviceState& ds = g_device[dev];
+  std::vector<PlanBlock*> out;
+  {
+    std::lock_guard<std::mutex> lock(ds.mu);
+    ds.idle.push_back(b);
+    ds.idle_bytes += b->bytes;
+    while (ds.idle.size() > kKeepBlocks || ds.idle_bytes > kKeepBytes) {
+      out.push_back(ds.idle.front());
+      ds.idle_bytes -= ds.idle.front()->bytes;
+      ds.idle.erase(ds.idle.begin());
+    }
+  }
+  for (PlanBlock* x : out) free_block(x);
+}
+
+// At the end of every compute call: the block is in use until the work queued so far on `st` is done (calls on one
+// plan are stream-ordered, so the last event covers the earlier calls).  Work recorded into a graph can run at any later
+// time: such a plan's block is never handed on.
+void mark_used(const fcp_plan* plan, cudaStream_t st) {
+  if (!plan->block) return;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
+      cudaEventRecord(plan->block->used, st) != cudaSuccess) {
+    plan->block_pinned = true;
+    cudaGetLastError();
+  }
+}
+}  // namespace
+
+extern "C" int fcp_release_cached(void) {
+  int dev = 0;
+  FCP_CUDA_CHECK(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= kMaxDevices) return FCP_OK;
+  std::vector<PlanBlock*> out;
+  {
+    std::lock_guard<std::mutex> lock(g_device[dev].mu);
+    out.swap(g_device[dev].idle);
+    g_device[dev].idle_bytes = 0;
+  }
+  for (PlanBlock* b : out) free_block(b);
+  return FCP_OK;
+}
+
 extern "C" int fcp_plan_upload(fcp_plan* plan, void* stream) {
+  (void)stream;                  // the call is complete when it returns, whatever is queued there
   if (!plan) return FCP_ERR_INVALID_ARG;
   if (plan->d_blob) return FCP_OK;
   int dev = 0;
   FCP_CUDA_CHECK(cudaGetDevice(&dev));
-  cudaDeviceProp prop;
-  FCP_CUDA_CHECK(cudaGetDeviceProperties(&prop, dev));
-  if (prop.major != 10) {
-    fcp_set_error("device %d is sm_%d%d; this library is built for sm_100a only", dev, prop.major, prop.minor);
-    return FCP_ERR_CUDA;
+  if (dev < 0 || dev >= kMaxDevices) {
+    fcp_set_error("device index %d not supported", dev);
+    return FCP_ERR_UNSUPPORTED;
   }
-  plan->device = dev;
-  plan->sm_count = prop.multiProcessorCount;
+  DeviceState& ds = g_device[dev];
   constexpr int NT = 10;
   const std::vector<int32_t>* tabs[NT] = {&plan->fwd_units, &plan->bwd_units, &plan->bwd_qranges, &plan->merge_units,
                                           &plan->slot_offset, &plan->slot_rows, &plan->bwd_work, &plan->fused_units,
@@ -257,19 +398,36 @@ extern "C" int fcp_plan_upload(fcp_plan* plan, void* stream) {
     total += (tabs[i]->size() * 4 + 255) / 256 * 256;
   }
   off[NT] = total;
-  void* blob = nullptr;
-  FCP_CUDA_CHECK(cudaMalloc(&blob, total));
-  cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = cudaMemsetAsync(blob, 0, 256, st);
-  for (int i = 0; i < NT && e == cudaSuccess; ++i)
-    if (!tabs[i]->empty())
-      e = cudaMemcpyAsync((char*)blob + off[i], tabs[i]->data(), tabs[i]->size() * 4, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) {
-    cudaFree(blob);
+  PlanBlock* block = nullptr;
+  cudaStream_t copy = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(ds.mu);
+    int rc = device_setup(dev, ds);
+    if (rc == FCP_OK) rc = acquire_block(ds, total, &block);
+    if (rc != FCP_OK) return rc;
+    plan->sm_count = ds.sm_count;
+    copy = ds.copy;
+  }
+  if (cudaError_t e = cudaEventSynchronize(block->used); e != cudaSuccess) {
+    free_block(block);
     fcp_set_error("plan upload failed: %s", cudaGetErrorString(e));
     return FCP_ERR_CUDA;
   }
+  memset(block->host, 0, 256);
+  for (int i = 0; i < NT; ++i)
+    if (!tabs[i]->empty()) memcpy((char*)block->host + off[i], tabs[i]->data(), tabs[i]->size() * 4);
+  cudaError_t e = cudaMemcpyAsync(block->dev, block->host, total, cudaMemcpyHostToDevice, copy);
+  if (e == cudaSuccess) e = cudaEventRecord(block->used, copy);
+  if (e == cudaSuccess) e = cudaEventSynchronize(block->used);
+  if (e != cudaSuccess) {
+    free_block(block);
+    fcp_set_error("plan upload failed: %s", cudaGetErrorString(e));
+    return FCP_ERR_CUDA;
+  }
+  void* blob = block->dev;
+  plan->block = block;
+  plan->block_pinned = false;
+  plan->device = dev;
   plan->d_blob = blob;
   plan->d_status = (int32_t*)blob;
   plan->d_fwd_units = (int32_t*)((char*)blob + off[0]);
@@ -282,11 +440,6 @@ extern "C" int fcp_plan_upload(fcp_plan* plan, void* stream) {
   plan->d_fused_units = (int32_t*)((char*)blob + off[7]);
   plan->d_row_limit = plan->row_limit.empty() ? nullptr : (int32_t*)((char*)blob + off[8]);
   plan->d_first_query = plan->first_query.empty() ? nullptr : (int32_t*)((char*)blob + off[9]);
-  // opt in to the large dynamic shared memory of the tensor-core kernels once
-  FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<64>::DYN_BYTES));
-  FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<128>::DYN_BYTES));
-  FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_bwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<64>::DYN_BYTES));
-  FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_bwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<128>::DYN_BYTES));
   return FCP_OK;
 }
 
@@ -334,7 +487,7 @@ extern "C" int fcp_plan_destroy(fcp_plan* plan) {
   if (plan->host_out) cudaStreamDestroy((cudaStream_t)plan->host_out);
   plan->host_in = plan->host_out = nullptr;
   fcp_plan_set_profiling(plan, 0);
-  if (plan->d_blob) cudaFree(plan->d_blob);
+  if (plan->block) return_block(plan->device, plan->block, !plan->block_pinned);
   delete plan;
   return FCP_OK;
 }
@@ -453,16 +606,22 @@ int launch_merge(const fcp_plan* plan, const float* o_partial, const float* lse_
   FCP_CUDA_CHECK(cudaGetLastError());
   return FCP_OK;
 }
+
+// End of a compute call, also of one that failed half-way: part of its work may be queued.
+int used(const fcp_plan* plan, void* stream, int rc) {
+  if (plan) mark_used(plan, (cudaStream_t)stream);
+  return rc;
+}
 }  // namespace
 
 extern "C" int fcp_attn_fwd(const fcp_plan* plan, const void* q, const void* k, const void* v, int32_t head_begin,
                             int32_t head_count, float* o_partial, float* lse_partial, void* stream) {
-  return launch_fwd(plan, q, k, v, head_begin, head_count, o_partial, lse_partial, nullptr, nullptr, nullptr, false, stream);
+  return used(plan, stream, launch_fwd(plan, q, k, v, head_begin, head_count, o_partial, lse_partial, nullptr, nullptr, nullptr, false, stream));
 }
 
 extern "C" int fcp_attn_fwd_fused(const fcp_plan* plan, const void* q, const void* k, const void* v, int32_t head_begin,
                                   int32_t head_count, void* o, float* o_f32, float* lse, void* stream) {
-  return launch_fwd(plan, q, k, v, head_begin, head_count, nullptr, nullptr, o, lse, o_f32, true, stream);
+  return used(plan, stream, launch_fwd(plan, q, k, v, head_begin, head_count, nullptr, nullptr, o, lse, o_f32, true, stream));
 }
 
 extern "C" int fcp_attn_fwd_merged(const fcp_plan* plan, const void* q, const void* k, const void* v, int32_t head_begin,
@@ -473,8 +632,9 @@ extern "C" int fcp_attn_fwd_merged(const fcp_plan* plan, const void* q, const vo
     return FCP_ERR_INVALID_ARG;
   }
   int rc = launch_fwd(plan, q, k, v, head_begin, head_count, o_partial, lse_partial, o, lse, nullptr, false, stream);
-  if (rc != FCP_OK) return rc;
-  return launch_merge(plan, o_partial, lse_partial, head_begin, head_count, o, nullptr, lse, plan->n_merge_multi, stream);
+  if (rc == FCP_OK)
+    rc = launch_merge(plan, o_partial, lse_partial, head_begin, head_count, o, nullptr, lse, plan->n_merge_multi, stream);
+  return used(plan, stream, rc);
 }
 
 extern "C" int fcp_lse_merge(const fcp_plan* plan, const float* o_partial, const float* lse_partial,
@@ -491,8 +651,8 @@ extern "C" int fcp_lse_merge(const fcp_plan* plan, const float* o_partial, const
     fcp_set_error("fcp_lse_merge: the per-item partial path is causal only; this plan has bidirectional spans");
     return FCP_ERR_UNSUPPORTED;
   }
-  return launch_merge(plan, o_partial, lse_partial, head_begin, head_count, o, o_f32, lse,
-                      (int)(plan->merge_units.size() / FCP_MERGE_UNIT_W), stream);
+  return used(plan, stream, launch_merge(plan, o_partial, lse_partial, head_begin, head_count, o, o_f32, lse,
+                                         (int)(plan->merge_units.size() / FCP_MERGE_UNIT_W), stream));
 }
 
 namespace {
@@ -619,8 +779,8 @@ extern "C" int fcp_attn_bwd_heads(const fcp_plan* plan, const void* q, const voi
   }
   const BwdTables tb{plan->d_bwd_units, plan->d_bwd_qranges, plan->d_bwd_work, plan->d_first_query, plan->d_status,
                      plan->d_status + 16, plan->sm_count};
-  return run_bwd(plan, tb, q, k, v, o, d_o, lse, kv_head_begin, kv_head_count, dq, dk, dv, scratch, plan,
-                 (cudaStream_t)stream);
+  return used(plan, stream, run_bwd(plan, tb, q, k, v, o, d_o, lse, kv_head_begin, kv_head_count, dq, dk, dv, scratch, plan,
+                                    (cudaStream_t)stream));
 }
 
 extern "C" int fcp_attn_bwd(const fcp_plan* plan, const void* q, const void* k, const void* v, const void* o,
@@ -875,7 +1035,6 @@ extern "C" int fcp_attn_fwd_bwd_host(const fcp_plan* plan, const void* q_host, c
 static __device__ __align__(256) unsigned char g_noalloc_arena[FCP_NOALLOC_MAX_BYTES];
 
 namespace {
-constexpr int kMaxDevices = 64;
 unsigned char* g_noalloc_ptr[kMaxDevices] = {};   // device address of the arena, per device
 int g_noalloc_sms[kMaxDevices] = {};
 

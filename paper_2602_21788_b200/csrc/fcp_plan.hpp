@@ -24,6 +24,8 @@ enum { BU_KV_ROW0 = 0, BU_KV_ROWS, BU_FIRST_QRANGE, BU_N_QRANGES, BU_T_FIRST, BU
 enum { BQ_BEGIN = 0, BQ_END, BQ_DIAG, BQ_RSV };
 enum { MU_TOK_BEGIN = 0, MU_N_TOK, MU_CHUNK, MU_CHUNK_TOK_BEGIN };
 
+struct PlanBlock;                      // device block of an uploaded plan (fcp_kernels.cu)
+
 struct fcp_plan {
   fcp_params params{};
   int32_t B = 0;
@@ -38,7 +40,9 @@ struct fcp_plan {
 
   // device copy (fcp_plan_upload)
   int device = -1;
-  void* d_blob = nullptr;      // one allocation holding every table below
+  PlanBlock* block = nullptr;
+  mutable bool block_pinned = false;   // the block's event does not cover all work that may read it (graph capture)
+  void* d_blob = nullptr;      // the block's device memory: holds every table below
   int32_t* d_fwd_units = nullptr;
   int32_t* d_bwd_units = nullptr;
   int32_t* d_bwd_qranges = nullptr;

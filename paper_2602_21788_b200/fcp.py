@@ -27,7 +27,7 @@ INFO = dict(T=0, R=1, n_pairs=2, n_items=3, n_fwd_units=4, n_bwd_units=5, n_merg
             n_fused_units=9)
 
 EXPORTS = ["fcp_plan_strategy", "fcp_plan_blocks", "fcp_plan_blocks_spans", "fcp_span_mask_efficiency", "fcp_plan_get", "fcp_plan_info", "fcp_plan_workspace_bytes",
-           "fcp_plan_bwd_scratch_bytes", "fcp_plan_upload", "fcp_plan_destroy", "fcp_attn_fwd", "fcp_attn_fwd_merged",
+           "fcp_plan_bwd_scratch_bytes", "fcp_plan_upload", "fcp_release_cached", "fcp_plan_destroy", "fcp_attn_fwd", "fcp_attn_fwd_merged",
            "fcp_attn_fwd_fused", "fcp_lse_merge", "fcp_attn_bwd", "fcp_attn_bwd_heads",
            "fcp_host_workspace_bytes", "fcp_attn_fwd_bwd_host", "fcp_last_device_status", "fcp_plan_set_profiling",
            "fcp_plan_kernel_ms", "fcp_noalloc_bytes_needed", "fcp_attn_bwd_noalloc", "fcp_noalloc_device_status",
@@ -73,6 +73,7 @@ def lib() -> C.CDLL:
     L.fcp_plan_workspace_bytes.argtypes = [vp, C.c_int32, i64p, i64p, i64p]
     L.fcp_plan_upload.argtypes = [vp, vp]
     L.fcp_plan_destroy.argtypes = [vp]
+    L.fcp_release_cached.argtypes = []
     L.fcp_attn_fwd.argtypes = [vp, vp, vp, vp, C.c_int32, C.c_int32, vp, vp, vp]
     L.fcp_lse_merge.argtypes = [vp, vp, vp, C.c_int32, C.c_int32, vp, vp, vp, vp]
     L.fcp_attn_fwd_merged.argtypes = [vp, vp, vp, vp, C.c_int32, C.c_int32, vp, vp, vp, vp, vp]
@@ -216,6 +217,11 @@ class Plan:
         st = np.zeros(4, dtype=np.int32)
         _check(lib().fcp_last_device_status(self.handle, st.ctypes.data_as(C.POINTER(C.c_int32))))
         return st
+
+
+def fcp_release_cached():
+    """Frees the device blocks that destroyed plans left for later ones (current device)."""
+    _check(lib().fcp_release_cached())
 
 
 def fcp_plan_blocks(seqlens, cp_degrees, hq, hkv, head_dim, scale=0.0) -> Plan:

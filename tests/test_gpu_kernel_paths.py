@@ -51,3 +51,61 @@ def _check(w, **kw):
 ])
 def test_backward_d64_blocked_dq_accumulator(lens, hq, hkv, kv_pass):
     _check(_wl(lens, [1] * len(lens), hq, hkv, 64, seed=11), kv_heads_per_bwd_pass=kv_pass)
+
+
+def _fused(plan, q, k, v, hq, stream):
+    from paper_2602_21788_b200 import fcp
+    o = torch.empty_like(q)
+    lse = torch.empty(q.shape[:2], dtype=torch.float32, device="cuda")
+    fcp.fcp_attn_fwd_fused(plan, q, k, v, o, lse, stream=stream.cuda_stream)
+    return o, lse
+
+
+@pytest.mark.parametrize("threads", [1, 3])
+def test_plan_blocks_are_handed_on_only_after_the_work_that_reads_them(threads):
+    """Plans that are dropped right after their calls were queued, with the next plan (of another batch) uploaded at
+    once: from one thread over two streams, and from several threads with a stream each."""
+    import threading
+    from paper_2602_21788_b200 import fcp
+    hq, hkv, D = 8, 2, 128
+    batches = [[3000, 1000, 96], [128] * 32, [4096], [700, 650, 1300, 1446]]
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q, k, v = (torch.randn((4096, h, D), dtype=torch.bfloat16, device="cuda", generator=g) for h in (hq, hkv, hkv))
+    main = torch.cuda.current_stream()
+    want = {}
+    for i, lens in enumerate(batches):
+        plan = fcp.Plan(lens, [1] * len(lens), hq, hkv, D).upload()
+        want[i] = _fused(plan, q, k, v, hq, main)
+    torch.cuda.synchronize()
+    got, failed = [], []
+
+    def work(t):
+        try:
+            streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+            busy = torch.zeros(1 << 27, device="cuda")
+            torch.cuda.synchronize()
+            for r in range(12):
+                i, st = (r + t) % len(batches), streams[r & 1]
+                with torch.cuda.stream(st):
+                    busy.add_(1.0)                      # keeps the stream busy: the calls below stay queued for a while
+                    plan = fcp.Plan(batches[i], [1] * len(batches[i]), hq, hkv, D).upload(st.cuda_stream)
+                    got.append((i, _fused(plan, q, k, v, hq, st)))
+                del plan
+        except Exception as e:                          # a thread's failure must reach the test
+            failed.append(e)
+
+    ts = [threading.Thread(target=work, args=(t,)) for t in range(threads)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed, failed
+    assert len(got) == 12 * threads
+    for i, (o, lse) in got:
+        assert torch.equal(o, want[i][0]) and torch.equal(lse, want[i][1]), i
+    fcp.fcp_release_cached()
+    plan = fcp.Plan(batches[0], [1, 1, 1], hq, hkv, D).upload()
+    o, lse = _fused(plan, q, k, v, hq, main)
+    torch.cuda.synchronize()
+    assert torch.equal(o, want[0][0]) and torch.equal(lse, want[0][1])
