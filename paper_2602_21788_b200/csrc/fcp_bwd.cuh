@@ -173,6 +173,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
   if ((sbase & 1023u) != 0) {                  // uniform across the grid: nobody touches a barrier
+    grid_begin();
     if (threadIdx.x == 0 && blockIdx.x == 0) {
       a.status[0] = -5;
       a.status[1] = 199;
@@ -227,6 +228,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_begin();
 
   const int g = a.hq / a.hkv;
 

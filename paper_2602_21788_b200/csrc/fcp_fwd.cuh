@@ -62,7 +62,7 @@ struct FwdArgs {
   int32_t head_begin, head_count, hq, hkv;
   int32_t head_group;     // heads that are adjacent in the work order: hq/hkv when the head range is made of whole
                           // KV-head groups, else 1; head_count % head_group == 0
-  int32_t* work_counter;  // zero before the launch: the grid's next work item
+  int32_t* work_counter;  // the grid's next work item: zero before the launch, and again after it
   float scale_log2;       // softmax scale * log2(e)
   float* o_partial;       // [R][head_count][D]
   float* lse_partial;     // [R][head_count]
@@ -137,6 +137,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_begin();
 
   const int64_t n_work = (int64_t)a.n_units * a.head_count;
   const int g = a.hq / a.hkv;
@@ -171,10 +172,12 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       uint32_t kv_it = 0, qcnt[2] = {0, 0}, nw = 0;
-      bool ok = true;
+      bool ok = true, taken_all = false;
 #pragma unroll 1
       while (ok) {
         const int64_t w = atomicAdd(a.work_counter, 1);
+        taken_all = w >= n_work;
+        if (w == n_work + (int)gridDim.x - 1) *a.work_counter = 0;   // every producer takes one item past the end: this is the last
         const uint32_t slot = nw % FWD_WORK_SLOTS;
         ok = mbar_wait(BAR(B_WEMPTY + slot), ((nw / FWD_WORK_SLOTS) & 1) ^ 1, wctx, 41);
         if (!ok) break;
@@ -225,6 +228,13 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             ++kv_it;
           }
         }
+      }
+      // after a wait that gave up: take the rest of the list, so that the counter comes back to zero
+#pragma unroll 1
+      while (!taken_all) {
+        const int64_t w = atomicAdd(a.work_counter, 1);
+        taken_all = w >= n_work;
+        if (w == n_work + (int)gridDim.x - 1) *a.work_counter = 0;
       }
     }
   } else if (warp == 1) {

