@@ -250,13 +250,13 @@ int fcp_attn_bwd_heads(const fcp_plan* plan, const void* q, const void* k, const
  * runs fcp_attn_fwd_fused and fcp_attn_bwd, and copies o, lse, dq, dk, dv back.  `workspace` is a
  * caller-owned DEVICE buffer of `workspace_bytes` >= fcp_host_workspace_bytes(plan); host pointers
  * should be pinned for the copies to be asynchronous.
- * The batch is cut into up to 8 runs of consecutive sequences (packed tensors are token-major, so a
- * run is one contiguous slice of every tensor), and a run of several hundred megabytes further into
- * passes over whole KV heads (strided slices); the inputs of the next slice come in and the results
- * of the previous one go out while the kernels of the current slice execute (two internal copy
- * streams, ordered after the work already queued on `stream`).  The first call on a plan is the
- * one exception to "compute calls do not allocate": it builds and uploads the plans of the runs
- * and creates the copy streams and events (small allocations, all released by fcp_plan_destroy).
+ * The batch is cut into up to 16 slices: passes over whole KV heads (strided copies) and, where there
+ * are few KV heads, runs of consecutive sequences (packed tensors are token-major, so a run is one
+ * contiguous slice of every tensor).  The inputs of later slices come in and the results of earlier
+ * ones go out while kernels execute (two internal copy streams and a second kernel stream, ordered
+ * after the work already queued on `stream`).  The first call on a plan is the one exception to
+ * "compute calls do not allocate": it builds and uploads the plans of the runs and creates the
+ * streams and events (small allocations, all released by fcp_plan_destroy).
  * Synchronises `stream` before returning; every output is complete then.  On an error return the
  * work already queued has been waited for, so nothing writes into the caller's buffers afterwards.
  */

@@ -173,7 +173,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
   if ((sbase & 1023u) != 0) {                  // uniform across the grid: nobody touches a barrier
-    grid_begin();
+    grid_wait();
     if (threadIdx.x == 0 && blockIdx.x == 0) {
       a.status[0] = -5;
       a.status[1] = 199;
@@ -228,7 +228,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  grid_begin();
+  grid_wait();
 
   const int g = a.hq / a.hkv;
 
@@ -262,7 +262,10 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         work_ring[2 * slot] = unit;
         work_ring[2 * slot + 1] = hk;
         mbar_arrive(BAR(B_WFULL + slot));     // release: the two stores above are visible to the waiters
-        if (last) break;
+        if (last) {
+          grid_launch_next();
+          break;
+        }
         const int32_t* U = a.units + (size_t)unit * FCP_BWD_UNIT_W;
         const int kv_row0 = __ldg(U + BU_KV_ROW0);
         ok = mbar_wait(BAR(B_KVFREE), (n & 1) ^ 1, wctx, 110);

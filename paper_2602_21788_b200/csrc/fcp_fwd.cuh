@@ -137,7 +137,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  grid_begin();
+  grid_wait();
 
   const int64_t n_work = (int64_t)a.n_units * a.head_count;
   const int g = a.hq / a.hkv;
@@ -192,7 +192,10 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         work_ring[2 * slot + 1] = h;
         mbar_arrive(BAR(B_WFULL + slot));      // release: the two stores above are visible to the waiters
         ++nw;
-        if (last) break;
+        if (last) {
+          grid_launch_next();
+          break;
+        }
         const int32_t* U = a.units + (size_t)unit * FCP_FWD_UNIT_W;
         const int hk = h / g;
         const int nt[2] = {__ldg(U + FU_NT_STAGE0), __ldg(U + FU_NT_STAGE1)};

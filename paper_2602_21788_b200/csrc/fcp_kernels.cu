@@ -529,7 +529,8 @@ extern "C" int fcp_plan_destroy(fcp_plan* plan) {
   plan->host_events.clear();
   if (plan->host_in) cudaStreamDestroy((cudaStream_t)plan->host_in);
   if (plan->host_out) cudaStreamDestroy((cudaStream_t)plan->host_out);
-  plan->host_in = plan->host_out = nullptr;
+  if (plan->host_lane) cudaStreamDestroy((cudaStream_t)plan->host_lane);
+  plan->host_in = plan->host_out = plan->host_lane = nullptr;
   fcp_plan_set_profiling(plan, 0);
   if (plan->block) return_block(plan->device, plan->block, !plan->block_pinned);
   delete plan;
@@ -579,10 +580,11 @@ static int check_heads(const fcp_plan* plan, int head_begin, int head_count) {
 }
 
 namespace {
-// `fused`: run the merge-on-the-fly units (every row goes straight to o_direct / lse_direct, no partials)
+// `fused`: run the merge-on-the-fly units (every row goes straight to o_direct / lse_direct, no partials).
+// `lane`: which work counter of the plan to use (two calls that may overlap use different ones).
 int launch_fwd(const fcp_plan* plan, const void* q, const void* k, const void* v, int32_t head_begin, int32_t head_count,
                float* o_partial, float* lse_partial, void* o_direct, float* lse_direct, float* o_f32_direct, bool fused,
-               void* stream) {
+               void* stream, int lane = 0) {
   int rc = check_plan(plan);
   if (rc != FCP_OK) return rc;
   if (!q || !k || !v || (!fused && (!o_partial || !lse_partial)) || (fused && (!o_direct || !lse_direct))) {
@@ -623,8 +625,8 @@ int launch_fwd(const fcp_plan* plan, const void* q, const void* k, const void* v
   const int grid = (int)std::min<int64_t>(n_work, plan->sm_count);
   if (grid == 0) return FCP_OK;
   cudaStream_t st = (cudaStream_t)stream;
-  // the grid's work counter (the status block's word 17; word 16 is the backward grid's): zero from the upload on
-  a.work_counter = plan->d_status + 17;
+  // the grid's work counter (status block: words 16 + 2 * lane backward, 17 + 2 * lane forward): zero from the upload on
+  a.work_counter = plan->d_status + 17 + 2 * lane;
   ProfScope prof(plan, 0, st);
   if (P.head_dim == 128)
     FCP_CUDA_CHECK(launch(fcp_fwd_kernel<128>, grid, FWD_THREADS, FwdSmem<128>::DYN_BYTES, st, tq, tk, tv, a));
@@ -796,9 +798,10 @@ extern "C" int fcp_plan_bwd_scratch_bytes(const fcp_plan* plan, int32_t kv_head_
   return FCP_OK;
 }
 
-extern "C" int fcp_attn_bwd_heads(const fcp_plan* plan, const void* q, const void* k, const void* v, const void* o,
-                                  const void* d_o, const float* lse, int32_t kv_head_begin, int32_t kv_head_count,
-                                  void* dq, void* dk, void* dv, void* scratch, int64_t scratch_bytes, void* stream) {
+namespace {
+int bwd_heads(const fcp_plan* plan, const void* q, const void* k, const void* v, const void* o, const void* d_o, const float* lse,
+              int32_t kv_head_begin, int32_t kv_head_count, void* dq, void* dk, void* dv, void* scratch, int64_t scratch_bytes,
+              void* stream, int lane) {
   int rc = check_plan(plan);
   if (rc != FCP_OK) return rc;
   if (!q || !k || !v || !o || !d_o || !lse || !dq || !dk || !dv || !scratch) {
@@ -815,9 +818,16 @@ extern "C" int fcp_attn_bwd_heads(const fcp_plan* plan, const void* q, const voi
     return FCP_ERR_WORKSPACE;
   }
   const BwdTables tb{plan->d_bwd_units, plan->d_bwd_qranges, plan->d_bwd_work, plan->d_first_query, plan->d_status,
-                     plan->d_status + 16, plan->sm_count};
+                     plan->d_status + 16 + 2 * lane, plan->sm_count};
   return used(plan, stream, run_bwd(plan, tb, q, k, v, o, d_o, lse, kv_head_begin, kv_head_count, dq, dk, dv, scratch, plan,
                                     (cudaStream_t)stream));
+}
+}  // namespace
+
+extern "C" int fcp_attn_bwd_heads(const fcp_plan* plan, const void* q, const void* k, const void* v, const void* o,
+                                  const void* d_o, const float* lse, int32_t kv_head_begin, int32_t kv_head_count,
+                                  void* dq, void* dk, void* dv, void* scratch, int64_t scratch_bytes, void* stream) {
+  return bwd_heads(plan, q, k, v, o, d_o, lse, kv_head_begin, kv_head_count, dq, dk, dv, scratch, scratch_bytes, stream, 0);
 }
 
 extern "C" int fcp_attn_bwd(const fcp_plan* plan, const void* q, const void* k, const void* v, const void* o,
@@ -867,16 +877,27 @@ extern "C" int fcp_host_workspace_bytes(const fcp_plan* plan, int64_t* bytes) {
 }
 
 namespace {
-// Cuts the batch into runs of consecutive sequences of about equal token counts (at most 8 runs, at
-// least about 8192 tokens each) and plans each run on its own: packed tensors are token-major, so a run
-// is one contiguous slice of every tensor and can be copied, computed and copied back independently.
-// Also creates the two copy streams and the events the host entry point orders its work with; all of
-// it belongs to the plan and is released by fcp_plan_destroy.
+// How the host entry point cuts a batch: into passes over whole KV heads (strided slices, 2-D copies; these run at full
+// PCIe speed down to one head of 256 bytes per row: 52 of 55 GB/s) and, when there are too few KV heads, into runs of
+// consecutive sequences (packed tensors are token-major, so a run is one contiguous slice of every tensor) with a plan of
+// their own.  About kHostSliceBytes of inputs per slice and at most kHostSlices: what is not overlapped is the first
+// slice's way in and the last one's way out.  Heads come first because the work of a slice is then the same for all of
+// them; runs of a batch with one long sequence are as unequal as its sequences (32K tokens, half of them one sequence:
+// 24.1 ms with runs only).
+constexpr int64_t kHostSliceBytes = int64_t(32) << 20;
+constexpr int64_t kHostSlices = 16;
+
+// Builds the runs' plans and creates the streams and events the host entry point orders its work with; all of it belongs
+// to the plan and is released by fcp_plan_destroy.
 int build_host_groups(const fcp_plan* plan, void* stream) {
-  if (!plan->groups.empty()) return FCP_OK;
+  if (!plan->host_events.empty()) return FCP_OK;
   const int B = plan->B;
   const int64_t T = plan->T;
-  const int want = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(8, B), T / 8192));
+  const fcp_params& P = plan->params;
+  const int64_t in_bytes = 2 * T * (P.hq + P.hkv) * P.head_dim * 2;
+  const int64_t slices = std::max<int64_t>(1, std::min<int64_t>(kHostSlices, in_bytes / kHostSliceBytes));
+  const int32_t passes = (int32_t)std::min<int64_t>(P.hkv, slices);
+  const int want = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(slices / passes, B), T / 8192));
   std::vector<int32_t> lens(B), degs(B);
   for (int b = 0; b < B; ++b) {
     lens[b] = plan->cu_seqlens[b + 1] - plan->cu_seqlens[b];
@@ -888,7 +909,8 @@ int build_host_groups(const fcp_plan* plan, void* stream) {
     for (fcp_plan* x : groups) fcp_plan_destroy(x);
     return rc;
   };
-  int b0 = 0;
+  int b0 = want > 1 ? 0 : B;                     // one run: the plan itself
+  if (want == 1) tok0.push_back(0);
   for (int g = 0; g < want && b0 < B; ++g) {
     int b1 = b0 + 1;
     if (g == want - 1) {
@@ -917,21 +939,13 @@ int build_host_groups(const fcp_plan* plan, void* stream) {
     b0 = b1;
   }
   tok0.push_back(T);
-  // A group whose query tensor alone is hundreds of megabytes (one very long sequence) is additionally cut into
-  // passes over whole KV heads, so that its copies overlap its own kernels too: at least ~256 MB of q per pass.
-  std::vector<int32_t> passes;
-  int64_t total_passes = 0;
-  for (size_t g = 0; g < groups.size(); ++g) {
-    const int64_t q_bytes = (tok0[g + 1] - tok0[g]) * plan->params.hq * plan->params.head_dim * 2;
-    const int32_t np = (int32_t)std::max<int64_t>(1, std::min<int64_t>(plan->params.hkv, q_bytes / (int64_t(256) << 20)));
-    passes.push_back(np);
-    total_passes += np;
-  }
-  // streams and events: [0] start, [1] last copy out, then per (group, pass): q, k, v up; dO up; forward done; backward done
-  cudaStream_t in = nullptr, out = nullptr;
-  std::vector<void*> ev(2 + 4 * (size_t)total_passes, nullptr);
+  const size_t total_passes = (tok0.size() - 1) * passes;
+  // streams and events: [0] start, [1] last copy out, [2] second lane done, then per (run, pass): q, k, v up; dO up; forward done; backward done
+  cudaStream_t in = nullptr, out = nullptr, lane = nullptr;
+  std::vector<void*> ev(3 + 4 * total_passes, nullptr);
   cudaError_t e = cudaStreamCreateWithFlags(&in, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&out, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&lane, cudaStreamNonBlocking);
   for (size_t i = 0; i < ev.size() && e == cudaSuccess; ++i) {
     cudaEvent_t x = nullptr;
     e = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
@@ -941,28 +955,31 @@ int build_host_groups(const fcp_plan* plan, void* stream) {
     for (void* x : ev) if (x) cudaEventDestroy((cudaEvent_t)x);
     if (in) cudaStreamDestroy(in);
     if (out) cudaStreamDestroy(out);
+    if (lane) cudaStreamDestroy(lane);
     fcp_set_error("fcp_attn_fwd_bwd_host: creating copy streams failed: %s", cudaGetErrorString(e));
     return fail(FCP_ERR_CUDA);
   }
   plan->host_in = in;
   plan->host_out = out;
+  plan->host_lane = lane;
   plan->host_events = std::move(ev);
   plan->groups = std::move(groups);
   plan->group_tok0 = std::move(tok0);
-  plan->group_passes = std::move(passes);
+  plan->host_passes = passes;
   return FCP_OK;
 }
 
 // On any early exit of the host entry point: wait for the copies and kernels already queued, so that
 // nothing still writes into the caller's buffers after the call has returned an error.
 struct HostDrain {
-  cudaStream_t a, b, c;
+  cudaStream_t a, b, c, d;
   bool armed = true;
   ~HostDrain() {
     if (!armed) return;
     cudaStreamSynchronize(a);
     cudaStreamSynchronize(b);
     cudaStreamSynchronize(c);
+    cudaStreamSynchronize(d);
   }
 };
 }  // namespace
@@ -989,31 +1006,35 @@ extern "C" int fcp_attn_fwd_bwd_host(const fcp_plan* plan, const void* q_host, c
   const int64_t D = P.head_dim;
   const int64_t rq = (int64_t)P.hq * D * 2, rkv = (int64_t)P.hkv * D * 2, rl = (int64_t)P.hq * 4;   // bytes per token
   char* w = (char*)workspace;
-  const int G = (int)plan->groups.size();
-  // Three streams: inputs of group g+1 come in and results of group g-1 go out while the kernels of
-  // group g run on `stream`.  Everything is ordered after the work already queued on `stream` and is
+  const int G = (int)plan->group_tok0.size() - 1;
+  // Inputs of later slices come in (s_in) and results of earlier ones go out (s_out) while kernels run.  The kernels of
+  // consecutive slices alternate between `stream` and a second lane: a slice has few work units, and the next one fills
+  // the SMs that its longest units leave idle.  Everything is ordered after the work already queued on `stream` and is
   // complete when this call returns.
-  cudaStream_t s_in = (cudaStream_t)plan->host_in, s_out = (cudaStream_t)plan->host_out;
+  cudaStream_t s_in = (cudaStream_t)plan->host_in, s_out = (cudaStream_t)plan->host_out, s_lane = (cudaStream_t)plan->host_lane;
   auto EV = [&](int i) { return (cudaEvent_t)plan->host_events[i]; };
-  // Work is cut twice: into groups (runs of consecutive sequences: contiguous token slices) and, for large groups,
-  // into passes over whole KV heads with their query heads (strided slices of every token row: 2-D copies).  The
-  // forward pass of a slice needs q, k, v only: dO follows them and arrives while the forward kernel runs; o and
-  // lse leave while the backward kernels run (they only read them).
-  struct Slice { int g, hk0, hkc, ev0; };
+  // The forward pass of a slice needs q, k, v only: dO follows them and arrives while the forward kernel runs; o leaves
+  // while the backward kernels run (they only read it), the log-sum-exps of a run when its last forward pass is done
+  // (the few bytes per row of one pass would make a slow strided copy).
+  struct Slice { int g, hk0, hkc, ev0; bool last; };
   std::vector<Slice> slices;
+  const int per = (P.hkv + plan->host_passes - 1) / plan->host_passes;
+  int64_t lane_scratch = 0;                      // scratch of the largest slice
   {
-    int ev0 = 2;
-    for (int g = 0; g < G; ++g) {
-      const int np = plan->group_passes[g];
-      const int per = (P.hkv + np - 1) / np;
-      for (int hk0 = 0; hk0 < P.hkv; hk0 += per, ev0 += 4) slices.push_back(Slice{g, hk0, std::min(per, P.hkv - hk0), ev0});
-    }
+    int ev0 = 3;
+    for (int g = 0; g < G; ++g)
+      for (int hk0 = 0; hk0 < P.hkv; hk0 += per, ev0 += 4) {
+        slices.push_back(Slice{g, hk0, std::min(per, P.hkv - hk0), ev0, hk0 + per >= P.hkv});
+        lane_scratch = std::max(lane_scratch, al(bwd_scratch_need(plan->groups.empty() ? plan : plan->groups[g], per)));
+      }
   }
+  const bool two_lanes = slices.size() > 1 && 2 * lane_scratch <= al(bwd_scratch_need(plan, P.hkv));
   const int gq = P.hq / P.hkv;
-  HostDrain drain{s_in, s_out, st};
+  HostDrain drain{s_in, s_out, st, s_lane};
   FCP_CUDA_CHECK(cudaEventRecord(EV(0), st));
   FCP_CUDA_CHECK(cudaStreamWaitEvent(s_in, EV(0), 0));
   FCP_CUDA_CHECK(cudaStreamWaitEvent(s_out, EV(0), 0));
+  FCP_CUDA_CHECK(cudaStreamWaitEvent(s_lane, EV(0), 0));
   // copies of the heads [h0, h0 + hc) of nt token rows: width hc * bytes per head, pitch = the row of all heads
   auto copy_heads = [&](char* dst, const char* src, int64_t t0, int64_t nt, int64_t row_bytes, int64_t head_bytes, int h0, int hc,
                         cudaMemcpyKind kind, cudaStream_t cs) {
@@ -1031,31 +1052,39 @@ extern "C" int fcp_attn_fwd_bwd_host(const fcp_plan* plan, const void* q_host, c
     FCP_CUDA_CHECK(copy_heads(w + L.d_o, (const char*)d_o_host, t0, nt, rq, hb, h0, hc, cudaMemcpyHostToDevice, s_in));
     FCP_CUDA_CHECK(cudaEventRecord(EV(sl.ev0 + 1), s_in));
   }
-  for (const Slice& sl : slices) {
-    const fcp_plan* sub = plan->groups[sl.g];
+  for (size_t i = 0; i < slices.size(); ++i) {
+    const Slice& sl = slices[i];
+    const fcp_plan* sub = plan->groups.empty() ? plan : plan->groups[sl.g];
+    const int lane = two_lanes ? (int)(i & 1) : 0;
+    cudaStream_t sk = lane ? s_lane : st;
     const int64_t t0 = plan->group_tok0[sl.g], nt = plan->group_tok0[sl.g + 1] - t0;
     const int h0 = sl.hk0 * gq, hc = sl.hkc * gq;
-    FCP_CUDA_CHECK(cudaStreamWaitEvent(st, EV(sl.ev0), 0));
-    if ((rc = fcp_attn_fwd_fused(sub, w + L.q + t0 * rq, w + L.k + t0 * rkv, w + L.v + t0 * rkv, h0, hc, w + L.o + t0 * rq,
-                                 nullptr, (float*)(w + L.lse + t0 * rl), st)) != FCP_OK)
+    FCP_CUDA_CHECK(cudaStreamWaitEvent(sk, EV(sl.ev0), 0));
+    if ((rc = launch_fwd(sub, w + L.q + t0 * rq, w + L.k + t0 * rkv, w + L.v + t0 * rkv, h0, hc, nullptr, nullptr, w + L.o + t0 * rq,
+                         (float*)(w + L.lse + t0 * rl), nullptr, true, sk, lane)) != FCP_OK)
       return rc;
-    FCP_CUDA_CHECK(cudaEventRecord(EV(sl.ev0 + 2), st));
+    FCP_CUDA_CHECK(cudaEventRecord(EV(sl.ev0 + 2), sk));
     FCP_CUDA_CHECK(cudaStreamWaitEvent(s_out, EV(sl.ev0 + 2), 0));
     FCP_CUDA_CHECK(copy_heads((char*)o_host, w + L.o, t0, nt, rq, hb, h0, hc, cudaMemcpyDeviceToHost, s_out));
-    FCP_CUDA_CHECK(copy_heads((char*)lse_host, w + L.lse, t0, nt, rl, 4, h0, hc, cudaMemcpyDeviceToHost, s_out));
-    FCP_CUDA_CHECK(cudaStreamWaitEvent(st, EV(sl.ev0 + 1), 0));
-    if ((rc = fcp_attn_bwd_heads(sub, w + L.q + t0 * rq, w + L.k + t0 * rkv, w + L.v + t0 * rkv, w + L.o + t0 * rq,
-                                 w + L.d_o + t0 * rq, (float*)(w + L.lse + t0 * rl), sl.hk0, sl.hkc, w + L.dq + t0 * rq,
-                                 w + L.dk + t0 * rkv, w + L.dv + t0 * rkv, w + L.scratch, bwd_scratch_need(sub, sl.hkc), st)) != FCP_OK)
+    if (sl.last)
+      FCP_CUDA_CHECK(cudaMemcpyAsync((char*)lse_host + t0 * rl, w + L.lse + t0 * rl, nt * rl, cudaMemcpyDeviceToHost, s_out));
+    FCP_CUDA_CHECK(cudaStreamWaitEvent(sk, EV(sl.ev0 + 1), 0));
+    if ((rc = bwd_heads(sub, w + L.q + t0 * rq, w + L.k + t0 * rkv, w + L.v + t0 * rkv, w + L.o + t0 * rq, w + L.d_o + t0 * rq,
+                        (float*)(w + L.lse + t0 * rl), sl.hk0, sl.hkc, w + L.dq + t0 * rq, w + L.dk + t0 * rkv, w + L.dv + t0 * rkv,
+                        w + L.scratch + lane * lane_scratch, bwd_scratch_need(sub, sl.hkc), sk, lane)) != FCP_OK)
       return rc;
-    FCP_CUDA_CHECK(cudaEventRecord(EV(sl.ev0 + 3), st));
+    FCP_CUDA_CHECK(cudaEventRecord(EV(sl.ev0 + 3), sk));
     FCP_CUDA_CHECK(cudaStreamWaitEvent(s_out, EV(sl.ev0 + 3), 0));
     FCP_CUDA_CHECK(copy_heads((char*)dq_host, w + L.dq, t0, nt, rq, hb, h0, hc, cudaMemcpyDeviceToHost, s_out));
     FCP_CUDA_CHECK(copy_heads((char*)dk_host, w + L.dk, t0, nt, rkv, hb, sl.hk0, sl.hkc, cudaMemcpyDeviceToHost, s_out));
     FCP_CUDA_CHECK(copy_heads((char*)dv_host, w + L.dv, t0, nt, rkv, hb, sl.hk0, sl.hkc, cudaMemcpyDeviceToHost, s_out));
   }
+  FCP_CUDA_CHECK(cudaEventRecord(EV(2), s_lane));
+  FCP_CUDA_CHECK(cudaStreamWaitEvent(st, EV(2), 0));
   FCP_CUDA_CHECK(cudaEventRecord(EV(1), s_out));
   FCP_CUDA_CHECK(cudaStreamWaitEvent(st, EV(1), 0));
+  for (const fcp_plan* sub : plan->groups) mark_used(sub, st);   // after both lanes
+  mark_used(plan, st);
   FCP_CUDA_CHECK(cudaStreamSynchronize(st));
   drain.armed = false;
   return FCP_OK;

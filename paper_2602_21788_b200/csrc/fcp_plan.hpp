@@ -56,14 +56,15 @@ struct fcp_plan {
   int32_t* d_status = nullptr; // [4]: status word, diagnostic
   int sm_count = 0;
 
-  // Sub-plans over runs of consecutive sequences, built and uploaded at the first call of the host
-  // entry point, which pipelines copies and kernels over them (owned by this plan).
+  // Host entry point, set up at its first call and owned by this plan: sub-plans over runs of consecutive sequences
+  // (none when one run, this plan itself, is enough), streams and events.
   mutable std::vector<fcp_plan*> groups;
-  mutable std::vector<int64_t> group_tok0;   // first packed token of each group, plus T at the end
-  mutable void* host_in = nullptr;           // cudaStream_t: host -> device copies of the host entry point
+  mutable std::vector<int64_t> group_tok0;   // first packed token of each run, plus T at the end
+  mutable void* host_in = nullptr;           // cudaStream_t: host -> device copies
   mutable void* host_out = nullptr;          // cudaStream_t: device -> host copies
-  mutable std::vector<int32_t> group_passes; // KV-head passes of each group (large groups are also pipelined by KV head)
-  mutable std::vector<void*> host_events;    // cudaEvent_t: start, last copy out, then four per (group, pass)
+  mutable void* host_lane = nullptr;         // cudaStream_t: kernels of every second slice
+  mutable int32_t host_passes = 1;           // KV-head passes of each run
+  mutable std::vector<void*> host_events;    // cudaEvent_t: start, last copy out, second lane, then four per (run, pass)
 
   // optional kernel timing: ring of event pairs per kernel kind (void* = cudaEvent_t)
   bool profiling = false;

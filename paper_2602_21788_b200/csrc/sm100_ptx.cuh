@@ -35,12 +35,15 @@ __device__ __forceinline__ bool elect_one() {
 }
 
 // ----------------------------------------------------------------------------- programmatic launch
-// Every kernel of the library lets the next one of the stream be launched at once (its blocks start as SMs become
-// free) and waits for the work before it, memory included, before it touches global memory.  Because every kernel
-// waits, "the grid before is complete" covers all grids before that one too.
+// Every kernel of the library waits (grid_wait) for the work before it, memory included, before it touches global
+// memory, so that "the grid before is complete" covers all grids before that one too.  The short kernels let the next
+// one of the stream be launched at once; the persistent ones only when a CTA sees the end of the work list, because
+// blocks that wait on an SM keep other streams' work off it.
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_begin() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_launch_next();
+  grid_wait();
 }
 
 // ----------------------------------------------------------------------------- mbarrier
