@@ -878,14 +878,15 @@ extern "C" int fcp_host_workspace_bytes(const fcp_plan* plan, int64_t* bytes) {
 
 namespace {
 // How the host entry point cuts a batch: into passes over whole KV heads (strided slices, 2-D copies; these run at full
-// PCIe speed down to one head of 256 bytes per row: 52 of 55 GB/s) and, when there are too few KV heads, into runs of
-// consecutive sequences (packed tensors are token-major, so a run is one contiguous slice of every tensor) with a plan of
-// their own.  About kHostSliceBytes of inputs per slice and at most kHostSlices: what is not overlapped is the first
-// slice's way in and the last one's way out.  Heads come first because the work of a slice is then the same for all of
-// them; runs of a batch with one long sequence are as unequal as its sequences (32K tokens, half of them one sequence:
-// 24.1 ms with runs only).
-constexpr int64_t kHostSliceBytes = int64_t(32) << 20;
-constexpr int64_t kHostSlices = 16;
+// PCIe speed down to 512 bytes per row, 48 of 55 GB/s with both directions busy, 42 at 256 bytes) and, to get to
+// kHostSlices, into runs of consecutive sequences (packed tensors are token-major, so a run is one contiguous slice of
+// every tensor) with a plan of their own.  About kHostSliceBytes of inputs per slice: what is not overlapped is the
+// first slice's way in and the last one's way out (11K tokens of 4 heads, D = 64: 1.4 ms with slices of 32 MB, 1.0 with
+// 8 MB; 32K tokens of 32/32 heads: 28.7 ms with 16 passes, 26.5 with 8 in two runs).  Heads come first because every
+// pass has the same work; runs of a batch with one long sequence are as unequal as its sequences (32K tokens of 32/8
+// heads, half of them one sequence: 23.0 ms with runs only, 17.5 now; the copies alone take 13.6).
+constexpr int64_t kHostSliceBytes = int64_t(8) << 20;
+constexpr int64_t kHostSlices = 16, kHostPasses = 8;
 
 // Builds the runs' plans and creates the streams and events the host entry point orders its work with; all of it belongs
 // to the plan and is released by fcp_plan_destroy.
@@ -896,7 +897,7 @@ int build_host_groups(const fcp_plan* plan, void* stream) {
   const fcp_params& P = plan->params;
   const int64_t in_bytes = 2 * T * (P.hq + P.hkv) * P.head_dim * 2;
   const int64_t slices = std::max<int64_t>(1, std::min<int64_t>(kHostSlices, in_bytes / kHostSliceBytes));
-  const int32_t passes = (int32_t)std::min<int64_t>(P.hkv, slices);
+  const int32_t passes = (int32_t)std::min<int64_t>(std::min<int64_t>(P.hkv, kHostPasses), slices);
   const int want = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(slices / passes, B), T / 8192));
   std::vector<int32_t> lens(B), degs(B);
   for (int b = 0; b < B; ++b) {

@@ -109,3 +109,33 @@ def test_plan_blocks_are_handed_on_only_after_the_work_that_reads_them(threads):
     o, lse = _fused(plan, q, k, v, hq, main)
     torch.cuda.synchronize()
     assert torch.equal(o, want[0][0]) and torch.equal(lse, want[0][1])
+
+
+@pytest.mark.parametrize("lens,hq,hkv,D", [
+    ([900, 130], 2, 1, 128),                        # a single slice
+    ([12000, 7000, 1001], 6, 3, 64),                # odd number of KV heads: one pass each, two kernel lanes
+    ([5000, 9000, 6000, 4000], 8, 1, 128),          # one KV head: runs of sequences only
+    ([11000, 8000, 1500, 6000], 20, 10, 128),       # passes of two KV heads and runs
+])
+def test_host_entry_point_slices(lens, hq, hkv, D):
+    """fcp_attn_fwd_bwd_host == the device calls, bit for bit where those are deterministic, on a first and a second call."""
+    from paper_2602_21788_b200 import fcp
+    from paper_2602_21788_b200.runner import DeviceState
+    w = _wl(lens, [1] * len(lens), hq, hkv, D, seed=13)
+    ds = DeviceState(w, *w.device_tensors(), partials=False)
+    ds.forward_fused()
+    ds.backward()
+    torch.cuda.synchronize()
+    ds.check_status()
+    pin = lambda t: t.cpu().pin_memory()
+    ins = [pin(t) for t in (ds.q, ds.k, ds.v, ds.do)]
+    nbytes = ds.plan.host_workspace_bytes()
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        out = [torch.zeros(t.shape, dtype=t.dtype).pin_memory() for t in (ds.o, ds.lse, ds.dq, ds.dk, ds.dv)]
+        fcp.fcp_attn_fwd_bwd_host(ds.plan, *ins, *out, ws, nbytes, torch.cuda.current_stream().cuda_stream)
+        assert ds.plan.device_status()[0] == 0
+        for got, ref in zip((out[0], out[1], out[3], out[4]), (ds.o, ds.lse, ds.dk, ds.dv)):
+            assert torch.equal(got, ref.cpu())
+        a, b = out[2].float(), ds.dq.float().cpu()
+        assert (a - b).norm() <= 1e-2 * b.norm()
