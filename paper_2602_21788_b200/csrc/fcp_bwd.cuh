@@ -30,21 +30,27 @@
 namespace fcp {
 
 constexpr int BWD_THREADS = 512;
-constexpr int BWD_QDO_STAGES = 2;
+constexpr int BWD_Q_STAGES = 2;
 constexpr int BWD_MATH_WARPS = 8;
 constexpr int BWD_DRAIN_WARPS = 4;
+constexpr int BWD_RED_COLS = 32;         // dQ columns per staged piece
+constexpr int BWD_RED_BYTES = 128 * BWD_RED_COLS * 4;
 
 template <int D>
 struct BwdSmem {
+  // D = 128 has room for one dO tile: it is read by T2 at the start of a tile's turn and last by T3, and the next tile's T2
+  // comes three products later, time enough for the load.
+  static constexpr int DO_STAGES = D == 128 ? 1 : 2;
   static constexpr int TILE_BYTES = 128 * D * 2;
   static constexpr int K_OFF = 0;
   static constexpr int V_OFF = TILE_BYTES;
   static constexpr int DS_OFF = 2 * TILE_BYTES;                         // [2][128 keys][64 q] bf16, swizzled
   static constexpr int Q_OFF = DS_OFF + 128 * 128 * 2;
-  static constexpr int DO_OFF = Q_OFF + BWD_QDO_STAGES * TILE_BYTES;
-  static constexpr int ROWS_OFF = DO_OFF + BWD_QDO_STAGES * TILE_BYTES;  // [2 buffers][lse2[128], delta[128]] fp32
+  static constexpr int DO_OFF = Q_OFF + BWD_Q_STAGES * TILE_BYTES;
+  static constexpr int RED_OFF = DO_OFF + DO_STAGES * TILE_BYTES;       // two pieces of a dQ tile on their way to the accumulator
+  static constexpr int ROWS_OFF = RED_OFF + 2 * BWD_RED_BYTES;          // [2 buffers][lse2[128], delta[128]] fp32
   static constexpr int BAR_OFF = ROWS_OFF + 2048;
-  static constexpr int N_BARS = 2 + 2 * BWD_QDO_STAGES + 9 + 4;
+  static constexpr int N_BARS = 2 + 2 * BWD_Q_STAGES + 4 + 9 + 4 + 4;
   static constexpr int MISC_OFF = BAR_OFF + N_BARS * 8;                  // tmem base, abort flag, work ring [2][2]
   static constexpr int TOTAL = MISC_OFF + 32;
   // The tiles need 1024-byte alignment.  The dynamic shared window of a kernel without static shared
@@ -66,7 +72,7 @@ struct BwdArgs {
   const float* delta_t;     // [hq_acc][t_stride], minus delta, already multiplied by the softmax scale
   const float* lse2_t;      // [hq_acc][t_stride], minus the log-sum-exp, log2 units
   const int32_t* first_query;   // [T] or nullptr (causal): first query (packed index) that sees key t
-  float* dq_acc;            // fp32, zero-initialised: [T][hq_acc][D] (D = 128), blocked for D = 64 (see dq_block)
+  float* dq_acc;            // [hq_acc][T][D] fp32, zero-initialised, tile by tile in the order of dq_tile
   __nv_bfloat16* dk;        // [T][hkv][D]
   __nv_bfloat16* dv;
   int32_t* status;
@@ -126,24 +132,23 @@ struct BwdIter {
 __device__ __forceinline__ void red_add_f32(float* p, float v) {
   asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
 }
-__device__ __forceinline__ void red_add_v4_f32(float* p, float a, float b, float c, float d) {
-  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+// dQ accumulator: the rows of one Q tile (128 packed rows from the start of a sequence on, fewer at its end) of one head
+// are rows * D consecutive floats, ordered [D / 4][rows][4].  A drain thread holds one query row, so its 16-byte pieces
+// lie next to those of its neighbours both in shared memory (no bank conflicts) and here, and a piece of 32 columns is
+// one contiguous reduction of 16 KB.
+__device__ __forceinline__ float* dq_tile(float* acc, int64_t T, int D, int h, int64_t row0) {
+  return acc + ((int64_t)h * T + row0) * D;
 }
-
-// dQ accumulator of D = 64: per query head, blocks of 128 packed token rows (the last one of T % 128 rows), within a block
-// [D / 4][rows][4].  The dQ tile has the query rows along the TMEM lanes (a transposed one would be an M = 64 product at
-// half the rate), so a drain warp holds 32 consecutive rows, one per lane, and each of its 16-byte reductions covers 512
-// contiguous bytes whatever row the tile starts at; with plain rows every lane would touch a line of its own.  Returns
-// the address of (head, row t, columns 0..3); `step` is the distance in bytes to the next four columns.
-// Ragged 16K batch, D = 64: kernel 308 -> 221 us (249 without the pauses between the reductions).
-// At D = 128 the same layout is slower (128K bimodal batch 102 -> 117 ms): there the rate of the reductions in the L2
-// bounds, and the transposed tile's 128-byte scalar ones run faster than four-wide ones.
-template <int D>
-__device__ __forceinline__ char* dq_block(float* acc, int64_t T, int h, int64_t t, uint32_t& step) {
-  const int64_t blk = t >> 7;
-  step = 16u * (uint32_t)(blk == (T >> 7) ? (T & 127) : 128);
-  return reinterpret_cast<char*>(acc) + ((int64_t)h * T + (blk << 7)) * (D * 4) + (t & 127) * 16;
+// Asynchronous reduction of `bytes` contiguous fp32 values from shared into global memory.
+__device__ __forceinline__ void bulk_red_add_f32(float* dst, uint32_t src, uint32_t bytes) {
+  asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {   // all but the last N reductions have read their shared memory
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // Two element-wise operations of a math warp, as one two-wide instruction (WIDE) or two scalar ones.  Both give the same
 // bits.  Two-wide is faster at D = 64 (kernel -4 %), where the tile's products are short and the math warps are what
@@ -168,7 +173,6 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   constexpr uint32_t BLK_BYTES = 128 * 128;
   constexpr uint32_t TMEM_COLS = 512;
   constexpr uint32_t C_S = 0, C_DP = 128, C_DV = 256, C_DK = 384;
-  constexpr bool DQ_T = (D == 128);            // dQ tile kept transposed in TMEM (rows = head-dim index)
 
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sbase = smem_u32(smem);
@@ -182,10 +186,12 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   }
   const uint32_t bar0 = sbase + SM::BAR_OFF;
   auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
-  const int B_KVFULL = 0, B_KVFREE = 1, B_QDOFULL = 2, B_QDOFREE = 2 + BWD_QDO_STAGES, B0 = 2 + 2 * BWD_QDO_STAGES;
+  constexpr int DO_STAGES = SM::DO_STAGES;
+  const int B_KVFULL = 0, B_KVFREE = 1, B_QFULL = 2, B_QFREE = B_QFULL + BWD_Q_STAGES, B_DOFULL = B_QFREE + BWD_Q_STAGES,
+            B_DOFREE = B_DOFULL + 2, B0 = B_DOFREE + 2;
   const int B_SFULL = B0, B_DPFULL = B0 + 1, B_PFULL = B0 + 2, B_DSFULL = B0 + 3, B_DQFULL = B0 + 4,
             B_DQEMPTY = B0 + 5, B_ACCFULL = B0 + 6, B_ACCEMPTY = B0 + 7, B_ROWS = B0 + 8, B_WFULL = B0 + 9,
-            B_WEMPTY = B0 + 11;
+            B_WEMPTY = B0 + 11, B_REDFULL = B0 + 13, B_REDFREE = B0 + 15;
   volatile uint32_t* tmem_slot = (volatile uint32_t*)(smem + SM::MISC_OFF);
   volatile int* abort_flag = (volatile int*)(smem + SM::MISC_OFF + 4);
   volatile int* work_ring = (volatile int*)(smem + SM::MISC_OFF + 8);    // [2 slots][unit, kv head]
@@ -197,9 +203,13 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     *abort_flag = 0;
     mbar_init(BAR(B_KVFULL), 1);
     mbar_init(BAR(B_KVFREE), 1);
-    for (int i = 0; i < BWD_QDO_STAGES; ++i) {
-      mbar_init(BAR(B_QDOFULL + i), 1);
-      mbar_init(BAR(B_QDOFREE + i), 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(BAR(B_QFULL + i), 1);
+      mbar_init(BAR(B_QFREE + i), 1);
+      mbar_init(BAR(B_DOFULL + i), 1);
+      mbar_init(BAR(B_DOFREE + i), 1);
+      mbar_init(BAR(B_REDFULL + i), BWD_DRAIN_WARPS);
+      mbar_init(BAR(B_REDFREE + i), 1);
     }
     mbar_init(BAR(B_SFULL), 1);
     mbar_init(BAR(B_DPFULL), 1);
@@ -212,7 +222,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     mbar_init(BAR(B_ROWS), BWD_MATH_WARPS);
     for (int i = 0; i < 2; ++i) {
       mbar_init(BAR(B_WFULL + i), 1);
-      mbar_init(BAR(B_WEMPTY + i), 1 + BWD_MATH_WARPS + BWD_DRAIN_WARPS);   // issuer + one lane per consumer warp
+      mbar_init(BAR(B_WEMPTY + i), 2 + BWD_MATH_WARPS + BWD_DRAIN_WARPS);   // issuer, reducer + one lane per consumer warp
     }
     fence_mbar_init();
     prefetch_tmap(&tm_q);
@@ -280,24 +290,27 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         BwdIter iter;
 #pragma unroll 1
         for (iter.init(U, a.qranges, g); iter.valid; iter.advance(), ++it) {
-          const uint32_t st = it % BWD_QDO_STAGES;
-          ok = mbar_wait(BAR(B_QDOFREE + st), ((it / BWD_QDO_STAGES) & 1) ^ 1, wctx, 111);
-          if (!ok) break;
-          mbar_expect_tx(BAR(B_QDOFULL + st), 2 * SM::TILE_BYTES);
+          const uint32_t st = it % BWD_Q_STAGES, sd = it % DO_STAGES;
           const int h = hk * g + iter.hh;
+          ok = mbar_wait(BAR(B_QFREE + st), ((it / BWD_Q_STAGES) & 1) ^ 1, wctx, 111);
+          if (!ok) break;
+          mbar_expect_tx(BAR(B_QFULL + st), SM::TILE_BYTES);
 #pragma unroll 1
-          for (int kb = 0; kb < KBLK; ++kb) {
-            tma_load_3d(sbase + SM::Q_OFF + st * SM::TILE_BYTES + kb * BLK_BYTES, &tm_q, BAR(B_QDOFULL + st), kb * 64, h, iter.q_row);
-            tma_load_3d(sbase + SM::DO_OFF + st * SM::TILE_BYTES + kb * BLK_BYTES, &tm_do, BAR(B_QDOFULL + st), kb * 64, h, iter.q_row);
-          }
+          for (int kb = 0; kb < KBLK; ++kb)
+            tma_load_3d(sbase + SM::Q_OFF + st * SM::TILE_BYTES + kb * BLK_BYTES, &tm_q, BAR(B_QFULL + st), kb * 64, h, iter.q_row);
+          ok = mbar_wait(BAR(B_DOFREE + sd), ((it / DO_STAGES) & 1) ^ 1, wctx, 113);
+          if (!ok) break;
+          mbar_expect_tx(BAR(B_DOFULL + sd), SM::TILE_BYTES);
+#pragma unroll 1
+          for (int kb = 0; kb < KBLK; ++kb)
+            tma_load_3d(sbase + SM::DO_OFF + sd * SM::TILE_BYTES + kb * BLK_BYTES, &tm_do, BAR(B_DOFULL + sd), kb * 64, h, iter.q_row);
         }
       }
     } else if (warp == 1 && lane == 0) {
       // ------------------------------------------------------------------ UMMA issuer
       constexpr uint32_t IDESC_ST = make_idesc(128, 128, 0, 0);   // K-major x K-major -> [keys][queries]
       constexpr uint32_t IDESC_ACC = make_idesc(128, D, 0, 1);    // TMEM A, MN-major B -> dV, dK
-      constexpr uint32_t IDESC_DQ = DQ_T ? make_idesc(128, 128, 1, 1)   // K^T (MN-major) x dS^T (MN-major)
-                                         : make_idesc(128, D, 1, 1);    // dS (MN-major) x K (MN-major)
+      constexpr uint32_t IDESC_DQ = make_idesc(128, D, 1, 1);     // dS (MN-major) x K (MN-major)
       uint32_t n = 0, it = 0;
       bool ok = true;
       const uint32_t kbase = sbase + SM::K_OFF, vbase = sbase + SM::V_OFF, dsbase = sbase + SM::DS_OFF;
@@ -319,21 +332,23 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll 1
         for (int i = -1; i < n_iter && ok; ++i) {
           const bool cur = i >= 0, next = i + 1 < n_iter;
-          const uint32_t st = (it + 1) % BWD_QDO_STAGES, st_next = it % BWD_QDO_STAGES;   // tile i is tile it - 1
-          const uint32_t qbase = sbase + SM::Q_OFF + st * SM::TILE_BYTES, dobase = sbase + SM::DO_OFF + st * SM::TILE_BYTES;
+          const uint32_t st = (it + 1) % BWD_Q_STAGES, st_next = it % BWD_Q_STAGES;   // tile i is tile it - 1
+          const uint32_t sd = (it + DO_STAGES - 1) % DO_STAGES, sd_next = it % DO_STAGES;
+          const uint32_t qbase = sbase + SM::Q_OFF + st * SM::TILE_BYTES, dobase = sbase + SM::DO_OFF + sd * SM::TILE_BYTES;
           bool q_ready = false, ds_ready = false;
           if (cur) {
             // T3: dV += P^T dO
             if (!p_ready) ok = mbar_wait(BAR(B_PFULL), (it - 1) & 1, wctx, 123);
             if (ok && i == 0) ok = mbar_wait(BAR(B_ACCEMPTY), (n & 1) ^ 1, wctx, 124);
             if (!ok) break;
-            if (next) q_ready = mbar_test(BAR(B_QDOFULL + st_next), (it / BWD_QDO_STAGES) & 1);
+            if (next) q_ready = mbar_test(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1);
             tc_fence_after();
             umma_loop_ts(true, tmem + C_DV, tmem + C_S, true, dobase, IDESC_ACC, i > 0 ? 1u : 0u);
+            tc_commit(BAR(B_DOFREE + sd));
           }
           // T1 of the next tile: S^T has been read by the math warps and P^T is consumed in order
           if (next) {
-            if (!q_ready) ok = mbar_wait(BAR(B_QDOFULL + st_next), (it / BWD_QDO_STAGES) & 1, wctx, 126);
+            if (!q_ready) ok = mbar_wait(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1, wctx, 126);
             if (!ok) break;
             if (cur) ds_ready = mbar_test(BAR(B_DSFULL), (it - 1) & 1);
             tc_fence_after();
@@ -346,20 +361,20 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (!ds_ready) ok = mbar_wait(BAR(B_DSFULL), (it - 1) & 1, wctx, 125);
             if (!ok) break;
             tc_fence_after();
-            if (DQ_T) umma_loop_mm(true, tmem + C_DP, kbase, dsbase, IDESC_DQ);
-            else umma_loop_mm(true, tmem + C_DP, dsbase, kbase, IDESC_DQ);
+            umma_loop_mm(true, tmem + C_DP, dsbase, kbase, IDESC_DQ);
             tc_commit(BAR(B_DQFULL));
             umma_loop_km(true, tmem + C_DK, dsbase, qbase, IDESC_ACC, i > 0 ? 1u : 0u);
-            tc_commit(BAR(B_QDOFREE + st));
+            tc_commit(BAR(B_QFREE + st));
           }
           // T2 of the next tile once the drain warps have emptied the dQ tile of the one before it
           p_ready = false;
           if (next) {
-            ok = mbar_wait(BAR(B_DQEMPTY), (it & 1) ^ 1, wctx, 127);
+            ok = mbar_wait(BAR(B_DOFULL + sd_next), (it / DO_STAGES) & 1, wctx, 128);
+            if (ok) ok = mbar_wait(BAR(B_DQEMPTY), (it & 1) ^ 1, wctx, 127);
             if (!ok) break;
             p_ready = mbar_test(BAR(B_PFULL), it & 1);
             tc_fence_after();
-            umma_loop_kk<D / 16>(true, tmem + C_DP, vbase, sbase + SM::DO_OFF + st_next * SM::TILE_BYTES, IDESC_ST);
+            umma_loop_kk<D / 16>(true, tmem + C_DP, vbase, sbase + SM::DO_OFF + sd_next * SM::TILE_BYTES, IDESC_ST);
             tc_commit(BAR(B_DPFULL));
             ++it;
           }
@@ -369,6 +384,36 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         tc_commit(BAR(B_KVFREE));
         ++n;
       }
+    } else if (warp == 2 && lane == 0) {
+      // ------------------------------------------------------------------ dQ reducer
+      uint32_t n = 0, piece = 0;
+      bool ok = true;
+      while (ok) {
+        const uint32_t slot = n & 1;
+        ok = mbar_wait(BAR(B_WFULL + slot), (n >> 1) & 1, wctx, 142);
+        if (!ok) break;
+        const int unit = work_ring[2 * slot], hk = work_ring[2 * slot + 1];
+        mbar_arrive(BAR(B_WEMPTY + slot));
+        if (unit < 0) break;
+        ++n;
+        BwdIter iter;
+#pragma unroll 1
+        for (iter.init(a.units + (size_t)unit * FCP_BWD_UNIT_W, a.qranges, g); iter.valid && ok; iter.advance()) {
+          float* dst = dq_tile(a.dq_acc, a.T, D, (hk - a.hk_begin) * g + iter.hh, iter.q_row);
+#pragma unroll 1
+          for (int c = 0; c < D / BWD_RED_COLS; ++c, ++piece) {
+            ok = mbar_wait(BAR(B_REDFULL + (piece & 1)), (piece >> 1) & 1, wctx, 143);
+            if (!ok) break;
+            bulk_red_add_f32(dst, sbase + SM::RED_OFF + (piece & 1) * BWD_RED_BYTES, iter.q_valid * BWD_RED_COLS * 4);
+            dst += iter.q_valid * BWD_RED_COLS;
+            if (piece > 0) {                 // the piece before this one has left shared memory
+              bulk_wait_read<1>();
+              mbar_arrive(BAR(B_REDFREE + ((piece - 1) & 1)));
+            }
+          }
+        }
+      }
+      bulk_wait_all();
     }
   } else if (warp < 4 + BWD_MATH_WARPS) {
     // ------------------------------------------------------------------ math warps: C1, C2
@@ -506,10 +551,10 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     // ------------------------------------------------------------------ drain warps: C3, dK/dV epilogue
     asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
     const int rb = warp & 3;
-    const int row = rb * 32 + lane;             // TMEM lane: head-dim index of dQ^T (or query row), key row of dK/dV
+    const int row = rb * 32 + lane;             // TMEM lane: query row of dQ, key row of dK/dV
     const uint32_t t_dq = tmem_addr(tmem, rb * 32, C_DP);
     const uint32_t t_dv = tmem_addr(tmem, rb * 32, C_DV), t_dk = tmem_addr(tmem, rb * 32, C_DK);
-    uint32_t n = 0, it = 0;
+    uint32_t n = 0, it = 0, piece = 0;
     bool ok = true;
     while (true) {
       int hk = 0;
@@ -519,85 +564,35 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       BwdIter iter;
 #pragma unroll 1
       for (iter.init(U, a.qranges, g); iter.valid; iter.advance(), ++it) {
-        const int h = (hk - a.hk_begin) * g + iter.hh;   // head index within the accumulators of this pass
-        const int q_row = iter.q_row, q_valid = iter.q_valid;
+        const int q_valid = iter.q_valid;
         ok = mbar_wait_warp(BAR(B_DQFULL), it & 1, wctx, 132);
         if (!ok) break;
         tc_fence_after();
-        if constexpr (DQ_T) {
-          // thread = head-dim index, columns = queries: a warp adds 32 consecutive floats per query.
-          char* dst = reinterpret_cast<char*>(a.dq_acc + ((int64_t)q_row * a.hq_acc + h) * D + row);
-          const int64_t stride = (int64_t)a.hq_acc * D * 4;
-          if (q_valid == 128) {
-            // whole tile into registers, columns handed back at once, then the reductions: they are
-            // slow (L2 round trips) and must not sit between the tile and the issuer's next product
-            uint32_t qa[64], qb[64];
+        // whole tile into registers and the columns handed back at once, then piece by piece through shared memory
+        uint32_t qv[D];
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-              tmem_ld32(t_dq + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&qa[c * 32]));
-              tmem_ld32(t_dq + 64 + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&qb[c * 32]));
-            }
-            tc_wait_ld();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(BAR(B_DQEMPTY));
-            // two rolled trips of 64 reductions (the second half moves down in between): half the
-            // code of a fully unrolled tile, which matters more to the instruction cache than the moves.
-            // The reductions are paced (a short sleep after every 16) so that they spread over the time
-            // a tile takes: sent back to back they keep the load/store queues of the SM full, and every
-            // barrier poll and shared-memory access of the other warps then waits behind them.  Measured:
-            // any pause that sums to 1.2-2 us per tile gives the same gain; 3 us makes this warp the bound.
-#pragma unroll 1
-            for (int hlf = 0; hlf < 2; ++hlf) {
+        for (int c = 0; c < D / 32; ++c) tmem_ld32(t_dq + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&qv[c * 32]));
+        tc_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(BAR(B_DQEMPTY));
 #pragma unroll
-              for (int c = 0; c < 64; ++c) {
-                red_add_f32(reinterpret_cast<float*>(dst), __uint_as_float(qa[c]));
-                dst += stride;
-                if ((c & 15) == 15) __nanosleep(200);
-              }
-#pragma unroll
-              for (int c = 0; c < 64; ++c) qa[c] = qb[c];
-            }
-          } else {
-            // ragged tile (end of a chunk): rolled loop over 16-query slices
-#pragma unroll 1
-            for (int c16 = 0; c16 < 8; ++c16) {
-              uint32_t qv[16];
-              tmem_ld16(t_dq + c16 * 16, qv);
-              tc_wait_ld();
-              if (c16 == 7) {
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(BAR(B_DQEMPTY));
-              }
-              const int nv = q_valid - c16 * 16;
-#pragma unroll
-              for (int c = 0; c < 16; ++c) {
-                if (c < nv) red_add_f32(reinterpret_cast<float*>(dst), __uint_as_float(qv[c]));
-                dst += stride;
-              }
-            }
-          }
-        } else {
-          uint32_t qv[D];
-#pragma unroll
-          for (int c = 0; c < D / 32; ++c) tmem_ld32(t_dq + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&qv[c * 32]));
-          tc_wait_ld();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(BAR(B_DQEMPTY));
-          uint32_t step;
-          char* dst = dq_block<D>(a.dq_acc, a.T, h, (int64_t)q_row + row, step);
+        for (int c = 0; c < D / BWD_RED_COLS; ++c, ++piece) {
+          ok = mbar_wait_warp(BAR(B_REDFREE + (piece & 1)), ((piece >> 1) & 1) ^ 1, wctx, 135);
+          if (!ok) break;
+          uint8_t* dst = smem + SM::RED_OFF + (piece & 1) * BWD_RED_BYTES + row * 16;
           if (row < q_valid) {
 #pragma unroll
-            for (int c = 0; c < D / 4; ++c) {
-              red_add_v4_f32(reinterpret_cast<float*>(dst), __uint_as_float(qv[4 * c]), __uint_as_float(qv[4 * c + 1]),
-                             __uint_as_float(qv[4 * c + 2]), __uint_as_float(qv[4 * c + 3]));
-              dst += step;
-              if ((c & 3) == 3) __nanosleep(200);
+            for (int i = 0; i < BWD_RED_COLS / 4; ++i) {
+              const uint32_t* v = &qv[c * BWD_RED_COLS + 4 * i];
+              *reinterpret_cast<uint4*>(dst + i * q_valid * 16) = make_uint4(v[0], v[1], v[2], v[3]);
             }
           }
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(BAR(B_REDFULL + (piece & 1)));
         }
+        if (!ok) break;
       }
       if (!ok) break;
       // unit epilogue: dK, dV rows of this key tile

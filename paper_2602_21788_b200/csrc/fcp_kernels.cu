@@ -227,41 +227,22 @@ __global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* __r
   }
 }
 
-// fp32 dQ accumulator [T][hc][D] -> bf16 dq [T][hq][D], heads [h0, h0 + hc); n8 = T*hc*D/8 groups of
-// eight values, row8 = hc*D/8 groups per token of the accumulator
+// fp32 dQ accumulator (tiles of dq_tile: [D / 4][rows][4]) -> bf16 dq [T][hq][D], heads [h0, h0 + gridDim.y).  One CTA per
+// (tile, head): it reads rows * D contiguous floats with lanes along the rows and turns them round in shared memory, so
+// that both sides move whole sectors.  Q tiles are cut like key tiles, so the backward units list them.
+template <int D>
 __global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq,
-                                                             int64_t n8, int64_t row8, int64_t dst_row8, int64_t dst_off8) {
+                                                             const int32_t* __restrict__ units, int64_t T, int hq, int h0) {
   grid_begin();
-  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n8; i += (int64_t)gridDim.x * 256) {
-    const float4 a = __ldcs(reinterpret_cast<const float4*>(acc) + 2 * i);
-    const float4 b = __ldcs(reinterpret_cast<const float4*>(acc) + 2 * i + 1);
-    uint4 pk;
-    pk.x = pack_bf16(a.x, a.y); pk.y = pack_bf16(a.z, a.w);
-    pk.z = pack_bf16(b.x, b.y); pk.w = pack_bf16(b.z, b.w);
-    int64_t j = i;
-    if (row8 != dst_row8) {
-      const int64_t t = i / row8;
-      j = t * dst_row8 + dst_off8 + (i - t * row8);
-    }
-    reinterpret_cast<uint4*>(dq)[j] = pk;
-  }
-}
-
-// The same from the blocked accumulator of D = 64 (dq_block): one CTA per (block of 128 rows, head) reads the block's
-// contiguous 128 * D floats with lanes along the rows and turns it round in shared memory, so that both sides move
-// whole sectors.
-__global__ void __launch_bounds__(256) fcp_dq_convert_blocked_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq,
-                                                                     int64_t T, int hq, int h0) {
-  grid_begin();
-  constexpr int D = 64;
   constexpr int PITCH = D + 8;                // bf16 elements per row in shared memory: 16 bytes of padding
   __shared__ __align__(16) __nv_bfloat16 tile[128 * PITCH];
-  const int64_t t0 = (int64_t)blockIdx.x * 128;
-  const int rows = (int)min((int64_t)128, T - t0);
+  const int32_t* U = units + (size_t)blockIdx.x * FCP_BWD_UNIT_W;
+  const int64_t t0 = __ldg(U + BU_KV_ROW0);
+  const int rows = __ldg(U + BU_KV_ROWS);
   const float4* src = reinterpret_cast<const float4*>(acc + ((int64_t)blockIdx.y * T + t0) * D);
   const int row = threadIdx.x & 127;
   if (row < rows) {
-#pragma unroll
+#pragma unroll 8
     for (int c = threadIdx.x >> 7; c < D / 4; c += 2) {
       const float4 v = __ldcs(src + c * rows + row);
       *reinterpret_cast<uint2*>(tile + row * PITCH + c * 4) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
@@ -776,14 +757,12 @@ int run_bwd(const fcp_plan* plan, const BwdTables& tb, const void* q, const void
       FCP_CUDA_CHECK(launch(fcp_bwd_kernel<64>, grid, BWD_THREADS, BwdSmem<64>::DYN_BYTES, st, tq, tk, tv, tdo, a));
   }
   {
-    const int64_t n8 = T * hc * D / 8;
-    const int blocks = (int)std::min<int64_t>((n8 + 255) / 256, (int64_t)tb.sm_count * 16);
+    const dim3 grid_c((unsigned)a.n_units, (unsigned)hc);
     ProfScope ps(prof, 4, st);
     if (D == 128)
-      FCP_CUDA_CHECK(launch(fcp_dq_convert_kernel, blocks, 256, 0, st, dq_acc, (__nv_bfloat16*)dq, n8, hc * D / 8, P.hq * D / 8, h0 * D / 8));
+      FCP_CUDA_CHECK(launch(fcp_dq_convert_kernel<128>, grid_c, 256, 0, st, dq_acc, (__nv_bfloat16*)dq, tb.units, T, P.hq, h0));
     else
-      FCP_CUDA_CHECK(launch(fcp_dq_convert_blocked_kernel, dim3((unsigned)((T + 127) / 128), (unsigned)hc), 256, 0, st, dq_acc,
-                            (__nv_bfloat16*)dq, T, P.hq, h0));
+      FCP_CUDA_CHECK(launch(fcp_dq_convert_kernel<64>, grid_c, 256, 0, st, dq_acc, (__nv_bfloat16*)dq, tb.units, T, P.hq, h0));
   }
   return FCP_OK;
 }

@@ -542,11 +542,11 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
   // Backward: one unit per 128-key tile; it visits the Q rows of all block pairs whose kv_chunk holds
   // its keys (q_chunk >= kv_chunk), the DIAG pair from its own tile on.  The Q ranges of a KV chunk
   // are its pairs in q_chunk order with adjacent ranges joined (a DIAG range followed by the FULL
-  // ranges of the later chunks is one DIAG range up to their end).  When every KV chunk of a sequence
-  // ends up with the single range [chunk start, sequence end) DIAG -- the causal plan -- the key
-  // tiles are cut from the start of the sequence instead of from each chunk start (a key tile may
-  // then span two KV chunks; the causal mask only depends on token positions), so that neither key
-  // tiles nor query tiles are cut at chunk edges.
+  // ranges of the later chunks is one DIAG range up to their end).  Every KV chunk of a sequence ends
+  // up with the single range [chunk start, sequence end) DIAG, so the key tiles are cut from the start
+  // of the sequence instead of from each chunk start (a key tile may then span two KV chunks; the
+  // causal mask only depends on token positions): neither key tiles nor query tiles are cut at chunk
+  // edges, and a query tile has the same rows for every key tile.
   struct BU { int32_t f[FCP_BWD_UNIT_W]; };
   std::vector<BU> bus;
   {
@@ -607,18 +607,13 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
         }
         return first;
       };
-      if (causal_seq) {
-        const std::vector<Range> whole{Range{t0, t1, 1}};
-        emit_tiles(t0, t1, push_ranges(whole), whole, has_spans);
-      } else {
-        if (has_spans) {
-          delete p;
-          fcp_set_error("fcp_plan_blocks_spans: sequence %d has spans but its block pairs are not the causal set", b);
-          return FCP_ERR_UNSUPPORTED;
-        }
-        for (int c = 0; c < nc; ++c)
-          if (!kv_cover[c].empty()) emit_tiles(cbp[c], cbp[c + 1], push_ranges(kv_cover[c]), kv_cover[c], false);
+      if (!causal_seq) {                         // the dQ accumulator is laid out by Q tiles cut from the sequence start
+        delete p;
+        fcp_set_error("fcp_plan_blocks: the block pairs of sequence %d are not the causal set", b);
+        return FCP_ERR_UNSUPPORTED;
       }
+      const std::vector<Range> whole{Range{t0, t1, 1}};
+      emit_tiles(t0, t1, push_ranges(whole), whole, has_spans);
     }
   }
   for (const BU& u : bus) p->bwd_units.insert(p->bwd_units.end(), u.f, u.f + FCP_BWD_UNIT_W);
