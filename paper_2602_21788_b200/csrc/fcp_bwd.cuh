@@ -327,7 +327,8 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         if (!ok) break;
         // Software pipeline over the unit's tiles: trip i issues T3, T4, T5 of tile i and T1, T2 of tile
         // i + 1; trip -1 only starts the first tile.  `it` counts the tiles whose T1/T2 have been issued.
-        // Each barrier is looked at (mbar_test) one UMMA batch before it is needed.
+        // Each barrier is looked at (mbar_test) two UMMAs before the end of the product in front of its use: late enough for
+        // it to be complete, early enough for the answer to arrive while those two are issued.
         bool p_ready = false;
 #pragma unroll 1
         for (int i = -1; i < n_iter && ok; ++i) {
@@ -335,24 +336,26 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           const uint32_t st = (it + 1) % BWD_Q_STAGES, st_next = it % BWD_Q_STAGES;   // tile i is tile it - 1
           const uint32_t sd = (it + DO_STAGES - 1) % DO_STAGES, sd_next = it % DO_STAGES;
           const uint32_t qbase = sbase + SM::Q_OFF + st * SM::TILE_BYTES, dobase = sbase + SM::DO_OFF + sd * SM::TILE_BYTES;
-          bool q_ready = false, ds_ready = false;
+          bool q_ready = false, ds_ready = false, do_ready = false, dq_free = false;
           if (cur) {
             // T3: dV += P^T dO
             if (!p_ready) ok = mbar_wait(BAR(B_PFULL), (it - 1) & 1, wctx, 123);
             if (ok && i == 0) ok = mbar_wait(BAR(B_ACCEMPTY), (n & 1) ^ 1, wctx, 124);
             if (!ok) break;
-            if (next) q_ready = mbar_test(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1);
             tc_fence_after();
-            umma_loop_ts(true, tmem + C_DV, tmem + C_S, true, dobase, IDESC_ACC, i > 0 ? 1u : 0u);
+            umma_loop_ts<0, 6>(true, tmem + C_DV, tmem + C_S, true, dobase, IDESC_ACC, i > 0 ? 1u : 0u);
+            if (next) q_ready = mbar_test(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1);
+            umma_loop_ts<6, 8>(true, tmem + C_DV, tmem + C_S, true, dobase, IDESC_ACC, 1u);
             tc_commit(BAR(B_DOFREE + sd));
           }
           // T1 of the next tile: S^T has been read by the math warps and P^T is consumed in order
           if (next) {
             if (!q_ready) ok = mbar_wait(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1, wctx, 126);
             if (!ok) break;
-            if (cur) ds_ready = mbar_test(BAR(B_DSFULL), (it - 1) & 1);
             tc_fence_after();
-            umma_loop_kk<D / 16>(true, tmem + C_S, kbase, sbase + SM::Q_OFF + st_next * SM::TILE_BYTES, IDESC_ST);
+            umma_loop_kk<0, D / 16 - 2>(true, tmem + C_S, kbase, sbase + SM::Q_OFF + st_next * SM::TILE_BYTES, IDESC_ST);
+            if (cur) ds_ready = mbar_test(BAR(B_DSFULL), (it - 1) & 1);
+            umma_loop_kk<D / 16 - 2, D / 16>(true, tmem + C_S, kbase, sbase + SM::Q_OFF + st_next * SM::TILE_BYTES, IDESC_ST);
             tc_commit(BAR(B_SFULL));
           }
           if (cur) {
@@ -363,18 +366,22 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             tc_fence_after();
             umma_loop_mm(true, tmem + C_DP, dsbase, kbase, IDESC_DQ);
             tc_commit(BAR(B_DQFULL));
-            umma_loop_km(true, tmem + C_DK, dsbase, qbase, IDESC_ACC, i > 0 ? 1u : 0u);
+            if (next) do_ready = mbar_test(BAR(B_DOFULL + sd_next), (it / DO_STAGES) & 1);
+            umma_loop_km<0, 6>(true, tmem + C_DK, dsbase, qbase, IDESC_ACC, i > 0 ? 1u : 0u);
+            if (next) dq_free = mbar_test(BAR(B_DQEMPTY), (it & 1) ^ 1);
+            umma_loop_km<6, 8>(true, tmem + C_DK, dsbase, qbase, IDESC_ACC, 1u);
             tc_commit(BAR(B_QFREE + st));
           }
           // T2 of the next tile once the drain warps have emptied the dQ tile of the one before it
           p_ready = false;
           if (next) {
-            ok = mbar_wait(BAR(B_DOFULL + sd_next), (it / DO_STAGES) & 1, wctx, 128);
-            if (ok) ok = mbar_wait(BAR(B_DQEMPTY), (it & 1) ^ 1, wctx, 127);
+            if (!do_ready) ok = mbar_wait(BAR(B_DOFULL + sd_next), (it / DO_STAGES) & 1, wctx, 128);
+            if (ok && !dq_free) ok = mbar_wait(BAR(B_DQEMPTY), (it & 1) ^ 1, wctx, 127);
             if (!ok) break;
-            p_ready = mbar_test(BAR(B_PFULL), it & 1);
             tc_fence_after();
-            umma_loop_kk<D / 16>(true, tmem + C_DP, vbase, sbase + SM::DO_OFF + sd_next * SM::TILE_BYTES, IDESC_ST);
+            umma_loop_kk<0, D / 16 - 2>(true, tmem + C_DP, vbase, sbase + SM::DO_OFF + sd_next * SM::TILE_BYTES, IDESC_ST);
+            p_ready = mbar_test(BAR(B_PFULL), it & 1);
+            umma_loop_kk<D / 16 - 2, D / 16>(true, tmem + C_DP, vbase, sbase + SM::DO_OFF + sd_next * SM::TILE_BYTES, IDESC_ST);
             tc_commit(BAR(B_DPFULL));
             ++it;
           }
@@ -420,11 +427,15 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
     const int rb = warp & 3;                    // TMEM lane quarter
     const int half = (warp - 4) >> 2;           // which 64 of the 128 query columns
-    const int row = rb * 32 + lane;             // key row of S^T / dP^T
     const int mtid = threadIdx.x - 128;         // 0..255 among the math threads
     const uint32_t t_s = tmem_addr(tmem, rb * 32, C_S + half * 64), t_dp = tmem_addr(tmem, rb * 32, C_DP + half * 64);
     const float2 c22 = make_float2(a.scale_log2, a.scale_log2), s22 = make_float2(a.scale, a.scale);
-    uint8_t* ds_row = smem + SM::DS_OFF + half * BLK_BYTES + row * 128;
+    // A thread holds fragments of the tile: key rows frow + 8 * i (i = 0..3) and, in each group of 8 queries, the queries
+    // fcol and fcol + 1.  Four rows share every per-query statistic that is read from shared memory.
+    const int frow = rb * 32 + (lane >> 2), fcol = 2 * (lane & 3);
+    // this lane's row of the 8 x 8 matrices it addresses for stmatrix_x4 (rows + 8 * (matrix % 2)), and its 16-byte chunk
+    const int mrow = rb * 32 + (lane & 7) + ((lane >> 3) & 1) * 8, mch = lane >> 4;
+    const uint32_t ds_row = sbase + SM::DS_OFF + half * BLK_BYTES + mrow * 128;
     // this thread's share of the per-query-row statistics: lse2 (threads 0..127) or delta (128..255)
     const float* my_rows = (mtid < 128 ? a.lse2_t : a.delta_t) + (mtid & 127);
     auto load_row = [&](const BwdIter& x, int hk) -> float {
@@ -438,8 +449,13 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const int32_t* U = next_work(n++, hk, ok);
       if (!U) break;
       const int kv_row0 = __ldg(U + BU_KV_ROW0), kv_rows = __ldg(U + BU_KV_ROWS);
-      // first query that sees this thread's key row: the key itself, or the begin of its span
-      const int first_q = (a.first_query != nullptr && row < kv_rows) ? __ldg(a.first_query + kv_row0 + row) : kv_row0 + row;
+      // first query that sees each of this thread's key rows: the key itself, or the begin of its span
+      int first_q[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int row = frow + 8 * i;
+        first_q[i] = (a.first_query != nullptr && row < kv_rows) ? __ldg(a.first_query + kv_row0 + row) : kv_row0 + row;
+      }
       BwdIter iter;
       iter.init(U, a.qranges, g);
       float pre = load_row(iter, hk);
@@ -466,43 +482,43 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         ok = mbar_wait_warp(BAR(B_SFULL), it & 1, wctx, 130);
         if (!ok) break;
         tc_fence_after();
-        // P^T of this key row and column half as bf16 pairs: pa = query columns [0,32), pb = [32,64).
-        // C1 and C2 run as two rolled trips of 32 columns; between the trips the pair arrays rotate
-        // (register arrays cannot be indexed by the trip), which halves the code of this loop.
+        // P^T fragments as bf16 pairs: pa = query columns [0,32) of this half, pb = [32,64); element 8 * g + 2 * j + i is
+        // the pair of row frow + 16 * g + 8 * i and query group j.  C1 and C2 run as two rolled trips of 32 columns;
+        // between the trips the pair arrays rotate (register arrays cannot be indexed by the trip), which halves the
+        // code of this loop.
         uint32_t pa[16], pb[16] = {};
-        unsigned long long keep = ~0ull;
-        if (need_mask) {
-          // valid query columns of this key row, relative to this warp's half: [lo, hi).  Bit j of
-          // `keep` = column j survives; applied to the packed pairs.
-          const int hi = min(64, max(0, (row < kv_rows ? q_valid : 0) - half * 64));
-          const int lo = min(64, max(0, (causal ? first_q - q_row : 0) - half * 64));
-          keep = (hi > lo) ? ((hi == 64 ? ~0ull : ((1ull << hi) - 1)) & ~((1ull << lo) - 1)) : 0ull;
-        }
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           uint32_t sv[32];
-          tmem_ld32(t_s + c * 32, sv);
+          tmem_ld_frag(t_s + c * 32, sv);
+          tmem_ld_frag(t_s + (16u << 16) + c * 32, sv + 16);
 #pragma unroll
           for (int j = 0; j < 16; ++j) pa[j] = pb[j];
           tc_wait_ld();
-          const float* lse_c = s_lse + c * 32;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float4 l4 = *reinterpret_cast<const float4*>(lse_c + 4 * i);
-            const float2 e0 = fma_pair<D == 64>(sv[4 * i], sv[4 * i + 1], c22, make_float2(l4.x, l4.y));
-            const float2 e1 = fma_pair<D == 64>(sv[4 * i + 2], sv[4 * i + 3], c22, make_float2(l4.z, l4.w));
-            pb[2 * i] = pack_bf16(ex2(e0.x), ex2(e0.y));
-            pb[2 * i + 1] = pack_bf16(ex2(e1.x), ex2(e1.y));
-          }
-          if (need_mask) {
-            const uint32_t k32 = (uint32_t)(keep >> (32 * c));
+          for (int j = 0; j < 4; ++j) {
+            const float2 l2 = *reinterpret_cast<const float2*>(s_lse + c * 32 + 8 * j + fcol);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const uint32_t b2 = (k32 >> (2 * j)) & 3u;
-              pb[j] &= (b2 & 1u ? 0x0000ffffu : 0u) | (b2 & 2u ? 0xffff0000u : 0u);
+            for (int g2 = 0; g2 < 4; ++g2) {               // row frow + 8 * g2
+              const uint32_t* x = &sv[(g2 >> 1) * 16 + 4 * j + 2 * (g2 & 1)];
+              const float2 e = fma_pair<D == 64>(x[0], x[1], c22, l2);
+              pb[(g2 >> 1) * 8 + 2 * j + (g2 & 1)] = pack_bf16(ex2(e.x), ex2(e.y));
             }
           }
-          tmem_st16(t_s + c * 16, pb);            // over this warp's own, already loaded, columns
+          if (need_mask) {
+            // columns of this trip a key row keeps: [lo, hi)
+#pragma unroll
+            for (int g2 = 0; g2 < 4; ++g2) {
+              const int off = half * 64 + c * 32 + fcol;
+              const int hi = (frow + 8 * g2 < kv_rows ? q_valid : 0) - off, lo = (causal ? first_q[g2] - q_row : 0) - off;
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                pb[(g2 >> 1) * 8 + 2 * j + (g2 & 1)] &= (8 * j >= lo && 8 * j < hi ? 0x0000ffffu : 0u) |
+                                                        (8 * j + 1 >= lo && 8 * j + 1 < hi ? 0xffff0000u : 0u);
+            }
+          }
+          tmem_st_frag(t_s + c * 16, pb);            // over this warp's own, already loaded, columns
+          tmem_st_frag(t_s + (16u << 16) + c * 16, pb + 8);
         }
         tc_wait_st();
         tc_fence_before();
@@ -514,30 +530,29 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         tc_fence_after();
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
-          uint32_t dv_[32];
-          tmem_ld32(t_dp + c * 32, dv_);
+          uint32_t dv_[32], out[16];
+          tmem_ld_frag(t_dp + c * 32, dv_);
+          tmem_ld_frag(t_dp + (16u << 16) + c * 32, dv_ + 16);
           tc_wait_ld();
-          const float* delta_c = s_delta + c * 32;
-          uint32_t out[16];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float4 d4 = *reinterpret_cast<const float4*>(delta_c + 4 * i);
-            const uint32_t pp = pa[2 * i], pq = pa[2 * i + 1];
-            const float2 f0 = fma_pair<D == 64>(dv_[4 * i], dv_[4 * i + 1], s22, make_float2(d4.x, d4.y));
-            const float2 f1 = fma_pair<D == 64>(dv_[4 * i + 2], dv_[4 * i + 3], s22, make_float2(d4.z, d4.w));
-            const float2 d0 = mul_pair<D == 64>(f0, pp), d1 = mul_pair<D == 64>(f1, pq);
-            out[2 * i] = pack_bf16(d0.x, d0.y);
-            out[2 * i + 1] = pack_bf16(d1.x, d1.y);
+          for (int j = 0; j < 4; ++j) {
+            const float2 d2 = *reinterpret_cast<const float2*>(s_delta + c * 32 + 8 * j + fcol);
+#pragma unroll
+            for (int g2 = 0; g2 < 4; ++g2) {
+              const uint32_t* x = &dv_[(g2 >> 1) * 16 + 4 * j + 2 * (g2 & 1)];
+              const int e = (g2 >> 1) * 8 + 2 * j + (g2 & 1);
+              const float2 d = mul_pair<D == 64>(fma_pair<D == 64>(x[0], x[1], s22, d2), pa[e]);
+              out[e] = pack_bf16(d.x, d.y);
+            }
           }
 #pragma unroll
           for (int j = 0; j < 16; ++j) pa[j] = pb[j];
-          // 32 values -> shared memory, keys x queries with queries contiguous (the K-major A operand
-          // of the dK product and the MN-major B operand of the dQ product): 4 x 16-byte chunks, 128-byte swizzle
+          // 32 x 32 values -> shared memory, keys x queries with queries contiguous (the K-major A operand of the dK
+          // product and the MN-major A operand of the dQ product), 128-byte swizzle: 16-byte chunk ^ (row & 7)
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
-            const int cc = c * 4 + ch;                          // 16-byte chunk within this half's 128-byte row
-            uint4 v4 = make_uint4(out[ch * 4], out[ch * 4 + 1], out[ch * 4 + 2], out[ch * 4 + 3]);
-            *reinterpret_cast<uint4*>(ds_row + ((cc ^ (row & 7)) << 4)) = v4;
+          for (int m = 0; m < 4; ++m) {                    // rows + 16 * (m / 2), query groups 2 * (m % 2) and the next
+            const int cc = c * 4 + 2 * (m & 1) + mch;
+            stmatrix_x4(ds_row + (m >> 1) * 2048 + ((cc ^ (lane & 7)) << 4), &out[(m >> 1) * 8 + 4 * (m & 1)]);
           }
         }
         fence_proxy_async_smem();

@@ -274,7 +274,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (!ok) break;
             if (sb) ++xcnt1; else ++xcnt0;
             tc_fence_after();
-            umma_loop_kk<D / 16>(true, tmem + S_COL0 + sb * 128, sbase + SM::Q_OFF + s * SM::Q_TILE_BYTES,
+            umma_loop_kk<0, D / 16>(true, tmem + S_COL0 + sb * 128, sbase + SM::Q_OFF + s * SM::Q_TILE_BYTES,
                                  sbase + SM::KV_OFF + slot * SM::KV_TILE_BYTES, IDESC_QK);
             tc_commit(BAR(B_SFULL + s));
             if (j == nts - 1) tc_commit(BAR(B_QEMPTY + s));
@@ -314,7 +314,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (s) ++pcnt1; else ++pcnt0;
             if (!ok) break;
             tc_fence_after();
-            umma_loop_ts(true, tmem + O_COL0 + s * O_STRIDE, tmem + P_COL0 + s * 64, false,
+            umma_loop_ts<0, 8>(true, tmem + O_COL0 + s * O_STRIDE, tmem + P_COL0 + s * 64, false,
                          sbase + SM::KV_OFF + slot * SM::KV_TILE_BYTES, IDESC_PV, j > 0 ? 1u : 0u);
             tc_commit(BAR(B_PFREE + s));
             if (j == nts - 1) tc_commit(BAR(B_OFINAL + s));

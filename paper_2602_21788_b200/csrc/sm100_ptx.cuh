@@ -250,11 +250,12 @@ __device__ __forceinline__ uint64_t sdesc_pack(uint32_t lo, uint32_t hi) {
 // The helpers are called by a whole warp in uniform control flow; only `leader` (one lane) executes
 // the UMMA itself.  Keeping the descriptor arithmetic outside the divergent part lets the compiler
 // hold it in the warp-uniform datapath instead of re-deriving it in one lane's registers.
-template <int KSTEPS>
+// K steps [K0, K1); the first step of the product (K0 = 0) overwrites D.
+template <int K0, int K1>
 __device__ __forceinline__ void umma_loop_kk(bool leader, uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc) {
   const uint32_t hi = sdesc_hi(1024), alo = sdesc_lo(a_addr, 16), blo = sdesc_lo(b_addr, 16);
 #pragma unroll
-  for (int k = 0; k < KSTEPS; ++k) {
+  for (int k = K0; k < K1; ++k) {
     const uint32_t off = (uint32_t)(k >> 2) * (16384u >> 4) + (uint32_t)(k & 3) * 2u;
     const uint64_t ad = sdesc_pack(alo + off, hi), bd = sdesc_pack(blo + off, hi);
     if (leader) umma_ss(d_tmem, ad, bd, idesc, k > 0 ? 1u : 0u);
@@ -271,26 +272,29 @@ __device__ __forceinline__ void umma_loop_mm(bool leader, uint32_t d_tmem, uint3
 }
 // K-major A ([128][64]-element swizzled blocks, as in umma_loop_kk) and MN-major B (as in
 // umma_loop_mm); `acc` = accumulate into D from the first step on.
+// K steps [K0, K1).
+template <int K0, int K1>
 __device__ __forceinline__ void umma_loop_km(bool leader, uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc,
                                              uint32_t acc) {
   const uint32_t hi = sdesc_hi(1024), alo = sdesc_lo(a_addr, 16), blo = sdesc_lo(b_addr, 16384);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
+  for (int k = K0; k < K1; ++k) {
     const uint32_t off = (uint32_t)(k >> 2) * (16384u >> 4) + (uint32_t)(k & 3) * 2u;
     const uint64_t ad = sdesc_pack(alo + off, hi), bd = sdesc_pack(blo + k * 128u, hi);
-    if (leader) umma_ss(d_tmem, ad, bd, idesc, (acc | (k > 0)) ? 1u : 0u);
+    if (leader) umma_ss(d_tmem, ad, bd, idesc, (acc | (k > K0)) ? 1u : 0u);
   }
 }
 // A from TMEM (bf16 pairs, 8 columns per K step; with `split` the second four steps start at
-// column 64), MN-major B.  `acc` = accumulate into D from the first step on.
+// column 64), MN-major B, K steps [K0, K1).  `acc` = accumulate into D from the first step on.
+template <int K0, int K1>
 __device__ __forceinline__ void umma_loop_ts(bool leader, uint32_t d_tmem, uint32_t a_tmem, bool split, uint32_t b_addr,
                                              uint32_t idesc, uint32_t acc) {
   const uint32_t hi = sdesc_hi(1024), blo = sdesc_lo(b_addr, 16384);
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
+  for (int k = K0; k < K1; ++k) {
     const uint32_t col = (split && k >= 4) ? 64u + 8u * (k - 4) : 8u * k;
     const uint64_t bd = sdesc_pack(blo + k * 128u, hi);
-    if (leader) umma_ts(d_tmem, a_tmem + col, bd, idesc, (acc | (k > 0)) ? 1u : 0u);
+    if (leader) umma_ts(d_tmem, a_tmem + col, bd, idesc, (acc | (k > K0)) ? 1u : 0u);
   }
 }
 // TMEM address = (lane << 16) | column.
@@ -343,6 +347,31 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
       ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
         "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
+}
+
+// 16 lanes x 32 columns in matrix fragments: thread t gets, for each group j of 8 columns, the columns 8j + 2 * (t % 4) and
+// the next of lane t / 4 (r[4j], r[4j + 1]) and of lane t / 4 + 8 (r[4j + 2], r[4j + 3]).
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+// 16 lanes x 16 columns of bf16 pairs, the pairs of the fragment above: thread t gives column 4j + t % 4 of lane t / 4
+// (r[2j]) and of lane t / 4 + 8 (r[2j + 1]).
+__device__ __forceinline__ void tmem_st_frag(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+// Four 8 x 8 bf16 matrices to shared memory: register m of thread t holds columns 2 * (t % 4), + 1 of row t / 4 of matrix m;
+// lane l gives the address of row l % 8 of matrix l / 8.
+__device__ __forceinline__ void stmatrix_x4(uint32_t saddr, const uint32_t* r) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared::cta.b16 [%0], {%1, %2, %3, %4};"
+               ::"r"(saddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
 }
 
 __device__ __forceinline__ float ex2(float x) {
