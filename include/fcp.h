@@ -137,6 +137,9 @@ int fcp_span_mask_efficiency(int32_t length, const int32_t* spans, int32_t n_spa
 #define FCP_TABLE_FUSED_UNITS  12  /* [n_fused_units][16]       derived: work units of fcp_attn_fwd_fused       */
 #define FCP_TABLE_ROW_LIMIT    13  /* [T] or empty              first key (packed index) query t does not see   */
 #define FCP_TABLE_FIRST_QUERY  14  /* [T] or empty              first query (packed index) that sees key t      */
+#define FCP_TABLE_FWD_GROUPS   16  /* [n][4]  first unit, units, KV heads per block, 0: execution order of FWD_UNITS */
+#define FCP_TABLE_FUSED_GROUPS 17  /* [n][4]  the same of FUSED_UNITS                                            */
+#define FCP_TABLE_BWD_GROUPS   18  /* [n][4]  the same of BWD_WORK                                               */
 #define FCP_TABLE_SPAN_PAIRS   15  /* [n][5]  seq, rank, step, q_chunk, kv_chunk (> q_chunk): pairs a span adds  */
 
 /* fcp_plan_get: *host_ptr = first element of the table, *count = number of int32 elements. */

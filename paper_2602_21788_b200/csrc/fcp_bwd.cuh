@@ -20,9 +20,7 @@
 // as C1 has read S^T, and T2 of the next tile as soon as C3 has drained dQ, so the tensor core, the
 // math warps and the drain warps work on different tiles at the same time.
 //
-// Work items are handed out through a global counter: KV heads one after the other, within a head
-// the units in plan order (one sequence after the other, keys ascending), so that the dQ rows being
-// reduced into stay in L2.
+// Work items are handed out through a global counter in the order of the plan's work groups.
 #pragma once
 #include "fcp_plan.hpp"
 #include "sm100_ptx.cuh"
@@ -62,8 +60,9 @@ struct BwdSmem {
 struct BwdArgs {
   const int32_t* units;     // [n_units][8]
   const int32_t* qranges;   // [n][4]
-  const int32_t* work;      // [n_units]: units in execution order; work item w = (work[w % n_units], hk_begin + w / n_units)
-  int32_t n_work, n_units, hq, hkv;
+  const int32_t* work;      // [n_units]: units in execution order
+  const int32_t* groups;    // work groups of that order (fcp_plan.hpp)
+  int32_t n_work, n_heads, hq, hkv;   // n_heads: KV heads of this pass
   int32_t hk_begin;         // first KV head of this pass
   int32_t hq_acc;           // query heads held by dq_acc / delta_t / lse2_t: those of the pass, numbered from 0
   int32_t* counter;         // work counter, zero before the launch
@@ -261,14 +260,19 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       // ------------------------------------------------------------------ TMA producer + scheduler
       uint32_t n = 0, it = 0;
       bool ok = true;
+      WorkOrder order;
       while (ok) {
         const int w = atomicAdd(a.counter, 1);
         const uint32_t slot = n & 1;
         ok = mbar_wait(BAR(B_WEMPTY + slot), ((n >> 1) & 1) ^ 1, wctx, 112);
         if (!ok) break;
         const bool last = w >= a.n_work;
-        const int unit = last ? -1 : __ldg(a.work + w % a.n_units);
-        const int hk = last ? 0 : a.hk_begin + w / a.n_units;
+        int unit = -1, hk = 0;
+        if (!last) {
+          order.locate(a.groups, w, a.n_heads, 1, unit, hk);
+          unit = __ldg(a.work + unit);
+          hk += a.hk_begin;
+        }
         work_ring[2 * slot] = unit;
         work_ring[2 * slot + 1] = hk;
         mbar_arrive(BAR(B_WFULL + slot));     // release: the two stores above are visible to the waiters

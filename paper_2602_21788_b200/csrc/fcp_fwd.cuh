@@ -59,6 +59,7 @@ struct FwdSmem {
 struct FwdArgs {
   const int32_t* units;   // [n_units][16]
   int32_t n_units;
+  const int32_t* groups;  // work groups of the units, in execution order (fcp_plan.hpp)
   int32_t head_begin, head_count, hq, hkv;
   int32_t head_group;     // heads that are adjacent in the work order: hq/hkv when the head range is made of whole
                           // KV-head groups, else 1; head_count % head_group == 0
@@ -141,12 +142,11 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 
   const int64_t n_work = (int64_t)a.n_units * a.head_count;
   const int g = a.hq / a.hkv;
-  // Work order.  Item w = (head within a group of gi heads, unit, group), innermost first; gi = the query heads of
-  // one KV head when the head range is made of whole KV-head groups, else 1.  Units are sorted by cost, so the CTAs
-  // that run at the same time work on adjacent units of the same KV head and stream the same K/V tiles: one copy in
-  // L2 serves them all.  Items are handed out dynamically: the producer thread takes item numbers from a global
-  // counter and passes (unit, head) through a small ring in shared memory to the issuing threads and the softmax
-  // and epilogue warps, which all consume every item in order; -1 ends the list.
+  // Work items = (unit, query head), in the order of the work groups; the gi query heads of one KV head (gi = 1 when the head
+  // range cuts KV-head groups) are always adjacent, so that one copy of its K/V tiles in L2 serves them all.  Items are
+  // handed out dynamically: the producer thread takes item numbers from a global counter and passes (unit, head)
+  // through a small ring in shared memory to the issuing threads and the softmax and epilogue warps, which all consume
+  // every item in order; -1 ends the list.
   const int gi = a.head_group;
   // returns 1 with (U, h) of the next item, 0 at the end of the list, -1 if the CTA is aborting
   auto take_item = [&](uint32_t& n, const int32_t*& U, int& h, bool whole_warp) -> int {
@@ -173,6 +173,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     if (lane == 0) {
       uint32_t kv_it = 0, qcnt[2] = {0, 0}, nw = 0;
       bool ok = true, taken_all = false;
+      WorkOrder order;
 #pragma unroll 1
       while (ok) {
         const int64_t w = atomicAdd(a.work_counter, 1);
@@ -184,9 +185,8 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const bool last = w >= n_work;
         int unit = -1, h = 0;
         if (!last) {
-          const int64_t t = w / gi;
-          unit = (int)(t % a.n_units);
-          h = a.head_begin + (int)(t / a.n_units) * gi + (int)(w % gi);
+          order.locate(a.groups, w, a.head_count / gi, gi, unit, h);
+          h += a.head_begin;
         }
         work_ring[2 * slot] = unit;
         work_ring[2 * slot + 1] = h;

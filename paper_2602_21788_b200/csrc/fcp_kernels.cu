@@ -412,10 +412,11 @@ extern "C" int fcp_plan_upload(fcp_plan* plan, void* stream) {
     return FCP_ERR_UNSUPPORTED;
   }
   DeviceState& ds = g_device[dev];
-  constexpr int NT = 10;
+  constexpr int NT = 13;
   const std::vector<int32_t>* tabs[NT] = {&plan->fwd_units, &plan->bwd_units, &plan->bwd_qranges, &plan->merge_units,
                                           &plan->slot_offset, &plan->slot_rows, &plan->bwd_work, &plan->fused_units,
-                                          &plan->row_limit, &plan->first_query};
+                                          &plan->row_limit, &plan->first_query, &plan->fwd_groups, &plan->bwd_groups,
+                                          &plan->fused_groups};
   size_t off[NT + 1];
   size_t total = 256;  // status words first
   for (int i = 0; i < NT; ++i) {
@@ -463,6 +464,9 @@ extern "C" int fcp_plan_upload(fcp_plan* plan, void* stream) {
   plan->d_slot_rows = (int32_t*)((char*)blob + off[5]);
   plan->d_bwd_work = (int32_t*)((char*)blob + off[6]);
   plan->d_fused_units = (int32_t*)((char*)blob + off[7]);
+  plan->d_fwd_groups = (int32_t*)((char*)blob + off[10]);
+  plan->d_bwd_groups = (int32_t*)((char*)blob + off[11]);
+  plan->d_fused_groups = (int32_t*)((char*)blob + off[12]);
   plan->d_row_limit = plan->row_limit.empty() ? nullptr : (int32_t*)((char*)blob + off[8]);
   plan->d_first_query = plan->first_query.empty() ? nullptr : (int32_t*)((char*)blob + off[9]);
   return FCP_OK;
@@ -586,6 +590,7 @@ int launch_fwd(const fcp_plan* plan, const void* q, const void* k, const void* v
   FwdArgs a;
   a.units = fused ? plan->d_fused_units : plan->d_fwd_units;
   a.n_units = (int32_t)((fused ? plan->fused_units.size() : plan->fwd_units.size()) / FCP_FWD_UNIT_W);
+  a.groups = fused ? plan->d_fused_groups : plan->d_fwd_groups;
   a.head_begin = head_begin;
   a.head_count = head_count;
   a.hq = P.hq;
@@ -685,7 +690,7 @@ namespace {
 // work counter, SM count.  fcp_attn_bwd_heads takes them from the uploaded plan, fcp_attn_bwd_noalloc
 // from the built-in arena.
 struct BwdTables {
-  const int32_t *units, *qranges, *order, *first_query;
+  const int32_t *units, *qranges, *order, *groups, *first_query;
   int32_t* status;
   int32_t* counter;
   int sm_count;
@@ -730,8 +735,10 @@ int run_bwd(const fcp_plan* plan, const BwdTables& tb, const void* q, const void
   a.units = tb.units;
   a.qranges = tb.qranges;
   a.work = tb.order;
-  a.n_units = (int32_t)plan->bwd_work.size();
-  a.n_work = a.n_units * hkc;
+  a.groups = tb.groups;
+  a.n_heads = hkc;
+  const int32_t n_units = (int32_t)plan->bwd_work.size();
+  a.n_work = n_units * hkc;
   a.counter = tb.counter;
   a.hq = P.hq;
   a.hkv = P.hkv;
@@ -757,7 +764,7 @@ int run_bwd(const fcp_plan* plan, const BwdTables& tb, const void* q, const void
       FCP_CUDA_CHECK(launch(fcp_bwd_kernel<64>, grid, BWD_THREADS, BwdSmem<64>::DYN_BYTES, st, tq, tk, tv, tdo, a));
   }
   {
-    const dim3 grid_c((unsigned)a.n_units, (unsigned)hc);
+    const dim3 grid_c((unsigned)n_units, (unsigned)hc);
     ProfScope ps(prof, 4, st);
     if (D == 128)
       FCP_CUDA_CHECK(launch(fcp_dq_convert_kernel<128>, grid_c, 256, 0, st, dq_acc, (__nv_bfloat16*)dq, tb.units, T, P.hq, h0));
@@ -796,7 +803,7 @@ int bwd_heads(const fcp_plan* plan, const void* q, const void* k, const void* v,
     fcp_set_error("fcp_attn_bwd: scratch of %lld bytes, %lld needed", (long long)scratch_bytes, (long long)need);
     return FCP_ERR_WORKSPACE;
   }
-  const BwdTables tb{plan->d_bwd_units, plan->d_bwd_qranges, plan->d_bwd_work, plan->d_first_query, plan->d_status,
+  const BwdTables tb{plan->d_bwd_units, plan->d_bwd_qranges, plan->d_bwd_work, plan->d_bwd_groups, plan->d_first_query, plan->d_status,
                      plan->d_status + 16 + 2 * lane, plan->sm_count};
   return used(plan, stream, run_bwd(plan, tb, q, k, v, o, d_o, lse, kv_head_begin, kv_head_count, dq, dk, dv, scratch, plan,
                                     (cudaStream_t)stream));
@@ -1110,7 +1117,7 @@ extern "C" int fcp_noalloc_bytes_needed(const fcp_plan* plan, int64_t* bytes) {
   int64_t scratch = 0;
   fcp_plan_workspace_bytes(plan, 1, nullptr, nullptr, &scratch);
   *bytes = 256 + al((int64_t)plan->bwd_units.size() * 4) + al((int64_t)plan->bwd_qranges.size() * 4) +
-           al((int64_t)plan->bwd_work.size() * 4) + al(scratch);
+           al((int64_t)plan->bwd_work.size() * 4) + al((int64_t)plan->bwd_groups.size() * 4) + al(scratch);
   return FCP_OK;
 }
 
@@ -1150,6 +1157,7 @@ extern "C" int fcp_attn_bwd_noalloc(const fcp_plan* plan, const void* q, const v
   int32_t* d_units = (int32_t*)(base + off);    off += al((int64_t)plan->bwd_units.size() * 4);
   int32_t* d_qranges = (int32_t*)(base + off);  off += al((int64_t)plan->bwd_qranges.size() * 4);
   int32_t* d_work = (int32_t*)(base + off);     off += al((int64_t)plan->bwd_work.size() * 4);
+  int32_t* d_groups = (int32_t*)(base + off);   off += al((int64_t)plan->bwd_groups.size() * 4);
   unsigned char* d_scratch = base + off;
 
   // the arena still holds the previous call's data: status, work counter and the dQ accumulator
@@ -1162,7 +1170,10 @@ extern "C" int fcp_attn_bwd_noalloc(const fcp_plan* plan, const void* q, const v
   if (!plan->bwd_work.empty())
     FCP_CUDA_CHECK(cudaMemcpyAsync(d_work, plan->bwd_work.data(), plan->bwd_work.size() * 4, cudaMemcpyHostToDevice, st));
 
-  const BwdTables tb{d_units, d_qranges, d_work, nullptr, d_status, d_status + 16, g_noalloc_sms[dev]};
+  if (!plan->bwd_groups.empty())
+    FCP_CUDA_CHECK(cudaMemcpyAsync(d_groups, plan->bwd_groups.data(), plan->bwd_groups.size() * 4, cudaMemcpyHostToDevice, st));
+
+  const BwdTables tb{d_units, d_qranges, d_work, d_groups, nullptr, d_status, d_status + 16, g_noalloc_sms[dev]};
   return run_bwd(plan, tb, q, k, v, o, d_o, lse, 0, P.hkv, dq, dk, dv, d_scratch, nullptr, st);
 }
 

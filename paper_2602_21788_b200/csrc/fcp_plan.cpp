@@ -187,6 +187,48 @@ struct Pair {
 
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
+// Puts a unit list into execution order and describes it in work groups (fcp_plan.hpp).  Two things pull against each
+// other.  Long units must come early, over all KV heads, or the last head's long units run alone at the end; and the
+// CTAs that run together should share what one (sequence, KV head) keeps in L2: the K/V tiles of the forward pass, the
+// dQ rows of the backward pass (reductions that miss the L2 run at less than half the speed).  So sequences go longest
+// first, sequences whose data of one KV head fit kOrderBytes together form a group, as many KV heads as fit form a
+// block, and within (group, block) the units go by cost.  Backward kernel, whole lists per KV head -> groups of 64 MB:
+// 8K-token batch 341 -> 290 us, ragged 16K D = 64 225 -> 184 us, large batches unchanged.  Groups of 32 MB: 328 us, of
+// 128 MB: 275 us but 128K bimodal batch +2 %; no limit (all heads by cost): 128K bimodal batch 93 -> 146 ms.
+constexpr int64_t kOrderBytes = int64_t(64) << 20;
+
+void order_units(const std::vector<int32_t>& seq, const std::vector<int32_t>& cost, const int32_t* seqlens, int B,
+                 int64_t bytes_per_token, std::vector<int32_t>& order, std::vector<int32_t>& groups) {
+  std::vector<int32_t> by_len(B), group_of(B), group_heads;
+  std::iota(by_len.begin(), by_len.end(), 0);
+  std::stable_sort(by_len.begin(), by_len.end(), [&](int a, int b) { return seqlens[a] > seqlens[b]; });
+  int64_t bytes = 0;
+  for (int i = 0; i < B; ++i) {
+    const int64_t b = seqlens[by_len[i]] * bytes_per_token;
+    if (i == 0 || bytes + b > kOrderBytes) {
+      group_heads.push_back(1);
+      bytes = 0;
+    }
+    bytes += b;
+    group_of[by_len[i]] = (int32_t)group_heads.size() - 1;
+    group_heads.back() = (int32_t)std::max<int64_t>(1, std::min<int64_t>(kOrderBytes / bytes, 1 << 16));
+  }
+  order.resize(seq.size());
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+    const int ga = group_of[seq[a]], gb = group_of[seq[b]];
+    return ga != gb ? ga < gb : cost[a] > cost[b];
+  });
+  for (size_t i = 0; i < order.size();) {
+    size_t n = i;
+    const int g = group_of[seq[order[i]]];
+    while (n < order.size() && group_of[seq[order[n]]] == g) ++n;
+    const int32_t row[FCP_WORK_GROUP_W] = {(int32_t)i, (int32_t)(n - i), group_heads[g], 0};
+    groups.insert(groups.end(), row, row + FCP_WORK_GROUP_W);
+    i = n;
+  }
+}
+
 }  // namespace
 
 extern "C" int fcp_plan_blocks(const int32_t* seqlens, const int32_t* cp_degrees, int32_t B,
@@ -384,6 +426,17 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
   // item are its pairs in kv_chunk order, so a DIAG range (kv_chunk == q_chunk) is always last.
   struct FU { int32_t f[FCP_FWD_UNIT_W]; };
   std::vector<FU> fus;
+  std::vector<int32_t> fu_seq;
+  const int64_t kv_token_bytes = (int64_t)params->head_dim * 4;                                   // K and V, bf16
+  const int64_t dq_token_bytes = (int64_t)params->head_dim * 4 * (params->hq / params->hkv);      // fp32 dQ rows
+  auto emit_fwd = [&](const std::vector<FU>& units, const std::vector<int32_t>& seq, std::vector<int32_t>& rows,
+                      std::vector<int32_t>& groups) {
+    std::vector<int32_t> cost, order;
+    for (const FU& u : units) cost.push_back(u.f[FU_NT_STAGE0] + u.f[FU_NT_STAGE1]);
+    order_units(seq, cost, seqlens, B, kv_token_bytes, order, groups);
+    rows.reserve(units.size() * FCP_FWD_UNIT_W);
+    for (int32_t i : order) rows.insert(rows.end(), units[i].f, units[i].f + FCP_FWD_UNIT_W);
+  };
   const int n_items = (int)(p->items.size() / 8);
   for (int it = 0; it < n_items; ++it) {
     const int32_t* I = &p->items[(size_t)it * 8];
@@ -425,13 +478,10 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
         u.f[FU_SINGLE_SLOT] = p->slot_offset[ci + 1] - p->slot_offset[ci] == 1;
       }
       fus.push_back(u);
+      fu_seq.push_back(b);
     }
   }
-  std::stable_sort(fus.begin(), fus.end(), [](const FU& a, const FU& b) {
-    return a.f[FU_NT_STAGE0] + a.f[FU_NT_STAGE1] > b.f[FU_NT_STAGE0] + b.f[FU_NT_STAGE1];
-  });
-  p->fwd_units.reserve(fus.size() * FCP_FWD_UNIT_W);
-  for (const FU& u : fus) p->fwd_units.insert(p->fwd_units.end(), u.f, u.f + FCP_FWD_UNIT_W);
+  emit_fwd(fus, fu_seq, p->fwd_units, p->fwd_groups);
 
   // Fused forward (merge on the fly): all items of a Q chunk run on one CTA, so the KV ranges of the
   // chunk's block pairs are swept in one online softmax and no partial leaves the SM.  The ranges of
@@ -461,8 +511,9 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
   }
   {
     std::vector<FU> gus;
+    std::vector<int32_t> gu_seq;
     // rows [r0, r1) of the sequence [t0, t1) attend to [t0, row] (and, inside a span, on to the span's end)
-    auto emit_run = [&](int32_t t0, int32_t t1, int32_t r0, int32_t r1) {
+    auto emit_run = [&](int32_t b, int32_t t0, int32_t t1, int32_t r0, int32_t r1) {
       for (int32_t off = 0; off < r1 - r0; off += FCP_FWD_UNIT_ROWS) {
         FU u{};
         const int32_t rows = std::min<int32_t>(FCP_FWD_UNIT_ROWS, r1 - r0 - off);
@@ -481,6 +532,7 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
         u.f[FU_ITEM] = -1;
         u.f[FU_SINGLE_SLOT] = 1;
         gus.push_back(u);
+        gu_seq.push_back(b);
       }
     };
     for (int b = 0; b < B; ++b) {
@@ -495,11 +547,11 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
                             (rg.size() == 2 && !rg[0].diag && rg[0].b == t0 && rg[0].e == q0 && rg[1].diag && rg[1].b == q0);
         if (prefix) {
           if (run0 < 0) run0 = q0;
-          else if (run1 != q0) { emit_run(t0, t1, run0, run1); run0 = q0; }
+          else if (run1 != q0) { emit_run(b, t0, t1, run0, run1); run0 = q0; }
           run1 = q1;
           continue;
         }
-        if (run0 >= 0) { emit_run(t0, t1, run0, run1); run0 = -1; }
+        if (run0 >= 0) { emit_run(b, t0, t1, run0, run1); run0 = -1; }
         // a chunk whose ranges are not a causal prefix keeps them as they are (at most two per unit)
         if (rg.empty() || rg.size() > 2 || has_spans) {
           delete p;
@@ -528,15 +580,12 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
           u.f[FU_ITEM] = -1;
           u.f[FU_SINGLE_SLOT] = 1;
           gus.push_back(u);
+          gu_seq.push_back(b);
         }
       }
-      if (run0 >= 0) emit_run(t0, t1, run0, run1);
+      if (run0 >= 0) emit_run(b, t0, t1, run0, run1);
     }
-    std::stable_sort(gus.begin(), gus.end(), [](const FU& a, const FU& b) {
-      return a.f[FU_NT_STAGE0] + a.f[FU_NT_STAGE1] > b.f[FU_NT_STAGE0] + b.f[FU_NT_STAGE1];
-    });
-    p->fused_units.reserve(gus.size() * FCP_FWD_UNIT_W);
-    for (const FU& u : gus) p->fused_units.insert(p->fused_units.end(), u.f, u.f + FCP_FWD_UNIT_W);
+    emit_fwd(gus, gu_seq, p->fused_units, p->fused_groups);
   }
 
   // Backward: one unit per 128-key tile; it visits the Q rows of all block pairs whose kv_chunk holds
@@ -617,19 +666,13 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
     }
   }
   for (const BU& u : bus) p->bwd_units.insert(p->bwd_units.end(), u.f, u.f + FCP_BWD_UNIT_W);
-  // Execution order of the backward units within one KV head (the kernel runs the KV heads one after
-  // the other, each over this list).  dQ is accumulated with fp32 reductions in global memory, which
-  // only run at L2 speed while the rows they touch stay resident: so all CTAs work on one
-  // (sequence, KV head) panel at a time, key tiles in ascending position (descending cost), and
-  // sweep the query tiles roughly in step.  Sequences go longest first.
   {
-    std::vector<int> seq_order(B);
-    std::iota(seq_order.begin(), seq_order.end(), 0);
-    std::stable_sort(seq_order.begin(), seq_order.end(), [&](int a, int b) { return seqlens[a] > seqlens[b]; });
-    std::vector<std::vector<int32_t>> units_of(B);
-    for (size_t i = 0; i < bus.size(); ++i) units_of[bus[i].f[BU_SEQ]].push_back((int32_t)i);   // ascending key position
-    for (int b : seq_order)
-      for (int32_t u : units_of[b]) p->bwd_work.push_back(u);
+    std::vector<int32_t> seq, cost;
+    for (const BU& u : bus) {
+      seq.push_back(u.f[BU_SEQ]);
+      cost.push_back(u.f[BU_COST]);
+    }
+    order_units(seq, cost, seqlens, B, dq_token_bytes, p->bwd_work, p->bwd_groups);
   }
 
   // Merge: runs of up to FCP_MERGE_TOKENS tokens inside one chunk.  Chunks with two or more slots
@@ -695,6 +738,9 @@ extern "C" int fcp_plan_get(const fcp_plan* plan, int32_t which, const int32_t**
     case FCP_TABLE_FUSED_UNITS: v = &plan->fused_units; break;
     case FCP_TABLE_ROW_LIMIT: v = &plan->row_limit; break;
     case FCP_TABLE_FIRST_QUERY: v = &plan->first_query; break;
+    case FCP_TABLE_FWD_GROUPS: v = &plan->fwd_groups; break;
+    case FCP_TABLE_FUSED_GROUPS: v = &plan->fused_groups; break;
+    case FCP_TABLE_BWD_GROUPS: v = &plan->bwd_groups; break;
     case FCP_TABLE_SPAN_PAIRS: v = &plan->span_pairs; break;
     default: fcp_set_error("fcp_plan_get: unknown table %d", which); return FCP_ERR_INVALID_ARG;
   }

@@ -23,6 +23,10 @@ enum {
 enum { BU_KV_ROW0 = 0, BU_KV_ROWS, BU_FIRST_QRANGE, BU_N_QRANGES, BU_T_FIRST, BU_COST, BU_SEQ, BU_T_MASK_END };
 enum { BQ_BEGIN = 0, BQ_END, BQ_DIAG, BQ_RSV };
 enum { MU_TOK_BEGIN = 0, MU_N_TOK, MU_CHUNK, MU_CHUNK_TOK_BEGIN };
+// Execution order of the two persistent grids: groups of units (consecutive in the unit list); within a group the KV heads go
+// in blocks of WG_HEADS, within a block the units in list order, and innermost the heads of the block.
+constexpr int FCP_WORK_GROUP_W = 4;
+enum { WG_FIRST = 0, WG_N_UNITS, WG_HEADS, WG_RSV };
 
 struct PlanBlock;                      // device block of an uploaded plan (fcp_kernels.cu)
 
@@ -35,6 +39,7 @@ struct fcp_plan {
   int32_t n_merge_multi = 0;   // merge units of chunks with two or more slots (they come first in merge_units)
   std::vector<int32_t> cu_seqlens, chunk_offset, chunk_bounds, pairs, items, slot_offset, slot_rows;
   std::vector<int32_t> fwd_units, bwd_units, bwd_qranges, merge_units, bwd_work, fused_units;
+  std::vector<int32_t> fwd_groups, bwd_groups, fused_groups;   // work groups of the three unit lists
   std::vector<int32_t> row_limit, first_query, span_pairs;   // empty unless the plan has bidirectional spans
   std::vector<int32_t> span_offset, spans;                   // the caller's span list ([B+1], [n][2]); empty if none
 
@@ -49,6 +54,9 @@ struct fcp_plan {
   int32_t* d_merge_units = nullptr;
   int32_t* d_bwd_work = nullptr;
   int32_t* d_fused_units = nullptr;
+  int32_t* d_fwd_groups = nullptr;
+  int32_t* d_bwd_groups = nullptr;
+  int32_t* d_fused_groups = nullptr;
   int32_t* d_row_limit = nullptr;      // nullptr for a causal plan
   int32_t* d_first_query = nullptr;
   int32_t* d_slot_offset = nullptr;

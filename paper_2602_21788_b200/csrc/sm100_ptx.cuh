@@ -8,6 +8,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "fcp_plan.hpp"
+
 namespace fcp {
 
 constexpr unsigned long long FCP_WAIT_NS = 2000000000ull;  // 2 s: far above any legitimate wait
@@ -140,6 +142,29 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, co
   const bool ok = mbar_wait(bar, parity, ctx, where);
   return __all_sync(0xffffffffu, ok);
 }
+
+// ----------------------------------------------------------------------------- work order
+// Position of a work item in the execution order described by work groups (fcp_plan.hpp).  Items are asked for in ascending
+// order by one thread, which remembers the group it is in.
+struct WorkOrder {
+  int g = 0;              // current group
+  int64_t first = 0;      // its first work item
+  // `heads` KV heads of `per` adjacent items each; returns the unit's place in the list and head * per + item
+  __device__ __forceinline__ void locate(const int32_t* groups, int64_t w, int heads, int per, int& unit, int& h) {
+    const int32_t* G = groups + g * FCP_WORK_GROUP_W;
+    while (w - first >= (int64_t)__ldg(G + WG_N_UNITS) * heads * per) {
+      first += (int64_t)__ldg(G + WG_N_UNITS) * heads * per;
+      ++g;
+      G += FCP_WORK_GROUP_W;
+    }
+    const int n = __ldg(G + WG_N_UNITS), gh = min(__ldg(G + WG_HEADS), heads);
+    const int64_t r = w - first, block = (int64_t)n * gh * per;
+    const int hb = (int)(r / block), rest = (int)(r - hb * block);
+    const int inner = min(gh, heads - hb * gh) * per;
+    unit = __ldg(G + WG_FIRST) + rest / inner;
+    h = hb * gh * per + rest % inner;
+  }
+};
 
 // ----------------------------------------------------------------------------- TMA
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* m) {

@@ -20,9 +20,9 @@ FCP_MAX_DEGREE = 64
 
 TABLES = dict(cu_seqlens=0, chunk_offset=1, chunk_bounds=2, pairs=3, items=4, slot_offset=5, slot_rows=6,
               fwd_units=7, bwd_units=8, bwd_qranges=9, merge_units=10, bwd_work=11, fused_units=12, row_limit=13,
-              first_query=14, span_pairs=15)
+              first_query=14, span_pairs=15, fwd_groups=16, fused_groups=17, bwd_groups=18)
 _TABLE_WIDTH = dict(pairs=6, items=8, fwd_units=16, bwd_units=8, bwd_qranges=4, merge_units=4, fused_units=16,
-                    span_pairs=5)
+                    span_pairs=5, fwd_groups=4, fused_groups=4, bwd_groups=4)
 INFO = dict(T=0, R=1, n_pairs=2, n_items=3, n_fwd_units=4, n_bwd_units=5, n_merge_units=6, B=7, n_merge_multi=8,
             n_fused_units=9)
 

@@ -1,0 +1,56 @@
+"""Execution order of the persistent grids: every (unit, head) once, whatever the head range, longest sequences first."""
+import numpy as np
+import pytest
+
+from paper_2602_21788_b200 import build, fcp
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+
+
+def _items(groups, heads, per):
+    """(place in the unit list, head) of work items 0, 1, ... as the kernels' producer thread computes them."""
+    out = []
+    for first, n, gh, _ in groups.tolist():
+        gh = min(gh, heads)
+        block = n * gh * per
+        for r in range(n * heads * per):
+            hb, rest = divmod(r, block)
+            inner = min(gh, heads - hb * gh) * per
+            out.append((first + rest // inner, hb * gh * per + rest % inner))
+    return out
+
+
+CASES = [
+    ([5], 1, 1, 64),
+    ([300, 4000, 129, 2000, 2000, 64], 8, 2, 128),
+    ([70000, 70000, 900, 1500, 300], 32, 8, 128),      # one sequence's dQ rows of a KV head exceed a group: blocks of one head
+    ([9000, 20000, 9000, 128], 24, 8, 128),            # blocks of several heads, the last one smaller
+]
+
+
+@pytest.mark.parametrize("lens,hq,hkv,D", CASES)
+@pytest.mark.parametrize("heads", [None, 1, 3])
+def test_work_order_visits_every_item_once(lens, hq, hkv, D, heads):
+    plan = fcp.Plan(lens, [1] * len(lens), hq, hkv, D)
+    n_kv = min(heads or hkv, hkv)
+    for table, n_units, per in (("fwd_groups", plan.info("n_fwd_units"), hq // hkv), ("fused_groups", plan.info("n_fused_units"), hq // hkv),
+                                ("bwd_groups", plan.info("n_bwd_units"), 1), ("fwd_groups", plan.info("n_fwd_units"), 1)):
+        items = _items(plan.table(table), n_kv, per)
+        assert len(items) == len(set(items)) == n_units * n_kv * per
+        assert {u for u, _ in items} == set(range(n_units)) and {h for _, h in items} == set(range(n_kv * per))
+
+
+@pytest.mark.parametrize("lens,hq,hkv,D", CASES)
+def test_groups_go_longest_sequence_first_and_by_cost_within(lens, hq, hkv, D):
+    plan = fcp.Plan(lens, [1] * len(lens), hq, hkv, D)
+    units = plan.table("bwd_units")[plan.table("bwd_work")]
+    shortest_so_far = max(lens)
+    for first, n, _, _ in plan.table("bwd_groups").tolist():
+        g = units[first:first + n]
+        group_lens = [lens[b] for b in g[:, 6]]
+        assert max(group_lens) <= shortest_so_far
+        shortest_so_far = min(group_lens)
+        assert np.all(np.diff(g[:, 5]) <= 0)
