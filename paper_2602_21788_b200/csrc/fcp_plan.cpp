@@ -195,10 +195,16 @@ inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 // block, and within (group, block) the units go by cost.  Backward kernel, whole lists per KV head -> groups of 64 MB:
 // 8K-token batch 341 -> 290 us, ragged 16K D = 64 225 -> 184 us, large batches unchanged.  Groups of 32 MB: 328 us, of
 // 128 MB: 275 us but 128K bimodal batch +2 %; no limit (all heads by cost): 128K bimodal batch 93 -> 146 ms.
+// The cheapest units of all sequences wait for the end, all KV heads together: they level out what the last block's
+// long units leave uneven.  Half of the longest unit per SM is enough (simulated with measured unit times: 16K new
+// batch 1421 us -> 1250 us for a mean of 1240, 8K batch 248 -> 226 for 220), at most 15 % of the work, and only where
+// the longest unit is over a quarter of an SM's share: these units touch the ends of all sequences and share little (64K
+// batch, 15 %: backward +2 % when they wait).  Measured: 8K step 501 -> 485 us, 16K new batch 2.50 -> 2.37 ms.
 constexpr int64_t kOrderBytes = int64_t(64) << 20;
+constexpr int64_t kOrderSms = 148;
 
 void order_units(const std::vector<int32_t>& seq, const std::vector<int32_t>& cost, const int32_t* seqlens, int B,
-                 int64_t bytes_per_token, std::vector<int32_t>& order, std::vector<int32_t>& groups) {
+                 int32_t heads, int64_t bytes_per_token, std::vector<int32_t>& order, std::vector<int32_t>& groups) {
   std::vector<int32_t> by_len(B), group_of(B), group_heads;
   std::iota(by_len.begin(), by_len.end(), 0);
   std::stable_sort(by_len.begin(), by_len.end(), [&](int a, int b) { return seqlens[a] > seqlens[b]; });
@@ -215,14 +221,29 @@ void order_units(const std::vector<int32_t>& seq, const std::vector<int32_t>& co
   }
   order.resize(seq.size());
   std::iota(order.begin(), order.end(), 0);
+  std::vector<int32_t> unit_group(seq.size());
+  for (size_t i = 0; i < seq.size(); ++i) unit_group[i] = group_of[seq[i]];
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] < cost[b]; });
+  {
+    int64_t total = 0, late = 0;
+    for (int32_t c : cost) total += c;
+    const int64_t longest = kOrderSms * (order.empty() ? 0 : cost[order.back()]) / heads;   // on every SM, per KV head
+    const int64_t most = 4 * longest > total ? std::min<int64_t>(longest / 2, total * 15 / 100) : 0;
+    const int32_t last = (int32_t)group_heads.size();
+    group_heads.push_back(1 << 16);
+    for (int32_t i : order) {
+      late += cost[i];
+      if (late > most) break;
+      unit_group[i] = last;
+    }
+  }
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-    const int ga = group_of[seq[a]], gb = group_of[seq[b]];
-    return ga != gb ? ga < gb : cost[a] > cost[b];
+    return unit_group[a] != unit_group[b] ? unit_group[a] < unit_group[b] : cost[a] > cost[b];
   });
   for (size_t i = 0; i < order.size();) {
     size_t n = i;
-    const int g = group_of[seq[order[i]]];
-    while (n < order.size() && group_of[seq[order[n]]] == g) ++n;
+    const int g = unit_group[order[i]];
+    while (n < order.size() && unit_group[order[n]] == g) ++n;
     const int32_t row[FCP_WORK_GROUP_W] = {(int32_t)i, (int32_t)(n - i), group_heads[g], 0};
     groups.insert(groups.end(), row, row + FCP_WORK_GROUP_W);
     i = n;
@@ -433,7 +454,7 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
                       std::vector<int32_t>& groups) {
     std::vector<int32_t> cost, order;
     for (const FU& u : units) cost.push_back(u.f[FU_NT_STAGE0] + u.f[FU_NT_STAGE1]);
-    order_units(seq, cost, seqlens, B, kv_token_bytes, order, groups);
+    order_units(seq, cost, seqlens, B, params->hkv, kv_token_bytes, order, groups);
     rows.reserve(units.size() * FCP_FWD_UNIT_W);
     for (int32_t i : order) rows.insert(rows.end(), units[i].f, units[i].f + FCP_FWD_UNIT_W);
   };
@@ -672,7 +693,7 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
       seq.push_back(u.f[BU_SEQ]);
       cost.push_back(u.f[BU_COST]);
     }
-    order_units(seq, cost, seqlens, B, dq_token_bytes, p->bwd_work, p->bwd_groups);
+    order_units(seq, cost, seqlens, B, params->hkv, dq_token_bytes, p->bwd_work, p->bwd_groups);
   }
 
   // Merge: runs of up to FCP_MERGE_TOKENS tokens inside one chunk.  Chunks with two or more slots

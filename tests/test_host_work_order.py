@@ -48,9 +48,15 @@ def test_groups_go_longest_sequence_first_and_by_cost_within(lens, hq, hkv, D):
     plan = fcp.Plan(lens, [1] * len(lens), hq, hkv, D)
     units = plan.table("bwd_units")[plan.table("bwd_work")]
     shortest_so_far = max(lens)
-    for first, n, _, _ in plan.table("bwd_groups").tolist():
+    groups = plan.table("bwd_groups").tolist()
+    late = groups.pop() if len(groups) > 1 and groups[-1][2] == 1 << 16 else None   # the cheapest units of all sequences
+    for first, n, _, _ in groups:
         g = units[first:first + n]
         group_lens = [lens[b] for b in g[:, 6]]
         assert max(group_lens) <= shortest_so_far
         shortest_so_far = min(group_lens)
         assert np.all(np.diff(g[:, 5]) <= 0)
+    if late:
+        g = units[late[0]:]
+        assert np.all(np.diff(g[:, 5]) <= 0) and g[:, 5].sum() <= 0.15 * units[:, 5].sum()
+        assert g[:, 5].max() <= min(units[f:f + n, 5].min() for f, n, _, _ in groups)
