@@ -63,6 +63,7 @@ struct FwdArgs {
   int32_t head_begin, head_count, hq, hkv;
   int32_t head_group;     // heads that are adjacent in the work order: hq/hkv when the head range is made of whole
                           // KV-head groups, else 1; head_count % head_group == 0
+  int32_t split;          // 1: the two Q tiles of a unit are work items of their own
   int32_t* work_counter;  // the grid's next work item: zero before the launch, and again after it
   float scale_log2;       // softmax scale * log2(e)
   float* o_partial;       // [R][head_count][D]
@@ -140,7 +141,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   const uint32_t tmem = *tmem_slot;
   grid_wait();
 
-  const int64_t n_work = (int64_t)a.n_units * a.head_count;
+  const int64_t n_work = (int64_t)a.n_units * a.head_count << a.split;
   const int g = a.hq / a.hkv;
   // Work items = (unit, query head), in the order of the work groups; the gi query heads of one KV head (gi = 1 when the head
   // range cuts KV-head groups) are always adjacent, so that one copy of its K/V tiles in L2 serves them all.  Items are
@@ -148,8 +149,10 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   // through a small ring in shared memory to the issuing threads and the softmax and epilogue warps, which all consume
   // every item in order; -1 ends the list.
   const int gi = a.head_group;
-  // returns 1 with (U, h) of the next item, 0 at the end of the list, -1 if the CTA is aborting
-  auto take_item = [&](uint32_t& n, const int32_t*& U, int& h, bool whole_warp) -> int {
+  // The ring holds (unit, head | mask of the Q tiles that are not part of the item << 30).
+  // returns 1 with (U, h) and the key tiles of the two Q tiles of the next item, 0 at the end of the list, -1 if the CTA is
+  // aborting
+  auto take_item = [&](uint32_t& n, const int32_t*& U, int& h, int& nt0, int& nt1, bool whole_warp) -> int {
     const uint32_t slot = n % FWD_WORK_SLOTS, par = (n / FWD_WORK_SLOTS) & 1;
     const bool got = whole_warp ? mbar_wait_warp(BAR(B_WFULL + slot), par, wctx, 40) : mbar_wait(BAR(B_WFULL + slot), par, wctx, 40);
     if (!got) return -1;
@@ -164,6 +167,9 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     ++n;
     if (unit < 0) return 0;
     U = a.units + (size_t)unit * FCP_FWD_UNIT_W;
+    nt0 = (h & (1 << 30)) ? 0 : __ldg(U + FU_NT_STAGE0);
+    nt1 = (h & (1u << 31)) ? 0 : __ldg(U + FU_NT_STAGE1);
+    h &= (1 << 30) - 1;
     return 1;
   };
 
@@ -184,12 +190,14 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         if (!ok) break;
         const bool last = w >= n_work;
         int unit = -1, h = 0;
+        uint32_t skip = 0;                       // Q tiles that are not part of this item
         if (!last) {
-          order.locate(a.groups, w, a.head_count / gi, gi, unit, h);
+          order.locate(a.groups, w >> a.split, a.head_count / gi, gi, unit, h);
           h += a.head_begin;
+          if (a.split) skip = 1u << ((w & 1) ^ 1);
         }
         work_ring[2 * slot] = unit;
-        work_ring[2 * slot + 1] = h;
+        work_ring[2 * slot + 1] = (int)((uint32_t)h | (skip << 30));
         mbar_arrive(BAR(B_WFULL + slot));      // release: the two stores above are visible to the waiters
         ++nw;
         if (last) {
@@ -198,7 +206,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
         const int32_t* U = a.units + (size_t)unit * FCP_FWD_UNIT_W;
         const int hk = h / g;
-        const int nt[2] = {__ldg(U + FU_NT_STAGE0), __ldg(U + FU_NT_STAGE1)};
+        const int nt[2] = {(skip & 1) ? 0 : __ldg(U + FU_NT_STAGE0), (skip & 2) ? 0 : __ldg(U + FU_NT_STAGE1)};
         const int q_row0 = __ldg(U + FU_Q_ROW0);
 #pragma unroll 1
         for (int s = 0; s < 2 && ok; ++s) {
@@ -251,10 +259,9 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll 1
       while (ok) {
         const int32_t* U;
-        int h;
-        const int r = take_item(nw, U, h, false);
+        int h, nt0, nt1;
+        const int r = take_item(nw, U, h, nt0, nt1, false);
         if (r <= 0) { ok = r == 0; break; }
-        const int nt0 = __ldg(U + FU_NT_STAGE0), nt1 = __ldg(U + FU_NT_STAGE1);
         const int n_max = max(nt0, nt1);
 #pragma unroll 1
         for (int j = 0; j < n_max && ok; ++j, kv_it += 2) {
@@ -292,10 +299,9 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll 1
       while (ok) {
         const int32_t* U;
-        int h;
-        const int r = take_item(nw, U, h, false);
+        int h, nt0, nt1;
+        const int r = take_item(nw, U, h, nt0, nt1, false);
         if (r <= 0) { ok = r == 0; break; }
-        const int nt0 = __ldg(U + FU_NT_STAGE0), nt1 = __ldg(U + FU_NT_STAGE1);
         const int n_max = max(nt0, nt1);
 #pragma unroll 1
         for (int j = 0; j < n_max && ok; ++j, kv_it += 2) {
@@ -342,10 +348,10 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll 1
     while (ok) {
       const int32_t* U;
-      int h;
-      const int r = take_item(nw, U, h, true);
+      int h, nt0, nt1;
+      const int r = take_item(nw, U, h, nt0, nt1, true);
       if (r <= 0) { ok = r == 0; break; }
-      const int nts = __ldg(U + FU_NT_STAGE0 + s);
+      const int nts = s ? nt1 : nt0;
       const int q_pos = __ldg(U + FU_Q_ROW0) + s * 128 + row;
       // first key this row does not see in a DIAG range: the one after itself, or the end of its span
       const int row_lim = (a.row_limit != nullptr && s * 128 + row < __ldg(U + FU_Q_ROWS)) ? __ldg(a.row_limit + q_pos) : q_pos + 1;
@@ -467,8 +473,8 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll 1
     while (ok) {
       const int32_t* U;
-      int h;
-      const int r = take_item(nw, U, h, true);
+      int h, nt0, nt1;
+      const int r = take_item(nw, U, h, nt0, nt1, true);
       if (r <= 0) { ok = r == 0; break; }
       const int hl = h - a.head_begin;
       const int q_rows = __ldg(U + FU_Q_ROWS);
@@ -479,7 +485,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const int64_t trow0 = (int64_t)__ldg(U + FU_Q_ROW0);
 #pragma unroll 1
       for (int s = 0; s < 2 && ok; ++s) {
-        if (__ldg(U + FU_NT_STAGE0 + s) == 0) continue;
+        if ((s ? nt1 : nt0) == 0) continue;
         const float* stat = (const float*)(smem + SM::STAT_OFF) + s * 256;
         const uint32_t ph = (s ? ecnt1 : ecnt0) & 1;
         if (s) ++ecnt1; else ++ecnt0;

@@ -607,7 +607,10 @@ int launch_fwd(const fcp_plan* plan, const void* q, const void* k, const void* v
   a.o_f32_direct = o_f32_direct;
   a.row_limit = fused ? plan->d_row_limit : nullptr;
   a.status = plan->d_status;
-  const int64_t n_work = (int64_t)a.n_units * head_count;
+  // With fewer items than SMs every item runs at once and the longest one is the launch: then its two Q tiles go to two
+  // SMs (a tile alone does not wait for the other one's turn in the MUFU and the tensor core): 4K-token forward 23.2 -> 21.2 us.
+  a.split = (int64_t)a.n_units * head_count < plan->sm_count ? 1 : 0;
+  const int64_t n_work = (int64_t)a.n_units * head_count << a.split;
   const int grid = (int)std::min<int64_t>(n_work, plan->sm_count);
   if (grid == 0) return FCP_OK;
   cudaStream_t st = (cudaStream_t)stream;

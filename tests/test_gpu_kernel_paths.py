@@ -139,3 +139,12 @@ def test_host_entry_point_slices(lens, hq, hkv, D):
             assert torch.equal(got, ref.cpu())
         a, b = out[2].float(), ds.dq.float().cpu()
         assert (a - b).norm() <= 1e-2 * b.norm()
+
+
+@pytest.mark.parametrize("lens,hq,hkv,D", [
+    ([1000], 2, 1, 128),                 # 8 items on 148 SMs: the Q tiles of a unit are items of their own
+    ([129, 128, 1], 3, 3, 64),           # units with one Q tile
+    ([2560] * 9 + [70], 16, 2, 64),      # more items than SMs: both tiles of a unit together
+])
+def test_forward_with_split_and_whole_units(lens, hq, hkv, D):
+    _check(_wl(lens, [1] * len(lens), hq, hkv, D, seed=17))
