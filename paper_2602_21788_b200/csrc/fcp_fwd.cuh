@@ -33,6 +33,7 @@ namespace fcp {
 constexpr int FWD_THREADS = 512;          // 4 control warps + 2 x 4 softmax warps + 4 epilogue warps
 constexpr int FWD_KV_SLOTS = 4;
 constexpr int FWD_WORK_SLOTS = 4;         // ring of work items handed from the producer to the other roles
+constexpr int FWD_CLAIM_AHEAD = 3;        // key tiles before the end of an item's loads at which the next item is claimed
 // register budgets per thread of the three roles: 128 * 48 + 256 * 192 + 128 * 80 = 512 * 128
 #define FCP_FWD_REGS_CTRL "48"
 #define FCP_FWD_REGS_SOFTMAX "192"
@@ -141,7 +142,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   const uint32_t tmem = *tmem_slot;
   grid_wait();
 
-  const int64_t n_work = (int64_t)a.n_units * a.head_count << a.split;
+  const uint32_t n_work = (uint32_t)a.n_units * a.head_count << a.split;   // below 2^31 (checked at the launch)
   const int g = a.hq / a.hkv;
   // Work items = (unit, query head), in the order of the work groups; the gi query heads of one KV head (gi = 1 when the head
   // range cuts KV-head groups) are always adjacent, so that one copy of its K/V tiles in L2 serves them all.  Items are
@@ -177,21 +178,24 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
+      // The next item is claimed FWD_CLAIM_AHEAD key tiles before the loads of this one end: the way from the counter
+      // to its first load (an atomic, the place in the work order, the unit's row: dependent trips to the L2, 5000-6000 clk) then runs
+      // beside this item's last steps.
       uint32_t kv_it = 0, qcnt[2] = {0, 0}, nw = 0;
-      bool ok = true, taken_all = false;
+      bool taken_all = false;
       WorkOrder order;
-#pragma unroll 1
-      while (ok) {
-        const int64_t w = atomicAdd(a.work_counter, 1);
+      int unit, h;
+      uint32_t skip;                             // Q tiles that are not part of the item
+      auto claim = [&]() -> int {                // 1: (unit, h, skip) is the next item, 0: end of the list, -1: aborting
+        const uint32_t w = atomicAdd(a.work_counter, 1);
         taken_all = w >= n_work;
-        if (w == n_work + (int)gridDim.x - 1) *a.work_counter = 0;   // every producer takes one item past the end: this is the last
+        if (w == n_work + gridDim.x - 1) *a.work_counter = 0;   // every producer takes one item past the end: this is the last
         const uint32_t slot = nw % FWD_WORK_SLOTS;
-        ok = mbar_wait(BAR(B_WEMPTY + slot), ((nw / FWD_WORK_SLOTS) & 1) ^ 1, wctx, 41);
-        if (!ok) break;
-        const bool last = w >= n_work;
-        int unit = -1, h = 0;
-        uint32_t skip = 0;                       // Q tiles that are not part of this item
-        if (!last) {
+        if (!mbar_wait(BAR(B_WEMPTY + slot), ((nw / FWD_WORK_SLOTS) & 1) ^ 1, wctx, 41)) return -1;
+        unit = -1;
+        h = 0;
+        skip = 0;
+        if (!taken_all) {
           order.locate(a.groups, w >> a.split, a.head_count / gi, gi, unit, h);
           h += a.head_begin;
           if (a.split) skip = 1u << ((w & 1) ^ 1);
@@ -200,29 +204,21 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         work_ring[2 * slot + 1] = (int)((uint32_t)h | (skip << 30));
         mbar_arrive(BAR(B_WFULL + slot));      // release: the two stores above are visible to the waiters
         ++nw;
-        if (last) {
-          grid_launch_next();
-          break;
-        }
+        if (taken_all) grid_launch_next();
+        return taken_all ? 0 : 1;
+      };
+      int state = claim();
+#pragma unroll 1
+      while (state == 1) {
         const int32_t* U = a.units + (size_t)unit * FCP_FWD_UNIT_W;
-        const int hk = h / g;
+        const int hc = h, hk = h / g;
         const int nt[2] = {(skip & 1) ? 0 : __ldg(U + FU_NT_STAGE0), (skip & 2) ? 0 : __ldg(U + FU_NT_STAGE1)};
         const int q_row0 = __ldg(U + FU_Q_ROW0);
-#pragma unroll 1
-        for (int s = 0; s < 2 && ok; ++s) {
-          if (nt[s] == 0) continue;
-          ok = mbar_wait(BAR(B_QEMPTY + s), (qcnt[s] & 1) ^ 1, wctx, 10 + s);
-          if (!ok) break;
-          mbar_expect_tx(BAR(B_QFULL + s), SM::Q_TILE_BYTES);
-#pragma unroll 1
-          for (int kb = 0; kb < KBLK; ++kb)
-            tma_load_3d(sbase + SM::Q_OFF + s * SM::Q_TILE_BYTES + kb * BLK_BYTES, &tm_q, BAR(B_QFULL + s), kb * 64, h,
-                        q_row0 + s * 128);
-          ++qcnt[s];
-        }
         const int n_max = max(nt[0], nt[1]);
         const int nr0 = __ldg(U + FU_NT_RANGE0);
         const int kv0 = __ldg(U + FU_KV0_BEGIN), kv1 = __ldg(U + FU_KV1_BEGIN);
+        bool ok = true;
+        state = -1;
 #pragma unroll 1
         for (int j = 0; j < n_max && ok; ++j) {
           const int row = j < nr0 ? kv0 + j * 128 : kv1 + (j - nr0) * 128;
@@ -237,15 +233,36 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               tma_load_3d(sbase + SM::KV_OFF + slot * SM::KV_TILE_BYTES + kb * BLK_BYTES, t == 0 ? &tm_k : &tm_v,
                           BAR(B_KVFULL + slot), kb * 64, hk, row);
             ++kv_it;
+            if (j == 0 && t == 0) {        // the Q tiles behind the first K tile, whose ring slot is free earlier
+#pragma unroll 1
+              for (int s = 0; s < 2 && ok; ++s) {
+                if (nt[s] == 0) continue;
+                ok = mbar_wait(BAR(B_QEMPTY + s), (qcnt[s] & 1) ^ 1, wctx, 10 + s);
+                if (!ok) break;
+                mbar_expect_tx(BAR(B_QFULL + s), SM::Q_TILE_BYTES);
+#pragma unroll 1
+                for (int kb = 0; kb < KBLK; ++kb)
+                  tma_load_3d(sbase + SM::Q_OFF + s * SM::Q_TILE_BYTES + kb * BLK_BYTES, &tm_q, BAR(B_QFULL + s), kb * 64, hc,
+                              q_row0 + s * 128);
+                ++qcnt[s];
+              }
+              if (!ok) break;
+            }
+          }
+          if (ok && j == max(0, n_max - FWD_CLAIM_AHEAD)) {
+            state = claim();
+            if (state < 0) ok = false;
           }
         }
+        if (n_max == 0) state = claim();   // a split unit without a second tile
+        if (!ok) break;
       }
       // after a wait that gave up: take the rest of the list, so that the counter comes back to zero
 #pragma unroll 1
       while (!taken_all) {
-        const int64_t w = atomicAdd(a.work_counter, 1);
+        const uint32_t w = atomicAdd(a.work_counter, 1);
         taken_all = w >= n_work;
-        if (w == n_work + (int)gridDim.x - 1) *a.work_counter = 0;
+        if (w == n_work + gridDim.x - 1) *a.work_counter = 0;
       }
     }
   } else if (warp == 1) {

@@ -611,6 +611,10 @@ int launch_fwd(const fcp_plan* plan, const void* q, const void* k, const void* v
   // SMs (a tile alone does not wait for the other one's turn in the MUFU and the tensor core): 4K-token forward 23.2 -> 21.2 us.
   a.split = (int64_t)a.n_units * head_count < plan->sm_count ? 1 : 0;
   const int64_t n_work = (int64_t)a.n_units * head_count << a.split;
+  if (n_work >= int64_t(1) << 31) {
+    fcp_set_error("forward attention: %lld work items exceed the 2^31 limit", (long long)n_work);
+    return FCP_ERR_INVALID_ARG;
+  }
   const int grid = (int)std::min<int64_t>(n_work, plan->sm_count);
   if (grid == 0) return FCP_OK;
   cudaStream_t st = (cudaStream_t)stream;

@@ -148,21 +148,22 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, co
 // order by one thread, which remembers the group it is in.
 struct WorkOrder {
   int g = 0;              // current group
-  int64_t first = 0;      // its first work item
+  uint32_t first = 0;     // its first work item
   // `heads` KV heads of `per` adjacent items each; returns the unit's place in the list and head * per + item
-  __device__ __forceinline__ void locate(const int32_t* groups, int64_t w, int heads, int per, int& unit, int& h) {
+  __device__ __forceinline__ void locate(const int32_t* groups, uint32_t w, uint32_t heads, uint32_t per, int& unit, int& h) {
     const int32_t* G = groups + g * FCP_WORK_GROUP_W;
-    while (w - first >= (int64_t)__ldg(G + WG_N_UNITS) * heads * per) {
-      first += (int64_t)__ldg(G + WG_N_UNITS) * heads * per;
+    while (w - first >= (uint32_t)__ldg(G + WG_N_UNITS) * heads * per) {
+      first += (uint32_t)__ldg(G + WG_N_UNITS) * heads * per;
       ++g;
       G += FCP_WORK_GROUP_W;
     }
-    const int n = __ldg(G + WG_N_UNITS), gh = min(__ldg(G + WG_HEADS), heads);
-    const int64_t r = w - first, block = (int64_t)n * gh * per;
-    const int hb = (int)(r / block), rest = (int)(r - hb * block);
-    const int inner = min(gh, heads - hb * gh) * per;
-    unit = __ldg(G + WG_FIRST) + rest / inner;
-    h = hb * gh * per + rest % inner;
+    const uint32_t gh = min((uint32_t)__ldg(G + WG_HEADS), heads);
+    const uint32_t r = w - first, block = (uint32_t)__ldg(G + WG_N_UNITS) * gh * per;
+    const uint32_t hb = r / block, rest = r - hb * block;
+    const uint32_t inner = min(gh, heads - hb * gh) * per;
+    const uint32_t u = rest / inner;
+    unit = __ldg(G + WG_FIRST) + (int)u;
+    h = (int)(hb * gh * per + rest - u * inner);
   }
 };
 
