@@ -255,7 +255,8 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   };
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+    // registers per thread: control 88, math 128, drain 168 (80 / 128 / 176 spilled in the issuing thread: kernel +2 %)
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
     if (warp == 0 && lane == 0) {
       // ------------------------------------------------------------------ TMA producer + scheduler
       uint32_t n = 0, it = 0;
@@ -568,7 +569,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   } else {
     // ------------------------------------------------------------------ drain warps: C3, dK/dV epilogue
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
     const int rb = warp & 3;
     const int row = rb * 32 + lane;             // TMEM lane: query row of dQ, key row of dK/dV
     const uint32_t t_dq = tmem_addr(tmem, rb * 32, C_DP);
