@@ -388,6 +388,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       int ks = __ldg(U + FU_KV0_BEGIN);
       const int nr0 = __ldg(U + FU_NT_RANGE0);
       float m_ref = -INFINITY;
+      bool s_ready = false;                      // the next step's scores were there at the last look (D = 64)
       float2 l01 = make_float2(0.f, 0.f), l23 = make_float2(0.f, 0.f);
 #pragma unroll 1
       for (int j = 0; j < nts; ++j, ++pcnt) {
@@ -398,7 +399,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const int limit = lim - ks;                // valid columns of this tile for this row
         ks += 128;
         const bool masked = __any_sync(0xffffffffu, limit < 128);
-        ok = mbar_wait_warp(BAR(B_SFULL + s), pcnt & 1, wctx, 30 + s);
+        if (!s_ready) ok = mbar_wait_warp(BAR(B_SFULL + s), pcnt & 1, wctx, 30 + s);
         if (!ok) break;
         tc_fence_after();
         uint32_t sv[4][32];
@@ -470,8 +471,12 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         ok = mbar_wait_warp(BAR(B_PFREE + s), (pcnt & 1) ^ 1, wctx, 34 + s);
         if (!ok) break;
         tc_fence_after();
+        // D = 64 has a score buffer per Q tile, so the next scores are mostly there: look before the stores of P instead of
+        // behind them (ragged 16K batch 91 -> 89 us); at D = 128 they are still being computed.
+        if (D == 64) s_ready = mbar_test(BAR(B_SFULL + s), (pcnt & 1) ^ 1);
 #pragma unroll
         for (int b = 0; b < 4; ++b) tmem_st16(t_p + b * 16, pk[b]);
+        if (D == 64) s_ready = __all_sync(0xffffffffu, s_ready) && j + 1 < nts;
         tc_wait_st();
         tc_fence_before();
         __syncwarp();
