@@ -463,23 +463,24 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       }
       BwdIter iter;
       iter.init(U, a.qranges, g);
-      float pre = load_row(iter, hk);
+      // Statistics of the unit's first tile -> shared memory, for all math warps.  Those of a later tile are written one tile
+      // ahead, into the other buffer, without a barrier of their own: lse after this tile's S^T has been seen (T1 comes
+      // after every warp's P^T of the tile before, the last use of that buffer) and before this tile's P^T is handed over,
+      // which T1 of the next tile waits for; delta in the same way between dP^T and dS^T.
+      float* rows0 = (float*)(smem + SM::ROWS_OFF);                              // [2][lse2[128] | delta[128]]
+      rows0[(it & 1) * 256 + mtid] = load_row(iter, hk);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(BAR(B_ROWS));
+      ok = mbar_wait_warp(BAR(B_ROWS), (n - 1) & 1, wctx, 134);
+      if (!ok) break;
 #pragma unroll 1
       for (; iter.valid; ++it) {
         const int q_row = iter.q_row, q_valid = iter.q_valid;
         const bool causal = iter.causal;
-        // Per-query-row statistics of this tile -> shared memory, double buffered by tile parity: a
-        // thread that gets here has passed the previous tile's barrier, so every thread has finished
-        // the tile before that one, the last reader of this buffer.  The next tile's values are
-        // fetched now and stay in flight while this tile is processed.
-        float* s_rows = (float*)(smem + SM::ROWS_OFF) + (it & 1) * 256;      // lse2[128] | delta[128]
-        s_rows[mtid] = pre;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(BAR(B_ROWS));
         iter.advance();
-        if (iter.valid) pre = load_row(iter, hk);
-        ok = mbar_wait_warp(BAR(B_ROWS), it & 1, wctx, 134);
-        if (!ok) break;
+        const float next_row = iter.valid ? load_row(iter, hk) : 0.f;            // in flight while this tile is processed
+        const float* s_rows = rows0 + (it & 1) * 256;
+        float* my_next = rows0 + ((it & 1) ^ 1) * 256 + mtid;
         const float* s_lse = s_rows + half * 64;
         const float* s_delta = s_rows + 128 + half * 64;
         const bool need_mask = causal || q_valid < 128 || kv_rows < 128;   // uniform across the CTA
@@ -487,6 +488,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         ok = mbar_wait_warp(BAR(B_SFULL), it & 1, wctx, 130);
         if (!ok) break;
         tc_fence_after();
+        if (mtid < 128) *my_next = next_row;
         // P^T fragments as bf16 pairs: pa = query columns [0,32) of this half, pb = [32,64); element 8 * g + 2 * j + i is
         // the pair of row frow + 16 * g + 8 * i and query group j.  C1 and C2 run as two rolled trips of 32 columns;
         // between the trips the pair arrays rotate (register arrays cannot be indexed by the trip), which halves the
@@ -533,6 +535,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         ok = mbar_wait_warp(BAR(B_DPFULL), it & 1, wctx, 131);
         if (!ok) break;
         tc_fence_after();
+        if (mtid >= 128) *my_next = next_row;
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           uint32_t dv_[32], out[16];
