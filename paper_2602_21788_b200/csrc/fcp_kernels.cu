@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* __r
     const int64_t t = t0 + i * RPP;
     if (t < T) {
       const int64_t src = t * hq + h0 + hl;
-      a[i] = __ldg(reinterpret_cast<const uint4*>(o + src * D + sub * 8));
+      a[i] = __ldcs(reinterpret_cast<const uint4*>(o + src * D + sub * 8));   // not read again: leaves the L2 to dO
       b[i] = __ldg(reinterpret_cast<const uint4*>(d_o + src * D + sub * 8));
     } else {
       a[i] = b[i] = make_uint4(0, 0, 0, 0);
