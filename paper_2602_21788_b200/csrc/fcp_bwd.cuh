@@ -8,19 +8,27 @@
 //   C1  P^T  = exp2(S^T*c - lse2[q])   (CUDA cores, thread = key row x half of the queries), bf16 over S^T
 //   T3  dV  += P^T dO                  (UMMA, TMEM x smem)      TMEM cols [256,384)
 //   C2  dS^T = P^T o (dP^T*scale - delta[q]*scale)               bf16 to smem
-//   T5  dQ^T = K^T dS^T  (D = 128; rows = head-dim index)  or  dQ = dS K  (D = 64; rows = queries)
-//                                      (UMMA, smem x smem)      over dP^T
+//   T5  dQ   = dS K                    (UMMA, smem x smem)      over dP^T
 //   T4  dK  += dS^T Q                  (UMMA, smem x smem)      TMEM cols [384,512); issued after T5 so
 //                                      that it runs while the drain warps read the dQ tile
-//   C3  dQ accumulator += tile         fp32 reductions to global memory, whole sectors per warp
+//   C3  dQ accumulator += tile         through shared memory, bulk fp32 reductions to global memory
 //
-// 16 warps: warp 0 TMA producer and work scheduler, warp 1 UMMA issuer (warps 2-3 idle), warps 4..11
-// the element-wise math C1/C2 (two warps per TMEM lane quarter, each half of the query columns),
-// warps 12..15 the dQ drain C3 and the dK/dV epilogue.  The issuer runs T1 of the next tile as soon
-// as C1 has read S^T, and T2 of the next tile as soon as C3 has drained dQ, so the tensor core, the
-// math warps and the drain warps work on different tiles at the same time.
+// 16 warps: warp 0 TMA producer and work scheduler, warp 1 UMMA issuer, warp 2 sends the dQ reductions (warp 3
+// idle), warps 4..11 the element-wise math C1/C2 (two warps per TMEM lane quarter, each half of the query
+// columns, on matrix fragments), warps 12..15 the dQ drain C3 and the dK/dV epilogue.  The issuer runs T1 of the
+// next tile as soon as T3 has consumed P^T, and T2 of the next tile as soon as C3 has drained dQ, so the tensor
+// core, the math warps and the drain warps work on different tiles at the same time.
 //
 // Work items are handed out through a global counter in the order of the plan's work groups.
+//
+// What bounds it (D = 128): about 4360 clk per 128 x 128 tile and head, of which the five products need 2570 when they
+// run alone (514-517 clk each).  S^T | dP^T | dV | dK fill the 512 columns of tensor memory, so there is no second tile in
+// flight behind which the hand-overs of P^T, dS^T and the drained dQ could hide.  The shared-memory data pipe is nearly as
+// full: 2310 wavefronts of operands and 1610 of the other warps per tile (counted before the statistics were written ahead).
+// Left out one by one on a 64K-token batch (19.4 ms): bulk reductions 17.1 ms, staging stores 18.7, exponentials 19.3.
+// The bulk reductions took the period from 5090 to 4412 clk.  Kernel with all of it, before -> now: 128K bimodal batch
+// 102 -> 92 ms, 64K log-normal batch 12.9 -> 11.6 ms, 8K batch 405 -> 260 us (there the work order counts most).
+// The math loops stay rolled: unrolling their trips costs 3-7 %.
 #pragma once
 #include "fcp_plan.hpp"
 #include "sm100_ptx.cuh"
@@ -128,9 +136,6 @@ struct BwdIter {
   }
 };
 
-__device__ __forceinline__ void red_add_f32(float* p, float v) {
-  asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
-}
 // dQ accumulator: the rows of one Q tile (128 packed rows from the start of a sequence on, fewer at its end) of one head
 // are rows * D consecutive floats, ordered [D / 4][rows][4].  A drain thread holds one query row, so its 16-byte pieces
 // lie next to those of its neighbours both in shared memory (no bank conflicts) and here, and a piece of 32 columns is
@@ -149,18 +154,13 @@ __device__ __forceinline__ void bulk_wait_read() {   // all but the last N reduc
 }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// Two element-wise operations of a math warp, as one two-wide instruction (WIDE) or two scalar ones.  Both give the same
-// bits.  Two-wide is faster at D = 64 (kernel -4 %), where the tile's products are short and the math warps are what
-// the tile waits for; at D = 128 it is slower (64K log-normal batch 12.9 -> 13.6 ms).
-template <bool WIDE>
+// Two element-wise operations of a math warp in one instruction, with the bits of two scalar ones.  Scalar at D = 128:
+// 64K log-normal batch 11.9 against 11.6 ms, 128K bimodal batch 93.8 against 92.0 ms, 8K batch 265 against 260 us.
 __device__ __forceinline__ float2 fma_pair(uint32_t x, uint32_t y, float2 m, float2 add) {
-  const float2 v = make_float2(__uint_as_float(x), __uint_as_float(y));
-  return WIDE ? fma2(v, m, add) : make_float2(fmaf(v.x, m.x, add.x), fmaf(v.y, m.y, add.y));
+  return fma2(make_float2(__uint_as_float(x), __uint_as_float(y)), m, add);
 }
-template <bool WIDE>
 __device__ __forceinline__ float2 mul_pair(float2 a, uint32_t bf16x2) {
-  const float2 b = make_float2(__uint_as_float(bf16x2 << 16), __uint_as_float(bf16x2 & 0xffff0000u));
-  return WIDE ? mul2(a, b) : make_float2(a.x * b.x, a.y * b.y);
+  return mul2(a, make_float2(__uint_as_float(bf16x2 << 16), __uint_as_float(bf16x2 & 0xffff0000u)));
 }
 
 template <int D>
@@ -508,7 +508,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll
             for (int g2 = 0; g2 < 4; ++g2) {               // row frow + 8 * g2
               const uint32_t* x = &sv[(g2 >> 1) * 16 + 4 * j + 2 * (g2 & 1)];
-              const float2 e = fma_pair<D == 64>(x[0], x[1], c22, l2);
+              const float2 e = fma_pair(x[0], x[1], c22, l2);
               pb[(g2 >> 1) * 8 + 2 * j + (g2 & 1)] = pack_bf16(ex2(e.x), ex2(e.y));
             }
           }
@@ -549,7 +549,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             for (int g2 = 0; g2 < 4; ++g2) {
               const uint32_t* x = &dv_[(g2 >> 1) * 16 + 4 * j + 2 * (g2 & 1)];
               const int e = (g2 >> 1) * 8 + 2 * j + (g2 & 1);
-              const float2 d = mul_pair<D == 64>(fma_pair<D == 64>(x[0], x[1], s22, d2), pa[e]);
+              const float2 d = mul_pair(fma_pair(x[0], x[1], s22, d2), pa[e]);
               out[e] = pack_bf16(d.x, d.y);
             }
           }
