@@ -879,7 +879,18 @@ namespace {
 // pass has the same work; runs of a batch with one long sequence are as unequal as its sequences (32K tokens of 32/8
 // heads, half of them one sequence: 23.0 ms with runs only, 17.5 now; the copies alone take 13.6).
 constexpr int64_t kHostSliceBytes = int64_t(8) << 20;
-constexpr int64_t kHostSlices = 16, kHostPasses = 8;
+//
+// That is for batches whose copies take as long as their kernels.  Above kHostFlopsPerByte (kernels at 1000 TFLOP/s against
+// input copies at 50 GB/s) the batch is cut by heads alone, into kHostSlices passes where it has as many heads: a run that
+// is one long sequence ends with few units left, pass after pass, while a pass over the whole batch has short ones for
+// that.  256K tokens with one of 128K, 98 000 flop/byte: 618 ms with runs, 585 without; 64K tokens of the 32/8-head
+// log-normal batch, 4 800 flop/byte: 32.1 ms with, 33.2 without.
+constexpr int64_t kHostSlices = 16, kHostPasses = 8, kHostFlopsPerByte = 20000;
+// Slices with fewer backward units than this per SM take turns on two kernel lanes, so that one fills the SMs that the
+// other's last units leave idle (30K tokens of 16/4 heads, D = 64, half a unit: 5.0 ms, one lane 6.7).  Larger ones fill the
+// chip by themselves, and two at once share its L2 (384K sequence, 20 units: 8390 ms, one lane 8125; 128K sequence, 7 units:
+// 625 and 609; 64K tokens, 2 units: both 32.9).
+constexpr int64_t kHostLaneUnits = 4;
 
 // Builds the runs' plans and creates the streams and events the host entry point orders its work with; all of it belongs
 // to the plan and is released by fcp_plan_destroy.
@@ -890,13 +901,17 @@ int build_host_groups(const fcp_plan* plan, void* stream) {
   const fcp_params& P = plan->params;
   const int64_t in_bytes = 2 * T * (P.hq + P.hkv) * P.head_dim * 2;
   const int64_t slices = std::max<int64_t>(1, std::min<int64_t>(kHostSlices, in_bytes / kHostSliceBytes));
-  const int32_t passes = (int32_t)std::min<int64_t>(std::min<int64_t>(P.hkv, kHostPasses), slices);
-  const int want = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(slices / passes, B), T / 8192));
   std::vector<int32_t> lens(B), degs(B);
+  double flops = 0;
   for (int b = 0; b < B; ++b) {
     lens[b] = plan->cu_seqlens[b + 1] - plan->cu_seqlens[b];
     degs[b] = (plan->chunk_offset[b + 1] - plan->chunk_offset[b] - 1) / 2;
+    flops += 7.0 * lens[b] * lens[b] * P.hq * P.head_dim;
   }
+  const bool by_heads = flops > (double)kHostFlopsPerByte * in_bytes;
+  const int64_t most = std::min<int64_t>(by_heads ? kHostSlices : kHostPasses, slices);
+  const int32_t passes = (int32_t)std::min<int64_t>(P.hkv, most);
+  const int want = by_heads ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(slices / passes, B), T / 8192));
   std::vector<fcp_plan*> groups;
   std::vector<int64_t> tok0;
   auto fail = [&](int rc) {
@@ -1002,9 +1017,8 @@ extern "C" int fcp_attn_fwd_bwd_host(const fcp_plan* plan, const void* q_host, c
   char* w = (char*)workspace;
   const int G = (int)plan->group_tok0.size() - 1;
   // Inputs of later slices come in (s_in) and results of earlier ones go out (s_out) while kernels run.  The kernels of
-  // consecutive slices alternate between `stream` and a second lane: a slice has few work units, and the next one fills
-  // the SMs that its longest units leave idle.  Everything is ordered after the work already queued on `stream` and is
-  // complete when this call returns.
+  // consecutive slices alternate between `stream` and a second lane where a slice has few work units.  Everything is
+  // ordered after the work already queued on `stream` and is complete when this call returns.
   cudaStream_t s_in = (cudaStream_t)plan->host_in, s_out = (cudaStream_t)plan->host_out, s_lane = (cudaStream_t)plan->host_lane;
   auto EV = [&](int i) { return (cudaEvent_t)plan->host_events[i]; };
   // The forward pass of a slice needs q, k, v only: dO follows them and arrives while the forward kernel runs; o leaves
@@ -1013,16 +1027,18 @@ extern "C" int fcp_attn_fwd_bwd_host(const fcp_plan* plan, const void* q_host, c
   struct Slice { int g, hk0, hkc, ev0; bool last; };
   std::vector<Slice> slices;
   const int per = (P.hkv + plan->host_passes - 1) / plan->host_passes;
-  int64_t lane_scratch = 0;                      // scratch of the largest slice
+  int64_t lane_scratch = 0, lane_units = 0;      // scratch and backward units of the largest slice
   {
     int ev0 = 3;
-    for (int g = 0; g < G; ++g)
-      for (int hk0 = 0; hk0 < P.hkv; hk0 += per, ev0 += 4) {
+    for (int g = 0; g < G; ++g) {
+      const fcp_plan* sub = plan->groups.empty() ? plan : plan->groups[g];
+      lane_scratch = std::max(lane_scratch, al(bwd_scratch_need(sub, per)));
+      lane_units = std::max(lane_units, (int64_t)(sub->bwd_units.size() / FCP_BWD_UNIT_W) * per);
+      for (int hk0 = 0; hk0 < P.hkv; hk0 += per, ev0 += 4)
         slices.push_back(Slice{g, hk0, std::min(per, P.hkv - hk0), ev0, hk0 + per >= P.hkv});
-        lane_scratch = std::max(lane_scratch, al(bwd_scratch_need(plan->groups.empty() ? plan : plan->groups[g], per)));
-      }
+    }
   }
-  const bool two_lanes = slices.size() > 1 && 2 * lane_scratch <= al(bwd_scratch_need(plan, P.hkv));
+  const bool two_lanes = slices.size() > 1 && lane_units < kHostLaneUnits * plan->sm_count && 2 * lane_scratch <= al(bwd_scratch_need(plan, P.hkv));
   const int gq = P.hq / P.hkv;
   HostDrain drain{s_in, s_out, st, s_lane};
   FCP_CUDA_CHECK(cudaEventRecord(EV(0), st));

@@ -116,6 +116,8 @@ def test_plan_blocks_are_handed_on_only_after_the_work_that_reads_them(threads):
     ([12000, 7000, 1001], 6, 3, 64),                # odd number of KV heads: one pass each, two kernel lanes
     ([5000, 9000, 6000, 4000], 8, 1, 128),          # one KV head: runs of sequences only
     ([11000, 8000, 1500, 6000], 20, 10, 128),       # passes of two KV heads and runs
+    ([19100, 300, 129], 8, 4, 128),                 # long enough for its copies to be cut by heads alone, two lanes
+    ([24700, 300], 64, 64, 64),                     # the same with slices that fill the chip: one lane
 ])
 def test_host_entry_point_slices(lens, hq, hkv, D):
     """fcp_attn_fwd_bwd_host == the device calls, bit for bit where those are deterministic, on a first and a second call."""
