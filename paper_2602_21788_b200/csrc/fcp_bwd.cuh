@@ -21,12 +21,13 @@
 //
 // Work items are handed out through a global counter in the order of the plan's work groups.
 //
-// What bounds it (D = 128): about 4360 clk per 128 x 128 tile and head, of which the five products need 2570 when they
-// run alone (514-517 clk each).  S^T | dP^T | dV | dK fill the 512 columns of tensor memory, so there is no second tile in
+// What bounds it (D = 128): about 3880 clk per 128 x 128 tile and head (tensor pipe 66 % busy, one 128K sequence among short
+// ones, 5 heads), of which the five products need 2570 when they run alone (514-517 clk each).  S^T | dP^T | dV | dK fill the 512 columns of tensor memory, so there is no second tile in
 // flight behind which the hand-overs of P^T, dS^T and the drained dQ could hide.  The shared-memory data pipe is nearly as
-// full: 2310 wavefronts of operands and 1610 of the other warps per tile (counted before the statistics were written ahead).
+// full: 2310 wavefronts of operands and 1610 of the other warps per tile (counted before the statistics were written ahead, at 4360 clk).
 // Left out one by one on a 64K-token batch (19.4 ms): bulk reductions 17.1 ms, staging stores 18.7, exponentials 19.3.
-// The bulk reductions took the period from 5090 to 4412 clk.  Kernel with all of it, before -> now: 128K bimodal batch
+// The bulk reductions took the period from 5090 to 4412 clk, what followed to 3880; under the power cap the clock falls
+// meanwhile, so that the time goes down less.  Kernel with all of it, before -> now: 128K bimodal batch
 // 102 -> 92 ms, 64K log-normal batch 12.9 -> 11.6 ms, 8K batch 405 -> 260 us (there the work order counts most).
 // The math loops stay rolled: unrolling their trips costs 3-7 %.
 #pragma once
