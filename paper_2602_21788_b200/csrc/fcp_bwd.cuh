@@ -446,7 +446,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const float* my_rows = (mtid < 128 ? a.lse2_t : a.delta_t) + (mtid & 127);
     auto load_row = [&](const BwdIter& x, int hk) -> float {
       const int64_t t = (int64_t)x.q_row + (mtid & 127);
-      return t < a.T ? __ldg(my_rows + (int64_t)((hk - a.hk_begin) * g + x.hh) * a.t_stride + x.q_row) : 0.f;
+      return t < a.T ? ld_f32(my_rows + (int64_t)((hk - a.hk_begin) * g + x.hh) * a.t_stride + x.q_row) : 0.f;
     };
     uint32_t n = 0, it = 0;
     bool ok = true;

@@ -124,8 +124,8 @@ int check_plan(const fcp_plan* plan) {
 // ---------------------------------------------------------------------------------------------
 template <int D>
 __global__ void __launch_bounds__(256) fcp_merge_kernel(const int32_t* __restrict__ units, const int32_t* __restrict__ slot_offset,
-                                                        const int32_t* __restrict__ slot_rows, const float* __restrict__ o_partial,
-                                                        const float* __restrict__ lse_partial, int head_begin, int head_count,
+                                                        const int32_t* __restrict__ slot_rows, const float* o_partial,
+                                                        const float* lse_partial, int head_begin, int head_count,
                                                         int hq, __nv_bfloat16* __restrict__ o, float* __restrict__ o_f32, float* __restrict__ lse) {
   grid_begin();
   constexpr int TPR = D / 8;                 // threads per (token, head) row
@@ -139,17 +139,17 @@ __global__ void __launch_bounds__(256) fcp_merge_kernel(const int32_t* __restric
     const int t = tok0 + r / head_count, hl = r % head_count;
     const int64_t rel = t - ctok0;
     float m = -INFINITY;
-    for (int s = 0; s < ns; ++s) m = fmaxf(m, __ldg(lse_partial + ((int64_t)slot_rows[s0 + s] + rel) * head_count + hl));
+    for (int s = 0; s < ns; ++s) m = fmaxf(m, ld_f32(lse_partial + ((int64_t)slot_rows[s0 + s] + rel) * head_count + hl));
     float z = 0.f;
     for (int s = 0; s < ns; ++s)
-      z += __expf(__ldg(lse_partial + ((int64_t)slot_rows[s0 + s] + rel) * head_count + hl) - m);
+      z += __expf(ld_f32(lse_partial + ((int64_t)slot_rows[s0 + s] + rel) * head_count + hl) - m);
     const float L = m + __logf(z);
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (int s = 0; s < ns; ++s) {
       const int64_t prow = ((int64_t)slot_rows[s0 + s] + rel) * head_count + hl;
-      const float wgt = __expf(__ldg(lse_partial + prow) - L);
-      const float4* src = reinterpret_cast<const float4*>(o_partial + prow * D + sub * 8);
-      const float4 a0 = __ldcs(src), a1 = __ldcs(src + 1);
+      const float wgt = __expf(ld_f32(lse_partial + prow) - L);
+      const float* src = o_partial + prow * D + sub * 8;
+      const float4 a0 = ld_stream_f4(src), a1 = ld_stream_f4(src + 4);
       acc[0] += wgt * a0.x; acc[1] += wgt * a0.y; acc[2] += wgt * a0.z; acc[3] += wgt * a0.w;
       acc[4] += wgt * a1.x; acc[5] += wgt * a1.y; acc[6] += wgt * a1.z; acc[7] += wgt * a1.w;
     }
@@ -176,8 +176,8 @@ __global__ void __launch_bounds__(256) fcp_merge_kernel(const int32_t* __restric
 // that the transposed statistics leave as whole sectors.
 constexpr int DELTA_TOKENS = 64;
 template <int D>
-__global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
-                                                        const float* __restrict__ lse, int64_t T, int hq, int h0, int hc,
+__global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* o, const __nv_bfloat16* d_o,
+                                                        const float* lse, int64_t T, int hq, int h0, int hc,
                                                         int64_t t_stride, float scale, float* __restrict__ delta_t,
                                                         float* __restrict__ lse2_t, float* __restrict__ dq_acc,
                                                         int32_t* __restrict__ counter) {
@@ -193,8 +193,8 @@ __global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* __r
     const int64_t t = t0 + i * RPP;
     if (t < T) {
       const int64_t src = t * hq + h0 + hl;
-      a[i] = __ldcs(reinterpret_cast<const uint4*>(o + src * D + sub * 8));   // not read again: leaves the L2 to dO
-      b[i] = __ldg(reinterpret_cast<const uint4*>(d_o + src * D + sub * 8));
+      a[i] = ld_stream_v4(o + src * D + sub * 8);   // leaves the L2 to dO
+      b[i] = ld_v4(d_o + src * D + sub * 8);
     } else {
       a[i] = b[i] = make_uint4(0, 0, 0, 0);
     }
@@ -220,18 +220,17 @@ __global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* __r
     }
 #pragma unroll
     for (int off = TPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (t < T && sub == 0) {
-      delta_t[hl * t_stride + t] = -acc * scale;
-      lse2_t[hl * t_stride + t] = lse[t * hq + h0 + hl] * -1.4426950408889634f;
-    }
+    if (t < T && sub == 0) delta_t[hl * t_stride + t] = -acc * scale;
   }
+  const int64_t tl = t0 - threadIdx.x / TPR + threadIdx.x;               // a thread per row for the log-sum-exps
+  if (threadIdx.x < DELTA_TOKENS && tl < T) lse2_t[hl * t_stride + tl] = ld_f32(lse + tl * hq + h0 + hl) * -1.4426950408889634f;
 }
 
 // fp32 dQ accumulator (tiles of dq_tile: [D / 4][rows][4]) -> bf16 dq [T][hq][D], heads [h0, h0 + gridDim.y).  One CTA per
 // (tile, head): it reads rows * D contiguous floats with lanes along the rows and turns them round in shared memory, so
 // that both sides move whole sectors.  Q tiles are cut like key tiles, so the backward units list them.
 template <int D>
-__global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq,
+__global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* acc, __nv_bfloat16* __restrict__ dq,
                                                              const int32_t* __restrict__ units, int64_t T, int hq, int h0) {
   grid_begin();
   constexpr int PITCH = D + 8;                // bf16 elements per row in shared memory: 16 bytes of padding
@@ -239,13 +238,19 @@ __global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* __rest
   const int32_t* U = units + (size_t)blockIdx.x * FCP_BWD_UNIT_W;
   const int64_t t0 = __ldg(U + BU_KV_ROW0);
   const int rows = __ldg(U + BU_KV_ROWS);
-  const float4* src = reinterpret_cast<const float4*>(acc + ((int64_t)blockIdx.y * T + t0) * D);
+  const float* src = acc + ((int64_t)blockIdx.y * T + t0) * D;
   const int row = threadIdx.x & 127;
   if (row < rows) {
-#pragma unroll 8
-    for (int c = threadIdx.x >> 7; c < D / 4; c += 2) {
-      const float4 v = __ldcs(src + c * rows + row);
-      *reinterpret_cast<uint2*>(tile + row * PITCH + c * 4) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+    constexpr int N = 8;                      // loads in flight per thread
+#pragma unroll
+    for (int c0 = 0; c0 < D / 4; c0 += 2 * N) {
+      float4 v[N];
+#pragma unroll
+      for (int i = 0; i < N; ++i) v[i] = ld_stream_f4(src + ((c0 + 2 * i + (threadIdx.x >> 7)) * rows + row) * 4);
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        *reinterpret_cast<uint2*>(tile + row * PITCH + (c0 + 2 * i + (threadIdx.x >> 7)) * 4) =
+            make_uint2(pack_bf16(v[i].x, v[i].y), pack_bf16(v[i].z, v[i].w));
     }
   }
   __syncthreads();

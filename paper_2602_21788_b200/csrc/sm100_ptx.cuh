@@ -47,6 +47,29 @@ __device__ __forceinline__ void grid_begin() {
   grid_launch_next();
   grid_wait();
 }
+// A kernel is therefore resident while the one before it still writes, and its inputs are not read-only for as long as it
+// lives, which ld.global.nc (__ldg, or a const __restrict__ parameter) requires; such a load, and one of the unmarked load
+// intrinsics (__ldcs), may also be scheduled above the wait.  So everything that an earlier kernel may have written is read
+// with the loads below (or by TMA); __ldg is for the plan's tables, which are complete before any launch that reads them.
+__device__ __forceinline__ float ld_f32(const float* p) {
+  float x;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ uint4 ld_v4(const void* p) {
+  uint4 x;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ uint4 ld_stream_v4(const void* p) {   // not needed again: first out of the L2
+  uint4 x;
+  asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ float4 ld_stream_f4(const float* p) {
+  const uint4 x = ld_stream_v4(p);
+  return make_float4(__uint_as_float(x.x), __uint_as_float(x.y), __uint_as_float(x.z), __uint_as_float(x.w));
+}
 
 // ----------------------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
