@@ -226,19 +226,20 @@ __global__ void __launch_bounds__(256) fcp_delta_kernel(const __nv_bfloat16* o, 
   if (threadIdx.x < DELTA_TOKENS && tl < T) lse2_t[hl * t_stride + tl] = ld_f32(lse + tl * hq + h0 + hl) * -1.4426950408889634f;
 }
 
-// fp32 dQ accumulator (tiles of dq_tile: [D / 4][rows][4]) -> bf16 dq [T][hq][D], heads [h0, h0 + gridDim.y).  One CTA per
-// (tile, head): it reads rows * D contiguous floats with lanes along the rows and turns them round in shared memory, so
+// fp32 dQ accumulator (tiles of dq_tile: [D / 4][rows][4]) -> bf16 dq [T][hq][D], heads from h0 on.  One CTA per (head,
+// tile), all in one grid dimension (the others end at 65535): it reads rows * D contiguous floats with lanes along the rows and turns them round in shared memory, so
 // that both sides move whole sectors.  Q tiles are cut like key tiles, so the backward units list them.
 template <int D>
 __global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* acc, __nv_bfloat16* __restrict__ dq,
-                                                             const int32_t* __restrict__ units, int64_t T, int hq, int h0) {
+                                                             const int32_t* __restrict__ units, int n_units, int64_t T, int hq, int h0) {
   grid_begin();
   constexpr int PITCH = D + 8;                // bf16 elements per row in shared memory: 16 bytes of padding
   __shared__ __align__(16) __nv_bfloat16 tile[128 * PITCH];
-  const int32_t* U = units + (size_t)blockIdx.x * FCP_BWD_UNIT_W;
+  const int hl = blockIdx.x / n_units;
+  const int32_t* U = units + (size_t)(blockIdx.x - hl * n_units) * FCP_BWD_UNIT_W;
   const int64_t t0 = __ldg(U + BU_KV_ROW0);
   const int rows = __ldg(U + BU_KV_ROWS);
-  const float* src = acc + ((int64_t)blockIdx.y * T + t0) * D;
+  const float* src = acc + ((int64_t)hl * T + t0) * D;
   const int row = threadIdx.x & 127;
   if (row < rows) {
     constexpr int N = 8;                      // loads in flight per thread
@@ -255,7 +256,7 @@ __global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* acc, _
   }
   __syncthreads();
   constexpr int TPR = D / 8;                  // threads per row, 16 bytes each
-  __nv_bfloat16* dst = dq + ((t0 * hq) + h0 + blockIdx.y) * (int64_t)D;
+  __nv_bfloat16* dst = dq + ((t0 * hq) + h0 + hl) * (int64_t)D;
   for (int r = threadIdx.x / TPR; r < rows; r += 256 / TPR) {
     const int c = (threadIdx.x % TPR) * 8;
     *reinterpret_cast<uint4*>(dst + (int64_t)r * hq * D + c) = *reinterpret_cast<const uint4*>(tile + r * PITCH + c);
@@ -776,12 +777,12 @@ int run_bwd(const fcp_plan* plan, const BwdTables& tb, const void* q, const void
       FCP_CUDA_CHECK(launch(fcp_bwd_kernel<64>, grid, BWD_THREADS, BwdSmem<64>::DYN_BYTES, st, tq, tk, tv, tdo, a));
   }
   {
-    const dim3 grid_c((unsigned)n_units, (unsigned)hc);
+    const unsigned grid_c = (unsigned)n_units * hc;
     ProfScope ps(prof, 4, st);
     if (D == 128)
-      FCP_CUDA_CHECK(launch(fcp_dq_convert_kernel<128>, grid_c, 256, 0, st, dq_acc, (__nv_bfloat16*)dq, tb.units, T, P.hq, h0));
+      FCP_CUDA_CHECK(launch(fcp_dq_convert_kernel<128>, grid_c, 256, 0, st, dq_acc, (__nv_bfloat16*)dq, tb.units, n_units, T, P.hq, h0));
     else
-      FCP_CUDA_CHECK(launch(fcp_dq_convert_kernel<64>, grid_c, 256, 0, st, dq_acc, (__nv_bfloat16*)dq, tb.units, T, P.hq, h0));
+      FCP_CUDA_CHECK(launch(fcp_dq_convert_kernel<64>, grid_c, 256, 0, st, dq_acc, (__nv_bfloat16*)dq, tb.units, n_units, T, P.hq, h0));
   }
   return FCP_OK;
 }

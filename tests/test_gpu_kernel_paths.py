@@ -150,3 +150,14 @@ def test_host_entry_point_slices(lens, hq, hkv, D):
 ])
 def test_forward_with_split_and_whole_units(lens, hq, hkv, D):
     _check(_wl(lens, [1] * len(lens), hq, hkv, D, seed=17))
+
+
+@pytest.mark.parametrize("hq", [65535, 65600])     # around the limit of a grid's second dimension
+def test_backward_of_more_query_heads_than_a_grid_dimension_holds(hq):
+    from paper_2602_21788_b200.runner import run_fwd_bwd
+    w = _wl([2, 1], [1, 1], hq, 1, 64, seed=19)
+    q, k, v, do = w.tensors()
+    res = run_fwd_bwd(w, q, k, v, do, fused=True, want_o_f32=False)
+    some = np.r_[0:3, hq - 67:hq - 62, hq - 2:hq]  # query heads that share the one KV head are independent
+    dq_ref, _, _ = A.attention_bwd_packed(f64(q[:, some]), f64(k), f64(v), f64(do[:, some]), w.cu_seqlens)
+    assert _rel(res["dq"][:, some], dq_ref) <= 2e-2
