@@ -1117,6 +1117,9 @@ extern "C" int fcp_attn_fwd_bwd_host(const fcp_plan* plan, const void* q_host, c
 static __device__ __align__(256) unsigned char g_noalloc_arena[FCP_NOALLOC_MAX_BYTES];
 
 namespace {
+// The work groups of the backward list lie in the 256 bytes of the status words, from word 32 on: eight rows fit, and an arena
+// of half a group's 64 MB of dQ rows (order_units of fcp_plan.cpp) holds batches of two at most, one and its tail.
+constexpr int kNoallocGroupsWord = 32, kNoallocGroupsWords = 32;
 unsigned char* g_noalloc_ptr[kMaxDevices] = {};   // device address of the arena, per device
 int g_noalloc_sms[kMaxDevices] = {};
 
@@ -1146,7 +1149,7 @@ extern "C" int fcp_noalloc_bytes_needed(const fcp_plan* plan, int64_t* bytes) {
   int64_t scratch = 0;
   fcp_plan_workspace_bytes(plan, 1, nullptr, nullptr, &scratch);
   *bytes = 256 + al((int64_t)plan->bwd_units.size() * 4) + al((int64_t)plan->bwd_qranges.size() * 4) +
-           al((int64_t)plan->bwd_work.size() * 4) + al((int64_t)plan->bwd_groups.size() * 4) + al(scratch);
+           al((int64_t)plan->bwd_work.size() * 4) + al(scratch);
   return FCP_OK;
 }
 
@@ -1162,7 +1165,7 @@ extern "C" int fcp_attn_bwd_noalloc(const fcp_plan* plan, const void* q, const v
   }
   int64_t need = 0;
   fcp_noalloc_bytes_needed(plan, &need);
-  if (need > (int64_t)FCP_NOALLOC_MAX_BYTES) {
+  if (need > (int64_t)FCP_NOALLOC_MAX_BYTES || plan->bwd_groups.size() > kNoallocGroupsWords) {
     fcp_set_error("fcp_attn_bwd_noalloc: this batch needs %lld bytes of scratch, the built-in arena holds %lld; "
                   "use fcp_attn_bwd with a caller-provided scratch buffer",
                   (long long)need, (long long)FCP_NOALLOC_MAX_BYTES);
@@ -1180,13 +1183,13 @@ extern "C" int fcp_attn_bwd_noalloc(const fcp_plan* plan, const void* q, const v
   cudaStream_t st = (cudaStream_t)stream;
   const fcp_params& P = plan->params;
 
-  // carve the arena: [status, counter | units | qranges | work | scratch]
+  // carve the arena: [status, counter, groups | units | qranges | work | scratch]
   int64_t off = 256;
   int32_t* d_status = (int32_t*)base;
   int32_t* d_units = (int32_t*)(base + off);    off += al((int64_t)plan->bwd_units.size() * 4);
   int32_t* d_qranges = (int32_t*)(base + off);  off += al((int64_t)plan->bwd_qranges.size() * 4);
   int32_t* d_work = (int32_t*)(base + off);     off += al((int64_t)plan->bwd_work.size() * 4);
-  int32_t* d_groups = (int32_t*)(base + off);   off += al((int64_t)plan->bwd_groups.size() * 4);
+  int32_t* d_groups = d_status + kNoallocGroupsWord;
   unsigned char* d_scratch = base + off;
 
   // the arena still holds the previous call's data: status, work counter and the dQ accumulator

@@ -60,3 +60,19 @@ def test_groups_go_longest_sequence_first_and_by_cost_within(lens, hq, hkv, D):
         g = units[late[0]:]
         assert np.all(np.diff(g[:, 5]) <= 0) and g[:, 5].sum() <= 0.15 * units[:, 5].sum()
         assert g[:, 5].max() <= min(units[f:f + n, 5].min() for f, n, _, _ in groups)
+
+
+@pytest.mark.parametrize("lens,hq,hkv,D", [
+    ([64486, 1], 1, 1, 128),              # exactly the built-in arena
+    ([63487] + [1] * 12, 2, 1, 64),       # the same, thirteen sequences
+    ([1500, 300, 77], 4, 2, 128),
+    ([32243] + [1] * 7, 2, 1, 128),
+])
+def test_noalloc_arena_holds_tables_and_scratch_and_nothing_for_the_order(lens, hq, hkv, D):
+    al = lambda x: (x + 255) // 256 * 256
+    T, tpad = sum(lens), al(sum(lens)) + 256
+    units = sum(-(-n // 128) for n in lens)
+    need = 256 + al(32 * units) + al(16 * len(lens)) + al(4 * units) + al(4 * T * hq * D + 8 * tpad * hq)
+    plan = fcp.Plan(lens, [1] * len(lens), hq, hkv, D)
+    assert fcp.fcp_noalloc_bytes_needed(plan) == need <= fcp.FCP_NOALLOC_MAX_BYTES
+    assert len(plan.table("bwd_groups")) <= 2

@@ -78,3 +78,23 @@ def test_noalloc_rejects_batches_beyond_the_builtin_arena():
         fcp.fcp_attn_bwd_noalloc(big, x, x, x, x, x, x, x, x, x, 0)
     assert e.value.status == fcp.FCP_ERR_WORKSPACE
     assert "arena" in str(e.value)
+
+
+def test_noalloc_runs_a_batch_that_fills_the_builtin_arena():
+    from paper_2602_21788_b200 import fcp
+    from paper_2602_21788_b200.runner import DeviceState
+    w = synth.Workload(name="full", seed=23, seqlens=np.asarray([64486, 1], np.int32), cp_degrees=np.asarray([1, 1], np.int32),
+                       hq=1, hkv=1, head_dim=128)
+    ds = DeviceState(w, *w.device_tensors(), partials=False)
+    ds.forward_fused()
+    ds.backward()
+    torch.cuda.synchronize()
+    ds.check_status()
+    host_plan = fcp.fcp_plan_blocks(w.seqlens, w.cp_degrees, 1, 1, 128)
+    dq, dk, dv = torch.empty_like(ds.dq), torch.empty_like(ds.dk), torch.empty_like(ds.dv)
+    fcp.fcp_attn_bwd_noalloc(host_plan, ds.q, ds.k, ds.v, ds.o, ds.do, ds.lse, dq, dk, dv,
+                             torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert fcp.fcp_noalloc_device_status()[0] == 0
+    assert torch.equal(dk, ds.dk) and torch.equal(dv, ds.dv)
+    assert (dq.float() - ds.dq.float()).norm() <= 1e-2 * ds.dq.float().norm()
