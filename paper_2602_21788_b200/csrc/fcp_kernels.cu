@@ -268,23 +268,22 @@ __global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* acc, _
 // ---------------------------------------------------------------------------------------------
 // Device blocks for the plans' tables.  Every new batch uploads a plan and drops the one before it, and cudaMalloc,
 // cudaFree (which waits for the whole device), the device query and the kernel attributes cost milliseconds each time:
-// a 16K-token batch took 6.8 ms for 2.8 ms of kernels.  So a destroyed plan's block goes to a short list per device and
-// is handed to the next plan once the event recorded after the last compute call that read it has completed; nothing
-// waits for it.  The list holds at most 8 blocks and 32 MB (the oldest leave first), larger blocks are never kept, and
-// fcp_release_cached gives all idle ones back.
+// with them a 16K-token batch takes 6.8 ms for 2.8 ms of kernels.  So a destroyed plan's block goes to a short list and
+// is handed to the next plan once the event recorded after the last compute call that read it has completed.  The list
+// holds at most 8 blocks and 32 MB (the oldest leave first), larger blocks are never kept, and fcp_release_cached gives
+// all idle ones back.
+// Memory, streams and kernel attributes belong to a CUDA context, so each context has a list of its own.
+struct PlanPool;
 struct PlanBlock {
   void* dev = nullptr;           // tables
   void* host = nullptr;          // pinned staging of the same size: one copy per upload
   size_t bytes = 0;
   cudaEvent_t used = nullptr;    // after the last compute call that read the block
+  PlanPool* pool = nullptr;
 };
 
-namespace {
-constexpr int kMaxDevices = 64;
-constexpr size_t kBlockMin = size_t(64) << 10, kBlockKeepMax = size_t(8) << 20, kKeepBytes = size_t(32) << 20;
-constexpr size_t kKeepBlocks = 8;
-
-struct DeviceState {
+struct PlanPool {
+  unsigned long long context = 0;
   std::mutex mu;
   bool ready = false;            // device checked, attributes set, stream created
   int sm_count = 0;
@@ -292,7 +291,42 @@ struct DeviceState {
   std::vector<PlanBlock*> idle;  // oldest first
   size_t idle_bytes = 0;
 };
-DeviceState g_device[kMaxDevices];
+
+namespace {
+constexpr int kMaxDevices = 64;
+constexpr size_t kBlockMin = size_t(64) << 10, kBlockKeepMax = size_t(8) << 20, kKeepBytes = size_t(32) << 20;
+constexpr size_t kKeepBlocks = 8;
+
+// The current context's pool.  Pools are never taken down: the id of a context is not used again.
+int current_pool(PlanPool** out) {
+  typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long*);
+  static CtxGetIdFn get_id = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    return cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess
+               ? (CtxGetIdFn)p : nullptr;
+  }();
+  static std::mutex mu;
+  static std::vector<PlanPool*>& pools = *new std::vector<PlanPool*>();
+  unsigned long long id = 0;
+  if (!get_id || get_id(nullptr, &id) != CUDA_SUCCESS) {
+    FCP_CUDA_CHECK(cudaFree(nullptr));           // a thread without a context yet: the runtime makes the device's current
+    if (!get_id || get_id(nullptr, &id) != CUDA_SUCCESS) {
+      fcp_set_error("cuCtxGetId failed");
+      return FCP_ERR_CUDA;
+    }
+  }
+  std::lock_guard<std::mutex> lock(mu);
+  for (PlanPool* p : pools)
+    if (p->context == id) {
+      *out = p;
+      return FCP_OK;
+    }
+  pools.push_back(new PlanPool());
+  pools.back()->context = id;
+  *out = pools.back();
+  return FCP_OK;
+}
 
 void free_block(PlanBlock* b) {
   if (b->dev) cudaFree(b->dev);
@@ -301,10 +335,11 @@ void free_block(PlanBlock* b) {
   delete b;
 }
 
-// Once per device: architecture check, shared-memory opt-in of the tensor-core kernels, the upload stream.
-int device_setup(int dev, DeviceState& ds) {
-  if (ds.ready) return FCP_OK;
-  int major = 0, sms = 0;
+// Once per context: architecture check, shared-memory opt-in of the tensor-core kernels, the upload stream.
+int pool_setup(PlanPool& pool) {
+  if (pool.ready) return FCP_OK;
+  int dev = 0, major = 0, sms = 0;
+  FCP_CUDA_CHECK(cudaGetDevice(&dev));
   FCP_CUDA_CHECK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
   FCP_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   if (major != 10) {
@@ -315,33 +350,38 @@ int device_setup(int dev, DeviceState& ds) {
   FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<128>::DYN_BYTES));
   FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_bwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<64>::DYN_BYTES));
   FCP_CUDA_CHECK(cudaFuncSetAttribute(fcp_bwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdSmem<128>::DYN_BYTES));
-  FCP_CUDA_CHECK(cudaStreamCreateWithFlags(&ds.copy, cudaStreamNonBlocking));
-  ds.sm_count = sms;
-  ds.ready = true;
+  FCP_CUDA_CHECK(cudaStreamCreateWithFlags(&pool.copy, cudaStreamNonBlocking));
+  pool.sm_count = sms;
+  pool.ready = true;
   return FCP_OK;
+}
+
+// Whether no queued work reads the block any more.  (cudaErrorNotReady is left behind as the thread's last error.)
+bool is_free(const PlanBlock* b) {
+  const cudaError_t e = cudaEventQuery(b->used);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess;
 }
 
 // A block of at least `bytes`: the smallest idle one that fits and that no queued work reads any more; with a full list
 // the oldest one that fits, whose event the caller then waits for (a new block would push out one in use, and freeing
 // that waits for the whole device); else a new one.
-int acquire_block(DeviceState& ds, size_t bytes, PlanBlock** out) {
-  size_t best = ds.idle.size();
-  for (size_t i = 0; i < ds.idle.size(); ++i) {
-    PlanBlock* b = ds.idle[i];
-    if (b->bytes >= bytes && (best == ds.idle.size() || b->bytes < ds.idle[best]->bytes) &&
-        cudaEventQuery(b->used) == cudaSuccess)
-      best = i;
+int acquire_block(PlanPool& pool, size_t bytes, PlanBlock** out) {
+  size_t best = pool.idle.size();
+  for (size_t i = 0; i < pool.idle.size(); ++i) {
+    PlanBlock* b = pool.idle[i];
+    if (b->bytes >= bytes && (best == pool.idle.size() || b->bytes < pool.idle[best]->bytes) && is_free(b)) best = i;
   }
-  cudaGetLastError();            // cudaErrorNotReady of a query is no error
-  if (best == ds.idle.size() && ds.idle.size() >= kKeepBlocks)
-    for (best = 0; best < ds.idle.size() && ds.idle[best]->bytes < bytes;) ++best;
-  if (best < ds.idle.size()) {
-    *out = ds.idle[best];
-    ds.idle_bytes -= (*out)->bytes;
-    ds.idle.erase(ds.idle.begin() + best);
+  if (best == pool.idle.size() && pool.idle.size() >= kKeepBlocks)
+    for (best = 0; best < pool.idle.size() && pool.idle[best]->bytes < bytes;) ++best;
+  if (best < pool.idle.size()) {
+    *out = pool.idle[best];
+    pool.idle_bytes -= (*out)->bytes;
+    pool.idle.erase(pool.idle.begin() + best);
     return FCP_OK;
   }
   PlanBlock* b = new PlanBlock();
+  b->pool = &pool;
   b->bytes = kBlockMin;
   while (b->bytes < bytes && b->bytes < kBlockKeepMax) b->bytes *= 2;
   b->bytes = std::max(b->bytes, bytes);
@@ -359,21 +399,21 @@ int acquire_block(DeviceState& ds, size_t bytes, PlanBlock** out) {
 
 // `keep`: the event of the block covers all work that may still read it.  Otherwise (and for large blocks) the memory
 // is freed, which waits for the device.
-void return_block(int dev, PlanBlock* b, bool keep) {
-  if (!keep || b->bytes > kBlockKeepMax || dev < 0 || dev >= kMaxDevices) {
+void return_block(PlanBlock* b, bool keep) {
+  if (!keep || b->bytes > kBlockKeepMax) {
     free_block(b);
     return;
   }
-  DeviceState& ds = g_device[dev];
+  PlanPool& pool = *b->pool;
   std::vector<PlanBlock*> out;
   {
-    std::lock_guard<std::mutex> lock(ds.mu);
-    ds.idle.push_back(b);
-    ds.idle_bytes += b->bytes;
-    while (ds.idle.size() > kKeepBlocks || ds.idle_bytes > kKeepBytes) {
-      out.push_back(ds.idle.front());
-      ds.idle_bytes -= ds.idle.front()->bytes;
-      ds.idle.erase(ds.idle.begin());
+    std::lock_guard<std::mutex> lock(pool.mu);
+    pool.idle.push_back(b);
+    pool.idle_bytes += b->bytes;
+    while (pool.idle.size() > kKeepBlocks || pool.idle_bytes > kKeepBytes) {
+      out.push_back(pool.idle.front());
+      pool.idle_bytes -= pool.idle.front()->bytes;
+      pool.idle.erase(pool.idle.begin());
     }
   }
   for (PlanBlock* x : out) free_block(x);
@@ -394,14 +434,14 @@ void mark_used(const fcp_plan* plan, cudaStream_t st) {
 }  // namespace
 
 extern "C" int fcp_release_cached(void) {
-  int dev = 0;
-  FCP_CUDA_CHECK(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= kMaxDevices) return FCP_OK;
+  PlanPool* pool = nullptr;
+  int rc = current_pool(&pool);
+  if (rc != FCP_OK) return rc;
   std::vector<PlanBlock*> out;
   {
-    std::lock_guard<std::mutex> lock(g_device[dev].mu);
-    out.swap(g_device[dev].idle);
-    g_device[dev].idle_bytes = 0;
+    std::lock_guard<std::mutex> lock(pool->mu);
+    out.swap(pool->idle);
+    pool->idle_bytes = 0;
   }
   for (PlanBlock* b : out) free_block(b);
   return FCP_OK;
@@ -411,13 +451,9 @@ extern "C" int fcp_plan_upload(fcp_plan* plan, void* stream) {
   (void)stream;                  // the call is complete when it returns, whatever is queued there
   if (!plan) return FCP_ERR_INVALID_ARG;
   if (plan->d_blob) return FCP_OK;
-  int dev = 0;
-  FCP_CUDA_CHECK(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= kMaxDevices) {
-    fcp_set_error("device index %d not supported", dev);
-    return FCP_ERR_UNSUPPORTED;
-  }
-  DeviceState& ds = g_device[dev];
+  PlanPool* pool = nullptr;
+  int rc = current_pool(&pool);
+  if (rc != FCP_OK) return rc;
   constexpr int NT = 13;
   const std::vector<int32_t>* tabs[NT] = {&plan->fwd_units, &plan->bwd_units, &plan->bwd_qranges, &plan->merge_units,
                                           &plan->slot_offset, &plan->slot_rows, &plan->bwd_work, &plan->fused_units,
@@ -433,22 +469,20 @@ extern "C" int fcp_plan_upload(fcp_plan* plan, void* stream) {
   PlanBlock* block = nullptr;
   cudaStream_t copy = nullptr;
   {
-    std::lock_guard<std::mutex> lock(ds.mu);
-    int rc = device_setup(dev, ds);
-    if (rc == FCP_OK) rc = acquire_block(ds, total, &block);
+    std::lock_guard<std::mutex> lock(pool->mu);
+    rc = pool_setup(*pool);
+    if (rc == FCP_OK) rc = acquire_block(*pool, total, &block);
     if (rc != FCP_OK) return rc;
-    plan->sm_count = ds.sm_count;
-    copy = ds.copy;
+    plan->sm_count = pool->sm_count;
+    copy = pool->copy;
   }
-  if (cudaError_t e = cudaEventSynchronize(block->used); e != cudaSuccess) {
-    free_block(block);
-    fcp_set_error("plan upload failed: %s", cudaGetErrorString(e));
-    return FCP_ERR_CUDA;
+  cudaError_t e = cudaEventSynchronize(block->used);
+  if (e == cudaSuccess) {
+    memset(block->host, 0, 256);
+    for (int i = 0; i < NT; ++i)
+      if (!tabs[i]->empty()) memcpy((char*)block->host + off[i], tabs[i]->data(), tabs[i]->size() * 4);
+    e = cudaMemcpyAsync(block->dev, block->host, total, cudaMemcpyHostToDevice, copy);
   }
-  memset(block->host, 0, 256);
-  for (int i = 0; i < NT; ++i)
-    if (!tabs[i]->empty()) memcpy((char*)block->host + off[i], tabs[i]->data(), tabs[i]->size() * 4);
-  cudaError_t e = cudaMemcpyAsync(block->dev, block->host, total, cudaMemcpyHostToDevice, copy);
   if (e == cudaSuccess) e = cudaEventRecord(block->used, copy);
   if (e == cudaSuccess) e = cudaEventSynchronize(block->used);
   if (e != cudaSuccess) {
@@ -459,7 +493,6 @@ extern "C" int fcp_plan_upload(fcp_plan* plan, void* stream) {
   void* blob = block->dev;
   plan->block = block;
   plan->block_pinned = false;
-  plan->device = dev;
   plan->d_blob = blob;
   plan->d_status = (int32_t*)blob;
   plan->d_fwd_units = (int32_t*)((char*)blob + off[0]);
@@ -523,7 +556,7 @@ extern "C" int fcp_plan_destroy(fcp_plan* plan) {
   if (plan->host_lane) cudaStreamDestroy((cudaStream_t)plan->host_lane);
   plan->host_in = plan->host_out = plan->host_lane = nullptr;
   fcp_plan_set_profiling(plan, 0);
-  if (plan->block) return_block(plan->device, plan->block, !plan->block_pinned);
+  if (plan->block) return_block(plan->block, !plan->block_pinned);
   delete plan;
   return FCP_OK;
 }

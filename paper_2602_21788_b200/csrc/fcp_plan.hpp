@@ -44,7 +44,6 @@ struct fcp_plan {
   std::vector<int32_t> span_offset, spans;                   // the caller's span list ([B+1], [n][2]); empty if none
 
   // device copy (fcp_plan_upload)
-  int device = -1;
   PlanBlock* block = nullptr;
   mutable bool block_pinned = false;   // the block's event does not cover all work that may read it (graph capture)
   void* d_blob = nullptr;      // the block's device memory: holds every table below

@@ -220,7 +220,7 @@ class Plan:
 
 
 def fcp_release_cached():
-    """Frees the device blocks that destroyed plans left for later ones (current device)."""
+    """Frees the device blocks that destroyed plans left for later ones (current CUDA context)."""
     _check(lib().fcp_release_cached())
 
 
