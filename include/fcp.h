@@ -159,11 +159,12 @@ int fcp_plan_workspace_bytes(const fcp_plan* plan, int32_t heads_per_pass, int64
 int fcp_plan_bwd_scratch_bytes(const fcp_plan* plan, int32_t kv_head_count, int64_t* bytes);
 
 /* Copies the plan's work tables to the current device (the only device allocation the library
- * makes).  Must precede the compute calls.  Complete when it returns, without waiting for work that
+ * makes; 1 MB of page-locked host memory per CUDA context takes part and stays).  Must precede the
+ * compute calls.  Complete when it returns, without waiting for work that
  * is queued on `stream`.  fcp_plan_destroy does not wait for the plan's queued work either: the
  * tables' memory stays with the library (at most 8 blocks and 32 MB per CUDA context) and serves a later
  * plan once that work is done; a plan whose calls were captured into a graph must outlive the
- * graph's launches.  fcp_release_cached frees the idle blocks of the current context.            */
+ * graph's launches.  fcp_release_cached frees what is idle in the current context.               */
 int fcp_plan_upload(fcp_plan* plan, void* stream);
 int fcp_release_cached(void);
 int fcp_plan_destroy(fcp_plan* plan);

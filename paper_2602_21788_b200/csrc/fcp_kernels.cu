@@ -3,6 +3,7 @@
 // fcp_bwd.cuh.  No call here allocates device memory except fcp_plan_upload.
 #include <algorithm>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -276,7 +277,6 @@ __global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* acc, _
 struct PlanPool;
 struct PlanBlock {
   void* dev = nullptr;           // tables
-  void* host = nullptr;          // pinned staging of the same size: one copy per upload
   size_t bytes = 0;
   cudaEvent_t used = nullptr;    // after the last compute call that read the block
   PlanPool* pool = nullptr;
@@ -284,18 +284,22 @@ struct PlanBlock {
 
 struct PlanPool {
   unsigned long long context = 0;
-  std::mutex mu;
+  std::mutex mu;                 // the members up to `staging`
   bool ready = false;            // device checked, attributes set, stream created
   int sm_count = 0;
   cudaStream_t copy = nullptr;   // uploads: complete without waiting for the work queued on the caller's stream
   std::vector<PlanBlock*> idle;  // oldest first
   size_t idle_bytes = 0;
+  std::mutex staging_mu;         // one upload at a time passes its tables through `staging`
+  char* staging = nullptr;
+  bool staging_pinned = false;
 };
 
 namespace {
 constexpr int kMaxDevices = 64;
 constexpr size_t kBlockMin = size_t(64) << 10, kBlockKeepMax = size_t(8) << 20, kKeepBytes = size_t(32) << 20;
 constexpr size_t kKeepBlocks = 8;
+constexpr size_t kStagingBytes = size_t(1) << 20;
 
 // The current context's pool.  Pools are never taken down: the id of a context is not used again.
 int current_pool(PlanPool** out) {
@@ -330,7 +334,6 @@ int current_pool(PlanPool** out) {
 
 void free_block(PlanBlock* b) {
   if (b->dev) cudaFree(b->dev);
-  if (b->host) cudaFreeHost(b->host);
   if (b->used) cudaEventDestroy(b->used);
   delete b;
 }
@@ -386,7 +389,6 @@ int acquire_block(PlanPool& pool, size_t bytes, PlanBlock** out) {
   while (b->bytes < bytes && b->bytes < kBlockKeepMax) b->bytes *= 2;
   b->bytes = std::max(b->bytes, bytes);
   cudaError_t e = cudaMalloc(&b->dev, b->bytes);
-  if (e == cudaSuccess) e = cudaMallocHost(&b->host, b->bytes);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->used, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     free_block(b);
@@ -419,6 +421,36 @@ void return_block(PlanBlock* b, bool keep) {
   for (PlanBlock* x : out) free_block(x);
 }
 
+// Host tables -> device, in pieces through the pool's page-locked buffer (a pageable one where that is not to be had): the
+// pool keeps 1 MB of it, whatever the plans' number and sizes.  Complete on return.
+struct Staging {
+  PlanPool& pool;
+  char* dst;                     // where the first byte of the buffer goes
+  cudaEvent_t done;
+  size_t fill = 0;
+  cudaError_t flush() {
+    if (fill == 0) return cudaSuccess;
+    cudaError_t e = cudaMemcpyAsync(dst, pool.staging, fill, cudaMemcpyHostToDevice, pool.copy);
+    if (e == cudaSuccess) e = cudaEventRecord(done, pool.copy);
+    if (e == cudaSuccess) e = cudaEventSynchronize(done);
+    dst += fill;
+    fill = 0;
+    return e;
+  }
+  cudaError_t put(const void* src, size_t bytes) {         // src NULL: zeros
+    for (size_t i = 0; i < bytes;) {
+      const size_t n = std::min(bytes - i, kStagingBytes - fill);
+      if (src) memcpy(pool.staging + fill, (const char*)src + i, n);
+      else memset(pool.staging + fill, 0, n);
+      i += n;
+      fill += n;
+      if (fill == kStagingBytes)
+        if (cudaError_t e = flush(); e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
+};
+
 // At the end of every compute call: the block is in use until the work queued so far on `st` is done (calls on one
 // plan are stream-ordered, so the last event covers the earlier calls).  Work recorded into a graph can run at any later
 // time: such a plan's block is never handed on.
@@ -444,6 +476,10 @@ extern "C" int fcp_release_cached(void) {
     pool->idle_bytes = 0;
   }
   for (PlanBlock* b : out) free_block(b);
+  std::lock_guard<std::mutex> lock(pool->staging_mu);
+  if (pool->staging_pinned) cudaFreeHost(pool->staging);
+  else free(pool->staging);
+  pool->staging = nullptr;
   return FCP_OK;
 }
 
@@ -467,24 +503,32 @@ extern "C" int fcp_plan_upload(fcp_plan* plan, void* stream) {
   }
   off[NT] = total;
   PlanBlock* block = nullptr;
-  cudaStream_t copy = nullptr;
   {
     std::lock_guard<std::mutex> lock(pool->mu);
     rc = pool_setup(*pool);
     if (rc == FCP_OK) rc = acquire_block(*pool, total, &block);
     if (rc != FCP_OK) return rc;
     plan->sm_count = pool->sm_count;
-    copy = pool->copy;
   }
   cudaError_t e = cudaEventSynchronize(block->used);
   if (e == cudaSuccess) {
-    memset(block->host, 0, 256);
-    for (int i = 0; i < NT; ++i)
-      if (!tabs[i]->empty()) memcpy((char*)block->host + off[i], tabs[i]->data(), tabs[i]->size() * 4);
-    e = cudaMemcpyAsync(block->dev, block->host, total, cudaMemcpyHostToDevice, copy);
+    std::lock_guard<std::mutex> lock(pool->staging_mu);
+    if (!pool->staging) {
+      pool->staging_pinned = cudaMallocHost((void**)&pool->staging, kStagingBytes) == cudaSuccess;
+      if (!pool->staging_pinned) {
+        cudaGetLastError();
+        pool->staging = (char*)malloc(kStagingBytes);
+      }
+    }
+    if (!pool->staging) e = cudaErrorMemoryAllocation;
+    Staging up{*pool, (char*)block->dev, block->used};
+    if (e == cudaSuccess) e = up.put(nullptr, 256);
+    for (int i = 0; i < NT && e == cudaSuccess; ++i) {
+      e = up.put(tabs[i]->data(), tabs[i]->size() * 4);
+      if (e == cudaSuccess) e = up.put(nullptr, off[i + 1] - off[i] - tabs[i]->size() * 4);
+    }
+    if (e == cudaSuccess) e = up.flush();
   }
-  if (e == cudaSuccess) e = cudaEventRecord(block->used, copy);
-  if (e == cudaSuccess) e = cudaEventSynchronize(block->used);
   if (e != cudaSuccess) {
     free_block(block);
     fcp_set_error("plan upload failed: %s", cudaGetErrorString(e));

@@ -161,3 +161,26 @@ def test_backward_of_more_query_heads_than_a_grid_dimension_holds(hq):
     some = np.r_[0:3, hq - 67:hq - 62, hq - 2:hq]  # query heads that share the one KV head are independent
     dq_ref, _, _ = A.attention_bwd_packed(f64(q[:, some]), f64(k), f64(v), f64(do[:, some]), w.cu_seqlens)
     assert _rel(res["dq"][:, some], dq_ref) <= 2e-2
+
+
+@pytest.mark.parametrize("n_seq", [3, 1500, 3200])    # one piece of the upload buffer, several, and a block that is not kept
+def test_upload_in_pieces(n_seq):
+    """A sequence's results do not depend on where its rows lie in the tables: span plans, whose tables grow with the tokens."""
+    from paper_2602_21788_b200 import fcp
+    kinds = [(500, [(10, 200), (210, 499)]), (129, []), (700, [(0, 700)])]
+    some = sorted({0, 1, 2, n_seq // 2, n_seq - 2, n_seq - 1})
+    lens = [kinds[i % 3][0] for i in range(n_seq)]
+    cu = np.r_[0, np.cumsum(lens)]
+    g = torch.Generator(device="cuda").manual_seed(29)
+    q, k, v = (torch.randn((int(cu[-1]), 1, 64), dtype=torch.bfloat16, device="cuda", generator=g) for _ in range(3))
+    st = torch.cuda.current_stream()
+    plan = fcp.Plan(lens, [1] * n_seq, 1, 1, 64, spans=[kinds[i % 3][1] for i in range(n_seq)]).upload()
+    small = fcp.Plan([5, 129], [1, 1], 1, 1, 64).upload()          # another one's tables go through the same buffer
+    o, lse = _fused(plan, q, k, v, 1, st)
+    _fused(small, q[:134], k[:134], v[:134], 1, st)
+    assert plan.device_status()[0] == 0
+    for i in some:
+        a, b = int(cu[i]), int(cu[i + 1])
+        alone = fcp.Plan([lens[i]], [1], 1, 1, 64, spans=[kinds[i % 3][1]]).upload()
+        o1, lse1 = _fused(alone, *(t[a:b].contiguous() for t in (q, k, v)), 1, st)
+        assert torch.equal(o[a:b], o1) and torch.equal(lse[a:b], lse1), i
