@@ -160,11 +160,14 @@ int fcp_plan_bwd_scratch_bytes(const fcp_plan* plan, int32_t kv_head_count, int6
 
 /* Copies the plan's work tables to the current device (the only device allocation the library
  * makes; 1 MB of page-locked host memory per CUDA context takes part and stays).  Must precede the
- * compute calls.  Complete when it returns, without waiting for work that
- * is queued on `stream`.  fcp_plan_destroy does not wait for the plan's queued work either: the
- * tables' memory stays with the library (at most 8 blocks and 32 MB per CUDA context) and serves a later
- * plan once that work is done; a plan whose calls were captured into a graph must outlive the
- * graph's launches.  fcp_release_cached frees what is idle in the current context.               */
+ * compute calls.  Complete when it returns.  fcp_plan_destroy leaves the tables' memory with the
+ * library (at most 8 blocks and 32 MB per CUDA context) for a later plan, which gets it once the
+ * destroyed plan's queued work is done; fcp_release_cached frees what is idle in the current context.
+ * Neither upload nor destroy waits for queued work, with these exceptions: an upload that finds 8 idle
+ * blocks, all still read by queued work, waits for the oldest that fits; a destroy frees memory, which
+ * waits for the device, when 8 blocks or 32 MB are kept already, when the tables are larger than 8 MB,
+ * and when calls of the plan were captured into a graph.  A captured plan must outlive the graph's
+ * launches.                                                                                      */
 int fcp_plan_upload(fcp_plan* plan, void* stream);
 int fcp_release_cached(void);
 int fcp_plan_destroy(fcp_plan* plan);

@@ -271,8 +271,10 @@ __global__ void __launch_bounds__(256) fcp_dq_convert_kernel(const float* acc, _
 // cudaFree (which waits for the whole device), the device query and the kernel attributes cost milliseconds each time:
 // with them a 16K-token batch takes 6.8 ms for 2.8 ms of kernels.  So a destroyed plan's block goes to a short list and
 // is handed to the next plan once the event recorded after the last compute call that read it has completed.  The list
-// holds at most 8 blocks and 32 MB (the oldest leave first), larger blocks are never kept, and fcp_release_cached gives
-// all idle ones back.
+// holds at most 8 blocks and 32 MB; larger blocks are never kept, and fcp_release_cached gives all idle ones back.
+// Three things still wait for queued work: an upload that finds the list full of blocks in use (for the oldest that
+// fits), and, because cudaFree waits for the device, the release of a block that the list has no room for (one whose
+// work is done goes first) and of the block of a plan that was captured into a graph.
 // Memory, streams and kernel attributes belong to a CUDA context, so each context has a list of its own.
 struct PlanPool;
 struct PlanBlock {
@@ -413,9 +415,12 @@ void return_block(PlanBlock* b, bool keep) {
     pool.idle.push_back(b);
     pool.idle_bytes += b->bytes;
     while (pool.idle.size() > kKeepBlocks || pool.idle_bytes > kKeepBytes) {
-      out.push_back(pool.idle.front());
-      pool.idle_bytes -= pool.idle.front()->bytes;
-      pool.idle.erase(pool.idle.begin());
+      size_t i = 0;              // the oldest whose work is done, else the oldest
+      while (i < pool.idle.size() && !is_free(pool.idle[i])) ++i;
+      if (i == pool.idle.size()) i = 0;
+      out.push_back(pool.idle[i]);
+      pool.idle_bytes -= pool.idle[i]->bytes;
+      pool.idle.erase(pool.idle.begin() + i);
     }
   }
   for (PlanBlock* x : out) free_block(x);

@@ -184,3 +184,32 @@ def test_upload_in_pieces(n_seq):
         alone = fcp.Plan([lens[i]], [1], 1, 1, 64, spans=[kinds[i % 3][1]]).upload()
         o1, lse1 = _fused(alone, *(t[a:b].contiguous() for t in (q, k, v)), 1, st)
         assert torch.equal(o[a:b], o1) and torch.equal(lse[a:b], lse1), i
+
+
+@pytest.mark.parametrize("n_seq", [2, 300])     # tables in blocks of 64 KB: eight are kept; of 8 MB (spans): four
+def test_more_plans_in_flight_than_blocks_are_kept(n_seq):
+    """Twelve plans with queued work are dropped at once, so the list overflows with blocks in use and the uploads that follow
+    find it full of them; results must come from the plan's own tables throughout."""
+    from paper_2602_21788_b200 import fcp
+    batches = [[2000 - 100 * i] + [2000] * (n_seq - 2) + [2000 + 100 * i] for i in range(12)]
+    g = torch.Generator(device="cuda").manual_seed(31)
+    q, k, v = (torch.randn((2000 * n_seq, 1, 64), dtype=torch.bfloat16, device="cuda", generator=g) for _ in range(3))
+    st = torch.cuda.current_stream()
+    make = lambda lens: fcp.Plan(lens, [1] * n_seq, 1, 1, 64, spans=[[(0, 500)]] * n_seq).upload()
+    fcp.fcp_release_cached()
+    want = []
+    for lens in batches:
+        want.append(_fused(make(lens), q, k, v, 1, st))
+        torch.cuda.synchronize()
+    busy = torch.zeros(1 << 28, device="cuda")
+    got = []
+    for _ in range(2):
+        for _ in range(40):
+            busy.add_(1.0)                              # the calls below stay queued for about 15 ms
+        plans = [make(lens) for lens in batches]
+        got += [_fused(plan, q, k, v, 1, st) for plan in plans]
+        del plans
+        got += [_fused(make(lens), q, k, v, 1, st) for lens in batches]
+    torch.cuda.synchronize()
+    for i, (o, lse) in enumerate(got):
+        assert torch.equal(o, want[i % 12][0]) and torch.equal(lse, want[i % 12][1]), i
