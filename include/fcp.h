@@ -147,7 +147,8 @@ int fcp_plan_get(const fcp_plan* plan, int32_t which, const int32_t** host_ptr, 
 
 /* Scalar facts about a plan: which in {0: T, 1: R (partial rows), 2: n_pairs, 3: n_items,
  * 4: n_fwd_units, 5: n_bwd_units, 6: n_merge_units, 7: B, 8: the leading merge units that belong
- * to Q chunks with two or more slots (all that fcp_attn_fwd_merged has to merge), 9: n_fused_units}. */
+ * to Q chunks with two or more slots (all that fcp_attn_fwd_merged has to merge), 9: n_fused_units,
+ * 10: 1 if fcp_attn_fwd_fused over all heads hands out the two Q tiles of a unit one by one (B200)}. */
 int fcp_plan_info(const fcp_plan* plan, int32_t which, int64_t* value);
 
 /* Bytes the caller must provide: o_partial = R*heads_per_pass*D*4, lse_partial = R*heads_per_pass*4,

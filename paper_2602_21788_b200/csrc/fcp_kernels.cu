@@ -695,9 +695,11 @@ int launch_fwd(const fcp_plan* plan, const void* q, const void* k, const void* v
   a.o_f32_direct = o_f32_direct;
   a.row_limit = fused ? plan->d_row_limit : nullptr;
   a.status = plan->d_status;
-  // With fewer items than SMs every item runs at once and the longest one is the launch: then its two Q tiles go to two
-  // SMs (a tile alone does not wait for the other one's turn in the MUFU and the tensor core): 4K-token forward 23.2 -> 21.2 us.
-  a.split = (int64_t)a.n_units * head_count < plan->sm_count ? 1 : 0;
+  if (head_count == P.hq && plan->sm_count == FCP_PLAN_SMS)
+    a.split = fused ? plan->fused_split : plan->fwd_split;
+  else
+    a.split = split_units(fused ? plan->fused_units : plan->fwd_units, fused ? plan->fused_groups : plan->fwd_groups,
+                          head_count / a.head_group, a.head_group, plan->sm_count);
   const int64_t n_work = (int64_t)a.n_units * head_count << a.split;
   if (n_work >= int64_t(1) << 31) {
     fcp_set_error("forward attention: %lld work items exceed the 2^31 limit", (long long)n_work);

@@ -5,6 +5,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <limits>
 #include <numeric>
 #include <vector>
@@ -201,7 +202,7 @@ inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 // the longest unit is over a quarter of an SM's share: these units touch the ends of all sequences and share little (64K
 // batch, 15 %: backward +2 % when they wait).  Measured: 8K step 501 -> 485 us, 16K new batch 2.50 -> 2.37 ms.
 constexpr int64_t kOrderBytes = int64_t(64) << 20;
-constexpr int64_t kOrderSms = 148;
+constexpr int64_t kOrderSms = FCP_PLAN_SMS;
 
 void order_units(const std::vector<int32_t>& seq, const std::vector<int32_t>& cost, const int32_t* seqlens, int B,
                  int32_t heads, int64_t bytes_per_token, std::vector<int32_t>& order, std::vector<int32_t>& groups) {
@@ -251,6 +252,50 @@ void order_units(const std::vector<int32_t>& seq, const std::vector<int32_t>& co
 }
 
 }  // namespace
+
+// With fewer items than SMs every unit runs at once and the longest one is the launch.  Its two Q tiles as items of their
+// own take a quarter less time, because a tile alone does not wait for the other one's turn in the MUFU and the tensor core;
+// but with more than half as many units as SMs some SMs get a second item, which starts late, and the empty half of a unit
+// with one tile holds up what comes behind it too.  Measured, whole against split (kernel, us; n units of sequences of L tokens):
+//   D = 64:  L = 256, n = 74: 14.4, 13.8; n = 80: 14.4, 16.5; n = 144: 15.3, 19.2     L = 512, n = 80: equal; n = 144: 17.1, 21.0
+//            L = 1024, n = 112: 23.1, 22.3; n = 144: 23.8, 25.1                       L = 2048, n = 144: 36.5, 33.3
+//   D = 128: L = 256, n = 80: 14.9, 17.7; L = 1024, n = 112: 25.4, 23.8; n = 144: 25.4, 27.3; L = 2048, n = 144: 37.4, 36.2
+// So both launches are played through, in quarters of the time of one key tile of a Q tile alone: a tile 4, a second item 12
+// more (8 behind an empty half), a whole unit of two tiles 5 per key tile of the longer one and 6.  Over 224 measured lists of
+// equal and unequal units this takes the slower launch, by over 3 %, once; always splitting does 62 times, by up to 30 %.
+bool split_units(const std::vector<int32_t>& units, const std::vector<int32_t>& groups, int heads, int per, int sms) {
+  const int64_t n_units = (int64_t)(units.size() / FCP_FWD_UNIT_W);
+  if (n_units * heads * per >= sms) return false;
+  std::vector<int64_t> busy;                     // when each SM is done (a heap, the earliest on top, once all have an item)
+  int64_t split = 0, whole = 0;
+  bool two = false;
+  auto hand_out = [&](int64_t tiles) {
+    const int64_t t = tiles > 0 ? 4 * tiles : 8;
+    if ((int)busy.size() < sms) {
+      busy.push_back(2 * t + (tiles > 0));       // lowest bit: the SM's last item was not an empty half
+      std::push_heap(busy.begin(), busy.end(), std::greater<int64_t>());
+    } else {
+      std::pop_heap(busy.begin(), busy.end(), std::greater<int64_t>());
+      busy.back() = 2 * (busy.back() / 2 + (busy.back() & 1 ? 12 : 0) + t) + (tiles > 0);
+      std::push_heap(busy.begin(), busy.end(), std::greater<int64_t>());
+    }
+  };
+  for (size_t g = 0; g < groups.size(); g += FCP_WORK_GROUP_W)
+    for (int h0 = 0; h0 < heads; h0 += groups[g + WG_HEADS])                       // the order of WorkOrder::locate
+      for (int32_t u = 0; u < groups[g + WG_N_UNITS]; ++u) {
+        const int32_t* U = &units[(size_t)(groups[g + WG_FIRST] + u) * FCP_FWD_UNIT_W];
+        const int32_t a = U[FU_NT_STAGE0], b = U[FU_NT_STAGE1], most = std::max(a, b);
+        two = two || (a > 0 && b > 0);
+        whole = std::max<int64_t>(whole, a > 0 && b > 0 ? 5 * most + 6 : 4 * most);
+        for (int i = std::min(groups[g + WG_HEADS], heads - h0) * per; i > 0; --i) {
+          hand_out(a);
+          hand_out(b);
+        }
+      }
+  for (int64_t t : busy)
+    if (t & 1) split = std::max(split, t / 2);
+  return two && split <= whole;
+}
 
 extern "C" int fcp_plan_blocks(const int32_t* seqlens, const int32_t* cp_degrees, int32_t B,
                                const fcp_params* params, fcp_plan** out) {
@@ -503,6 +548,7 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
     }
   }
   emit_fwd(fus, fu_seq, p->fwd_units, p->fwd_groups);
+  p->fwd_split = split_units(p->fwd_units, p->fwd_groups, params->hkv, params->hq / params->hkv, FCP_PLAN_SMS);
 
   // Fused forward (merge on the fly): all items of a Q chunk run on one CTA, so the KV ranges of the
   // chunk's block pairs are swept in one online softmax and no partial leaves the SM.  The ranges of
@@ -607,6 +653,7 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
       if (run0 >= 0) emit_run(b, t0, t1, run0, run1);
     }
     emit_fwd(gus, gu_seq, p->fused_units, p->fused_groups);
+    p->fused_split = split_units(p->fused_units, p->fused_groups, params->hkv, params->hq / params->hkv, FCP_PLAN_SMS);
   }
 
   // Backward: one unit per 128-key tile; it visits the Q rows of all block pairs whose kv_chunk holds
@@ -783,6 +830,7 @@ extern "C" int fcp_plan_info(const fcp_plan* plan, int32_t which, int64_t* value
     case 7: *value = plan->B; break;
     case 8: *value = plan->n_merge_multi; break;
     case 9: *value = (int64_t)plan->fused_units.size() / FCP_FWD_UNIT_W; break;
+    case 10: *value = plan->fused_split; break;
     default: return FCP_ERR_INVALID_ARG;
   }
   return FCP_OK;

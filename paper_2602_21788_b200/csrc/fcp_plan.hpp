@@ -30,6 +30,11 @@ enum { WG_FIRST = 0, WG_N_UNITS, WG_HEADS, WG_RSV };
 
 struct PlanBlock;                      // device block of an uploaded plan (fcp_kernels.cu)
 
+// Whether the two Q tiles of a forward unit become work items of their own, in a launch over `heads` groups of `per` adjacent
+// query heads (fcp_plan.cpp).
+bool split_units(const std::vector<int32_t>& units, const std::vector<int32_t>& groups, int heads, int per, int sms);
+constexpr int FCP_PLAN_SMS = 148;      // what the planner takes the device to have
+
 struct fcp_plan {
   fcp_params params{};
   int32_t B = 0;
@@ -40,6 +45,7 @@ struct fcp_plan {
   std::vector<int32_t> cu_seqlens, chunk_offset, chunk_bounds, pairs, items, slot_offset, slot_rows;
   std::vector<int32_t> fwd_units, bwd_units, bwd_qranges, merge_units, bwd_work, fused_units;
   std::vector<int32_t> fwd_groups, bwd_groups, fused_groups;   // work groups of the three unit lists
+  bool fwd_split = false, fused_split = false;                 // split_units over all heads
   std::vector<int32_t> row_limit, first_query, span_pairs;   // empty unless the plan has bidirectional spans
   std::vector<int32_t> span_offset, spans;                   // the caller's span list ([B+1], [n][2]); empty if none
 

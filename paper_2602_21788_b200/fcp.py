@@ -24,7 +24,7 @@ TABLES = dict(cu_seqlens=0, chunk_offset=1, chunk_bounds=2, pairs=3, items=4, sl
 _TABLE_WIDTH = dict(pairs=6, items=8, fwd_units=16, bwd_units=8, bwd_qranges=4, merge_units=4, fused_units=16,
                     span_pairs=5, fwd_groups=4, fused_groups=4, bwd_groups=4)
 INFO = dict(T=0, R=1, n_pairs=2, n_items=3, n_fwd_units=4, n_bwd_units=5, n_merge_units=6, B=7, n_merge_multi=8,
-            n_fused_units=9)
+            n_fused_units=9, fused_split=10)
 
 EXPORTS = ["fcp_plan_strategy", "fcp_plan_blocks", "fcp_plan_blocks_spans", "fcp_span_mask_efficiency", "fcp_plan_get", "fcp_plan_info", "fcp_plan_workspace_bytes",
            "fcp_plan_bwd_scratch_bytes", "fcp_plan_upload", "fcp_release_cached", "fcp_plan_destroy", "fcp_attn_fwd", "fcp_attn_fwd_merged",

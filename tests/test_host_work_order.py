@@ -76,3 +76,16 @@ def test_noalloc_arena_holds_tables_and_scratch_and_nothing_for_the_order(lens, 
     plan = fcp.Plan(lens, [1] * len(lens), hq, hkv, D)
     assert fcp.fcp_noalloc_bytes_needed(plan) == need <= fcp.FCP_NOALLOC_MAX_BYTES
     assert len(plan.table("bwd_groups")) <= 2
+
+
+@pytest.mark.parametrize("lens,hq,split", [
+    ([256] * 74, 1, 1), ([256] * 80, 1, 0), ([256] * 36, 4, 0),      # second items on some SMs cost more than the tiles apart save
+    ([512] * 40, 1, 1), ([512] * 72, 1, 0),
+    ([1024] * 28, 1, 1), ([1024] * 36, 1, 0), ([1024] * 9, 4, 0),
+    ([2048] * 18, 1, 1), ([2048] * 6, 3, 1),
+    ([128] * 20, 2, 0), ([100, 128, 7], 3, 0),                       # one Q tile per unit
+    ([700, 520, 300, 1000, 450, 640, 130, 613], 4, 1),               # 88 items or so of a small model's batch
+    ([2560] * 15, 1, 0), ([256] * 37, 4, 0),                         # as many items as SMs, or more
+])
+def test_q_tiles_are_items_of_their_own_where_that_is_the_shorter_launch(lens, hq, split):
+    assert fcp.Plan(lens, [1] * len(lens), hq, 1, 64).info("fused_split") == split
