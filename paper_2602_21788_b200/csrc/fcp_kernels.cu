@@ -71,7 +71,7 @@ int make_thd_map(CUtensorMap* m, const void* base, int64_t T, int H, int D, int 
 // Launch that may begin while the kernel before it in the stream still runs (grid_begin of sm100_ptx.cuh); hides the
 // launch latency and the set-up of barriers and tensor memory: 4K-token step, seven queue entries before and four launches now, 59 -> 50 us.
 template <typename... P, typename... A>
-cudaError_t launch(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+cudaError_t launch_when(bool early, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
@@ -81,8 +81,12 @@ cudaError_t launch(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cu
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  return launch_when(true, kernel, grid, threads, smem, st, args...);
 }
 
 // Records an event pair around a kernel launch when the plan is in profiling mode.
@@ -724,11 +728,15 @@ int launch_merge(const fcp_plan* plan, const float* o_partial, const float* lse_
   if (n_units == 0) return FCP_OK;
   cudaStream_t st = (cudaStream_t)stream;
   ProfScope prof(plan, 1, st);
+  // Launched early, the CTAs go to the first SMs that the forward grid leaves, eight to each, and a grid of few CTAs stays on
+  // them (forward + merge, us, early against not; n CTAs): n = 60, 64 heads, D = 64: 327, 287; n = 112, 32 heads, D = 128: 163,
+  // 144; n = 448: 389, 375; n = 665: 639, 630; n = 3584: 10570, 10440; where the merge is short the launch costs 1-2 us more.
+  const bool early = n_units >= 4 * plan->sm_count;
   if (P.head_dim == 128)
-    FCP_CUDA_CHECK(launch(fcp_merge_kernel<128>, n_units, 256, 0, st, plan->d_merge_units, plan->d_slot_offset, plan->d_slot_rows,
+    FCP_CUDA_CHECK(launch_when(early, fcp_merge_kernel<128>, n_units, 256, 0, st, plan->d_merge_units, plan->d_slot_offset, plan->d_slot_rows,
                           o_partial, lse_partial, head_begin, head_count, P.hq, (__nv_bfloat16*)o, o_f32, lse));
   else
-    FCP_CUDA_CHECK(launch(fcp_merge_kernel<64>, n_units, 256, 0, st, plan->d_merge_units, plan->d_slot_offset, plan->d_slot_rows,
+    FCP_CUDA_CHECK(launch_when(early, fcp_merge_kernel<64>, n_units, 256, 0, st, plan->d_merge_units, plan->d_slot_offset, plan->d_slot_rows,
                           o_partial, lse_partial, head_begin, head_count, P.hq, (__nv_bfloat16*)o, o_f32, lse));
   FCP_CUDA_CHECK(cudaGetLastError());
   return FCP_OK;
