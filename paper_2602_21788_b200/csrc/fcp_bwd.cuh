@@ -164,6 +164,13 @@ __device__ __forceinline__ float2 mul_pair(float2 a, uint32_t bf16x2) {
   return mul2(a, make_float2(__uint_as_float(bf16x2 << 16), __uint_as_float(bf16x2 & 0xffff0000u)));
 }
 
+// Bits [first, first + n), cut off at bit 31.
+__device__ __forceinline__ uint32_t bit_range(int first, int n) {
+  uint32_t m;
+  asm("bmsk.clamp.b32 %0, %1, %2;" : "=r"(m) : "r"(first), "r"(n));
+  return m;
+}
+
 template <int D>
 __global__ void __launch_bounds__(BWD_THREADS, 1)
 fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -485,6 +492,10 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const float* s_lse = s_rows + half * 64;
         const float* s_delta = s_rows + 128 + half * 64;
         const bool need_mask = causal || q_valid < 128 || kv_rows < 128;   // uniform across the CTA
+        // A warp without any (key row, query) pair of the tile writes zeros, and the mask comes from one bit per column instead of
+        // four comparisons per pair of columns: 1841 sequences of 12 tokens, D = 64: 237 -> 208 us; 16K ragged batch, D = 64:
+        // 179.9 -> 173.5; 8K batch 257 -> 250.
+        const bool live = rb * 32 < kv_rows && half * 64 < q_valid;
 
         ok = mbar_wait_warp(BAR(B_SFULL), it & 1, wctx, 130);
         if (!ok) break;
@@ -495,6 +506,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         // between the trips the pair arrays rotate (register arrays cannot be indexed by the trip), which halves the
         // code of this loop.
         uint32_t pa[16], pb[16] = {};
+        if (live) {
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           uint32_t sv[32];
@@ -517,16 +529,25 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             // columns of this trip a key row keeps: [lo, hi)
 #pragma unroll
             for (int g2 = 0; g2 < 4; ++g2) {
-              const int off = half * 64 + c * 32 + fcol;
-              const int hi = (frow + 8 * g2 < kv_rows ? q_valid : 0) - off, lo = (causal ? first_q[g2] - q_row : 0) - off;
+              const int off = half * 64 + c * 32;
+              const int hi = min(32, (frow + 8 * g2 < kv_rows ? q_valid : 0) - off), lo = max(0, (causal ? first_q[g2] - q_row : 0) - off);
+              // one bit per column, then a byte of ones for the even and the odd column of each pair
+              const uint32_t keep = bit_range(lo, max(0, hi - lo)) >> fcol;
+              const uint32_t even = (keep & 0x01010101u) * 0xffu, odd = ((keep >> 1) & 0x01010101u) * 0xffu;
 #pragma unroll
-              for (int j = 0; j < 4; ++j)
-                pb[(g2 >> 1) * 8 + 2 * j + (g2 & 1)] &= (8 * j >= lo && 8 * j < hi ? 0x0000ffffu : 0u) |
-                                                        (8 * j + 1 >= lo && 8 * j + 1 < hi ? 0xffff0000u : 0u);
+              for (int j = 0; j < 4; ++j) pb[(g2 >> 1) * 8 + 2 * j + (g2 & 1)] &= __byte_perm(even, odd, 0x4400 + 0x1111 * j);
             }
           }
           tmem_st_frag(t_s + c * 16, pb);            // over this warp's own, already loaded, columns
           tmem_st_frag(t_s + (16u << 16) + c * 16, pb + 8);
+        }
+        } else {
+          const uint32_t zero[8] = {};
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            tmem_st_frag(t_s + c * 16, zero);
+            tmem_st_frag(t_s + (16u << 16) + c * 16, zero);
+          }
         }
         tc_wait_st();
         tc_fence_before();
@@ -537,6 +558,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         if (!ok) break;
         tc_fence_after();
         if (mtid >= 128) *my_next = next_row;
+        if (live) {
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           uint32_t dv_[32], out[16];
@@ -563,6 +585,12 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             const int cc = c * 4 + 2 * (m & 1) + mch;
             stmatrix_x4(ds_row + (m >> 1) * 2048 + ((cc ^ (lane & 7)) << 4), &out[(m >> 1) * 8 + 4 * (m & 1)]);
           }
+        }
+        } else {
+          const uint32_t zero[4] = {};
+#pragma unroll
+          for (int m = 0; m < 8; ++m)
+            stmatrix_x4(ds_row + ((m >> 1) & 1) * 2048 + ((((m >> 2) * 4 + 2 * (m & 1) + mch) ^ (lane & 7)) << 4), zero);
         }
         fence_proxy_async_smem();
         tc_fence_before();

@@ -213,3 +213,26 @@ def test_more_plans_in_flight_than_blocks_are_kept(n_seq):
     torch.cuda.synchronize()
     for i, (o, lse) in enumerate(got):
         assert torch.equal(o, want[i % 12][0]) and torch.equal(lse, want[i % 12][1]), i
+
+
+SHORT = [1, 2, 31, 32, 33, 63, 64, 65, 95, 96, 97, 127, 128, 129]
+
+
+@pytest.mark.parametrize("D,hq,hkv", [(64, 4, 2), (128, 2, 2)])
+@pytest.mark.parametrize("spans", [False, True])
+def test_short_sequences(D, hq, hkv, spans):
+    """Lengths around 32, 64, 96 and 128, where column blocks, key rows and whole warps of a tile have nothing to do."""
+    from oracle import span_attention_ref as S
+    if not spans:
+        return _check(_wl(SHORT + SHORT[::-1], [1] * (2 * len(SHORT)), hq, hkv, D, seed=37))
+    from paper_2602_21788_b200.runner import run_fwd_bwd
+    w = _wl(SHORT, [1] * len(SHORT), hq, hkv, D, seed=41)
+    w.spans = [[] if n < 31 else [(0, 30)] if n < 64 else [(3, 33), (40, n)] for n in SHORT]
+    q, k, v, do = w.tensors()
+    res = run_fwd_bwd(w, q, k, v, do, fused=True)
+    o_ref, lse_ref = S.span_attention_fwd_packed(f64(q), f64(k), f64(v), w.cu_seqlens, w.spans)
+    e = np.abs(res["o_f32"] - o_ref)
+    assert e.max() <= 1e-2 and e.mean() <= 1e-3 and np.abs(res["lse"] - lse_ref).max() <= 1e-3
+    refs = S.span_attention_bwd_packed(f64(q), f64(k), f64(v), f64(do), w.cu_seqlens, w.spans)
+    for name, ref in zip(("dq", "dk", "dv"), refs):
+        assert _rel(res[name], ref) <= 2e-2, name
