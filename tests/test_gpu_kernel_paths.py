@@ -236,3 +236,16 @@ def test_short_sequences(D, hq, hkv, spans):
     refs = S.span_attention_bwd_packed(f64(q), f64(k), f64(v), f64(do), w.cu_seqlens, w.spans)
     for name, ref in zip(("dq", "dk", "dv"), refs):
         assert _rel(res[name], ref) <= 2e-2, name
+
+
+@pytest.mark.parametrize("D,deg", [(64, 1), (64, 5), (128, 3)])
+def test_partial_path_of_short_sequences(D, deg):
+    """Items of at most 64 keys, diagonal and full ones, and longer ones."""
+    from paper_2602_21788_b200.runner import run_fwd_bwd
+    lens = SHORT + [200, 331, 640]
+    w = _wl(lens, [deg] * len(lens), 4, 2, D, seed=43)
+    q, k, v, _ = w.tensors()
+    res = run_fwd_bwd(w, q, k, v)
+    o_ref, lse_ref = A.attention_fwd_packed(f64(q), f64(k), f64(v), w.cu_seqlens)
+    e = np.abs(res["o_f32"] - o_ref)
+    assert e.max() <= 1e-2 and e.mean() <= 1e-3 and np.abs(res["lse"] - lse_ref).max() <= 1e-3
