@@ -174,17 +174,18 @@ struct WorkOrder {
   uint32_t first = 0;     // its first work item
   // `heads` KV heads of `per` adjacent items each; returns the unit's place in the list and head * per + item
   __device__ __forceinline__ void locate(const int32_t* groups, uint32_t w, uint32_t heads, uint32_t per, int& unit, int& h) {
-    int4 G = __ldg(reinterpret_cast<const int4*>(groups) + g);        // one load of WG_FIRST, WG_N_UNITS, WG_HEADS
-    while (w - first >= (uint32_t)G.y * heads * per) {
-      first += (uint32_t)G.y * heads * per;
-      G = __ldg(reinterpret_cast<const int4*>(groups) + ++g);
+    const int4* G = reinterpret_cast<const int4*>(groups);
+    int4 row = __ldg(G + g);                 // one load of WG_FIRST, WG_N_UNITS, WG_HEADS
+    while (w - first >= (uint32_t)row.y * heads * per) {
+      first += (uint32_t)row.y * heads * per;
+      row = __ldg(G + ++g);
     }
-    const uint32_t gh = min((uint32_t)G.z, heads);
-    const uint32_t r = w - first, block = (uint32_t)G.y * gh * per;
+    const uint32_t gh = min((uint32_t)row.z, heads);
+    const uint32_t r = w - first, block = (uint32_t)row.y * gh * per;
     const uint32_t hb = r / block, rest = r - hb * block;
     const uint32_t inner = min(gh, heads - hb * gh) * per;
     const uint32_t u = rest / inner;
-    unit = G.x + (int)u;
+    unit = row.x + (int)u;
     h = (int)(hb * gh * per + rest - u * inner);
   }
 };
