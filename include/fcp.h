@@ -260,7 +260,7 @@ int fcp_attn_bwd_heads(const fcp_plan* plan, const void* q, const void* k, const
  * should be pinned for the copies to be asynchronous.
  * The batch is cut into up to 16 slices: passes over whole KV heads (strided copies) and, where there
  * are few KV heads, runs of consecutive sequences (packed tensors are token-major, so a run is one
- * contiguous slice of every tensor).  The inputs of later slices come in and the results of earlier
+ * contiguous slice of every tensor); where a buffer is pageable, into up to 8 runs only.  The inputs of later slices come in and the results of earlier
  * ones go out while kernels execute (two internal copy streams and a second kernel stream, ordered
  * after the work already queued on `stream`).  The first call on a plan is the one exception to
  * "compute calls do not allocate": it builds and uploads the plans of the runs and creates the

@@ -600,10 +600,10 @@ extern "C" int fcp_plan_kernel_ms(const fcp_plan* plan, int32_t kind, int32_t* l
 
 extern "C" int fcp_plan_destroy(fcp_plan* plan) {
   if (!plan) return FCP_OK;
-  for (fcp_plan* g : plan->groups) fcp_plan_destroy(g);
-  plan->groups.clear();
-  for (void* e : plan->host_events) if (e) cudaEventDestroy((cudaEvent_t)e);
-  plan->host_events.clear();
+  for (HostCut& cut : plan->host_cuts) {
+    for (fcp_plan* g : cut.groups) fcp_plan_destroy(g);
+    for (void* e : cut.events) if (e) cudaEventDestroy((cudaEvent_t)e);
+  }
   if (plan->host_in) cudaStreamDestroy((cudaStream_t)plan->host_in);
   if (plan->host_out) cudaStreamDestroy((cudaStream_t)plan->host_out);
   if (plan->host_lane) cudaStreamDestroy((cudaStream_t)plan->host_lane);
@@ -621,10 +621,11 @@ extern "C" int fcp_last_device_status(const fcp_plan* plan, int32_t* status) {
   FCP_CUDA_CHECK(cudaDeviceSynchronize());
   FCP_CUDA_CHECK(cudaMemcpy(status, plan->d_status, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost));
   // kernels launched by the host entry point report into the status words of its sequence groups
-  for (const fcp_plan* g : plan->groups) {
-    if (status[0] != 0) break;
-    FCP_CUDA_CHECK(cudaMemcpy(status, g->d_status, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost));
-  }
+  for (const HostCut& cut : plan->host_cuts)
+    for (const fcp_plan* g : cut.groups) {
+      if (status[0] != 0) break;
+      FCP_CUDA_CHECK(cudaMemcpy(status, g->d_status, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    }
   return FCP_OK;
 }
 
@@ -990,10 +991,25 @@ constexpr int64_t kHostSlices = 16, kHostPasses = 8, kHostFlopsPerByte = 20000;
 // 625 and 609; 64K tokens, 2 units: both 32.9).
 constexpr int64_t kHostLaneUnits = 4;
 
+// Strided copies of pageable memory run at a fraction of the speed of contiguous ones, and copies wait for one another
+// whatever the slices are: such buffers are cut into up to eight runs of at least 8192 tokens and not by heads (8K tokens of
+// 32/8 heads: 37 ms by heads, 25 like this; 32K: 155, 104; 64K: 301, 204; 64K of 32/32 heads: 494, 345).
+constexpr int64_t kHostRuns = 8, kHostRunTokens = 8192;
+
+bool is_pageable(const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return a.type == cudaMemoryTypeUnregistered;
+}
+
 // Builds the runs' plans and creates the streams and events the host entry point orders its work with; all of it belongs
 // to the plan and is released by fcp_plan_destroy.
-int build_host_groups(const fcp_plan* plan, void* stream) {
-  if (!plan->host_events.empty()) return FCP_OK;
+int build_host_cut(const fcp_plan* plan, bool pageable, void* stream) {
+  HostCut& cut = plan->host_cuts[pageable];
+  if (!cut.tok0.empty()) return FCP_OK;
   const int B = plan->B;
   const int64_t T = plan->T;
   const fcp_params& P = plan->params;
@@ -1008,8 +1024,12 @@ int build_host_groups(const fcp_plan* plan, void* stream) {
   }
   const bool by_heads = flops > (double)kHostFlopsPerByte * in_bytes;
   const int64_t most = std::min<int64_t>(by_heads ? kHostSlices : kHostPasses, slices);
-  const int32_t passes = (int32_t)std::min<int64_t>(P.hkv, most);
-  const int want = by_heads ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(slices / passes, B), T / 8192));
+  int32_t passes = (int32_t)std::min<int64_t>(P.hkv, most);
+  int want = by_heads ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(slices / passes, B), T / kHostRunTokens));
+  if (pageable) {
+    passes = 1;
+    want = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(kHostRuns, B), T / kHostRunTokens));
+  }
   std::vector<fcp_plan*> groups;
   std::vector<int64_t> tok0;
   auto fail = [&](int rc) {
@@ -1047,12 +1067,15 @@ int build_host_groups(const fcp_plan* plan, void* stream) {
   }
   tok0.push_back(T);
   const size_t total_passes = (tok0.size() - 1) * passes;
-  // streams and events: [0] start, [1] last copy out, [2] second lane done, then per (run, pass): q, k, v up; dO up; forward done; backward done
-  cudaStream_t in = nullptr, out = nullptr, lane = nullptr;
+  // events: [0] start, [1] last copy out, [2] second lane done, then per (run, pass): q, k, v up; dO up; forward done; backward done
   std::vector<void*> ev(3 + 4 * total_passes, nullptr);
-  cudaError_t e = cudaStreamCreateWithFlags(&in, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&out, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&lane, cudaStreamNonBlocking);
+  cudaError_t e = cudaSuccess;
+  for (void** st : {&plan->host_in, &plan->host_out, &plan->host_lane})
+    if (!*st && e == cudaSuccess) {
+      cudaStream_t x = nullptr;
+      e = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
+      *st = x;
+    }
   for (size_t i = 0; i < ev.size() && e == cudaSuccess; ++i) {
     cudaEvent_t x = nullptr;
     e = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
@@ -1060,19 +1083,13 @@ int build_host_groups(const fcp_plan* plan, void* stream) {
   }
   if (e != cudaSuccess) {
     for (void* x : ev) if (x) cudaEventDestroy((cudaEvent_t)x);
-    if (in) cudaStreamDestroy(in);
-    if (out) cudaStreamDestroy(out);
-    if (lane) cudaStreamDestroy(lane);
     fcp_set_error("fcp_attn_fwd_bwd_host: creating copy streams failed: %s", cudaGetErrorString(e));
     return fail(FCP_ERR_CUDA);
   }
-  plan->host_in = in;
-  plan->host_out = out;
-  plan->host_lane = lane;
-  plan->host_events = std::move(ev);
-  plan->groups = std::move(groups);
-  plan->group_tok0 = std::move(tok0);
-  plan->host_passes = passes;
+  cut.events = std::move(ev);
+  cut.groups = std::move(groups);
+  cut.tok0 = std::move(tok0);
+  cut.passes = passes;
   return FCP_OK;
 }
 
@@ -1108,28 +1125,33 @@ extern "C" int fcp_attn_fwd_bwd_host(const fcp_plan* plan, const void* q_host, c
     return FCP_ERR_WORKSPACE;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  if ((rc = build_host_groups(plan, stream)) != FCP_OK) return rc;
+  bool pageable = false;
+  for (const void* p : {q_host, k_host, v_host, d_o_host, (const void*)o_host, (const void*)lse_host, (const void*)dq_host,
+                        (const void*)dk_host, (const void*)dv_host})
+    pageable = pageable || is_pageable(p);
+  if ((rc = build_host_cut(plan, pageable, stream)) != FCP_OK) return rc;
+  const HostCut& cut = plan->host_cuts[pageable];
   const fcp_params& P = plan->params;
   const int64_t D = P.head_dim;
   const int64_t rq = (int64_t)P.hq * D * 2, rkv = (int64_t)P.hkv * D * 2, rl = (int64_t)P.hq * 4;   // bytes per token
   char* w = (char*)workspace;
-  const int G = (int)plan->group_tok0.size() - 1;
+  const int G = (int)cut.tok0.size() - 1;
   // Inputs of later slices come in (s_in) and results of earlier ones go out (s_out) while kernels run.  The kernels of
   // consecutive slices alternate between `stream` and a second lane where a slice has few work units.  Everything is
   // ordered after the work already queued on `stream` and is complete when this call returns.
   cudaStream_t s_in = (cudaStream_t)plan->host_in, s_out = (cudaStream_t)plan->host_out, s_lane = (cudaStream_t)plan->host_lane;
-  auto EV = [&](int i) { return (cudaEvent_t)plan->host_events[i]; };
+  auto EV = [&](int i) { return (cudaEvent_t)cut.events[i]; };
   // The forward pass of a slice needs q, k, v only: dO follows them and arrives while the forward kernel runs; o leaves
   // while the backward kernels run (they only read it), the log-sum-exps of a run when its last forward pass is done
   // (the few bytes per row of one pass would make a slow strided copy).
   struct Slice { int g, hk0, hkc, ev0; bool last; };
   std::vector<Slice> slices;
-  const int per = (P.hkv + plan->host_passes - 1) / plan->host_passes;
+  const int per = (P.hkv + cut.passes - 1) / cut.passes;
   int64_t lane_scratch = 0, lane_units = 0;      // scratch and backward units of the largest slice
   {
     int ev0 = 3;
     for (int g = 0; g < G; ++g) {
-      const fcp_plan* sub = plan->groups.empty() ? plan : plan->groups[g];
+      const fcp_plan* sub = cut.groups.empty() ? plan : cut.groups[g];
       lane_scratch = std::max(lane_scratch, al(bwd_scratch_need(sub, per)));
       lane_units = std::max(lane_units, (int64_t)(sub->bwd_units.size() / FCP_BWD_UNIT_W) * per);
       for (int hk0 = 0; hk0 < P.hkv; hk0 += per, ev0 += 4)
@@ -1151,7 +1173,7 @@ extern "C" int fcp_attn_fwd_bwd_host(const fcp_plan* plan, const void* q_host, c
   };
   const int64_t hb = D * 2;   // bytes of one head of one token (bf16)
   for (const Slice& sl : slices) {
-    const int64_t t0 = plan->group_tok0[sl.g], nt = plan->group_tok0[sl.g + 1] - t0;
+    const int64_t t0 = cut.tok0[sl.g], nt = cut.tok0[sl.g + 1] - t0;
     const int h0 = sl.hk0 * gq, hc = sl.hkc * gq;
     FCP_CUDA_CHECK(copy_heads(w + L.q, (const char*)q_host, t0, nt, rq, hb, h0, hc, cudaMemcpyHostToDevice, s_in));
     FCP_CUDA_CHECK(copy_heads(w + L.k, (const char*)k_host, t0, nt, rkv, hb, sl.hk0, sl.hkc, cudaMemcpyHostToDevice, s_in));
@@ -1162,10 +1184,10 @@ extern "C" int fcp_attn_fwd_bwd_host(const fcp_plan* plan, const void* q_host, c
   }
   for (size_t i = 0; i < slices.size(); ++i) {
     const Slice& sl = slices[i];
-    const fcp_plan* sub = plan->groups.empty() ? plan : plan->groups[sl.g];
+    const fcp_plan* sub = cut.groups.empty() ? plan : cut.groups[sl.g];
     const int lane = two_lanes ? (int)(i & 1) : 0;
     cudaStream_t sk = lane ? s_lane : st;
-    const int64_t t0 = plan->group_tok0[sl.g], nt = plan->group_tok0[sl.g + 1] - t0;
+    const int64_t t0 = cut.tok0[sl.g], nt = cut.tok0[sl.g + 1] - t0;
     const int h0 = sl.hk0 * gq, hc = sl.hkc * gq;
     FCP_CUDA_CHECK(cudaStreamWaitEvent(sk, EV(sl.ev0), 0));
     if ((rc = launch_fwd(sub, w + L.q + t0 * rq, w + L.k + t0 * rkv, w + L.v + t0 * rkv, h0, hc, nullptr, nullptr, w + L.o + t0 * rq,
@@ -1191,7 +1213,7 @@ extern "C" int fcp_attn_fwd_bwd_host(const fcp_plan* plan, const void* q_host, c
   FCP_CUDA_CHECK(cudaStreamWaitEvent(st, EV(2), 0));
   FCP_CUDA_CHECK(cudaEventRecord(EV(1), s_out));
   FCP_CUDA_CHECK(cudaStreamWaitEvent(st, EV(1), 0));
-  for (const fcp_plan* sub : plan->groups) mark_used(sub, st);   // after both lanes
+  for (const fcp_plan* sub : cut.groups) mark_used(sub, st);   // after both lanes
   mark_used(plan, st);
   FCP_CUDA_CHECK(cudaStreamSynchronize(st));
   drain.armed = false;

@@ -35,6 +35,15 @@ struct PlanBlock;                      // device block of an uploaded plan (fcp_
 bool split_units(const std::vector<int32_t>& units, const std::vector<int32_t>& groups, int heads, int per, int sms);
 constexpr int FCP_PLAN_SMS = 148;      // what the planner takes the device to have
 
+// How the host entry point cuts a batch: sub-plans over runs of consecutive sequences (none when one run, the plan itself, is
+// enough), KV-head passes of each run, and the events between the slices.
+struct HostCut {
+  std::vector<fcp_plan*> groups;
+  std::vector<int64_t> tok0;                 // first packed token of each run, plus T at the end; empty: not set up yet
+  int32_t passes = 1;
+  std::vector<void*> events;                 // cudaEvent_t: start, last copy out, second lane, then four per (run, pass)
+};
+
 struct fcp_plan {
   fcp_params params{};
   int32_t B = 0;
@@ -69,15 +78,12 @@ struct fcp_plan {
   int32_t* d_status = nullptr; // [4]: status word, diagnostic
   int sm_count = 0;
 
-  // Host entry point, set up at its first call and owned by this plan: sub-plans over runs of consecutive sequences
-  // (none when one run, this plan itself, is enough), streams and events.
-  mutable std::vector<fcp_plan*> groups;
-  mutable std::vector<int64_t> group_tok0;   // first packed token of each run, plus T at the end
+  // Host entry point, set up at its first call and owned by this plan: streams, and one cut of the batch for page-locked
+  // and one for pageable buffers (fcp_kernels.cu).
+  mutable HostCut host_cuts[2];
   mutable void* host_in = nullptr;           // cudaStream_t: host -> device copies
   mutable void* host_out = nullptr;          // cudaStream_t: device -> host copies
   mutable void* host_lane = nullptr;         // cudaStream_t: kernels of every second slice
-  mutable int32_t host_passes = 1;           // KV-head passes of each run
-  mutable std::vector<void*> host_events;    // cudaEvent_t: start, last copy out, second lane, then four per (run, pass)
 
   // optional kernel timing: ring of event pairs per kernel kind (void* = cudaEvent_t)
   bool profiling = false;

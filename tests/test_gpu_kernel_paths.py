@@ -249,3 +249,27 @@ def test_partial_path_of_short_sequences(D, deg):
     o_ref, lse_ref = A.attention_fwd_packed(f64(q), f64(k), f64(v), w.cu_seqlens)
     e = np.abs(res["o_f32"] - o_ref)
     assert e.max() <= 1e-2 and e.mean() <= 1e-3 and np.abs(res["lse"] - lse_ref).max() <= 1e-3
+
+
+@pytest.mark.parametrize("lens,hq,hkv,D", [([700, 130], 4, 2, 64), ([9000, 12000, 7000, 1001], 8, 4, 128)])
+def test_host_entry_point_with_pageable_buffers(lens, hq, hkv, D):
+    """One plan's calls with page-locked and pageable buffers in turn, and with one pageable buffer among page-locked ones."""
+    from paper_2602_21788_b200 import fcp
+    from paper_2602_21788_b200.runner import DeviceState
+    w = _wl(lens, [1] * len(lens), hq, hkv, D, seed=47)
+    ds = DeviceState(w, *w.device_tensors(), partials=False)
+    ds.forward_fused()
+    ds.backward()
+    torch.cuda.synchronize()
+    nbytes = ds.plan.host_workspace_bytes()
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    host = [t.cpu() for t in (ds.q, ds.k, ds.v, ds.do)]
+    for locked in ("all", "none", "but dk", "all"):
+        pin = lambda i, t: t.pin_memory() if locked == "all" or (locked == "but dk" and i != 7) else t
+        ins = [pin(i, t) for i, t in enumerate(host)]
+        out = [pin(4 + i, torch.zeros(t.shape, dtype=t.dtype)) for i, t in enumerate((ds.o, ds.lse, ds.dq, ds.dk, ds.dv))]
+        fcp.fcp_attn_fwd_bwd_host(ds.plan, *ins, *out, ws, nbytes, torch.cuda.current_stream().cuda_stream)
+        assert ds.plan.device_status()[0] == 0
+        for got, ref in zip((out[0], out[1], out[3], out[4]), (ds.o, ds.lse, ds.dk, ds.dv)):
+            assert torch.equal(got, ref.cpu()), locked
+        assert (out[2].float() - ds.dq.float().cpu()).norm() <= 1e-2 * ds.dq.float().norm().item()
