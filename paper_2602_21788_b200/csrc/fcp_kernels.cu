@@ -985,6 +985,14 @@ constexpr int64_t kHostSliceBytes = int64_t(8) << 20;
 // that.  256K tokens with one of 128K, 98 000 flop/byte: 618 ms with runs, 585 without; 64K tokens of the 32/8-head
 // log-normal batch, 4 800 flop/byte: 32.1 ms with, 33.2 without.
 constexpr int64_t kHostSlices = 16, kHostPasses = 8, kHostFlopsPerByte = 20000;
+// Where the copies decide and would be of narrow rows (below kHostNarrowFlops, query rows of a pass of at most kHostNarrowRow
+// bytes; or below kHostCopyFlops at any width) and four even runs or more can be had (the longest sequence at most two of them),
+// runs come first, up to kHostRuns of kHostRunTokens, and heads are cut only down to K/V rows of kHostRowBytes.  Heads first
+// against this (ms, two GPUs where they differ): 32K tokens of 8/8 heads 8.1, 7.3; 64K of 12/4 heads, D = 64: 7.9, 7.2; 700
+// sequences of 300 tokens, 32/8 heads: 104, 100; but 64K of 32/32 heads (5800 flop/byte): 50.9, 53.4 and 50.1, 49.5; 64K of 32/8
+// heads (1024 bytes): 33.0, 33.9 and 32.5, 31.8.
+constexpr int64_t kHostNarrowRow = 512, kHostNarrowFlops = 5000, kHostCopyFlops = 1000, kHostRowBytes = 1024;
+constexpr int64_t kHostRuns = 8, kHostRunTokens = 8192;
 // Slices with fewer backward units than this per SM take turns on two kernel lanes, so that one fills the SMs that the
 // other's last units leave idle (30K tokens of 16/4 heads, D = 64, half a unit: 5.0 ms, one lane 6.7).  Larger ones fill the
 // chip by themselves, and two at once share its L2 (384K sequence, 20 units: 8390 ms, one lane 8125; 128K sequence, 7 units:
@@ -994,7 +1002,6 @@ constexpr int64_t kHostLaneUnits = 4;
 // Strided copies of pageable memory run at a fraction of the speed of contiguous ones, and copies wait for one another
 // whatever the slices are: such buffers are cut into up to eight runs of at least 8192 tokens and not by heads (8K tokens of
 // 32/8 heads: 37 ms by heads, 25 like this; 32K: 155, 104; 64K: 301, 204; 64K of 32/32 heads: 494, 345).
-constexpr int64_t kHostRuns = 8, kHostRunTokens = 8192;
 
 bool is_pageable(const void* p) {
   cudaPointerAttributes a;
@@ -1026,6 +1033,14 @@ int build_host_cut(const fcp_plan* plan, bool pageable, void* stream) {
   const int64_t most = std::min<int64_t>(by_heads ? kHostSlices : kHostPasses, slices);
   int32_t passes = (int32_t)std::min<int64_t>(P.hkv, most);
   int want = by_heads ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(slices / passes, B), T / kHostRunTokens));
+  const int64_t runs = std::min<int64_t>(std::min<int64_t>(kHostRuns, B), std::min<int64_t>(slices, T / kHostRunTokens));
+  const int64_t q_row = (int64_t)P.hq / P.hkv * P.head_dim * 2;
+  const bool copies = flops < (double)(q_row <= kHostNarrowRow ? kHostNarrowFlops : kHostCopyFlops) * in_bytes;
+  if (copies && runs >= 4 && plan->max_seqlen * runs <= 2 * T) {
+    const int64_t kv_row = (int64_t)P.hkv * P.head_dim * 2;
+    passes = (int32_t)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(P.hkv, kv_row / kHostRowBytes), kHostSlices / runs));
+    want = (int)runs;
+  }
   if (pageable) {
     passes = 1;
     want = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(kHostRuns, B), T / kHostRunTokens));

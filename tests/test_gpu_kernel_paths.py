@@ -273,3 +273,12 @@ def test_host_entry_point_with_pageable_buffers(lens, hq, hkv, D):
         for got, ref in zip((out[0], out[1], out[3], out[4]), (ds.o, ds.lse, ds.dk, ds.dv)):
             assert torch.equal(got, ref.cpu()), locked
         assert (out[2].float() - ds.dq.float().cpu()).norm() <= 1e-2 * ds.dq.float().norm().item()
+
+
+@pytest.mark.parametrize("lens,hq,hkv,D", [
+    ([1000] * 33, 8, 8, 128),             # narrow rows, even runs: four runs of two passes
+    ([4100] * 8, 4, 2, 64),               # the same with one pass
+    ([20000] + [1000] * 13, 4, 4, 64),    # a sequence longer than two runs: heads first
+])
+def test_host_entry_point_cuts_copy_bound_batches_into_runs(lens, hq, hkv, D):
+    test_host_entry_point_slices(lens, hq, hkv, D)
