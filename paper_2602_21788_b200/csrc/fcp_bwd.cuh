@@ -5,7 +5,7 @@
 //
 //   T1  S^T  = K Q^T                   (UMMA, smem x smem)      TMEM cols [  0,128)
 //   T2  dP^T = V dO^T                  (UMMA, smem x smem)      TMEM cols [128,256)
-//   C1  P^T  = exp2(S^T*c - lse2[q])   (CUDA cores, thread = key row x half of the queries), bf16 over S^T
+//   C1  P^T  = exp2(S^T*c - lse2[q])   (CUDA cores, matrix fragments), bf16 over S^T
 //   T3  dV  += P^T dO                  (UMMA, TMEM x smem)      TMEM cols [256,384)
 //   C2  dS^T = P^T o (dP^T*scale - delta[q]*scale)               bf16 to smem
 //   T5  dQ   = dS K                    (UMMA, smem x smem)      over dP^T
@@ -86,53 +86,39 @@ struct BwdArgs {
   int32_t* status;
 };
 
-// The (head-of-group, Q range, Q tile) iterations of one unit, in the order every role walks them.
-// The head is the outer loop: all CTAs of a (sequence, KV head) panel then sweep the query tiles of
-// one query head at a time, which keeps the dQ rows they reduce into (and the Q/dO tiles they
-// share) to one head's worth of L2.
+// The (head-of-group, Q tile) iterations of one unit, in the order every role walks them: Q tiles T_FIRST and on of the
+// unit's sequence (its one Q range), the tiles before T_MASK_END masked.  The head is the outer loop: all CTAs of a
+// (sequence, KV head) panel then sweep the query tiles of one query head at a time, which keeps the dQ rows they reduce into
+// (and the Q/dO tiles they share) to one head's worth of L2.
 struct BwdIter {
-  const int32_t* qr;     // Q ranges of the unit
-  int nq, t_first, t_mask_end, g;   // a DIAG range starts at Q tile t_first; tiles before t_mask_end need the mask
-  int r, t, hh;          // range, tile within range, head within group
-  int qb, qe, diag;
+  int qb, qe, t_first, t_mask_end, g;    // Q rows of the range; query heads of the group
+  int t, hh;                             // tile within the range, head within the group
   bool valid;
   int q_row, q_valid;
   bool causal;
 
-  __device__ __forceinline__ void load_range() {
-    const int32_t* Q = qr + (size_t)r * FCP_BWD_QRANGE_W;
-    qb = __ldg(Q + BQ_BEGIN);
-    qe = __ldg(Q + BQ_END);
-    diag = __ldg(Q + BQ_DIAG);
-    t = diag ? t_first : 0;
-  }
-  __device__ __forceinline__ void settle() {           // make (hh, r, t) point at an existing tile
-    while (valid && qb + t * 128 >= qe) {
-      if (++r >= nq) {
-        r = 0;
-        if (++hh >= g) { valid = false; break; }
-      }
-      load_range();
-    }
-    if (valid) {
-      q_row = qb + t * 128;
-      q_valid = min(128, qe - q_row);
-      causal = diag && t < t_mask_end;
-    }
+  __device__ __forceinline__ void settle() {
+    q_row = qb + t * 128;
+    q_valid = min(128, qe - q_row);
+    causal = t < t_mask_end;
   }
   __device__ __forceinline__ void init(const int32_t* U, const int32_t* qranges, int g_) {
-    qr = qranges + (size_t)__ldg(U + BU_FIRST_QRANGE) * FCP_BWD_QRANGE_W;
-    nq = __ldg(U + BU_N_QRANGES);
+    const int32_t* Q = qranges + (size_t)__ldg(U + BU_FIRST_QRANGE) * FCP_BWD_QRANGE_W;
+    qb = __ldg(Q + BQ_BEGIN);
+    qe = __ldg(Q + BQ_END);
     t_first = __ldg(U + BU_T_FIRST);
     t_mask_end = __ldg(U + BU_T_MASK_END);
     g = g_;
-    r = 0; hh = 0;
-    valid = nq > 0;
-    if (valid) load_range();
+    t = t_first;
+    hh = 0;
+    valid = true;                        // a key tile is seen by its own queries at least
     settle();
   }
   __device__ __forceinline__ void advance() {
-    ++t;
+    if (qb + ++t * 128 >= qe) {
+      t = t_first;
+      valid = ++hh < g;
+    }
     settle();
   }
 };
@@ -356,9 +342,9 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (ok && i == 0) ok = mbar_wait(BAR(B_ACCEMPTY), (n & 1) ^ 1, wctx, 124);
             if (!ok) break;
             tc_fence_after();
-            umma_loop_ts<0, 6>(true, tmem + C_DV, tmem + C_S, true, dobase, IDESC_ACC, i > 0 ? 1u : 0u);
+            umma_loop_ts<0, 6>(tmem + C_DV, tmem + C_S, true, dobase, IDESC_ACC, i > 0 ? 1u : 0u);
             if (next) q_ready = mbar_test(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1);
-            umma_loop_ts<6, 8>(true, tmem + C_DV, tmem + C_S, true, dobase, IDESC_ACC, 1u);
+            umma_loop_ts<6, 8>(tmem + C_DV, tmem + C_S, true, dobase, IDESC_ACC, 1u);
             tc_commit(BAR(B_DOFREE + sd));
           }
           // T1 of the next tile: S^T has been read by the math warps and P^T is consumed in order
@@ -366,9 +352,9 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (!q_ready) ok = mbar_wait(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1, wctx, 126);
             if (!ok) break;
             tc_fence_after();
-            umma_loop_kk<0, D / 16 - 2>(true, tmem + C_S, kbase, sbase + SM::Q_OFF + st_next * SM::TILE_BYTES, IDESC_ST);
+            umma_loop_kk<0, D / 16 - 2>(tmem + C_S, kbase, sbase + SM::Q_OFF + st_next * SM::TILE_BYTES, IDESC_ST);
             if (cur) ds_ready = mbar_test(BAR(B_DSFULL), (it - 1) & 1);
-            umma_loop_kk<D / 16 - 2, D / 16>(true, tmem + C_S, kbase, sbase + SM::Q_OFF + st_next * SM::TILE_BYTES, IDESC_ST);
+            umma_loop_kk<D / 16 - 2, D / 16>(tmem + C_S, kbase, sbase + SM::Q_OFF + st_next * SM::TILE_BYTES, IDESC_ST);
             tc_commit(BAR(B_SFULL));
           }
           if (cur) {
@@ -377,12 +363,12 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (!ds_ready) ok = mbar_wait(BAR(B_DSFULL), (it - 1) & 1, wctx, 125);
             if (!ok) break;
             tc_fence_after();
-            umma_loop_mm(true, tmem + C_DP, dsbase, kbase, IDESC_DQ);
+            umma_loop_mm(tmem + C_DP, dsbase, kbase, IDESC_DQ);
             tc_commit(BAR(B_DQFULL));
             if (next) do_ready = mbar_test(BAR(B_DOFULL + sd_next), (it / DO_STAGES) & 1);
-            umma_loop_km<0, 6>(true, tmem + C_DK, dsbase, qbase, IDESC_ACC, i > 0 ? 1u : 0u);
+            umma_loop_km<0, 6>(tmem + C_DK, dsbase, qbase, IDESC_ACC, i > 0 ? 1u : 0u);
             if (next) dq_free = mbar_test(BAR(B_DQEMPTY), (it & 1) ^ 1);
-            umma_loop_km<6, 8>(true, tmem + C_DK, dsbase, qbase, IDESC_ACC, 1u);
+            umma_loop_km<6, 8>(tmem + C_DK, dsbase, qbase, IDESC_ACC, 1u);
             tc_commit(BAR(B_QFREE + st));
           }
           // T2 of the next tile once the drain warps have emptied the dQ tile of the one before it
@@ -392,9 +378,9 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (ok && !dq_free) ok = mbar_wait(BAR(B_DQEMPTY), (it & 1) ^ 1, wctx, 127);
             if (!ok) break;
             tc_fence_after();
-            umma_loop_kk<0, D / 16 - 2>(true, tmem + C_DP, vbase, sbase + SM::DO_OFF + sd_next * SM::TILE_BYTES, IDESC_ST);
+            umma_loop_kk<0, D / 16 - 2>(tmem + C_DP, vbase, sbase + SM::DO_OFF + sd_next * SM::TILE_BYTES, IDESC_ST);
             p_ready = mbar_test(BAR(B_PFULL), it & 1);
-            umma_loop_kk<D / 16 - 2, D / 16>(true, tmem + C_DP, vbase, sbase + SM::DO_OFF + sd_next * SM::TILE_BYTES, IDESC_ST);
+            umma_loop_kk<D / 16 - 2, D / 16>(tmem + C_DP, vbase, sbase + SM::DO_OFF + sd_next * SM::TILE_BYTES, IDESC_ST);
             tc_commit(BAR(B_DPFULL));
             ++it;
           }

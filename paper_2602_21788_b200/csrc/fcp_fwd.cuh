@@ -309,7 +309,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (!ok) break;
             if (sb) ++xcnt1; else ++xcnt0;
             tc_fence_after();
-            umma_loop_kk<0, D / 16>(true, tmem + S_COL0 + sb * 128, sbase + SM::Q_OFF + s * SM::Q_TILE_BYTES,
+            umma_loop_kk<0, D / 16>(tmem + S_COL0 + sb * 128, sbase + SM::Q_OFF + s * SM::Q_TILE_BYTES,
                                  sbase + SM::KV_OFF + slot * SM::KV_TILE_BYTES, IDESC_QK);
             tc_commit(BAR(B_SFULL + s));
             if (j == nts - 1) tc_commit(BAR(B_QEMPTY + s));
@@ -348,7 +348,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (s) ++pcnt1; else ++pcnt0;
             if (!ok) break;
             tc_fence_after();
-            umma_loop_ts<0, 8>(true, tmem + O_COL0 + s * O_STRIDE, tmem + P_COL0 + s * 64, false,
+            umma_loop_ts<0, 8>(tmem + O_COL0 + s * O_STRIDE, tmem + P_COL0 + s * 64, false,
                          sbase + SM::KV_OFF + slot * SM::KV_TILE_BYTES, IDESC_PV, j > 0 ? 1u : 0u);
             tc_commit(BAR(B_PFREE + s));
             if (j == nts - 1) tc_commit(BAR(B_OFINAL + s));
@@ -496,7 +496,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           const float f = grow ? ex2(m_ref - m_new) : 1.f;    // m_ref = -inf -> 0
           l01.x *= f; l01.y *= f; l23.x *= f; l23.y *= f;
           if (j > 0) {
-            ok = mbar_wait_warp(BAR(B_PFREE + s), (pcnt & 1) ^ 1, wctx, 36);   // O is at rest once the last product is done
+            ok = mbar_wait_warp(BAR(B_PFREE + s), (pcnt & 1) ^ 1, wctx, 42);   // O is at rest once the last product is done
             if (!ok) break;
             tc_fence_after();
 #pragma unroll 1

@@ -28,14 +28,6 @@ __device__ __forceinline__ uint32_t globaltimer_lo() {
   return t;
 }
 
-__device__ __forceinline__ bool elect_one() {
-  uint32_t pred;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(pred));
-  return pred != 0;
-}
-
 // ----------------------------------------------------------------------------- programmatic launch
 // Every kernel of the library waits (grid_wait) for the work before it, memory included, before it touches global
 // memory, so that "the grid before is complete" covers all grids before that one too.  The short kernels let the next
@@ -266,17 +258,7 @@ __host__ __device__ constexpr uint32_t make_idesc(int M, int N, int a_mn_major, 
 // groups along M/N; LBO is not used by the swizzled K-major form.
 // MN-major operand (the 64 contiguous elements run along M/N): SBO = 1024 is the step between
 // 8-row groups along K; LBO is the step between 64-element column blocks along M/N.
-__device__ __forceinline__ uint64_t make_sdesc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
-// The same descriptor split into its two 32-bit words, so that issue loops only add a byte offset to
+// The descriptor is kept as its two 32-bit words, so that issue loops only add a byte offset to
 // the low word (start address field) instead of rebuilding all 64 bits per instruction.
 __device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr, uint32_t lbo_bytes) {
   return ((saddr & 0x3FFFFu) >> 4) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
@@ -295,55 +277,51 @@ __device__ __forceinline__ uint64_t sdesc_pack(uint32_t lo, uint32_t hi) {
 // 85 clocks per trip) would be slower than the 64 clocks a 128x128x16 UMMA takes to execute.
 // K-major A and B tiles of [128][64]-element swizzled blocks: K step k lives in block k/4 at byte
 // offset (k%4)*32 of every row.
-//
-// The helpers are called by a whole warp in uniform control flow; only `leader` (one lane) executes
-// the UMMA itself.  Keeping the descriptor arithmetic outside the divergent part lets the compiler
-// hold it in the warp-uniform datapath instead of re-deriving it in one lane's registers.
 // K steps [K0, K1); the first step of the product (K0 = 0) overwrites D.
 template <int K0, int K1>
-__device__ __forceinline__ void umma_loop_kk(bool leader, uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc) {
+__device__ __forceinline__ void umma_loop_kk(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc) {
   const uint32_t hi = sdesc_hi(1024), alo = sdesc_lo(a_addr, 16), blo = sdesc_lo(b_addr, 16);
 #pragma unroll
   for (int k = K0; k < K1; ++k) {
     const uint32_t off = (uint32_t)(k >> 2) * (16384u >> 4) + (uint32_t)(k & 3) * 2u;
     const uint64_t ad = sdesc_pack(alo + off, hi), bd = sdesc_pack(blo + off, hi);
-    if (leader) umma_ss(d_tmem, ad, bd, idesc, k > 0 ? 1u : 0u);
+    umma_ss(d_tmem, ad, bd, idesc, k > 0 ? 1u : 0u);
   }
 }
 // MN-major A and B (64-element blocks 16384 bytes apart): K step k is rows [16k, 16k+16) = +2048 bytes.
-__device__ __forceinline__ void umma_loop_mm(bool leader, uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc) {
+__device__ __forceinline__ void umma_loop_mm(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc) {
   const uint32_t hi = sdesc_hi(1024), alo = sdesc_lo(a_addr, 16384), blo = sdesc_lo(b_addr, 16384);
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const uint64_t ad = sdesc_pack(alo + k * 128u, hi), bd = sdesc_pack(blo + k * 128u, hi);
-    if (leader) umma_ss(d_tmem, ad, bd, idesc, k > 0 ? 1u : 0u);
+    umma_ss(d_tmem, ad, bd, idesc, k > 0 ? 1u : 0u);
   }
 }
 // K-major A ([128][64]-element swizzled blocks, as in umma_loop_kk) and MN-major B (as in
 // umma_loop_mm); `acc` = accumulate into D from the first step on.
 // K steps [K0, K1).
 template <int K0, int K1>
-__device__ __forceinline__ void umma_loop_km(bool leader, uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc,
+__device__ __forceinline__ void umma_loop_km(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc,
                                              uint32_t acc) {
   const uint32_t hi = sdesc_hi(1024), alo = sdesc_lo(a_addr, 16), blo = sdesc_lo(b_addr, 16384);
 #pragma unroll
   for (int k = K0; k < K1; ++k) {
     const uint32_t off = (uint32_t)(k >> 2) * (16384u >> 4) + (uint32_t)(k & 3) * 2u;
     const uint64_t ad = sdesc_pack(alo + off, hi), bd = sdesc_pack(blo + k * 128u, hi);
-    if (leader) umma_ss(d_tmem, ad, bd, idesc, (acc | (k > K0)) ? 1u : 0u);
+    umma_ss(d_tmem, ad, bd, idesc, (acc | (k > K0)) ? 1u : 0u);
   }
 }
 // A from TMEM (bf16 pairs, 8 columns per K step; with `split` the second four steps start at
 // column 64), MN-major B, K steps [K0, K1).  `acc` = accumulate into D from the first step on.
 template <int K0, int K1>
-__device__ __forceinline__ void umma_loop_ts(bool leader, uint32_t d_tmem, uint32_t a_tmem, bool split, uint32_t b_addr,
+__device__ __forceinline__ void umma_loop_ts(uint32_t d_tmem, uint32_t a_tmem, bool split, uint32_t b_addr,
                                              uint32_t idesc, uint32_t acc) {
   const uint32_t hi = sdesc_hi(1024), blo = sdesc_lo(b_addr, 16384);
 #pragma unroll
   for (int k = K0; k < K1; ++k) {
     const uint32_t col = (split && k >= 4) ? 64u + 8u * (k - 4) : 8u * k;
     const uint64_t bd = sdesc_pack(blo + k * 128u, hi);
-    if (leader) umma_ts(d_tmem, a_tmem + col, bd, idesc, (acc | (k > K0)) ? 1u : 0u);
+    umma_ts(d_tmem, a_tmem + col, bd, idesc, (acc | (k > K0)) ? 1u : 0u);
   }
 }
 // TMEM address = (lane << 16) | column.
@@ -371,22 +349,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
-}
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),
-        "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
-        "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
 }
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {

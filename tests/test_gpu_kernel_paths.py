@@ -282,3 +282,50 @@ def test_host_entry_point_with_pageable_buffers(lens, hq, hkv, D):
 ])
 def test_host_entry_point_cuts_copy_bound_batches_into_runs(lens, hq, hkv, D):
     test_host_entry_point_slices(lens, hq, hkv, D)
+
+
+@pytest.mark.parametrize("lens,hq,hkv,D", [([700, 130, 1], 4, 2, 64), ([2300, 900, 64], 8, 2, 128)])
+def test_captured_calls(lens, hq, hkv, D):
+    """Forward and backward captured into a graph, replayed over new inputs while other plans are uploaded, run and dropped: the
+    work counters come back to zero each time, and the captured plan's tables stay its own, also after the plan object is gone
+    from the pool's point of view (its block is never handed on)."""
+    from paper_2602_21788_b200 import fcp
+    from paper_2602_21788_b200.runner import DeviceState
+    w = _wl(lens, [1] * len(lens), hq, hkv, D, seed=53)
+    ds = DeviceState(w, *w.device_tensors(), partials=False)
+    other = [fcp.Plan([500 + 100 * i, 77], [1, 1], hq, hkv, D) for i in range(3)]
+    big = torch.randn((800, hq, D), device="cuda").bfloat16()
+    small = torch.randn((800, hkv, D), device="cuda").bfloat16()
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):                       # eager once, as before any capture
+        ds.forward_fused(side)
+        ds.backward(side)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ds.forward_fused()
+        ds.backward()
+    g = torch.Generator(device="cuda").manual_seed(59)
+    for r in range(4):
+        for t in (ds.q, ds.k, ds.v, ds.do):
+            t.copy_(torch.randn(t.shape, device="cuda", generator=g))
+        for t in (ds.o, ds.lse, ds.dq, ds.dk, ds.dv):
+            t.zero_()
+        graph.replay()
+        if r < 3:
+            plan = other[r].upload()
+            _fused(plan, big, small, small, hq, torch.cuda.current_stream())
+            other[r] = None
+            del plan
+        got = [t.clone() for t in (ds.o, ds.lse, ds.dk, ds.dv, ds.dq)]
+        fresh = DeviceState(w, ds.q, ds.k, ds.v, ds.do, partials=False)
+        fresh.forward_fused()
+        fresh.backward()
+        torch.cuda.synchronize()
+        ds.check_status()
+        for a, b in zip(got, (fresh.o, fresh.lse, fresh.dk, fresh.dv)):
+            assert torch.equal(a, b), r
+        assert (got[4].float() - fresh.dq.float()).norm() <= 1e-2 * fresh.dq.float().norm()
+        del fresh
+    del graph
