@@ -264,7 +264,8 @@ int fcp_attn_bwd_heads(const fcp_plan* plan, const void* q, const void* k, const
  * ones go out while kernels execute (two internal copy streams and a second kernel stream, ordered
  * after the work already queued on `stream`).  The first call on a plan is the one exception to
  * "compute calls do not allocate": it builds and uploads the plans of the runs and creates the
- * streams and events (small allocations, all released by fcp_plan_destroy).
+ * streams and events; fcp_plan_destroy releases the streams and events and destroys the runs' plans,
+ * whose tables' memory goes the way of every plan's (fcp_plan_upload).
  * Synchronises `stream` before returning; every output is complete then.  On an error return the
  * work already queued has been waited for, so nothing writes into the caller's buffers afterwards.
  */

@@ -28,7 +28,7 @@
 // Left out one by one on a 64K-token batch (19.4 ms): bulk reductions 17.1 ms, staging stores 18.7, exponentials 19.3.
 // The bulk reductions took the period from 5090 to 4412 clk, what followed to 3880; under the power cap the clock falls
 // meanwhile, so that the time goes down less.  Kernel with all of it, before -> now: 128K bimodal batch
-// 102 -> 92 ms, 64K log-normal batch 12.9 -> 11.6 ms, 8K batch 405 -> 260 us (there the work order counts most).
+// 102 -> 92 ms, 64K log-normal batch 12.9 -> 11.2 ms, 8K batch 405 -> 244 us (there the work order counts most).
 // The math loops stay rolled: unrolling their trips costs 3-7 %.
 #pragma once
 #include "fcp_plan.hpp"

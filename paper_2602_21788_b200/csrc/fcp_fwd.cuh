@@ -68,7 +68,7 @@ struct FwdArgs {
   int32_t head_begin, head_count, hq, hkv;
   int32_t head_group;     // heads that are adjacent in the work order: hq/hkv when the head range is made of whole
                           // KV-head groups, else 1; head_count % head_group == 0
-  int32_t split;          // 1: the two Q tiles of a unit are work items of their own
+  int32_t split;          // 1: the two Q tiles of a unit are work items of their own (split_units of fcp_plan.cpp)
   int32_t* work_counter;  // the grid's next work item: zero before the launch, and again after it
   float scale_log2;       // softmax scale * log2(e)
   float* o_partial;       // [R][head_count][D]

@@ -287,8 +287,7 @@ def test_host_entry_point_cuts_copy_bound_batches_into_runs(lens, hq, hkv, D):
 @pytest.mark.parametrize("lens,hq,hkv,D", [([700, 130, 1], 4, 2, 64), ([2300, 900, 64], 8, 2, 128)])
 def test_captured_calls(lens, hq, hkv, D):
     """Forward and backward captured into a graph, replayed over new inputs while other plans are uploaded, run and dropped: the
-    work counters come back to zero each time, and the captured plan's tables stay its own, also after the plan object is gone
-    from the pool's point of view (its block is never handed on)."""
+    work counters come back to zero each time, and the captured plan's tables stay its own."""
     from paper_2602_21788_b200 import fcp
     from paper_2602_21788_b200.runner import DeviceState
     w = _wl(lens, [1] * len(lens), hq, hkv, D, seed=53)
