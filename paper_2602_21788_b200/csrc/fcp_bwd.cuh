@@ -28,7 +28,7 @@
 // Left out one by one on a 64K-token batch (19.4 ms): bulk reductions 17.1 ms, staging stores 18.7, exponentials 19.3.
 // The bulk reductions took the period from 5090 to 4412 clk, what followed to 3880; under the power cap the clock falls
 // meanwhile, so that the time goes down less.  Kernel with all of it, before -> now: 128K bimodal batch
-// 102 -> 92 ms, 64K log-normal batch 12.9 -> 11.2 ms, 8K batch 405 -> 244 us (there the work order counts most).
+// 102 -> 92 ms, 64K log-normal batch 12.9 -> 11.2 ms, 8K batch 405 -> 243 us (there the work order counts most).
 // The math loops stay rolled: unrolling their trips costs 3-7 %.
 #pragma once
 #include "fcp_plan.hpp"
@@ -92,7 +92,7 @@ struct BwdArgs {
 // (and the Q/dO tiles they share) to one head's worth of L2.
 struct BwdIter {
   int qb, qe, t_first, t_mask_end, g;    // Q rows of the range; query heads of the group
-  int t, hh;                             // tile within the range, head within the group
+  int nt, t, hh;                         // tile within the range, head within the group
   bool valid;
   int q_row, q_valid;
   bool causal;
@@ -109,13 +109,14 @@ struct BwdIter {
     t_first = __ldg(U + BU_T_FIRST);
     t_mask_end = __ldg(U + BU_T_MASK_END);
     g = g_;
+    nt = (qe - qb + 127) >> 7;
     t = t_first;
     hh = 0;
     valid = true;                        // a key tile is seen by its own queries at least
     settle();
   }
   __device__ __forceinline__ void advance() {
-    if (qb + ++t * 128 >= qe) {
+    if (++t >= nt) {
       t = t_first;
       valid = ++hh < g;
     }
@@ -478,10 +479,6 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const float* s_lse = s_rows + half * 64;
         const float* s_delta = s_rows + 128 + half * 64;
         const bool need_mask = causal || q_valid < 128 || kv_rows < 128;   // uniform across the CTA
-        // A warp without any (key row, query) pair of the tile writes zeros, and the mask comes from one bit per column instead of
-        // four comparisons per pair of columns: 1841 sequences of 12 tokens, D = 64: 237 -> 208 us; 16K ragged batch, D = 64:
-        // 179.9 -> 173.5; 8K batch 257 -> 250.
-        const bool live = rb * 32 < kv_rows && half * 64 < q_valid;
 
         ok = mbar_wait_warp(BAR(B_SFULL), it & 1, wctx, 130);
         if (!ok) break;
@@ -492,7 +489,6 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         // between the trips the pair arrays rotate (register arrays cannot be indexed by the trip), which halves the
         // code of this loop.
         uint32_t pa[16], pb[16] = {};
-        if (live) {
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           uint32_t sv[32];
@@ -517,7 +513,10 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             for (int g2 = 0; g2 < 4; ++g2) {
               const int off = half * 64 + c * 32;
               const int hi = min(32, (frow + 8 * g2 < kv_rows ? q_valid : 0) - off), lo = max(0, (causal ? first_q[g2] - q_row : 0) - off);
-              // one bit per column, then a byte of ones for the even and the odd column of each pair
+              // One bit per column, then a byte of ones for the even and the odd column of each pair.  Four comparisons per
+              // pair instead (kernel, us): 1841 sequences of 12 tokens, D = 64: 222, now 196; 16K tokens, D = 64: 319, 312; 64K
+              // tokens: 4325, 4185.  Warps without any pair that write zeros instead: 181, 322, 4240, and 128K tokens in
+              // three sequences 43500 instead of 43080.
               const uint32_t keep = bit_range(lo, max(0, hi - lo)) >> fcol;
               const uint32_t even = (keep & 0x01010101u) * 0xffu, odd = ((keep >> 1) & 0x01010101u) * 0xffu;
 #pragma unroll
@@ -526,14 +525,6 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           }
           tmem_st_frag(t_s + c * 16, pb);            // over this warp's own, already loaded, columns
           tmem_st_frag(t_s + (16u << 16) + c * 16, pb + 8);
-        }
-        } else {
-          const uint32_t zero[8] = {};
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            tmem_st_frag(t_s + c * 16, zero);
-            tmem_st_frag(t_s + (16u << 16) + c * 16, zero);
-          }
         }
         tc_wait_st();
         tc_fence_before();
@@ -544,7 +535,6 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         if (!ok) break;
         tc_fence_after();
         if (mtid >= 128) *my_next = next_row;
-        if (live) {
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           uint32_t dv_[32], out[16];
@@ -571,12 +561,6 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             const int cc = c * 4 + 2 * (m & 1) + mch;
             stmatrix_x4(ds_row + (m >> 1) * 2048 + ((cc ^ (lane & 7)) << 4), &out[(m >> 1) * 8 + 4 * (m & 1)]);
           }
-        }
-        } else {
-          const uint32_t zero[4] = {};
-#pragma unroll
-          for (int m = 0; m < 8; ++m)
-            stmatrix_x4(ds_row + ((m >> 1) & 1) * 2048 + ((((m >> 2) * 4 + 2 * (m & 1) + mch) ^ (lane & 7)) << 4), zero);
         }
         fence_proxy_async_smem();
         tc_fence_before();
