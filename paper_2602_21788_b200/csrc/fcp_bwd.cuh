@@ -191,7 +191,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   volatile int* work_ring = (volatile int*)(smem + SM::MISC_OFF + 8);    // [2 slots][unit, kv head]
   const WaitCtx wctx{abort_flag, a.status, (uint32_t)FCP_WAIT_NS};
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: uniform for the compiler too
 
   if (threadIdx.x == 0) {
     *abort_flag = 0;
@@ -252,7 +252,9 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   if (warp < 4) {
     // registers per thread: control 88, math 128, drain 168 (80 / 128 / 176 spilled in the issuing thread: kernel +2 %)
     asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
-    if (warp == 0 && lane == 0) {
+    // (warp branches outside the lane branches: behind a divergent one the compiler takes the issuer's operands for divergent)
+    if (warp == 0) {
+      if (lane == 0) {
       // ------------------------------------------------------------------ TMA producer + scheduler
       uint32_t n = 0, it = 0;
       bool ok = true;
@@ -306,7 +308,8 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             tma_load_3d(sbase + SM::DO_OFF + sd * SM::TILE_BYTES + kb * BLK_BYTES, &tm_do, BAR(B_DOFULL + sd), kb * 64, h, iter.q_row);
         }
       }
-    } else if (warp == 1 && lane == 0) {
+      }
+    } else if (warp == 1) {
       // ------------------------------------------------------------------ UMMA issuer
       constexpr uint32_t IDESC_ST = make_idesc(128, 128, 0, 0);   // K-major x K-major -> [keys][queries]
       constexpr uint32_t IDESC_ACC = make_idesc(128, D, 0, 1);    // TMEM A, MN-major B -> dV, dK
@@ -316,14 +319,15 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const uint32_t kbase = sbase + SM::K_OFF, vbase = sbase + SM::V_OFF, dsbase = sbase + SM::DS_OFF;
       while (ok) {
         const uint32_t slot = n & 1;
-        ok = mbar_wait(BAR(B_WFULL + slot), (n >> 1) & 1, wctx, 141);
+        ok = mbar_wait_warp(BAR(B_WFULL + slot), (n >> 1) & 1, wctx, 141);
         if (!ok) break;
-        const int unit = work_ring[2 * slot];
-        mbar_arrive(BAR(B_WEMPTY + slot));
+        const int unit = __shfl_sync(0xffffffffu, work_ring[2 * slot], 0);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(BAR(B_WEMPTY + slot));
         if (unit < 0) break;
         const int32_t* U = a.units + (size_t)unit * FCP_BWD_UNIT_W;
-        const int n_iter = __ldg(U + BU_COST) * g;
-        ok = mbar_wait(BAR(B_KVFULL), n & 1, wctx, 120);
+        const int n_iter = __shfl_sync(0xffffffffu, __ldg(U + BU_COST) * g, 0);
+        ok = mbar_wait_warp(BAR(B_KVFULL), n & 1, wctx, 120);
         if (!ok) break;
         // Software pipeline over the unit's tiles: trip i issues T3, T4, T5 of tile i and T1, T2 of tile
         // i + 1; trip -1 only starts the first tile.  `it` counts the tiles whose T1/T2 have been issued.
@@ -339,48 +343,48 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           bool q_ready = false, ds_ready = false, do_ready = false, dq_free = false;
           if (cur) {
             // T3: dV += P^T dO
-            if (!p_ready) ok = mbar_wait(BAR(B_PFULL), (it - 1) & 1, wctx, 123);
-            if (ok && i == 0) ok = mbar_wait(BAR(B_ACCEMPTY), (n & 1) ^ 1, wctx, 124);
+            if (!p_ready) ok = mbar_wait_warp(BAR(B_PFULL), (it - 1) & 1, wctx, 123);
+            if (ok && i == 0) ok = mbar_wait_warp(BAR(B_ACCEMPTY), (n & 1) ^ 1, wctx, 124);
             if (!ok) break;
             tc_fence_after();
             umma_loop_ts<0, 6>(tmem + C_DV, tmem + C_S, true, dobase, IDESC_ACC, i > 0 ? 1u : 0u);
-            if (next) q_ready = mbar_test(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1);
+            if (next) q_ready = mbar_test_warp(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1);
             umma_loop_ts<6, 8>(tmem + C_DV, tmem + C_S, true, dobase, IDESC_ACC, 1u);
             tc_commit(BAR(B_DOFREE + sd));
           }
           // T1 of the next tile: S^T has been read by the math warps and P^T is consumed in order
           if (next) {
-            if (!q_ready) ok = mbar_wait(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1, wctx, 126);
+            if (!q_ready) ok = mbar_wait_warp(BAR(B_QFULL + st_next), (it / BWD_Q_STAGES) & 1, wctx, 126);
             if (!ok) break;
             tc_fence_after();
             umma_loop_kk<0, D / 16 - 2>(tmem + C_S, kbase, sbase + SM::Q_OFF + st_next * SM::TILE_BYTES, IDESC_ST);
-            if (cur) ds_ready = mbar_test(BAR(B_DSFULL), (it - 1) & 1);
+            if (cur) ds_ready = mbar_test_warp(BAR(B_DSFULL), (it - 1) & 1);
             umma_loop_kk<D / 16 - 2, D / 16>(tmem + C_S, kbase, sbase + SM::Q_OFF + st_next * SM::TILE_BYTES, IDESC_ST);
             tc_commit(BAR(B_SFULL));
           }
           if (cur) {
             // T5: dQ tile, handed to the drain warps at once; T4: dK += dS^T Q runs while they read it.
             // Both take dS^T from shared memory (K-major A for T4, MN-major B for T5).
-            if (!ds_ready) ok = mbar_wait(BAR(B_DSFULL), (it - 1) & 1, wctx, 125);
+            if (!ds_ready) ok = mbar_wait_warp(BAR(B_DSFULL), (it - 1) & 1, wctx, 125);
             if (!ok) break;
             tc_fence_after();
             umma_loop_mm(tmem + C_DP, dsbase, kbase, IDESC_DQ);
             tc_commit(BAR(B_DQFULL));
-            if (next) do_ready = mbar_test(BAR(B_DOFULL + sd_next), (it / DO_STAGES) & 1);
+            if (next) do_ready = mbar_test_warp(BAR(B_DOFULL + sd_next), (it / DO_STAGES) & 1);
             umma_loop_km<0, 6>(tmem + C_DK, dsbase, qbase, IDESC_ACC, i > 0 ? 1u : 0u);
-            if (next) dq_free = mbar_test(BAR(B_DQEMPTY), (it & 1) ^ 1);
+            if (next) dq_free = mbar_test_warp(BAR(B_DQEMPTY), (it & 1) ^ 1);
             umma_loop_km<6, 8>(tmem + C_DK, dsbase, qbase, IDESC_ACC, 1u);
             tc_commit(BAR(B_QFREE + st));
           }
           // T2 of the next tile once the drain warps have emptied the dQ tile of the one before it
           p_ready = false;
           if (next) {
-            if (!do_ready) ok = mbar_wait(BAR(B_DOFULL + sd_next), (it / DO_STAGES) & 1, wctx, 128);
-            if (ok && !dq_free) ok = mbar_wait(BAR(B_DQEMPTY), (it & 1) ^ 1, wctx, 127);
+            if (!do_ready) ok = mbar_wait_warp(BAR(B_DOFULL + sd_next), (it / DO_STAGES) & 1, wctx, 128);
+            if (ok && !dq_free) ok = mbar_wait_warp(BAR(B_DQEMPTY), (it & 1) ^ 1, wctx, 127);
             if (!ok) break;
             tc_fence_after();
             umma_loop_kk<0, D / 16 - 2>(tmem + C_DP, vbase, sbase + SM::DO_OFF + sd_next * SM::TILE_BYTES, IDESC_ST);
-            p_ready = mbar_test(BAR(B_PFULL), it & 1);
+            p_ready = mbar_test_warp(BAR(B_PFULL), it & 1);
             umma_loop_kk<D / 16 - 2, D / 16>(tmem + C_DP, vbase, sbase + SM::DO_OFF + sd_next * SM::TILE_BYTES, IDESC_ST);
             tc_commit(BAR(B_DPFULL));
             ++it;
@@ -494,16 +498,18 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           uint32_t sv[32];
           tmem_ld_frag(t_s + c * 32, sv);
           tmem_ld_frag(t_s + (16u << 16) + c * 32, sv + 16);
+          float2 l2[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) l2[j] = lds_f2(s_lse + c * 32 + 8 * j + fcol);
 #pragma unroll
           for (int j = 0; j < 16; ++j) pa[j] = pb[j];
           tc_wait_ld();
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const float2 l2 = *reinterpret_cast<const float2*>(s_lse + c * 32 + 8 * j + fcol);
 #pragma unroll
             for (int g2 = 0; g2 < 4; ++g2) {               // row frow + 8 * g2
               const uint32_t* x = &sv[(g2 >> 1) * 16 + 4 * j + 2 * (g2 & 1)];
-              const float2 e = fma_pair(x[0], x[1], c22, l2);
+              const float2 e = fma_pair(x[0], x[1], c22, l2[j]);
               pb[(g2 >> 1) * 8 + 2 * j + (g2 & 1)] = pack_bf16(ex2(e.x), ex2(e.y));
             }
           }
@@ -540,15 +546,17 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           uint32_t dv_[32], out[16];
           tmem_ld_frag(t_dp + c * 32, dv_);
           tmem_ld_frag(t_dp + (16u << 16) + c * 32, dv_ + 16);
+          float2 d2[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) d2[j] = lds_f2(s_delta + c * 32 + 8 * j + fcol);
           tc_wait_ld();
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const float2 d2 = *reinterpret_cast<const float2*>(s_delta + c * 32 + 8 * j + fcol);
 #pragma unroll
             for (int g2 = 0; g2 < 4; ++g2) {
               const uint32_t* x = &dv_[(g2 >> 1) * 16 + 4 * j + 2 * (g2 & 1)];
               const int e = (g2 >> 1) * 8 + 2 * j + (g2 & 1);
-              const float2 d = mul_pair(fma_pair(x[0], x[1], s22, d2), pa[e]);
+              const float2 d = mul_pair(fma_pair(x[0], x[1], s22, d2[j]), pa[e]);
               out[e] = pack_bf16(d.x, d.y);
             }
           }

@@ -114,7 +114,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   volatile int* work_ring = (volatile int*)(smem + SM::MISC_OFF + 16);   // [FWD_WORK_SLOTS][unit, head]
   const WaitCtx wctx{abort_flag, a.status, (uint32_t)FCP_WAIT_NS};
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: uniform for the compiler too
 
   if (threadIdx.x == 0) {
     *abort_flag = 0;
@@ -164,18 +164,12 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   // The ring holds (unit, head | mask of the Q tiles that are not part of the item << 30).
   // returns 1 with (U, h) and the key tiles of the two Q tiles of the next item, 0 at the end of the list, -1 if the CTA is
   // aborting
-  auto take_item = [&](uint32_t& n, const int32_t*& U, int& h, int& nt0, int& nt1, bool whole_warp) -> int {
-    const uint32_t slot = n % FWD_WORK_SLOTS, par = (n / FWD_WORK_SLOTS) & 1;
-    const bool got = whole_warp ? mbar_wait_warp(BAR(B_WFULL + slot), par, wctx, 40) : mbar_wait(BAR(B_WFULL + slot), par, wctx, 40);
-    if (!got) return -1;
-    const int unit = work_ring[2 * slot];
-    h = work_ring[2 * slot + 1];
-    if (whole_warp) {
-      __syncwarp();
-      if (lane == 0) mbar_arrive(BAR(B_WEMPTY + slot));
-    } else {
-      mbar_arrive(BAR(B_WEMPTY + slot));
-    }
+  auto take_item = [&](uint32_t& n, const int32_t*& U, int& h, int& nt0, int& nt1) -> int {
+    const uint32_t slot = n % FWD_WORK_SLOTS;
+    if (!mbar_wait_warp(BAR(B_WFULL + slot), (n / FWD_WORK_SLOTS) & 1, wctx, 40)) return -1;
+    const int unit = __shfl_sync(0xffffffffu, work_ring[2 * slot], 0);
+    h = __shfl_sync(0xffffffffu, work_ring[2 * slot + 1], 0);
+    if (lane == 0) mbar_arrive(BAR(B_WEMPTY + slot));
     ++n;
     if (unit < 0) return 0;
     U = a.units + (size_t)unit * FCP_FWD_UNIT_W;
@@ -280,7 +274,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     // ------------------------------------------------------------------ UMMA issuer 1: S = Q K^T of both Q tiles
     // The two issuing threads are split by product, not by Q tile: S of the next step only waits for a free score
     // buffer, so it is never queued behind the product that consumes the probabilities of an earlier step.
-    if (lane == 0) {
+    {
       constexpr uint32_t IDESC_QK = make_idesc(128, 128, 0, 0);
       uint32_t kv_it = 0, qcnt0 = 0, qcnt1 = 0, xcnt0 = 0, xcnt1 = 0, nw = 0;
       bool ok = true;
@@ -288,24 +282,26 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       while (ok) {
         const int32_t* U;
         int h, nt0, nt1;
-        const int r = take_item(nw, U, h, nt0, nt1, false);
+        const int r = take_item(nw, U, h, nt0, nt1);
         if (r <= 0) { ok = r == 0; break; }
+        nt0 = __shfl_sync(0xffffffffu, nt0, 0);
+        nt1 = __shfl_sync(0xffffffffu, nt1, 0);
         const int n_max = max(nt0, nt1);
 #pragma unroll 1
         for (int j = 0; j < n_max && ok; ++j, kv_it += 2) {
           const uint32_t slot = kv_it % FWD_KV_SLOTS;
-          ok = mbar_wait(BAR(B_KVFULL + slot), (kv_it / FWD_KV_SLOTS) & 1, wctx, 23);
+          ok = mbar_wait_warp(BAR(B_KVFULL + slot), (kv_it / FWD_KV_SLOTS) & 1, wctx, 23);
 #pragma unroll 1
           for (int s = 0; s < 2 && ok; ++s) {
             const int nts = s ? nt1 : nt0;
             if (j >= nts) continue;
             if (j == 0) {
-              ok = mbar_wait(BAR(B_QFULL + s), (s ? qcnt1 : qcnt0) & 1, wctx, 20 + s);
+              ok = mbar_wait_warp(BAR(B_QFULL + s), (s ? qcnt1 : qcnt0) & 1, wctx, 20 + s);
               if (s) ++qcnt1; else ++qcnt0;
               if (!ok) break;
             }
             const uint32_t sb = NS == 2 ? s : 0;
-            ok = mbar_wait(BAR(B_SFREE + sb), ((sb ? xcnt1 : xcnt0) & 1) ^ 1, wctx, 24);
+            ok = mbar_wait_warp(BAR(B_SFREE + sb), ((sb ? xcnt1 : xcnt0) & 1) ^ 1, wctx, 24);
             if (!ok) break;
             if (sb) ++xcnt1; else ++xcnt0;
             tc_fence_after();
@@ -320,7 +316,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------------ UMMA issuer 2: O (+)= P V of both Q tiles
-    if (lane == 0) {
+    {
       constexpr uint32_t IDESC_PV = make_idesc(128, D, 0, 1);
       uint32_t kv_it = 1, pcnt0 = 0, pcnt1 = 0, ocnt0 = 0, ocnt1 = 0, nw = 0;
       bool ok = true;
@@ -328,23 +324,25 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       while (ok) {
         const int32_t* U;
         int h, nt0, nt1;
-        const int r = take_item(nw, U, h, nt0, nt1, false);
+        const int r = take_item(nw, U, h, nt0, nt1);
         if (r <= 0) { ok = r == 0; break; }
+        nt0 = __shfl_sync(0xffffffffu, nt0, 0);
+        nt1 = __shfl_sync(0xffffffffu, nt1, 0);
         const int n_max = max(nt0, nt1);
 #pragma unroll 1
         for (int j = 0; j < n_max && ok; ++j, kv_it += 2) {
           const uint32_t slot = kv_it % FWD_KV_SLOTS;
-          ok = mbar_wait(BAR(B_KVFULL + slot), (kv_it / FWD_KV_SLOTS) & 1, wctx, 22);
+          ok = mbar_wait_warp(BAR(B_KVFULL + slot), (kv_it / FWD_KV_SLOTS) & 1, wctx, 22);
 #pragma unroll 1
           for (int s = 0; s < 2 && ok; ++s) {
             const int nts = s ? nt1 : nt0;
             if (j >= nts) continue;
             if (j == 0) {
-              ok = mbar_wait(BAR(B_OEMPTY + s), ((s ? ocnt1 : ocnt0) & 1) ^ 1, wctx, 25);
+              ok = mbar_wait_warp(BAR(B_OEMPTY + s), ((s ? ocnt1 : ocnt0) & 1) ^ 1, wctx, 25);
               if (s) ++ocnt1; else ++ocnt0;
               if (!ok) break;
             }
-            ok = mbar_wait(BAR(B_PFULL + s), (s ? pcnt1 : pcnt0) & 1, wctx, 26 + s);
+            ok = mbar_wait_warp(BAR(B_PFULL + s), (s ? pcnt1 : pcnt0) & 1, wctx, 26 + s);
             if (s) ++pcnt1; else ++pcnt0;
             if (!ok) break;
             tc_fence_after();
@@ -377,7 +375,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     while (ok) {
       const int32_t* U;
       int h, nt0, nt1;
-      const int r = take_item(nw, U, h, nt0, nt1, true);
+      const int r = take_item(nw, U, h, nt0, nt1);
       if (r <= 0) { ok = r == 0; break; }
       const int nts = s ? nt1 : nt0;
       const int q_pos = __ldg(U + FU_Q_ROW0) + s * 128 + row;
@@ -567,7 +565,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     while (ok) {
       const int32_t* U;
       int h, nt0, nt1;
-      const int r = take_item(nw, U, h, nt0, nt1, true);
+      const int r = take_item(nw, U, h, nt0, nt1);
       if (r <= 0) { ok = r == 0; break; }
       const int hl = h - a.head_begin;
       const int q_rows = __ldg(U + FU_Q_ROWS);

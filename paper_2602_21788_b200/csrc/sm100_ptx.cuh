@@ -28,6 +28,12 @@ __device__ __forceinline__ uint32_t globaltimer_lo() {
   return t;
 }
 
+__device__ __forceinline__ float2 lds_f2(const float* p) {       // stays where it is written among the other asm statements
+  float2 x;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(x.x), "=f"(x.y) : "r"(smem_u32(p)) : "memory");
+  return x;
+}
+
 // ----------------------------------------------------------------------------- programmatic launch
 // Every kernel of the library waits (grid_wait) for the work before it, memory included, before it touches global
 // memory, so that "the grid before is complete" covers all grids before that one too.  The short kernels let the next
@@ -121,7 +127,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
   uint32_t spins = 0, t0 = 0;
 #pragma unroll 1
   while (!mbar_try_wait(bar, parity)) {
-    if ((++spins & 2047u) == 0) {
+    if (__builtin_expect((++spins & 2047u) == 0, 0)) {
       // low word of the nanosecond timer: differences are exact modulo 2^32 (4.29 s), enough for
       // the 2 s limit as long as the clock is looked at more often than that
       const uint32_t now = globaltimer_lo();
@@ -157,6 +163,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, co
   const bool ok = mbar_wait(bar, parity, ctx, where);
   return __all_sync(0xffffffffu, ok);
 }
+__device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_test(bar, parity)); }
 
 // ----------------------------------------------------------------------------- work order
 // Position of a work item in the execution order described by work groups (fcp_plan.hpp).  Items are asked for in ascending
@@ -217,17 +224,28 @@ __device__ __forceinline__ void tc_fence_after() {
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Arrive on `bar` once every MMA issued so far by this thread has completed.
+// Products and commits are issued by a whole, converged warp, of which one elected lane (always the same) sends the
+// instruction.  In code that only one lane runs the compiler cannot keep the operands in uniform registers, and the moves in
+// front of every UMMA took 55-90 clk, where one of 128 x 128 x 16 executes in 64.  One election per product: one per UMMA is
+// a quarter more code for the whole kernel, which the instruction cache pays for.  Measured with all of it, one lane -> elected: forward
+// 16 x 2048 tokens of 32/8 heads 535 -> 508 us, one sequence of 60 000, 8 heads 4980 -> 4832; backward, D = 64, 8 x 3000
+// tokens of 12/4 heads 398 -> 370; D = 128, one of 60 000 18045 -> 17460.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t x;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(x));
+  return x != 0;
+}
+
+// Arrive on `bar` once every MMA issued so far by this warp has completed.
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+  if (elect_one()) asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 // D[tmem] (+)= A[smem] * B[smem]   (bf16 in, fp32 accumulate)
 __device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                         uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
@@ -235,8 +253,7 @@ __device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t a_desc, uint64
 __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                         uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
@@ -273,14 +290,15 @@ __device__ __forceinline__ uint64_t sdesc_pack(uint32_t lo, uint32_t hi) {
 }
 
 // One 128 x N x (16*KSTEPS) product.  Fully unrolled with the descriptor offsets folded into
-// constants: a single thread issues these, and a rolled loop's dependent integer arithmetic (about
-// 85 clocks per trip) would be slower than the 64 clocks a 128x128x16 UMMA takes to execute.
+// constants: a rolled loop's dependent integer arithmetic (about 85 clocks per trip) would be slower
+// than the 64 clocks a 128x128x16 UMMA takes to execute.
 // K-major A and B tiles of [128][64]-element swizzled blocks: K step k lives in block k/4 at byte
 // offset (k%4)*32 of every row.
 // K steps [K0, K1); the first step of the product (K0 = 0) overwrites D.
 template <int K0, int K1>
 __device__ __forceinline__ void umma_loop_kk(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc) {
   const uint32_t hi = sdesc_hi(1024), alo = sdesc_lo(a_addr, 16), blo = sdesc_lo(b_addr, 16);
+  if (!elect_one()) return;
 #pragma unroll
   for (int k = K0; k < K1; ++k) {
     const uint32_t off = (uint32_t)(k >> 2) * (16384u >> 4) + (uint32_t)(k & 3) * 2u;
@@ -291,6 +309,7 @@ __device__ __forceinline__ void umma_loop_kk(uint32_t d_tmem, uint32_t a_addr, u
 // MN-major A and B (64-element blocks 16384 bytes apart): K step k is rows [16k, 16k+16) = +2048 bytes.
 __device__ __forceinline__ void umma_loop_mm(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc) {
   const uint32_t hi = sdesc_hi(1024), alo = sdesc_lo(a_addr, 16384), blo = sdesc_lo(b_addr, 16384);
+  if (!elect_one()) return;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const uint64_t ad = sdesc_pack(alo + k * 128u, hi), bd = sdesc_pack(blo + k * 128u, hi);
@@ -304,6 +323,7 @@ template <int K0, int K1>
 __device__ __forceinline__ void umma_loop_km(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc,
                                              uint32_t acc) {
   const uint32_t hi = sdesc_hi(1024), alo = sdesc_lo(a_addr, 16), blo = sdesc_lo(b_addr, 16384);
+  if (!elect_one()) return;
 #pragma unroll
   for (int k = K0; k < K1; ++k) {
     const uint32_t off = (uint32_t)(k >> 2) * (16384u >> 4) + (uint32_t)(k & 3) * 2u;
@@ -317,6 +337,7 @@ template <int K0, int K1>
 __device__ __forceinline__ void umma_loop_ts(uint32_t d_tmem, uint32_t a_tmem, bool split, uint32_t b_addr,
                                              uint32_t idesc, uint32_t acc) {
   const uint32_t hi = sdesc_hi(1024), blo = sdesc_lo(b_addr, 16384);
+  if (!elect_one()) return;
 #pragma unroll
   for (int k = K0; k < K1; ++k) {
     const uint32_t col = (split && k >= 4) ? 64u + 8u * (k - 4) : 8u * k;
