@@ -297,3 +297,17 @@ def test_span_plan_without_spans_is_the_causal_plan_and_bad_spans_are_refused():
     with pytest.raises(fcp.FcpError) as e:
         fcp.fcp_span_mask_efficiency(10, [(3, 30)])
     assert e.value.status == fcp.FCP_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("lens,degs", [
+    ([8192, 300, 8191], [31, 1, 17]),          # a batch as the strategy search hands it out: one sequence on nearly every rank
+    ([4001], [64]), ([130, 127], [64, 33]),    # the largest degree; chunks of one or two tokens
+    ([20, 9000, 5], [64, 30, 3]),              # chunks without tokens beside full ones
+])
+def test_high_degrees_bit_exact_vs_oracle(lens, degs):
+    plan = fcp.fcp_plan_blocks(lens, degs, 8, 2, 128)
+    _compare(plan, P.plan_blocks(lens, degs))
+    # rows of the fused forward and keys of the backward pass tile every sequence from its start, whatever its chunks
+    cu = np.concatenate([[0], np.cumsum(lens)])
+    assert sorted(plan.table("fused_units")[:, 0].tolist()) == [int(a) + o for a, n in zip(cu, lens) for o in range(0, n, 256)]
+    assert plan.table("bwd_units")[:, 0].tolist() == [int(a) + o for a, n in zip(cu, lens) for o in range(0, n, 128)]

@@ -89,3 +89,21 @@ def test_noalloc_arena_holds_tables_and_scratch_and_nothing_for_the_order(lens, 
 ])
 def test_q_tiles_are_items_of_their_own_where_that_is_the_shorter_launch(lens, hq, split):
     assert fcp.Plan(lens, [1] * len(lens), hq, 1, 64).info("fused_split") == split
+
+
+@pytest.mark.parametrize("lens,degs,hq,hkv,D", [
+    ([300, 4000, 129, 2000, 2000, 64], [1, 5, 1, 3, 3, 2], 8, 2, 128),
+    ([8192, 700, 700, 1], [31, 1, 2, 1], 32, 8, 128),
+    ([512] * 30, [2] * 30, 4, 4, 64),                  # equal costs throughout
+])
+def test_units_of_equal_cost_keep_the_order_of_the_list(lens, degs, hq, hkv, D):
+    plan = fcp.Plan(lens, degs, hq, hkv, D)
+    order, cost = plan.table("bwd_work"), plan.table("bwd_units")[:, 5]
+    for first, n, _, _ in plan.table("bwd_groups").tolist():
+        g = order[first:first + n].tolist()
+        assert g == sorted(g, key=lambda u: (-cost[u], u))
+    f = plan.table("fwd_units")                        # item numbers are the places in the unsorted list
+    for first, n, _, _ in plan.table("fwd_groups").tolist():
+        rows = f[first:first + n]
+        keys = [(-(r[10] + r[11]), r[13], r[0]) for r in rows.tolist()]
+        assert keys == sorted(keys)
