@@ -132,7 +132,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
     for (int i = 0; i < FWD_WORK_SLOTS; ++i) {
       mbar_init(BAR(B_WFULL + i), 1);
-      mbar_init(BAR(B_WEMPTY + i), 2 + 8 + 4);   // two issuing threads, one lane of each softmax and epilogue warp
+      mbar_init(BAR(B_WEMPTY + i), 2 + 8 + 4);   // one lane of each issuing, softmax and epilogue warp
     }
     for (int i = 0; i < FWD_KV_SLOTS; ++i) {
       mbar_init(BAR(B_KVFULL + i), 1);
@@ -158,7 +158,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   // Work items = (unit, query head), in the order of the work groups; the gi query heads of one KV head (gi = 1 when the head
   // range cuts KV-head groups) are always adjacent, so that one copy of its K/V tiles in L2 serves them all.  Items are
   // handed out dynamically: the producer thread takes item numbers from a global counter and passes (unit, head)
-  // through a small ring in shared memory to the issuing threads and the softmax and epilogue warps, which all consume
+  // through a small ring in shared memory to the issuing, the softmax and epilogue warps, which all consume
   // every item in order; -1 ends the list.
   const int gi = a.head_group;
   // The ring holds (unit, head | mask of the Q tiles that are not part of the item << 30).
@@ -272,7 +272,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ UMMA issuer 1: S = Q K^T of both Q tiles
-    // The two issuing threads are split by product, not by Q tile: S of the next step only waits for a free score
+    // The two issuing warps are split by product, not by Q tile: S of the next step only waits for a free score
     // buffer, so it is never queued behind the product that consumes the probabilities of an earlier step.
     {
       constexpr uint32_t IDESC_QK = make_idesc(128, 128, 0, 0);
