@@ -251,7 +251,9 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 
   if (warp < 4) {
     // registers per thread: control 88, math 128, drain 168 (80 / 128 / 176 spilled in the issuing thread: kernel +2 %)
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+    // (D = 64, whose math warps hold two loads: control 72, math 136)
+    if constexpr (D == 64) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    else asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
     // (warp branches outside the lane branches: behind a divergent one the compiler takes the issuer's operands for divergent)
     if (warp == 0) {
       if (lane == 0) {
@@ -428,7 +430,8 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   } else if (warp < 4 + BWD_MATH_WARPS) {
     // ------------------------------------------------------------------ math warps: C1, C2
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
+    if constexpr (D == 64) asm volatile("setmaxnreg.inc.sync.aligned.u32 136;");
+    else asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
     const int rb = warp & 3;                    // TMEM lane quarter
     const int half = (warp - 4) >> 2;           // which 64 of the 128 query columns
     const int mtid = threadIdx.x - 128;         // 0..255 among the math threads
@@ -488,29 +491,22 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         if (!ok) break;
         tc_fence_after();
         if (mtid < 128) *my_next = next_row;
-        // P^T fragments as bf16 pairs: pa = query columns [0,32) of this half, pb = [32,64); element 8 * g + 2 * j + i is
-        // the pair of row frow + 16 * g + 8 * i and query group j.  C1 and C2 run as two rolled trips of 32 columns;
-        // between the trips the pair arrays rotate (register arrays cannot be indexed by the trip), which halves the
-        // code of this loop.
-        uint32_t pa[16], pb[16] = {};
-#pragma unroll 1
-        for (int c = 0; c < 2; ++c) {
-          uint32_t sv[32];
-          tmem_ld_frag(t_s + c * 32, sv);
-          tmem_ld_frag(t_s + (16u << 16) + c * 32, sv + 16);
-          float2 l2[4];
+        // C1 and C2 are two passes of 32 of this half's columns each.  P^T fragments as bf16 pairs: element 8 * g + 2 * j + i is the pair
+        // of row frow + 16 * g + 8 * i and query group j.
+        auto load = [&](uint32_t (&x)[32], float2 (&stat2)[4], uint32_t t, const float* stat, int c) {
+          tmem_ld_frag(t + c * 32, x);
+          tmem_ld_frag(t + (16u << 16) + c * 32, x + 16);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) l2[j] = lds_f2(s_lse + c * 32 + 8 * j + fcol);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) pa[j] = pb[j];
-          tc_wait_ld();
+          for (int j = 0; j < 4; ++j) stat2[j] = lds_f2(stat + c * 32 + 8 * j + fcol);
+        };
+        auto probs = [&](const uint32_t (&x)[32], const float2 (&l2)[4], uint32_t (&p)[16], int c) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
 #pragma unroll
             for (int g2 = 0; g2 < 4; ++g2) {               // row frow + 8 * g2
-              const uint32_t* x = &sv[(g2 >> 1) * 16 + 4 * j + 2 * (g2 & 1)];
-              const float2 e = fma_pair(x[0], x[1], c22, l2[j]);
-              pb[(g2 >> 1) * 8 + 2 * j + (g2 & 1)] = pack_bf16(ex2(e.x), ex2(e.y));
+              const uint32_t* v = &x[(g2 >> 1) * 16 + 4 * j + 2 * (g2 & 1)];
+              const float2 e = fma_pair(v[0], v[1], c22, l2[j]);
+              p[(g2 >> 1) * 8 + 2 * j + (g2 & 1)] = pack_bf16(ex2(e.x), ex2(e.y));
             }
           }
           if (need_mask) {
@@ -526,11 +522,58 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               const uint32_t keep = bit_range(lo, max(0, hi - lo)) >> fcol;
               const uint32_t even = (keep & 0x01010101u) * 0xffu, odd = ((keep >> 1) & 0x01010101u) * 0xffu;
 #pragma unroll
-              for (int j = 0; j < 4; ++j) pb[(g2 >> 1) * 8 + 2 * j + (g2 & 1)] &= __byte_perm(even, odd, 0x4400 + 0x1111 * j);
+              for (int j = 0; j < 4; ++j) p[(g2 >> 1) * 8 + 2 * j + (g2 & 1)] &= __byte_perm(even, odd, 0x4400 + 0x1111 * j);
             }
           }
-          tmem_st_frag(t_s + c * 16, pb);            // over this warp's own, already loaded, columns
-          tmem_st_frag(t_s + (16u << 16) + c * 16, pb + 8);
+          tmem_st_frag(t_s + c * 16, p);             // over this warp's own, already loaded, columns
+          tmem_st_frag(t_s + (16u << 16) + c * 16, p + 8);
+        };
+        auto grads = [&](const uint32_t (&x)[32], const float2 (&d2)[4], const uint32_t (&p)[16], int c) {
+          uint32_t out[16];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+#pragma unroll
+            for (int g2 = 0; g2 < 4; ++g2) {
+              const uint32_t* v = &x[(g2 >> 1) * 16 + 4 * j + 2 * (g2 & 1)];
+              const int e = (g2 >> 1) * 8 + 2 * j + (g2 & 1);
+              const float2 d = mul_pair(fma_pair(v[0], v[1], s22, d2[j]), p[e]);
+              out[e] = pack_bf16(d.x, d.y);
+            }
+          }
+          // 32 x 32 values -> shared memory, keys x queries with queries contiguous (the K-major A operand of the dK
+          // product and the MN-major A operand of the dQ product), 128-byte swizzle: 16-byte chunk ^ (row & 7)
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {                    // rows + 16 * (m / 2), query groups 2 * (m % 2) and the next
+            const int cc = c * 4 + 2 * (m & 1) + mch;
+            stmatrix_x4(ds_row + (m >> 1) * 2048 + ((cc ^ (lane & 7)) << 4), &out[(m >> 1) * 8 + 4 * (m & 1)]);
+          }
+        };
+        // D = 128: rolled, the pair arrays rotate between the passes (register arrays cannot be indexed by the pass), which halves
+        // the code of this loop.  D = 64, where the products are half as long and the clock is not held down by the power: the
+        // second pass is loaded while the first is worked on, 8 x 3000 tokens of 12/4 heads 340 -> 332 us, 20 000 tokens 1670 -> 1615;
+        // at D = 128 that way 64K tokens of 32/8 heads 12.24 -> 12.37 ms.
+        constexpr bool AHEAD = D == 64;
+        uint32_t pa[16], pb[16] = {};
+        if constexpr (AHEAD) {
+          uint32_t x0[32], x1[32];
+          float2 l0[4], l1[4];
+          load(x0, l0, t_s, s_lse, 0);
+          tc_wait_ld();
+          load(x1, l1, t_s, s_lse, 1);
+          probs(x0, l0, pa, 0);
+          tc_wait_ld();
+          probs(x1, l1, pb, 1);
+        } else {
+#pragma unroll 1
+          for (int c = 0; c < 2; ++c) {
+            uint32_t x[32];
+            float2 l2[4];
+            load(x, l2, t_s, s_lse, c);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) pa[j] = pb[j];
+            tc_wait_ld();
+            probs(x, l2, pb, c);
+          }
         }
         tc_wait_st();
         tc_fence_before();
@@ -541,33 +584,25 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         if (!ok) break;
         tc_fence_after();
         if (mtid >= 128) *my_next = next_row;
-#pragma unroll 1
-        for (int c = 0; c < 2; ++c) {
-          uint32_t dv_[32], out[16];
-          tmem_ld_frag(t_dp + c * 32, dv_);
-          tmem_ld_frag(t_dp + (16u << 16) + c * 32, dv_ + 16);
-          float2 d2[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) d2[j] = lds_f2(s_delta + c * 32 + 8 * j + fcol);
+        if constexpr (AHEAD) {
+          uint32_t x0[32], x1[32];
+          float2 d0[4], d1[4];
+          load(x0, d0, t_dp, s_delta, 0);
           tc_wait_ld();
+          load(x1, d1, t_dp, s_delta, 1);
+          grads(x0, d0, pa, 0);
+          tc_wait_ld();
+          grads(x1, d1, pb, 1);
+        } else {
+#pragma unroll 1
+          for (int c = 0; c < 2; ++c) {
+            uint32_t x[32];
+            float2 d2[4];
+            load(x, d2, t_dp, s_delta, c);
+            tc_wait_ld();
+            grads(x, d2, pa, c);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-#pragma unroll
-            for (int g2 = 0; g2 < 4; ++g2) {
-              const uint32_t* x = &dv_[(g2 >> 1) * 16 + 4 * j + 2 * (g2 & 1)];
-              const int e = (g2 >> 1) * 8 + 2 * j + (g2 & 1);
-              const float2 d = mul_pair(fma_pair(x[0], x[1], s22, d2[j]), pa[e]);
-              out[e] = pack_bf16(d.x, d.y);
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < 16; ++j) pa[j] = pb[j];
-          // 32 x 32 values -> shared memory, keys x queries with queries contiguous (the K-major A operand of the dK
-          // product and the MN-major A operand of the dQ product), 128-byte swizzle: 16-byte chunk ^ (row & 7)
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {                    // rows + 16 * (m / 2), query groups 2 * (m % 2) and the next
-            const int cc = c * 4 + 2 * (m & 1) + mch;
-            stmatrix_x4(ds_row + (m >> 1) * 2048 + ((cc ^ (lane & 7)) << 4), &out[(m >> 1) * 8 + 4 * (m & 1)]);
+            for (int j = 0; j < 16; ++j) pa[j] = pb[j];
           }
         }
         fence_proxy_async_smem();
