@@ -399,8 +399,11 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
   std::vector<Pair> pairs;
   {
     size_t n_pairs = 0;
-    for (int b = 0; b < B; ++b) n_pairs += (size_t)cp_degrees[b] * (2 * cp_degrees[b] + 1);
-    pairs.reserve(n_pairs);                      // fewer where chunks are empty
+    for (int b = 0; b < B; ++b) {                // a short sequence has one token in each of L chunks, the others are empty
+      const size_t n = std::min(2 * cp_degrees[b], seqlens[b]);
+      n_pairs += n * (n + 1) / 2;
+    }
+    pairs.reserve(n_pairs);
   }
   for (int b = 0; b < B; ++b) {
     const int64_t L = seqlens[b];

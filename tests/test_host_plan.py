@@ -4,6 +4,8 @@ import ctypes
 import math
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -311,3 +313,30 @@ def test_high_degrees_bit_exact_vs_oracle(lens, degs):
     cu = np.concatenate([[0], np.cumsum(lens)])
     assert sorted(plan.table("fused_units")[:, 0].tolist()) == [int(a) + o for a, n in zip(cu, lens) for o in range(0, n, 256)]
     assert plan.table("bwd_units")[:, 0].tolist() == [int(a) + o for a, n in zip(cu, lens) for o in range(0, n, 128)]
+
+
+_IN_BOUNDED_SPACE = """
+import resource, sys
+from paper_2602_21788_b200 import fcp
+fcp.lib()
+mapped = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (mapped + int(sys.argv[1]), resource.RLIM_INFINITY))
+n, length, degree = (int(x) for x in sys.argv[2:5])
+plan = fcp.Plan([length] * n, [degree] * n, 1, 1, 64)
+print(plan.info("n_pairs"), plan.info("n_fused_units"), plan.info("n_bwd_units"))
+"""
+
+
+def _plan_in_bounded_space(space, n, length, degree):
+    """Pairs, fused units and backward units of n equal sequences, planned by a process of its own that may map `space` bytes more than
+    the loaded library has."""
+    r = subprocess.run([sys.executable, "-c", _IN_BOUNDED_SPACE, str(space), str(n), str(length), str(degree)], cwd=ROOT,
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, (r.returncode, r.stderr[-500:])
+    return [int(x) for x in r.stdout.split()]
+
+
+@pytest.mark.parametrize("n,length,pairs", [(12000, 1, 1), (8000, 5, 15)])
+def test_short_sequences_at_high_degree_take_memory_for_the_pairs_they_have(n, length, pairs):
+    # d (2d + 1) rows of 24 bytes per sequence would be 1.6 to 2.4 GB
+    assert _plan_in_bounded_space(1200 << 20, n, length, 64) == [n * pairs, n, n]
