@@ -204,9 +204,8 @@ inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 constexpr int64_t kOrderBytes = int64_t(64) << 20;
 constexpr int64_t kOrderSms = FCP_PLAN_SMS;
 
-// Stable sort of indexes by an ascending key of [0, n_keys), in two passes over the list.  With this, the pairs put into order
-// as they are made, and their ranges read from a matrix instead of from sorted lists, the plan of a 16K-token batch with one
-// sequence of 8192 at degree 31 (1953 pairs, 1441 items) takes 202 us instead of 380.
+// Stable sort of indexes by an ascending key of [0, n_keys), in two passes over the list.  The plan of a 16K-token batch of ten
+// sequences, one of 8192 at degree 31 (1980 pairs, 1475 items, 1501 forward units), takes 145-160 us with it, 165-190 with std::stable_sort.
 template <typename Key>
 void sort_by_key(std::vector<int32_t>& order, size_t n_keys, Key key) {
   std::vector<int32_t> at(n_keys + 1, 0), out(order.size());
@@ -417,10 +416,10 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
       if (nonempty(qc) && nonempty(kc)) pairs.push_back(Pair{b, r, s, qc, kc, qc == kc ? 1 : 0});
     };
     const int last = 2 * d - 1;
-    for (int r = 0; r < d; ++r)
-      for (int s = 0; s < d; ++s) {
-        const int j = ((r - s) % d + d) % d;   // rank whose K/V visits at this ring step
-        const size_t first = pairs.size();
+    for (int r = 0; r < d; ++r) {
+      if (!nonempty(r) && !nonempty(last - r)) continue;   // all but L ranks of a sequence of L < d tokens
+      for (int s = 0; s < d; ++s) {              // the pairs of a step ascend as they are written here: r, j < d <= last - r, last - j
+        const int j = r >= s ? r - s : r - s + d;   // rank whose K/V visits at this ring step
         if (s == 0) {
           add(r, s, r, r);
           add(r, s, last - r, r);
@@ -432,8 +431,8 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
           add(r, s, last - r, j);
           add(r, s, last - r, last - j);
         }
-        std::sort(pairs.begin() + first, pairs.end());   // rank and step ascend already
       }
+    }
   }
   p->pairs.resize(pairs.size() * 6);
   for (size_t i = 0; i < pairs.size(); ++i) {
@@ -577,55 +576,29 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
   p->fwd_split = split_units(p->fwd_units, p->fwd_groups, params->hkv, params->hq / params->hkv, FCP_PLAN_SMS);
 
   // Fused forward (merge on the fly): all items of a Q chunk run on one CTA, so the KV ranges of the
-  // chunk's block pairs are swept in one online softmax and no partial leaves the SM.  The ranges of
-  // a Q chunk are its pairs in kv_chunk order with adjacent FULL ranges joined.  In a causal plan
-  // that is the prefix [sequence start, chunk start) plus the DIAG range of the chunk itself, which
-  // one DIAG range starting at the sequence start describes exactly (every key before the chunk
-  // precedes every row of it); consecutive Q chunks of that form are joined into one run of rows,
-  // tiled in units of two Q tiles from the start of the run, so no tile is cut at a chunk edge.
-  struct Range { int32_t b, e, diag; };
-  // Kind of the pair (q chunk, kv chunk) of a sequence, -1: the plan has none.  One byte per cell, so that the pairs of a chunk
-  // come in the order of the other without a list and a sort per chunk.
-  std::vector<size_t> cell0(B + 1, 0);
-  for (int b = 0; b < B; ++b) cell0[b + 1] = cell0[b] + (size_t)4 * cp_degrees[b] * cp_degrees[b];
-  std::vector<int8_t> cells(cell0[B], -1);
-  for (const Pair& x : pairs) cells[cell0[x.seq] + (size_t)x.qc * 2 * cp_degrees[x.seq] + x.kc] = (int8_t)x.kind;
-  auto kind_of = [&](int b, int qc, int kc) -> int { return cells[cell0[b] + (size_t)qc * 2 * cp_degrees[b] + kc]; };
-  std::vector<std::vector<Range>> q_cover(n_chunks_total);   // per Q chunk: joined KV ranges of its pairs
-  {
-    for (int b = 0; b < B; ++b) {
-      const int32_t* cbp = &p->chunk_bounds[p->chunk_offset[b]];
-      const int nc = 2 * cp_degrees[b];
-      for (int c = 0; c < nc; ++c) {
-        auto& out_r = q_cover[chunk_index0[b] + c];
-        for (int kc = 0; kc < nc; ++kc) {
-          const int kind = kind_of(b, c, kc);
-          if (kind < 0) continue;
-          const Range r{cbp[kc], cbp[kc + 1], kind};
-          if (!out_r.empty() && !out_r.back().diag && !r.diag && out_r.back().e == r.b) out_r.back().e = r.e;
-          else out_r.push_back(r);
-        }
-      }
-    }
-  }
+  // chunk's block pairs are swept in one online softmax and no partial leaves the SM.  The pairs of a
+  // Q chunk are every chunk with tokens before it and the DIAG pair of the chunk itself; every key
+  // before the chunk precedes every row of it, so one DIAG range from the sequence start describes
+  // them exactly, and the chunks of a sequence are one run of rows, tiled in units of two Q tiles
+  // from its start: no tile is cut at a chunk edge.  Inside a span a row sees keys up to the span's end.
   {
     std::vector<FU> gus;
     std::vector<int32_t> gu_seq;
-    // rows [r0, r1) of the sequence [t0, t1) attend to [t0, row] (and, inside a span, on to the span's end)
-    auto emit_run = [&](int32_t b, int32_t t0, int32_t t1, int32_t r0, int32_t r1) {
-      for (int32_t off = 0; off < r1 - r0; off += FCP_FWD_UNIT_ROWS) {
+    for (int b = 0; b < B; ++b) {
+      const int32_t t0 = p->cu_seqlens[b], t1 = p->cu_seqlens[b + 1];
+      for (int32_t row0 = t0; row0 < t1; row0 += FCP_FWD_UNIT_ROWS) {
         FU u{};
-        const int32_t rows = std::min<int32_t>(FCP_FWD_UNIT_ROWS, r1 - r0 - off);
-        u.f[FU_Q_ROW0] = r0 + off;
+        const int32_t rows = std::min<int32_t>(FCP_FWD_UNIT_ROWS, t1 - row0);
+        u.f[FU_Q_ROW0] = row0;
         u.f[FU_Q_ROWS] = rows;
         u.f[FU_N_RANGES] = 1;
-        u.f[FU_KV0_BEGIN] = t0; u.f[FU_KV0_END] = has_spans ? t1 : r1; u.f[FU_KV0_DIAG] = 1;
+        u.f[FU_KV0_BEGIN] = t0; u.f[FU_KV0_END] = t1; u.f[FU_KV0_DIAG] = 1;
         for (int s = 0; s < 2; ++s) {
           const int32_t rs = std::min<int32_t>(FCP_TILE, rows - s * FCP_TILE);
+          if (rs <= 0) continue;
           // key tiles up to the last key the stage's last row sees (row limits do not decrease along a sequence)
-          const int32_t last_row = r0 + off + s * FCP_TILE + rs - 1;
-          const int32_t key_end = rs > 0 ? (has_spans ? p->row_limit[last_row] : last_row + 1) : t0;
-          u.f[FU_NT_STAGE0 + s] = rs > 0 ? ceil_div(key_end - t0, FCP_TILE) : 0;
+          const int32_t last_row = row0 + s * FCP_TILE + rs - 1;
+          u.f[FU_NT_STAGE0 + s] = ceil_div((has_spans ? p->row_limit[last_row] : last_row + 1) - t0, FCP_TILE);
         }
         u.f[FU_NT_RANGE0] = 0x7fffffff;
         u.f[FU_ITEM] = -1;
@@ -633,142 +606,44 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
         gus.push_back(u);
         gu_seq.push_back(b);
       }
-    };
-    for (int b = 0; b < B; ++b) {
-      const int32_t* cbp = &p->chunk_bounds[p->chunk_offset[b]];
-      const int32_t t0 = cbp[0], t1 = cbp[2 * cp_degrees[b]];
-      int32_t run0 = -1, run1 = -1;
-      for (int c = 0; c < 2 * cp_degrees[b]; ++c) {
-        const int32_t q0 = cbp[c], q1 = cbp[c + 1];
-        if (q1 == q0) continue;
-        const auto& rg = q_cover[chunk_index0[b] + c];
-        const bool prefix = (rg.size() == 1 && rg[0].diag && rg[0].b == q0 && q0 == t0) ||
-                            (rg.size() == 2 && !rg[0].diag && rg[0].b == t0 && rg[0].e == q0 && rg[1].diag && rg[1].b == q0);
-        if (prefix) {
-          if (run0 < 0) run0 = q0;
-          else if (run1 != q0) { emit_run(b, t0, t1, run0, run1); run0 = q0; }
-          run1 = q1;
-          continue;
-        }
-        if (run0 >= 0) { emit_run(b, t0, t1, run0, run1); run0 = -1; }
-        // a chunk whose ranges are not a causal prefix keeps them as they are (at most two per unit)
-        if (rg.empty() || rg.size() > 2 || has_spans) {
-          delete p;
-          fcp_set_error("fcp_plan_blocks: Q chunk %d of sequence %d has %d disjoint KV ranges", c, b, (int)rg.size());
-          return FCP_ERR_UNSUPPORTED;
-        }
-        const int lastr = (int)rg.size() - 1;
-        const int nt_first = rg.size() == 2 ? ceil_div(rg[0].e - rg[0].b, FCP_TILE) : 0;
-        for (int32_t off = 0; off < q1 - q0; off += FCP_FWD_UNIT_ROWS) {
-          FU u{};
-          const int32_t rows = std::min<int32_t>(FCP_FWD_UNIT_ROWS, q1 - q0 - off);
-          u.f[FU_Q_ROW0] = q0 + off;
-          u.f[FU_Q_ROWS] = rows;
-          u.f[FU_N_RANGES] = (int32_t)rg.size();
-          u.f[FU_KV0_BEGIN] = rg[0].b; u.f[FU_KV0_END] = rg[0].e; u.f[FU_KV0_DIAG] = rg[0].diag;
-          if (rg.size() == 2) { u.f[FU_KV1_BEGIN] = rg[1].b; u.f[FU_KV1_END] = rg[1].e; u.f[FU_KV1_DIAG] = rg[1].diag; }
-          for (int s = 0; s < 2; ++s) {
-            const int32_t rs = std::min<int32_t>(FCP_TILE, rows - s * FCP_TILE);
-            int nt = 0;
-            if (rs > 0)
-              nt = nt_first + (rg[lastr].diag ? ceil_div((int64_t)(q0 + off - rg[lastr].b) + s * FCP_TILE + rs, FCP_TILE)
-                                              : ceil_div(rg[lastr].e - rg[lastr].b, FCP_TILE));
-            u.f[FU_NT_STAGE0 + s] = nt;
-          }
-          u.f[FU_NT_RANGE0] = rg.size() == 2 ? nt_first : 0x7fffffff;
-          u.f[FU_ITEM] = -1;
-          u.f[FU_SINGLE_SLOT] = 1;
-          gus.push_back(u);
-          gu_seq.push_back(b);
-        }
-      }
-      if (run0 >= 0) emit_run(b, t0, t1, run0, run1);
     }
     emit_fwd(gus, gu_seq, p->fused_units, p->fused_groups);
     p->fused_split = split_units(p->fused_units, p->fused_groups, params->hkv, params->hq / params->hkv, FCP_PLAN_SMS);
   }
 
   // Backward: one unit per 128-key tile; it visits the Q rows of all block pairs whose kv_chunk holds
-  // its keys (q_chunk >= kv_chunk), the DIAG pair from its own tile on.  The Q ranges of a KV chunk
-  // are its pairs in q_chunk order with adjacent ranges joined (a DIAG range followed by the FULL
-  // ranges of the later chunks is one DIAG range up to their end).  Every KV chunk of a sequence ends
-  // up with the single range [chunk start, sequence end) DIAG, so the key tiles are cut from the start
-  // of the sequence instead of from each chunk start (a key tile may then span two KV chunks; the
-  // causal mask only depends on token positions): neither key tiles nor query tiles are cut at chunk
-  // edges, and a query tile has the same rows for every key tile.
-  struct BU { int32_t f[FCP_BWD_UNIT_W]; };
-  std::vector<BU> bus;
-  {
-    for (int b = 0; b < B; ++b) {
-      const int32_t* cbp = &p->chunk_bounds[p->chunk_offset[b]];
-      const int nc = 2 * cp_degrees[b];
-      const int32_t t0 = cbp[0], t1 = cbp[nc];
-      std::vector<std::vector<Range>> kv_cover(nc);
-      bool causal_seq = true;
-      for (int c = 0; c < nc; ++c) {
-        auto& out_r = kv_cover[c];
-        for (int qc = 0; qc < nc; ++qc) {
-          const int kind = kind_of(b, qc, c);
-          if (kind < 0) continue;
-          const Range r{cbp[qc], cbp[qc + 1], kind};
-          if (!out_r.empty() && !r.diag && out_r.back().e == r.b) out_r.back().e = r.e;   // keeps the first range's kind
-          else out_r.push_back(r);
-        }
-        if (cbp[c + 1] > cbp[c])
-          causal_seq = causal_seq && out_r.size() == 1 && out_r[0].diag && out_r[0].b == cbp[c] && out_r[0].e == t1;
-      }
-      // `spans`: the tiles are cut from the sequence start and a DIAG range starts where the first key of the
-      // tile is first seen (earlier than the tile's own position when that key lies inside a span)
-      auto emit_tiles = [&](int32_t k0, int32_t k1, int32_t first, const std::vector<Range>& rg, bool spans_on) {
-        for (int32_t off = 0, t = 0; off < k1 - k0; off += FCP_TILE, ++t) {
-          BU u{};
-          const int32_t rows = std::min<int32_t>(FCP_TILE, k1 - k0 - off);
-          u.f[BU_KV_ROW0] = k0 + off;
-          u.f[BU_KV_ROWS] = rows;
-          u.f[BU_FIRST_QRANGE] = first;
-          u.f[BU_N_QRANGES] = (int32_t)rg.size();
-          // Q tiles of a DIAG range run from T_FIRST on; those before T_MASK_END hold (query, key) pairs the
-          // mask removes.  Causal: the tile on the diagonal only.
-          int32_t t_first = t, t_mask_end = t + 1;
-          if (spans_on) {
-            t_first = (p->first_query[k0 + off] - k0) / FCP_TILE;
-            t_mask_end = ceil_div(p->first_query[k0 + off + rows - 1] - k0, FCP_TILE);
-          }
-          u.f[BU_T_FIRST] = t_first;
-          u.f[BU_T_MASK_END] = t_mask_end;
-          int cost = 0;
-          for (const Range& r : rg) {
-            const int nt = ceil_div(r.e - r.b, FCP_TILE);
-            cost += r.diag ? std::max(0, nt - t_first) : nt;
-          }
-          u.f[BU_COST] = cost;
-          u.f[BU_SEQ] = b;
-          bus.push_back(u);
-        }
-      };
-      auto push_ranges = [&](const std::vector<Range>& rg) {
-        const int32_t first = (int32_t)(p->bwd_qranges.size() / FCP_BWD_QRANGE_W);
-        for (const Range& r : rg) {
-          const int32_t rowq[4] = {r.b, r.e, r.diag, 0};
-          p->bwd_qranges.insert(p->bwd_qranges.end(), rowq, rowq + 4);
-        }
-        return first;
-      };
-      if (!causal_seq) {                         // the dQ accumulator is laid out by Q tiles cut from the sequence start
-        delete p;
-        fcp_set_error("fcp_plan_blocks: the block pairs of sequence %d are not the causal set", b);
-        return FCP_ERR_UNSUPPORTED;
-      }
-      const std::vector<Range> whole{Range{t0, t1, 1}};
-      emit_tiles(t0, t1, push_ranges(whole), whole, has_spans);
-    }
-  }
-  for (const BU& u : bus) p->bwd_units.insert(p->bwd_units.end(), u.f, u.f + FCP_BWD_UNIT_W);
+  // its keys, that is of its own chunk (DIAG) and of every later one: one DIAG range from the chunk
+  // start to the sequence end.  So the key tiles are cut from the start of the sequence instead of
+  // from each chunk start (a key tile may then span two KV chunks; the causal mask only depends on
+  // token positions): neither key tiles nor query tiles are cut at chunk edges, and a query tile has
+  // the same rows for every key tile, by which the dQ accumulator is laid out.
   {
     std::vector<int32_t> seq, cost;
-    for (const BU& u : bus) {
-      seq.push_back(u.f[BU_SEQ]);
-      cost.push_back(u.f[BU_COST]);
+    for (int b = 0; b < B; ++b) {
+      const int32_t t0 = p->cu_seqlens[b], t1 = p->cu_seqlens[b + 1];
+      const int32_t rowq[FCP_BWD_QRANGE_W] = {t0, t1, 1, 0};
+      p->bwd_qranges.insert(p->bwd_qranges.end(), rowq, rowq + FCP_BWD_QRANGE_W);
+      for (int32_t k0 = t0, t = 0; k0 < t1; k0 += FCP_TILE, ++t) {
+        const int32_t rows = std::min<int32_t>(FCP_TILE, t1 - k0);
+        // Q tiles run from T_FIRST on; those before T_MASK_END hold (query, key) pairs the mask removes.  Causal: the tile on
+        // the diagonal only.  With spans a tile is first seen where its first key is (earlier than the tile's own position
+        // when that key lies inside a span).
+        const int32_t t_first = has_spans ? (p->first_query[k0] - t0) / FCP_TILE : t;
+        const int32_t t_mask_end = has_spans ? ceil_div(p->first_query[k0 + rows - 1] - t0, FCP_TILE) : t + 1;
+        const int32_t tiles = ceil_div(t1 - t0, FCP_TILE) - t_first;
+        int32_t u[FCP_BWD_UNIT_W] = {};
+        u[BU_KV_ROW0] = k0;
+        u[BU_KV_ROWS] = rows;
+        u[BU_FIRST_QRANGE] = b;
+        u[BU_N_QRANGES] = 1;
+        u[BU_T_FIRST] = t_first;
+        u[BU_COST] = tiles;
+        u[BU_SEQ] = b;
+        u[BU_T_MASK_END] = t_mask_end;
+        p->bwd_units.insert(p->bwd_units.end(), u, u + FCP_BWD_UNIT_W);
+        seq.push_back(b);
+        cost.push_back(tiles);
+      }
     }
     order_units(seq, cost, seqlens, B, params->hkv, dq_token_bytes, p->bwd_work, p->bwd_groups);
   }

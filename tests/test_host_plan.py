@@ -6,6 +6,7 @@ import os
 import re
 import subprocess
 import sys
+import time
 
 import numpy as np
 import pytest
@@ -340,3 +341,25 @@ def _plan_in_bounded_space(space, n, length, degree):
 def test_short_sequences_at_high_degree_take_memory_for_the_pairs_they_have(n, length, pairs):
     # d (2d + 1) rows of 24 bytes per sequence would be 1.6 to 2.4 GB
     assert _plan_in_bounded_space(1200 << 20, n, length, 64) == [n * pairs, n, n]
+
+
+def test_chunks_without_tokens_cost_no_more_than_their_bounds():
+    # 655 MB would be a byte per (q chunk, kv chunk) of every sequence; the chunk bounds and slot offsets are 41 MB
+    assert _plan_in_bounded_space(500 << 20, 40000, 1, 64) == [40000, 40000, 40000]
+
+    def seconds(degree):
+        best = math.inf
+        for _ in range(7):
+            t = time.process_time()
+            fcp.Plan([1] * 2000, [degree] * 2000, 1, 1, 64)
+            best = min(best, time.process_time() - t)
+        return best
+    # degree 64 has 64 times the chunk bounds of degree 1 and the same pairs: about 10 times the time (a matrix of chunks: 120 and more)
+    assert seconds(64) < 64 * seconds(1)
+
+
+def test_short_sequences_at_high_degree_bit_exact_vs_oracle():
+    rng = np.random.default_rng(9)
+    lens, degs = rng.integers(1, 140, 60).tolist(), rng.integers(1, 65, 60).tolist()
+    plan = fcp.fcp_plan_blocks(lens, degs, 4, 2, 64)
+    _compare(plan, P.plan_blocks(lens, degs))
