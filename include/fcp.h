@@ -47,6 +47,7 @@ extern "C" {
 #define FCP_ERR_CUDA          (-5)   /* a CUDA runtime/driver call failed, or no usable device        */
 #define FCP_ERR_TIMEOUT       (-6)   /* a bounded device-side wait expired (reported by fcp_last_device_status) */
 #define FCP_ERR_NOT_UPLOADED  (-7)   /* compute call on a plan without a device copy                  */
+#define FCP_ERR_NO_MEMORY     (-8)   /* planner: the host's memory does not suffice for the batch     */
 
 #define FCP_MAX_DEGREE 64            /* largest CP degree of one sequence                             */
 
@@ -78,7 +79,8 @@ typedef struct fcp_cost_coeffs {
  *   out: group_of[B] (group index of each sequence, groups in creation order), cp_degree[B]
  *        (degree of the sequence's group), *n_groups, *makespan = DP[K'][N]; any may be NULL.
  * Errors: FCP_ERR_INVALID_ARG (NULL inputs, B <= 0, N <= 0, E <= M_ms, non-positive length or
- * M_token), FCP_ERR_INFEASIBLE (sum of d_min > N), FCP_ERR_UNSUPPORTED (N > FCP_MAX_DEGREE).
+ * M_token), FCP_ERR_INFEASIBLE (sum of d_min > N), FCP_ERR_UNSUPPORTED (N > FCP_MAX_DEGREE),
+ * FCP_ERR_NO_MEMORY.
  */
 int fcp_plan_strategy(const int32_t* seqlens, int32_t B, int32_t N, double E, double M_token,
                       double M_ms, const fcp_cost_coeffs* coeffs, int32_t* group_of,
@@ -93,7 +95,7 @@ int fcp_plan_strategy(const int32_t* seqlens, int32_t B, int32_t N, double E, do
  *   in : seqlens[B], cp_degrees[B] (host), params
  *   out: *plan (release with fcp_plan_destroy)
  * Errors: INVALID_ARG (NULL, B <= 0, length <= 0, degree <= 0, T or R >= 2^31),
- * UNSUPPORTED (head_dim, head ratio, degree > FCP_MAX_DEGREE).
+ * UNSUPPORTED (head_dim, head ratio, degree > FCP_MAX_DEGREE), NO_MEMORY.
  */
 int fcp_plan_blocks(const int32_t* seqlens, const int32_t* cp_degrees, int32_t B,
                     const fcp_params* params, fcp_plan** plan);

@@ -7,6 +7,8 @@
 #include <cstring>
 #include <functional>
 #include <limits>
+#include <memory>
+#include <new>
 #include <numeric>
 #include <vector>
 
@@ -35,9 +37,18 @@ extern "C" const char* fcp_status_string(int status) {
     case FCP_ERR_CUDA: return "FCP_ERR_CUDA";
     case FCP_ERR_TIMEOUT: return "FCP_ERR_TIMEOUT";
     case FCP_ERR_NOT_UPLOADED: return "FCP_ERR_NOT_UPLOADED";
+    case FCP_ERR_NO_MEMORY: return "FCP_ERR_NO_MEMORY";
     default: return "FCP_ERR_UNKNOWN";
   }
 }
+
+namespace {
+// The two planners allocate by the size of the batch; no exception may leave a C entry point.
+int no_memory(const char* call) {
+  fcp_set_error("%s: the host's memory does not suffice for this batch", call);
+  return FCP_ERR_NO_MEMORY;
+}
+}  // namespace
 
 // ---------------------------------------------------------------------------------------------
 // Strategy planner
@@ -63,7 +74,7 @@ double group_time(const GroupSums& g, int d, const fcp_cost_coeffs& c) {
 extern "C" int fcp_plan_strategy(const int32_t* seqlens, int32_t B, int32_t N, double E,
                                  double M_token, double M_ms, const fcp_cost_coeffs* coeffs,
                                  int32_t* group_of, int32_t* cp_degree, int32_t* n_groups,
-                                 double* makespan) {
+                                 double* makespan) try {
   if (!seqlens || !coeffs || B <= 0 || N <= 0 || !(E > M_ms) || !(M_token > 0.0) || !(coeffs->v > 0.0)) {
     fcp_set_error("fcp_plan_strategy: invalid argument");
     return FCP_ERR_INVALID_ARG;
@@ -169,6 +180,8 @@ extern "C" int fcp_plan_strategy(const int32_t* seqlens, int32_t B, int32_t N, d
   if (n_groups) *n_groups = K;
   if (makespan) *makespan = best_makespan;
   return FCP_OK;
+} catch (const std::bad_alloc&) {
+  return no_memory("fcp_plan_strategy");
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -316,7 +329,7 @@ extern "C" int fcp_plan_blocks(const int32_t* seqlens, const int32_t* cp_degrees
 
 extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_degrees, int32_t B,
                                      const int32_t* span_offset, const int32_t* spans,
-                                     const fcp_params* params, fcp_plan** out) {
+                                     const fcp_params* params, fcp_plan** out) try {
   if (!seqlens || !cp_degrees || !params || !out || B <= 0 || (span_offset && !spans && span_offset[B] > 0)) {
     fcp_set_error("fcp_plan_blocks: invalid argument");
     return FCP_ERR_INVALID_ARG;
@@ -347,7 +360,8 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
     return FCP_ERR_INVALID_ARG;
   }
 
-  fcp_plan* p = new fcp_plan();
+  std::unique_ptr<fcp_plan> owner(new fcp_plan());
+  fcp_plan* const p = owner.get();
   p->params = *params;
   if (!(p->params.scale > 0.f)) p->params.scale = 1.0f / std::sqrt((float)params->head_dim);
   p->B = B;
@@ -371,14 +385,12 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
     for (int b = 0; b < B; ++b) {
       int32_t prev_end = 0;
       if (span_offset[b + 1] < span_offset[b]) {
-        delete p;
         fcp_set_error("fcp_plan_blocks_spans: span_offset decreases at sequence %d", b);
         return FCP_ERR_INVALID_ARG;
       }
       for (int32_t i = span_offset[b]; i < span_offset[b + 1]; ++i) {
         const int32_t a = spans[2 * i], e = spans[2 * i + 1];
         if (a < prev_end || e <= a || e > seqlens[b]) {
-          delete p;
           fcp_set_error("fcp_plan_blocks_spans: span [%d, %d) of sequence %d (length %d) is empty, out of range, "
                         "unsorted or overlaps the one before", a, e, b, seqlens[b]);
           return FCP_ERR_INVALID_ARG;
@@ -491,7 +503,6 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
     chunk_items[chunk_index0[x.seq] + x.qc].push_back({x.step, item});
     row += len;
     if (row >= (int64_t(1) << 31) - 2 * FCP_FWD_UNIT_ROWS) {
-      delete p;
       fcp_set_error("fcp_plan_blocks: partial rows exceed the 2^31 limit");
       return FCP_ERR_INVALID_ARG;
     }
@@ -666,8 +677,10 @@ extern "C" int fcp_plan_blocks_spans(const int32_t* seqlens, const int32_t* cp_d
     }
     if (pass == 0) p->n_merge_multi = (int32_t)(p->merge_units.size() / FCP_MERGE_UNIT_W);
   }
-  *out = p;
+  *out = owner.release();
   return FCP_OK;
+} catch (const std::bad_alloc&) {
+  return no_memory("fcp_plan_blocks");
 }
 
 extern "C" int fcp_span_mask_efficiency(int32_t length, const int32_t* spans, int32_t n_spans, double* eta) {

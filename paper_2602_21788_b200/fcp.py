@@ -15,7 +15,7 @@ LIB_PATH = os.path.join(_HERE, "libfcp.so")
 
 FCP_OK = 0
 FCP_ERR_INVALID_ARG, FCP_ERR_INFEASIBLE, FCP_ERR_UNSUPPORTED, FCP_ERR_WORKSPACE = -1, -2, -3, -4
-FCP_ERR_CUDA, FCP_ERR_TIMEOUT, FCP_ERR_NOT_UPLOADED = -5, -6, -7
+FCP_ERR_CUDA, FCP_ERR_TIMEOUT, FCP_ERR_NOT_UPLOADED, FCP_ERR_NO_MEMORY = -5, -6, -7, -8
 FCP_MAX_DEGREE = 64
 
 TABLES = dict(cu_seqlens=0, chunk_offset=1, chunk_bounds=2, pairs=3, items=4, slot_offset=5, slot_rows=6,

@@ -363,3 +363,25 @@ def test_short_sequences_at_high_degree_bit_exact_vs_oracle():
     lens, degs = rng.integers(1, 140, 60).tolist(), rng.integers(1, 65, 60).tolist()
     plan = fcp.fcp_plan_blocks(lens, degs, 4, 2, 64)
     _compare(plan, P.plan_blocks(lens, degs))
+
+
+def test_a_plan_that_the_memory_does_not_hold_is_refused_and_the_next_one_is_made():
+    # 8000 sequences of 128 tokens at degree 64: 66 million pairs of 24 bytes.  43 million sequences for the search: its two result
+    # arrays fit, an array of its own does not.  Then a batch that fits.
+    code = _IN_BOUNDED_SPACE.replace("plan = fcp.Plan([length] * n, [degree] * n, 1, 1, 64)", """
+for call in (lambda: fcp.Plan([length] * n, [degree] * n, 1, 1, 64),
+             lambda: fcp.Plan([length] * n, [degree] * n, 1, 1, 64, spans=[[(0, length)]] * n),
+             lambda: fcp.fcp_plan_strategy(ones, 64, 5e7, 1.0, 0.0, dict(alpha1=1, alpha2=1, alpha3=1, beta1=0, beta2=0, v=1))):
+    try:
+        call()
+        print("made")
+    except fcp.FcpError as e:
+        print(e.status, "memory" in str(e))
+plan = fcp.Plan([300, 5], [3, 2], 1, 1, 64)
+""").replace("fcp.lib()", "import numpy as np; ones = np.ones(43000000, np.int32); fcp.lib()")
+    r = subprocess.run([sys.executable, "-c", code, str(400 << 20), "8000", "128", "64"], cwd=ROOT, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, (r.returncode, r.stderr[-500:])
+    assert r.stdout.splitlines()[:3] == [f"{fcp.FCP_ERR_NO_MEMORY} True"] * 3
+    assert r.stdout.split()[-3:] == [str(fcp.Plan([300, 5], [3, 2], 1, 1, 64).info(k)) for k in ("n_pairs", "n_fused_units", "n_bwd_units")]
+    assert fcp.status_string(fcp.FCP_ERR_NO_MEMORY) == "FCP_ERR_NO_MEMORY"
