@@ -558,10 +558,10 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           uint32_t x0[32], x1[32];
           float2 l0[4], l1[4];
           load(x0, l0, t_s, s_lse, 0);
-          tc_wait_ld();
+          tc_wait_ld(x0);
           load(x1, l1, t_s, s_lse, 1);
           probs(x0, l0, pa, 0);
-          tc_wait_ld();
+          tc_wait_ld(x1);
           probs(x1, l1, pb, 1);
         } else {
 #pragma unroll 1
@@ -571,7 +571,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             load(x, l2, t_s, s_lse, c);
 #pragma unroll
             for (int j = 0; j < 16; ++j) pa[j] = pb[j];
-            tc_wait_ld();
+            tc_wait_ld(x);
             probs(x, l2, pb, c);
           }
         }
@@ -588,10 +588,10 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           uint32_t x0[32], x1[32];
           float2 d0[4], d1[4];
           load(x0, d0, t_dp, s_delta, 0);
-          tc_wait_ld();
+          tc_wait_ld(x0);
           load(x1, d1, t_dp, s_delta, 1);
           grads(x0, d0, pa, 0);
-          tc_wait_ld();
+          tc_wait_ld(x1);
           grads(x1, d1, pb, 1);
         } else {
 #pragma unroll 1
@@ -599,7 +599,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             uint32_t x[32];
             float2 d2[4];
             load(x, d2, t_dp, s_delta, c);
-            tc_wait_ld();
+            tc_wait_ld(x);
             grads(x, d2, pa, c);
 #pragma unroll
             for (int j = 0; j < 16; ++j) pa[j] = pb[j];
@@ -637,7 +637,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         uint32_t qv[D];
 #pragma unroll
         for (int c = 0; c < D / 32; ++c) tmem_ld32(t_dq + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&qv[c * 32]));
-        tc_wait_ld();
+        tc_wait_ld(qv);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(BAR(B_DQEMPTY));
@@ -674,7 +674,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         for (int c = 0; c < D / 16; ++c) {
           uint32_t av[16];
           tmem_ld16(t_acc + c * 16, av);
-          tc_wait_ld();
+          tc_wait_ld(av);
           if (row < kv_rows) {
 #pragma unroll
             for (int i = 0; i < 16; i += 8) {

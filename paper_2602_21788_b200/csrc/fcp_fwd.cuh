@@ -403,7 +403,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll 1
         for (int b = 0; b < blocks; ++b) {
           tmem_ld32(t_s + 32 * b, x);
-          tc_wait_ld();
+          tc_wait_ld(x);
 #pragma unroll
           for (int i = 0; i < 32; ++i)
             if (b * 32 + i < limit) mx = fmaxf(mx, __uint_as_float(x[i]));
@@ -417,7 +417,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         for (int b = 0; b < 4; ++b) {
           if (b < blocks) {
             tmem_ld32(t_s + 32 * b, x);
-            tc_wait_ld();
+            tc_wait_ld(x);
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
               const float s0 = b * 32 + 2 * i < limit ? __uint_as_float(x[2 * i]) : -INFINITY;
@@ -461,7 +461,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         uint32_t sv[4][32];
 #pragma unroll
         for (int b = 0; b < 4; ++b) tmem_ld32(t_s + 32 * b, sv[b]);
-        tc_wait_ld();
+        tc_wait_ld(*reinterpret_cast<uint32_t(*)[128]>(sv));
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(BAR(B_SFREE + sb));
@@ -501,7 +501,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             for (int c = 0; c < D / 16; ++c) {
               uint32_t ov[16];
               tmem_ld16(t_o + c * 16, ov);
-              tc_wait_ld();
+              tc_wait_ld(ov);
 #pragma unroll
               for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * f);
               tmem_st16(t_o + c * 16, ov);
@@ -599,7 +599,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           for (int c = 0; c < D / 32; ++c) {
             uint32_t ov[32];
             tmem_ld32(t_o + c * 32, ov);
-            tc_wait_ld();
+            tc_wait_ld(ov);
             if (row < rows_s) {
 #pragma unroll
               for (int i = 0; i < 32; i += 8)
@@ -617,7 +617,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             for (int c = 0; c < D / 32; ++c) {
               uint32_t ov[32];
               tmem_ld32(t_o + c * 32, ov);
-              tc_wait_ld();
+              tc_wait_ld(ov);
               if (row < rows_s) {
 #pragma unroll
                 for (int i = 0; i < 32; i += 4)
@@ -634,7 +634,7 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           for (int c = 0; c < D / 32; ++c) {
             uint32_t ov[32];
             tmem_ld32(t_o + c * 32, ov);
-            tc_wait_ld();
+            tc_wait_ld(ov);
             if (row < rows_s) {
 #pragma unroll
               for (int i = 0; i < 32; i += 4)

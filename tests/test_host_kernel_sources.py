@@ -41,3 +41,14 @@ def test_the_rule_sees_the_kernels():
     code = "".join(_code(f) for f in FILES)
     assert len(re.findall(r"__global__[^;{]*?\bfcp_\w+\(([^{;]*)\)\s*\{", code, flags=re.S)) == 6
     assert code.count("__ldg(") > 20
+
+
+@pytest.mark.parametrize("name", FILES)
+def test_the_wait_for_tensor_memory_loads_names_the_registers_they_fill(name):
+    """A load from tensor memory fills its registers until the wait behind it, but to the compiler it has written them at once: only
+    what passes through the wait is sure to be used behind it."""
+    code = _code(name)
+    assert not re.findall(r"tc_wait_ld\(\s*\)", code)
+    waited = set(re.findall(r"\b(\w+)\)*\s*\)\s*;", " ".join(re.findall(r"tc_wait_ld\([^;]*\);", code))))
+    filled = set(re.findall(r"tmem_ld(?:32|16)\([^;]*?(?:, |&)(\w+)(?:\[[^;]*)?\)+;", code)) | set(re.findall(r"\bload\((\w+),", code))
+    assert filled <= waited, filled - waited
