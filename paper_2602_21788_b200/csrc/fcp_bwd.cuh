@@ -21,15 +21,20 @@
 //
 // Work items are handed out through a global counter in the order of the plan's work groups.
 //
-// What bounds it (D = 128): about 3880 clk per 128 x 128 tile and head (tensor pipe 66 % busy, one 128K sequence among short
-// ones, 5 heads), of which the five products need 2570 when they run alone (514-517 clk each).  S^T | dP^T | dV | dK fill the 512 columns of tensor memory, so there is no second tile in
-// flight behind which the hand-overs of P^T, dS^T and the drained dQ could hide.  The shared-memory data pipe is nearly as
-// full: 2310 wavefronts of operands and 1610 of the other warps per tile (counted before the statistics were written ahead, at 4360 clk).
-// Left out one by one on a 64K-token batch (19.4 ms): bulk reductions 17.1 ms, staging stores 18.7, exponentials 19.3.
-// The bulk reductions took the period from 5090 to 4412 clk, what followed to 3880; under the power cap the clock falls
-// meanwhile, so that the time goes down less.  Kernel with all of it, before -> now: 128K bimodal batch
-// 102 -> 92 ms, 64K log-normal batch 12.9 -> 11.2 ms, 8K batch 405 -> 243 us (there the work order counts most).
-// The math loops stay rolled: unrolling their trips costs 3-7 %.
+// What bounds it (D = 128): 3820 clk per 128 x 128 tile and head (tensor pipe 67 % busy, one 128K sequence among short
+// ones, 5 heads), of which the five products need 2570 when they run alone (514-517 clk each).  S^T | dP^T | dV | dK fill the
+// 512 columns of tensor memory, so there is no second tile in flight behind which the hand-overs of P^T, dS^T and the drained
+// dQ could hide.  A timestamp trace (16K tokens, one sequence) shows the chain in the math warps: S^T seen to P^T handed over
+// 1720 clk, to dP^T seen 580-690, to dS^T handed over 1100, to the next S^T 400.  The shared-memory data pipe is nearly as
+// full: 2310 wavefronts of operands and 1610 of the other warps per tile (counted when the period was 4360 clk).
+// Left out one by one when a 64K-token batch took 19.4 ms: bulk reductions 17.1 ms, staging stores 18.7, exponentials 19.3.
+// The bulk reductions took the period from 5090 to 4412 clk, what followed to 3820; under the power cap the clock falls
+// meanwhile, so that the time goes down less.  Scalar reductions -> now: 128K bimodal batch 102 -> 88 ms, 64K log-normal
+// batch 12.9 -> 11.2 ms.
+// D = 64: the same chain, 1490, 150, 820 and 400 clk, 2860 in all (3070 over a launch of 20 000 tokens, 12/4 heads), against 1280 of
+// products and 1024 of exponentials; T2 of the next tile waits for the dQ tile, which lies over its dP^T, but the math warps are not
+// behind it: dP^T is there 150 clk after they hand over P^T.
+// At D = 128 the math loops stay rolled: unrolling their trips costs 3-7 %.
 #pragma once
 #include "fcp_plan.hpp"
 #include "sm100_ptx.cuh"
@@ -250,66 +255,66 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   };
 
   if (warp < 4) {
-    // registers per thread: control 88, math 128, drain 168 (80 / 128 / 176 spilled in the issuing thread: kernel +2 %)
-    // (D = 64, whose math warps hold two loads: control 72, math 136)
+    // registers per thread: control 88, math 128, drain 168; D = 64, whose math warps hold two loads: control 72, math 136.  A
+    // drain thread holds a dQ row.  (None of 80 / 128 / 176, 72 / 128 / 184 and 80 / 136 / 160 spills at D = 128 either.)
     if constexpr (D == 64) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     else asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
     // (warp branches outside the lane branches: behind a divergent one the compiler takes the issuer's operands for divergent)
     if (warp == 0) {
       if (lane == 0) {
-      // ------------------------------------------------------------------ TMA producer + scheduler
-      uint32_t n = 0, it = 0;
-      bool ok = true;
-      WorkOrder order;
-      while (ok) {
-        const int w = atomicAdd(a.counter, 1);
-        const uint32_t slot = n & 1;
-        ok = mbar_wait(BAR(B_WEMPTY + slot), ((n >> 1) & 1) ^ 1, wctx, 112);
-        if (!ok) break;
-        const bool last = w >= a.n_work;
-        int unit = -1, hk = 0;
-        if (!last) {
-          order.locate(a.groups, w, a.n_heads, 1, unit, hk);
-          unit = __ldg(a.work + unit);
-          hk += a.hk_begin;
-        }
-        work_ring[2 * slot] = unit;
-        work_ring[2 * slot + 1] = hk;
-        mbar_arrive(BAR(B_WFULL + slot));     // release: the two stores above are visible to the waiters
-        if (last) {
-          grid_launch_next();
-          break;
-        }
-        const int32_t* U = a.units + (size_t)unit * FCP_BWD_UNIT_W;
-        const int kv_row0 = __ldg(U + BU_KV_ROW0);
-        ok = mbar_wait(BAR(B_KVFREE), (n & 1) ^ 1, wctx, 110);
-        ++n;
-        if (!ok) break;
-        mbar_expect_tx(BAR(B_KVFULL), 2 * SM::TILE_BYTES);
-#pragma unroll 1
-        for (int kb = 0; kb < KBLK; ++kb) {
-          tma_load_3d(sbase + SM::K_OFF + kb * BLK_BYTES, &tm_k, BAR(B_KVFULL), kb * 64, hk, kv_row0);
-          tma_load_3d(sbase + SM::V_OFF + kb * BLK_BYTES, &tm_v, BAR(B_KVFULL), kb * 64, hk, kv_row0);
-        }
-        BwdIter iter;
-#pragma unroll 1
-        for (iter.init(U, a.qranges, g); iter.valid; iter.advance(), ++it) {
-          const uint32_t st = it % BWD_Q_STAGES, sd = it % DO_STAGES;
-          const int h = hk * g + iter.hh;
-          ok = mbar_wait(BAR(B_QFREE + st), ((it / BWD_Q_STAGES) & 1) ^ 1, wctx, 111);
+        // ------------------------------------------------------------------ TMA producer + scheduler
+        uint32_t n = 0, it = 0;
+        bool ok = true;
+        WorkOrder order;
+        while (ok) {
+          const int w = atomicAdd(a.counter, 1);
+          const uint32_t slot = n & 1;
+          ok = mbar_wait(BAR(B_WEMPTY + slot), ((n >> 1) & 1) ^ 1, wctx, 112);
           if (!ok) break;
-          mbar_expect_tx(BAR(B_QFULL + st), SM::TILE_BYTES);
-#pragma unroll 1
-          for (int kb = 0; kb < KBLK; ++kb)
-            tma_load_3d(sbase + SM::Q_OFF + st * SM::TILE_BYTES + kb * BLK_BYTES, &tm_q, BAR(B_QFULL + st), kb * 64, h, iter.q_row);
-          ok = mbar_wait(BAR(B_DOFREE + sd), ((it / DO_STAGES) & 1) ^ 1, wctx, 113);
+          const bool last = w >= a.n_work;
+          int unit = -1, hk = 0;
+          if (!last) {
+            order.locate(a.groups, w, a.n_heads, 1, unit, hk);
+            unit = __ldg(a.work + unit);
+            hk += a.hk_begin;
+          }
+          work_ring[2 * slot] = unit;
+          work_ring[2 * slot + 1] = hk;
+          mbar_arrive(BAR(B_WFULL + slot));     // release: the two stores above are visible to the waiters
+          if (last) {
+            grid_launch_next();
+            break;
+          }
+          const int32_t* U = a.units + (size_t)unit * FCP_BWD_UNIT_W;
+          const int kv_row0 = __ldg(U + BU_KV_ROW0);
+          ok = mbar_wait(BAR(B_KVFREE), (n & 1) ^ 1, wctx, 110);
+          ++n;
           if (!ok) break;
-          mbar_expect_tx(BAR(B_DOFULL + sd), SM::TILE_BYTES);
+          mbar_expect_tx(BAR(B_KVFULL), 2 * SM::TILE_BYTES);
 #pragma unroll 1
-          for (int kb = 0; kb < KBLK; ++kb)
-            tma_load_3d(sbase + SM::DO_OFF + sd * SM::TILE_BYTES + kb * BLK_BYTES, &tm_do, BAR(B_DOFULL + sd), kb * 64, h, iter.q_row);
+          for (int kb = 0; kb < KBLK; ++kb) {
+            tma_load_3d(sbase + SM::K_OFF + kb * BLK_BYTES, &tm_k, BAR(B_KVFULL), kb * 64, hk, kv_row0);
+            tma_load_3d(sbase + SM::V_OFF + kb * BLK_BYTES, &tm_v, BAR(B_KVFULL), kb * 64, hk, kv_row0);
+          }
+          BwdIter iter;
+#pragma unroll 1
+          for (iter.init(U, a.qranges, g); iter.valid; iter.advance(), ++it) {
+            const uint32_t st = it % BWD_Q_STAGES, sd = it % DO_STAGES;
+            const int h = hk * g + iter.hh;
+            ok = mbar_wait(BAR(B_QFREE + st), ((it / BWD_Q_STAGES) & 1) ^ 1, wctx, 111);
+            if (!ok) break;
+            mbar_expect_tx(BAR(B_QFULL + st), SM::TILE_BYTES);
+#pragma unroll 1
+            for (int kb = 0; kb < KBLK; ++kb)
+              tma_load_3d(sbase + SM::Q_OFF + st * SM::TILE_BYTES + kb * BLK_BYTES, &tm_q, BAR(B_QFULL + st), kb * 64, h, iter.q_row);
+            ok = mbar_wait(BAR(B_DOFREE + sd), ((it / DO_STAGES) & 1) ^ 1, wctx, 113);
+            if (!ok) break;
+            mbar_expect_tx(BAR(B_DOFULL + sd), SM::TILE_BYTES);
+#pragma unroll 1
+            for (int kb = 0; kb < KBLK; ++kb)
+              tma_load_3d(sbase + SM::DO_OFF + sd * SM::TILE_BYTES + kb * BLK_BYTES, &tm_do, BAR(B_DOFULL + sd), kb * 64, h, iter.q_row);
+          }
         }
-      }
       }
     } else if (warp == 1) {
       // ------------------------------------------------------------------ UMMA issuer
@@ -550,7 +555,7 @@ fcp_bwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         };
         // D = 128: rolled, the pair arrays rotate between the passes (register arrays cannot be indexed by the pass), which halves
         // the code of this loop.  D = 64, where the products are half as long and the clock is not held down by the power: the
-        // second pass is loaded while the first is worked on, 8 x 3000 tokens of 12/4 heads 340 -> 332 us, 20 000 tokens 1670 -> 1615;
+        // second pass is loaded while the first is worked on, 8 x 3000 tokens of 12/4 heads 345 -> 338 us, 20 000 tokens 1658 -> 1619;
         // at D = 128 that way 64K tokens of 32/8 heads 12.24 -> 12.37 ms.
         constexpr bool AHEAD = D == 64;
         uint32_t pa[16], pb[16] = {};

@@ -14,12 +14,12 @@
 // turn) | P0 | P1 | O0 | O1; D = 64 has room for a score buffer per Q tile.  The two Q tiles share every K/V tile.
 //
 // What bounds it: per K/V tile the two Q tiles need 2048 clk of UMMA time and 2048 clk of the MUFU (one warp per
-// scheduler and tile, 8 clk per warp-wide ex2); a timestamp trace (D = 128) shows a period of 2860 clk: scores seen to
-// loaded 136, maximum 367, exponentials 1415, wait for the free P 200, store and hand over 124, wait for the next
-// scores 613; without the trace it is about 2670 (tensor pipe 77 % busy, MUFU 77 %).  With P over its own S (each tile's next scores behind the product that consumes P, the groups taking
-// turns at the exponentials) the period was 4200 clk.  Long launches run under the power cap, where a third fewer
-// cycles give 13 to 16 % of the time, before -> now: one 128K sequence among short ones 167 -> 141 ms, 128K bimodal
-// batch 37.2 -> 32 ms, 64K log-normal batch 4.54 -> 3.95 ms, D = 64 ragged 16K batch 112 -> 89 us.
+// scheduler and tile, 8 clk per warp-wide ex2); counted over a launch (D = 128, one 128K sequence among short ones) it is 2535 clk, tensor
+// pipe and MUFU 81 % busy each.  A timestamp trace shows 2700: scores seen to loaded 160, maximum 270, exponentials 1570, wait for
+// the free P 190, store and hand over 140, wait for the next scores 370.  With P over its own S (each tile's next scores behind the
+// product that consumes P, the groups taking turns at the exponentials) the period was 4200 clk.  Long launches run under the
+// power cap, where two fifths fewer cycles gave 12 to 24 % of the time, that version -> now: one 128K sequence among short ones
+// 167 -> 139 ms, 128K bimodal batch 37.2 -> 30 ms, 64K log-normal batch 4.54 -> 4.0 ms, D = 64 ragged 16K batch 112 -> 85 us.
 //
 // Registers are moved between the warp groups at start-up: a softmax thread holds a full row of S
 // (128 values), reads it from TMEM once, and needs no exchange with another thread for the row

@@ -94,7 +94,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Non-blocking look at a barrier phase.  An issuing thread sends this ahead of a batch of UMMAs for
+// Non-blocking look at a barrier phase.  An issuing warp sends this ahead of a batch of UMMAs for
 // the barrier it will need after the batch: the answer travels while the batch is issued, and the
 // blocking wait (whose round trip through a busy memory pipe costs hundreds of clocks even when the
 // phase completed long ago) is skipped if it was already there.
@@ -233,10 +233,12 @@ __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sy
 
 // Products and commits are issued by a whole, converged warp, of which one elected lane (always the same) sends the
 // instruction.  In code that only one lane runs the compiler cannot keep the operands in uniform registers, and the moves in
-// front of every UMMA took 55-90 clk, where one of 128 x 128 x 16 executes in 64.  One election per product: one per UMMA is
-// a quarter more code for the whole kernel, which the instruction cache pays for.  One lane -> elected, us: forward, 16 x 2048
-// tokens of 32/8 heads 544 -> 518, 12 x 700 86 -> 80, 60 000 tokens of 8 heads 5070 -> 4930; backward, D = 64, 8 x 3000 tokens of
-// 12/4 heads 398 -> 346; D = 128 1312 -> 1290, 168 -> 162, 17470 -> 17460 (the power cap).
+// front of every UMMA took 55-90 clk, where one of 128 x 128 x 16 executes in 64.  One election per run of UMMAs (the backward
+// kernel looks at a barrier between the two runs of a product) and per commit: one per UMMA is a quarter more code for the
+// whole kernel, which the instruction cache pays for.  One lane -> elected, us: forward, 16 x 2048 tokens of 32/8 heads 544 -> 518,
+// 12 x 700 86 -> 80, 60 000 tokens of 8 heads 5070 -> 4930; backward, D = 64, 8 x 3000 tokens of 12/4 heads 398 -> 370, and 346 with
+// the branches on the warp in front of those on the lane and the statistics read before the wait for tensor memory; all three at
+// D = 128, the same batches as forward: 1312 -> 1290, 168 -> 162, 17470 -> 17460 (the power cap).
 __device__ __forceinline__ bool elect_one() {
   uint32_t x;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(x));
