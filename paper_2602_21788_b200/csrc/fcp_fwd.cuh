@@ -389,8 +389,8 @@ fcp_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       bool s_ready = false;                      // the next step's scores were there at the last look (D = 64)
       float2 l01 = make_float2(0.f, 0.f), l23 = make_float2(0.f, 0.f);
       // An item of at most 64 keys has one or two blocks of 32 columns instead of four, taken in rolled passes over TMEM: the same
-      // operations in the same order as below, where the other columns add zeros.  1841 sequences of 12 tokens, D = 64: 118 us
-      // like this, 164 without; 1159 of them, D = 128: 171, 211.  (In front of the loop at D = 64 and behind it at D = 128,
+      // operations in the same order as below, where the other columns add zeros.  1841 sequences of 12 tokens, D = 64: 111 us
+      // like this, 142 without; 1159 of them, D = 128: 162, 169.  (In front of the loop at D = 64 and behind it at D = 128,
       // because the other way round the loop itself is 1.5 % slower.)
       const bool few = nts == 1 && __ldg(U + FU_KV0_END) - ks <= 64;
       auto few_keys = [&]() -> bool {

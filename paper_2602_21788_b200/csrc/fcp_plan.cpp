@@ -282,9 +282,9 @@ void order_units(const std::vector<int32_t>& seq, const std::vector<int32_t>& co
 // own take a quarter less time, because a tile alone does not wait for the other one's turn in the MUFU and the tensor core;
 // but with more than half as many units as SMs some SMs get a second item, which starts late, and the empty half of a unit
 // with one tile holds up what comes behind it too.  Measured, whole against split (kernel, us; n units of sequences of L tokens):
-//   D = 64:  L = 256, n = 74: 14.4, 13.8; n = 80: 14.4, 16.5; n = 144: 15.3, 19.2     L = 512, n = 80: equal; n = 144: 17.1, 21.0
-//            L = 1024, n = 112: 23.1, 22.3; n = 144: 23.8, 25.1                       L = 2048, n = 144: 36.5, 33.3
-//   D = 128: L = 256, n = 80: 14.9, 17.7; L = 1024, n = 112: 25.4, 23.8; n = 144: 25.4, 27.3; L = 2048, n = 144: 37.4, 36.2
+//   D = 64:  L = 256, n = 74: 13.1, 12.8; n = 80: 13.2, 16.7; n = 144: 14.5, 17.7     L = 512, n = 80: equal; n = 144: 16.8, 18.9
+//            L = 1024, n = 112: 23.0, 20.9; n = 144: 23.0, 23.1                       L = 2048, n = 144: 35.7, 32.2
+//   D = 128: L = 256, n = 80: 14.8, 17.3; L = 1024, n = 112: 24.2, 22.9; n = 144: 24.8, 25.5; L = 2048, n = 144: 35.3, 34.8
 // So both launches are played through, in quarters of the time of one key tile of a Q tile alone: a tile 4, a second item 12
 // more (8 behind an empty half), a whole unit of two tiles 5 per key tile of the longer one and 6.  Over 224 measured lists of
 // equal and unequal units this takes the slower launch, by over 3 %, once; always splitting does 62 times, by up to 30 %.
